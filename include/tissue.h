@@ -229,10 +229,15 @@ typedef struct {
  * 256 < V <= 1024, 16 lanes, 2 warps per block and the recompute layout
  * above 2128 cells, else 32 lanes and 2 warps, prefix layout (the recompute
  * layout holds more cells per SM; the thresholds are one wave of the prefix
- * launch on a 152-SM GB300).  A recompute launch with more voxels per block
- * than lanes that the tissue's model cannot take (the promoter model, a
- * trace) runs the prefix launch of its cell size instead; results never
- * depend on it. */
+ * launch on a 152-SM GB300).  While the shape is one of these defaults, for
+ * whatever number of cells, the library may run the step with its sum-tree
+ * kernel instead, in a form that fits the number of cells; it uses up to
+ * 1.4 GB of device memory for the length of a call, and keeps to the shape
+ * when that cannot be had, while a trace is on, and in a stream capture that
+ * would need it.  Another shape is run as it is.  A recompute launch with
+ * more voxels per block than lanes that the tissue's model cannot take (the
+ * promoter model, a trace) runs the prefix launch of its cell size instead;
+ * results never depend on any of it. */
 int tissue_set_launch_config(tissue* t, const tissue_launch* config);
 int tissue_get_launch_config(const tissue* t, tissue_launch* config);
 
@@ -259,7 +264,9 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
  * layout, which also needs V <= lanes^2, or for a Notch-Delta class 16 lanes
  * and V <= 1024 or 8 lanes and V <= 256), shared-memory layout
  * TISSUE_LAYOUT_*.  The default is
- * the single-tissue default for that V.  Results never depend on it. */
+ * the single-tissue default for that V, and a default shape leaves the kernel
+ * to the library as for a single tissue (a batch holds the memory its sum-tree
+ * launches need while it exists).  Results never depend on it. */
 int tissue_batch_set_class_launch(tissue_batch* b, uint32_t V, uint32_t lanes_per_cell,
                                   uint32_t warps_per_block, uint32_t smem_layout);
 

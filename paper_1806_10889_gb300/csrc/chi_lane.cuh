@@ -1,0 +1,853 @@
+// K_chi, sum-tree form: the intracellular module chi (arXiv 1806.10889,
+// Sec. II-A1) over a work list of cells, G = 1..32 lanes of a warp per cell.
+//
+// Every cell keeps a tree of propensity sums, four children per node: the
+// voxel totals are the leaves, S_{LV-1}[q] the total of the four voxels of
+// quad q, S_l[i] that of four entries of S_{l+1}; S_1 has four entries.  An
+// event descends from the root in the direct method's voxel-major order,
+// finds the channel inside the voxel in closed form, changes one or two
+// voxels and adds the two differences along their paths: 350 to 500
+// instructions of one lane, with nothing in them to share out over lanes.  The
+// segmented kernel (chi_seg.cuh) finds a voxel with ballots and scans over 8
+// to 32 lanes, and its event loop (600 to 900 instructions) serves one to four
+// cells; here an instruction serves up to 32 (G = 1).
+//
+// What the G lanes of a cell share out is the work that does not depend on
+// the state: lane j of the cell draws the random numbers of event j of the
+// next G (about 360 instructions), and computes its waiting time (120).  The
+// waiting time only decides where the cell stops.  So the G events are applied
+// first, the total propensity A before each kept by its lane, then all G
+// waiting times are computed at once and added in order; the events past the
+// end of the step are undone (at most G a cell and step, on the counts only:
+// the sums are not used again).  The updates of the sums are shared out too,
+// an entry to a lane.
+//
+// Bound (one GB300, from ncu): few cells by the event chain -- one warp alone
+// issues every 3.6 cycles, 1,320 cycles an event with G = 32 (2,530 in the
+// segmented kernel); cells of up to 256 voxels that fill the chip by issue
+// (32 warp instructions per event with G = 1 against 171 and 227, 8x8 and
+// 16x16 voxels); larger ones by random accesses to L2 and DRAM (a dependent
+// 64-byte read and write per lane reaches 25 G/s in DRAM, 42 G/s in L2, and an
+// event makes about three).  Chi ms per step, before -> with this kernel: 2x2
+// cells of 8x8 voxels 2.9 -> 1.53, 64x64 of 16x16 21.1 -> 10.4, 48x48 of 32x32
+// 77.5 -> 52.9, 256x256 of 8x8 33.4 -> 7.9, 256x256 of 32x32 611 -> 187.
+//
+// Template parameters: MODEL 0 Notch-Delta without in-voxel binding (k_in =
+// k_off = 0), 1 Notch-Delta, 2 promoter; LV the levels of the tree (V <= 4^LV,
+// LV = 3, 4, 5); LEAF where the voxels live (chi_lane.h): in shared memory
+// (20 bytes a voxel and the sums: the shortest chain), or in a scratch array,
+// total and packed counts side by side so that a quad is one aligned 64-byte
+// block (about a hundred bytes to 2.8 KB of sums a cell stay in shared memory,
+// and hundreds of cells fit on an SM); ONE: G = 1 at compile time.
+//
+// Limits.  Counts below the tissue's `small` keep every total below 2^52
+// unchecked, and R below kLaneHill reads the Hill table unchecked.  With
+// shared leaves a cell past either goes on with exact checks; a packed cell
+// (20 bits a count) is left untouched and goes to the redo list, which the
+// launcher runs through the segmented kernel from the same state and random
+// streams.
+#pragma once
+#include "chi_lane.h"
+#include "tissue_dev.cuh"
+
+namespace tsg {
+
+namespace {
+
+// Rates of the cell a lane runs, in registers.
+template <int MODEL>
+struct LaneRates {
+  uint64_t hD, hN, hR, gD, gN, gR, kN;  // promoter: kN unused
+  uint64_t k_in, k_off, tD, kd;         // MODEL 1: k_in, k_off; MODEL 2: k_in (k_a), tD, kd
+  const uint64_t* hill;
+  uint32_t small;
+  __device__ __forceinline__ void load(const QRates& q) {
+    hD = q.hopD;
+    hN = q.hopN;
+    hR = q.hopR;
+    gD = q.gD;
+    gN = q.gN;
+    gR = q.gR;
+    kN = q.kN;
+    k_in = MODEL ? q.k_in : 0ull;
+    k_off = MODEL == 1 ? q.k_off : 0ull;
+    tD = MODEL == 2 ? q.tD : 0ull;
+    kd = MODEL == 2 ? q.kd : 0ull;
+    hill = q.hill;
+    small = q.small;
+  }
+};
+
+// Hill(R) from the table; counts past it are computed (their view is read
+// from memory: never in a running tissue).
+__device__ __forceinline__ uint64_t lane_hill(const uint64_t* hill, const TissueView* tv,
+                                              uint32_t R) {
+  return R < kHillTab ? __ldg(hill + R) : hill_direct(tv->q, R);
+}
+
+// Total propensity of a voxel with nn neighbours, modulo 2^64 (exact while
+// the counts are below `small`; larger ones are checked by exact_ovf).
+template <int MODEL>
+__device__ __forceinline__ uint64_t lane_total(const LaneRates<MODEL>& q, const TissueView* tv,
+                                               uint32_t D, uint32_t N, uint32_t R, uint32_t nn,
+                                               bool centre) {
+  uint64_t a = (q.gD + q.hD * nn) * D + (q.gN + q.hN * nn) * N;
+  if (MODEL == 2) {
+    const uint32_t F = static_cast<uint32_t>(centre) - R;
+    a += q.tD * F + q.kd * R + q.k_in * (static_cast<uint64_t>(N) * F);
+  } else {
+    a += (q.gR + q.k_off + q.hR * nn) * R + lane_hill(q.hill, tv, R) + q.kN;
+    if (MODEL == 1) a += q.k_in * (static_cast<uint64_t>(D) * N);
+  }
+  return a;
+}
+
+// Whether a voxel's total (or one of its products) reaches 2^52, for a voxel
+// holding a count of `small` or more.
+template <int MODEL>
+__device__ __noinline__ bool exact_ovf(const TissueView* tv, uint32_t D, uint32_t N, uint32_t R,
+                                       uint32_t nn, bool centre) {
+  const QRates& q = tv->q;
+  if ((D | N | R) < q.small) return false;
+  uint64_t a, X;
+  if (MODEL == 2) {
+    const uint32_t F = static_cast<uint32_t>(centre) - R;
+    a = q.tD * F + q.kd * R;
+    X = static_cast<uint64_t>(N) * F;
+  } else {
+    a = hill_q(q, R) + q.kN;
+    X = static_cast<uint64_t>(D) * N;
+  }
+  bool ovf = false;
+  a += mul_lim(q.gD + q.hopD * nn, D, ovf);
+  a += mul_lim(q.gN + q.hopN * nn, N, ovf);
+  a += mul_lim(q.gR + q.hopR * nn, R, ovf);
+  a += mul_lim(q.k_in, X, ovf);
+  a += mul_lim(q.k_off, R, ovf);
+  return ovf || (a >> 52) != 0ull;
+}
+
+// Whether the event that changed v (and u) took a count past its maximum or
+// a total past its limit (shared leaves).
+template <int MODEL>
+__device__ __noinline__ bool past_limits(const TissueView* tv, const int32_t* cp, uint32_t ps,
+                                         const unsigned char* lut, uint32_t v, uint32_t u,
+                                         uint32_t centre) {
+  bool o = false;
+  for (int k = 0; k < 2; ++k) {
+    const uint32_t x = k ? u : v;
+    const uint32_t D = static_cast<uint32_t>(cp[x]), N = static_cast<uint32_t>(cp[ps + x]);
+    const uint32_t R = static_cast<uint32_t>(cp[2u * ps + x]);
+    o |= exact_ovf<MODEL>(tv, D, N, R, lut[x] >> 4, MODEL == 2 && x == centre);
+    o |= max(D, max(N, R)) > static_cast<uint32_t>(kCountMax);
+  }
+  return o;
+}
+
+// The child of a node that r falls into: k = the number of leading children
+// whose running sum is at most r; r becomes the remainder inside it.  WIDE
+// compares with the three running sums at once (the shorter chain, for few
+// warps); otherwise the half first, then the child in it (fewer instructions).
+template <bool WIDE>
+__device__ __forceinline__ uint32_t pick_child(uint64_t s0, uint64_t s1, uint64_t s2, uint64_t& r) {
+  const uint64_t p1 = s0 + s1;
+  if (WIDE) {
+    const uint64_t p2 = p1 + s2;
+    const bool c0 = r >= s0, c1 = r >= p1, c2 = r >= p2;
+    r -= c2 ? p2 : c1 ? p1 : c0 ? s0 : 0ull;
+    return c2 ? 3u : c1 ? 2u : c0 ? 1u : 0u;
+  }
+  const bool up = r >= p1;
+  r -= up ? p1 : 0ull;
+  const uint64_t t = up ? s2 : s0;
+  const bool second = r >= t;
+  r -= second ? t : 0ull;
+  return (up ? 2u : 0u) + (second ? 1u : 0u);
+}
+
+struct U64x4 {
+  uint64_t a, b, c, d;
+};
+
+// 32 bytes of the scratch array with one load.
+__device__ __forceinline__ U64x4 load4(const uint64_t* p) {
+  U64x4 r;
+  asm volatile("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(r.a), "=l"(r.b), "=l"(r.c), "=l"(r.d)
+               : "l"(p)
+               : "memory");
+  return r;
+}
+
+// A voxel of the scratch array in one word: D in bits 0..19, N in 20..39, R
+// in 40..59, the neighbour mask in 60..63.
+__device__ __forceinline__ uint64_t pack_voxel(uint32_t D, uint32_t N, uint32_t R, uint32_t mask) {
+  return D | (static_cast<uint64_t>(N) << 20) | (static_cast<uint64_t>(R | (mask << 20)) << 40);
+}
+__device__ __forceinline__ uint32_t word_D(uint64_t w) {
+  return static_cast<uint32_t>(w) & 0xFFFFFu;
+}
+__device__ __forceinline__ uint32_t word_N(uint64_t w) {
+  return static_cast<uint32_t>(w >> 20) & 0xFFFFFu;
+}
+__device__ __forceinline__ uint32_t word_R(uint64_t w) {
+  return static_cast<uint32_t>(w >> 40) & 0xFFFFFu;
+}
+__device__ __forceinline__ uint32_t word_mask(uint64_t w) {
+  return static_cast<uint32_t>(w >> 60);
+}
+// The change of a word by one molecule of species s.
+__device__ __forceinline__ uint64_t word_unit(uint32_t s) {
+  const uint32_t lo = s == 0u ? 1u : s == 1u ? 1u << 20 : 0u, hi = s == 2u ? 1u << 8 : 0u;
+  return (static_cast<uint64_t>(hi) << 32) | lo;
+}
+
+// First entry of level l of a four-ary tree whose levels follow one another:
+// (4^l - 4) / 3.
+__device__ __forceinline__ constexpr uint32_t level_off(uint32_t l) {
+  return (0x55555555u & ((1u << (2u * l)) - 1u)) - 1u;
+}
+
+// Event codes of the undo log.
+constexpr uint32_t kEvBind = 5u, kEvRelease = 6u, kEvHop = 8u;  // 0..4: channel; 8 + species: hop
+
+template <int MODEL, int LV, int LEAF, bool ONE>
+__global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ? 7 : 14) k_chi_lane(const LaneArgs p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  static_assert(!ONE || LEAF != kLeafShared, "one lane per cell: records or nodes");
+  constexpr bool REC = LEAF != kLeafShared;   // voxels in the scratch array, packed
+  constexpr bool NODE8 = LEAF == kLeafNodes;  // with the quads' sums, eight to a node
+  constexpr uint32_t NQ = 1u << (2 * (LV - 1));  // quads of a full tree
+  // levels kept in shared memory above the quads' sums (NODE8: 2, 8, 32
+  // entries), or down to them
+  constexpr int SL = NODE8 ? LV - 2 : LV - 1;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const uint32_t G = ONE ? 1u : p.G;
+  const uint32_t slot = ONE ? lane : lane / G, sl = ONE ? 0u : lane % G;
+  const uint32_t slots = ONE ? 32u : 32u / G;
+  const int base_lane = ONE ? lane : lane - static_cast<int>(sl);
+  const bool lead = sl == 0u;
+  const uint32_t V = p.V, n = p.n, nq = (V + 3u) >> 2;
+  const uint32_t ps = nq * 4u;  // distance between the planes of D, N and R (shared leaves)
+  const uint32_t centre = MODEL == 2 ? (n >> 1) * n + (n >> 1) : 0u;
+  const bool vec = (V & 3u) == 0u;
+
+  // offsets u - v of the m-th existing direction for each neighbour mask, then
+  // (shared leaves) the voxels' masks: bits 0..3, and their number: bits 4..6
+  int16_t* hop_off = reinterpret_cast<int16_t*>(smem);
+  unsigned char* lut = smem + 128;
+  for (uint32_t i = threadIdx.x; i < 64u; i += blockDim.x) {
+    uint32_t b = i >> 2;
+    for (uint32_t k = i & 3u; k > 0u; --k) b &= b - 1u;
+    const int d = __ffs(static_cast<int>(b)) - 1;
+    hop_off[i] = static_cast<int16_t>(d < 0    ? 0
+                                      : d == 0 ? -1
+                                      : d == 1 ? 1
+                                      : d == 2 ? -static_cast<int>(n)
+                                               : static_cast<int>(n));
+  }
+  for (uint32_t v = threadIdx.x; v < nq * 4u; v += blockDim.x) {
+    const uint32_t vy = v / n, vx = v - vy * n;
+    const uint32_t m = static_cast<uint32_t>(vx > 0) | (static_cast<uint32_t>(vx < n - 1) << 1) |
+                       (static_cast<uint32_t>(vy > 0) << 2) |
+                       (static_cast<uint32_t>(vy < n - 1) << 3);
+    lut[v] = static_cast<unsigned char>(m | (__popc(m) << 4));
+  }
+  __syncthreads();
+
+  // A cell's shared memory: the rates {g, h} of D, N and R, the sums, and with
+  // shared leaves the voxel totals (the tree's last level) and the counts.
+  unsigned char* warp_cells =
+      smem + p.lut_bytes + static_cast<size_t>(wib) * slots * p.cell_stride;
+  unsigned char* cs = warp_cells + slot * p.cell_stride;
+  const ulonglong2* rates = reinterpret_cast<const ulonglong2*>(cs);
+  uint64_t* tree = reinterpret_cast<uint64_t*>(cs + 48);
+  constexpr uint32_t kCnt = level_off(LV);  // shared leaves: entry of the voxel totals
+  int32_t* cp = reinterpret_cast<int32_t*>(tree + kCnt + ps);
+  // a cell's scratch: NODE8 its quad sums, 256 of them; then 2 words per voxel,
+  // its total and its counts
+  constexpr uint32_t kNodeWords = NODE8 ? 256u : 0u;
+  const uint32_t rec_words = kNodeWords + 8u * nq;
+  uint64_t* warp_rec =
+      REC ? p.scratch + (static_cast<size_t>(blockIdx.x) * (blockDim.x >> 5) + wib) * slots * rec_words
+          : nullptr;
+  uint64_t* rec = warp_rec + static_cast<size_t>(slot) * rec_words;
+
+  LaneRates<MODEL> q{};
+  const TissueView* tv = p.views + (p.items ? p.items[0].x : 0u);
+  q.hill = tv->q.hill;
+  bool have = false, done = false;
+  uint32_t cell = 0, vidx = 0, step = 0, word3 = 0, key0 = 0, key1 = 0, e0 = 0;
+  uint64_t A = 0, over_mask = 0;
+  double tnow = 0.0;
+  int err = 0;
+  uint32_t lim = 0;
+  bool big = false;  // shared leaves: the cell holds, or held, a D or N of `small` or an R of
+                     // `lim` or more
+
+  for (;;) {
+    // ---- slots without a cell take the next work items, one after another --
+    unsigned want = __ballot_sync(kFull, !have && !done && lead);
+    while (want) {
+      const int src = __ffs(want) - 1;
+      want &= want - 1u;
+      const uint32_t sc = ONE ? static_cast<uint32_t>(src) : static_cast<uint32_t>(src) / G;
+      uint32_t it = 0;
+      if (lane == src) it = atomicAdd(p.counter, 1u);
+      it = __shfl_sync(kFull, it, src);
+      if (it >= p.n_items) {
+        if (slot == sc) done = true;
+        continue;
+      }
+      const uint2 w = p.items ? p.items[it] : make_uint2(0u, it);
+      const TissueView* ntv = p.views + w.x;
+      LaneRates<MODEL> nr;
+      nr.load(ntv->q);
+      const int32_t* g = ntv->counts + static_cast<size_t>(w.y) * 3u * V;
+      unsigned char* ncs = warp_cells + sc * p.cell_stride;
+      uint64_t* ntree = reinterpret_cast<uint64_t*>(ncs + 48);
+      int32_t* ncp = reinterpret_cast<int32_t*>(ntree + kCnt + ps);
+      uint64_t* nrec = warp_rec + static_cast<size_t>(sc) * rec_words;
+      if (lane < 3)
+        reinterpret_cast<ulonglong2*>(ncs)[lane] =
+            lane == 0   ? make_ulonglong2(nr.gD, nr.hD)
+            : lane == 1 ? make_ulonglong2(nr.gN, nr.hN)
+                        : make_ulonglong2(nr.gR + (MODEL == 1 ? nr.k_off : 0ull), nr.hR);
+      bool ovf = false, bad_state = false, nbig = false;
+      uint64_t total = 0, pair = 0;
+      for (uint32_t k = 0; k < (NQ + 31u) / 32u; ++k) {
+        const uint32_t qi = static_cast<uint32_t>(lane) + 32u * k;
+        uint64_t S = 0;
+        if (qi < nq) {
+          uint32_t d[4] = {0, 0, 0, 0}, m[4] = {0, 0, 0, 0}, r[4] = {0, 0, 0, 0};
+          if (vec) {
+            const uint4 x = reinterpret_cast<const uint4*>(g)[qi];
+            const uint4 y = reinterpret_cast<const uint4*>(g + V)[qi];
+            const uint4 z = reinterpret_cast<const uint4*>(g + 2u * V)[qi];
+            d[0] = x.x, d[1] = x.y, d[2] = x.z, d[3] = x.w;
+            m[0] = y.x, m[1] = y.y, m[2] = y.z, m[3] = y.w;
+            r[0] = z.x, r[1] = z.y, r[2] = z.z, r[3] = z.w;
+          } else {
+#pragma unroll
+            for (uint32_t i = 0; i < 4u; ++i)
+              if (4u * qi + i < V) {
+                d[i] = static_cast<uint32_t>(g[4u * qi + i]);
+                m[i] = static_cast<uint32_t>(g[V + 4u * qi + i]);
+                r[i] = static_cast<uint32_t>(g[2u * V + 4u * qi + i]);
+              }
+          }
+          uint64_t a[4], wd[4];
+#pragma unroll
+          for (uint32_t i = 0; i < 4u; ++i) {
+            const uint32_t v = 4u * qi + i;
+            a[i] = 0ull;
+            wd[i] = 0ull;
+            if (v < V) {
+              const uint32_t mk = lut[v], nn = mk >> 4;
+              const bool ctr = MODEL == 2 && v == centre;
+              if (MODEL == 2 && r[i] > static_cast<uint32_t>(ctr)) bad_state = true;
+              if (MODEL != 2 && r[i] >= kLaneHill) nbig = true;
+              if ((d[i] | m[i] | r[i]) >= nr.small) {
+                nbig = true;
+                if (!REC) ovf |= exact_ovf<MODEL>(ntv, d[i], m[i], r[i], nn, ctr);
+              }
+              if (REC) {
+                // past the packed word's range: to the redo list
+                nbig |= (d[i] | m[i]) >= kWordCount;
+                wd[i] = pack_voxel(d[i], m[i], r[i] & 0xFFFFFu, mk & 15u);
+              }
+              a[i] = lane_total<MODEL>(nr, ntv, d[i], m[i], r[i], nn, ctr);
+            }
+            S += a[i];
+          }
+          if (REC) {
+            ulonglong2* o = reinterpret_cast<ulonglong2*>(nrec + kNodeWords) + 4u * qi;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o[i] = make_ulonglong2(a[i], wd[i]);
+          } else {
+            ulonglong2* o = reinterpret_cast<ulonglong2*>(ntree + kCnt) + 2u * qi;
+            o[0] = make_ulonglong2(a[0], a[1]);
+            o[1] = make_ulonglong2(a[2], a[3]);
+            reinterpret_cast<uint4*>(ncp)[qi] = make_uint4(d[0], d[1], d[2], d[3]);
+            reinterpret_cast<uint4*>(ncp + ps)[qi] = make_uint4(m[0], m[1], m[2], m[3]);
+            reinterpret_cast<uint4*>(ncp + 2u * ps)[qi] = make_uint4(r[0], r[1], r[2], r[3]);
+          }
+        }
+        // the sums above the quads (entries past the last quad are zero)
+        if (NODE8) {
+          nrec[qi] = S;
+          uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
+          x += __shfl_xor_sync(kFull, x, 2);
+          x += __shfl_xor_sync(kFull, x, 4);
+          if ((lane & 7) == 0) ntree[10u + (qi >> 3)] = x;  // 32 sums of 8 quads
+          x += __shfl_xor_sync(kFull, x, 8);
+          x += __shfl_xor_sync(kFull, x, 16);
+          if (lane == 0) ntree[2u + (qi >> 5)] = x;         // 8 sums of 32
+          total += x;
+          if ((k & 3u) == 3u && lane == 0) ntree[k >> 2] = (k == 3u) ? total : total - pair;
+          if (k == 3u) pair = total;
+        } else {
+          if (qi < NQ) ntree[level_off(LV - 1) + qi] = S;
+          uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
+          x += __shfl_xor_sync(kFull, x, 2);
+          if (qi < NQ && (lane & 3) == 0) ntree[level_off(LV - 2) + (qi >> 2)] = x;
+          x += __shfl_xor_sync(kFull, x, 4);
+          x += __shfl_xor_sync(kFull, x, 8);
+          if (LV >= 4 && (lane & 15) == 0) ntree[level_off(LV >= 4 ? LV - 3 : 1) + (qi >> 4)] = x;
+          x += __shfl_xor_sync(kFull, x, 16);
+          if (LV == 5) {
+            pair = (k & 1u) ? pair + x : x;
+            if ((k & 1u) && lane == 0) ntree[k >> 1] = pair;
+          }
+          total += x;
+        }
+      }
+      const bool any_ovf = __any_sync(kFull, ovf), any_bad = __any_sync(kFull, bad_state);
+      nbig = __any_sync(kFull, nbig);
+      if (slot == sc) {
+        q = nr;
+        tv = ntv;
+        cell = w.y;
+        vidx = w.x;
+        step = *ntv->step + p.step_off;
+        key0 = static_cast<uint32_t>(ntv->seed);
+        key1 = static_cast<uint32_t>(ntv->seed >> 32);
+        word3 = ntv->tissue_id | (kTagChi << 24);
+        A = total;
+        tnow = 0.0;
+        e0 = 0;
+        big = nbig;
+        lim = min(nr.small, kLaneHill);
+        err = any_bad ? kErrState : any_ovf ? kErrOverflow : (REC && nbig) ? kErrNarrow : 0;
+        have = true;
+        if (REC) {
+          // the bits a count has once it reaches its limit (a power of two)
+          const uint32_t lc = min(q.small, kWordCount), lr = MODEL == 2 ? lc : min(q.small, kLaneHill);
+          const uint32_t mc = 0xFFFFFu & ~(lc - 1u), mr = 0xFFFFFu & ~(lr - 1u);
+          over_mask = pack_voxel(mc, mc, mr, 0u);
+        }
+      }
+    }
+    __syncwarp();
+    if (__all_sync(kFull, done)) break;
+
+    // ---- draws: lane j of a cell, event e0 + j -----------------------------
+    uint64_t Em, Rb;
+    int Ek;
+    draw_event(e0 + sl, step, cell, word3, key0, key1, Em, Ek, Rb);
+
+    // ---- G events of every cell, the whole warp in step --------------------
+    bool run = have && err == 0;
+    bool paused = false;    // shared leaves: a count reached its limit for the first time
+    const bool slow = !REC && __any_sync(kFull, run && big);
+    uint32_t m = 0;         // events applied
+    uint64_t Aj = 0;        // the total propensity before this lane's event
+    uint32_t log = 0;       // this lane's event: v, u, code
+    for (uint32_t i = 0; i < G; ++i) {
+      const uint64_t R64 = ONE ? Rb : __shfl_sync(kFull, Rb, base_lane + static_cast<int>(i));
+      uint64_t r = __umul64hi(R64, A);
+      // descent to a quad
+      uint32_t idx = 0;
+      if (NODE8) {
+        const uint64_t s0 = tree[0];
+        idx = r >= s0 ? 1u : 0u;
+        r -= idx ? s0 : 0ull;
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + (l ? 10u : 2u)) + 2u * idx;
+          const ulonglong2 x = nd[0], y = nd[1];
+          idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        }
+        // eight quad sums: the half, then the quad
+        const U64x4 x = load4(rec + 8u * idx), y = load4(rec + 8u * idx + 4u);
+        const uint64_t half = (x.a + x.b) + (x.c + x.d);
+        const bool up = r >= half;
+        r -= up ? half : 0ull;
+        idx = 8u * idx + (up ? 4u : 0u) +
+              pick_child<!ONE>(up ? y.a : x.a, up ? y.b : x.b, up ? y.c : x.c, r);
+      } else {
+#pragma unroll
+        for (uint32_t l = 1; l < LV; ++l) {
+          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) + 2u * idx;
+          const ulonglong2 x = nd[0], y = nd[1];
+          idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        }
+      }
+      if (kChecked && run && idx >= nq) err |= kErrBounds;
+      idx = min(idx, nq - 1u);  // never past the cell's quads, whatever the sums hold
+      // the voxel, its total, counts and neighbours
+      uint64_t a_v, w_v = 0;
+      uint32_t v, D, N, R, mask, nn;
+      if (REC) {
+        const U64x4 x = load4(rec + kNodeWords + 8u * idx);
+        const U64x4 y = load4(rec + kNodeWords + 8u * idx + 4u);
+        const uint32_t k = pick_child<!ONE>(x.a, x.c, y.a, r);
+        a_v = k == 0u ? x.a : k == 1u ? x.c : k == 2u ? y.a : y.c;
+        w_v = k == 0u ? x.b : k == 1u ? x.d : k == 2u ? y.b : y.d;
+        v = 4u * idx + k;
+        D = word_D(w_v);
+        N = word_N(w_v);
+        R = word_R(w_v);
+        mask = word_mask(w_v);
+        nn = __popc(mask);
+      } else {
+        const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + kCnt) + 2u * idx;
+        const ulonglong2 x = nd[0], y = nd[1];
+        v = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        a_v = tree[kCnt + v];
+        D = static_cast<uint32_t>(cp[v]);
+        N = static_cast<uint32_t>(cp[ps + v]);
+        R = static_cast<uint32_t>(cp[2u * ps + v]);
+        const uint32_t mk = lut[v];
+        mask = mk & 15u;
+        nn = mk >> 4;
+      }
+      // nothing left to happen (A = 0); else never while the sums are
+      // consistent (voxels past V have total 0)
+      if (run && r >= a_v) {
+        run = false;
+        err |= A != 0ull ? kErrInternal : 0;
+      }
+
+      // channel: hops are the last but the in-voxel bindings in channel order
+      const bool ctr = MODEL == 2 && v == centre;
+      const uint32_t F = MODEL == 2 ? static_cast<uint32_t>(ctr) - R : 0u;
+      const uint64_t X = MODEL == 2 ? static_cast<uint64_t>(N) * F : static_cast<uint64_t>(D) * N;
+      const uint64_t y17 = MODEL ? q.k_in * X : 0ull;
+      const uint64_t y18 = MODEL == 1 ? q.k_off * R : 0ull;
+      const uint64_t UD = q.hD * D, UN = q.hN * N, UR = MODEL == 2 ? 0ull : q.hR * R;
+      const uint64_t HD = UD * nn, H2 = HD + UN * nn, H3 = MODEL == 2 ? H2 : H2 + UR * nn;
+      const uint64_t top = a_v - y17 - y18, y = top - H3;
+      const bool hop = r >= y && (MODEL == 0 || r < top);
+      const uint64_t z0 = r - y;
+      const bool z1 = z0 >= HD, z2 = MODEL != 2 && z0 >= H2;
+      uint32_t s = z2 ? 2u : z1 ? 1u : 0u;  // the species a hop or a MODEL 0 channel changes
+      bool gain = false;                    // ... and whether by +1 at v
+      uint32_t code = kEvHop + s, u = v;
+      int dD = 0, dN = 0, dR = 0;           // MODEL 1, 2: the changes at v
+      if (hop) {
+        const uint64_t unit = z2 ? UR : z1 ? UN : UD, unit2 = unit + unit;
+        const uint64_t z3 = z0 - (z2 ? H2 : z1 ? HD : 0ull);
+        const bool b2 = z3 >= unit2;
+        const uint64_t z4 = z3 - (b2 ? unit2 : 0ull);
+        const int off = hop_off[(mask << 2) + (b2 ? 2u : 0u) + (z4 >= unit ? 1u : 0u)];
+        u = v + static_cast<uint32_t>(off);
+        if (kChecked && run && u >= V) err |= kErrBounds;
+        u = min(u, V - 1u);
+        if (MODEL) {
+          dD = s == 0u ? -1 : 0;
+          dN = s == 1u ? -1 : 0;
+          dR = s == 2u ? -1 : 0;
+        }
+      } else {
+        const uint64_t gDD = q.gD * D, gNN = q.gN * N;
+        uint64_t c0, c1;
+        if (MODEL == 2) {
+          c0 = q.tD * F;
+          c1 = c0 + q.kd * R;
+        } else {
+          c1 = y - q.gR * R - gNN - gDD;
+          c0 = c1 - q.kN;
+        }
+        const uint64_t c2 = c1 + gDD, c3 = c2 + gNN;
+        const uint32_t ch = static_cast<uint32_t>(r >= c0) + static_cast<uint32_t>(r >= c1) +
+                            static_cast<uint32_t>(r >= c2) + static_cast<uint32_t>(r >= c3);
+        code = ch;
+        s = ch == 4u ? 2u : (ch & 1u);  // D, N, D, N, R
+        gain = ch <= 1u;
+        if (MODEL) {
+          dD = ch == 0u ? 1 : ch == 2u ? -1 : 0;
+          dN = ch == 1u ? 1 : ch == 3u ? -1 : 0;
+          dR = ch == 4u ? -1 : (MODEL == 2 && ch == 1u) ? -1 : 0;
+          if (r >= top) {
+            const bool rel = MODEL == 1 && r >= top + y17;  // R -> D + N
+            code = rel ? kEvRelease : kEvBind;
+            dD = MODEL == 2 ? 0 : rel ? 1 : -1;
+            dN = rel ? 1 : -1;
+            dR = rel ? -1 : 1;
+          }
+        }
+      }
+      const bool move = run && hop;
+      // differences of the totals of v and u
+      const ulonglong2 gh = rates[s];
+      uint64_t dv, du = 0;
+      uint32_t nc = 0, newmax = 0;
+      if (MODEL == 0) {
+        const uint64_t c = gh.x + gh.y * nn;
+        dv = gain ? c : 0ull - c;
+        nc = (s == 0u ? D : s == 1u ? N : R) + (gain ? 1u : 0xFFFFFFFFu);
+        newmax = nc;
+      } else {
+        dv = lane_total<MODEL>(q, tv, D + dD, N + dN, R + dR, nn, ctr) - a_v;
+        newmax = (D + dD) | (N + dN) | (R + dR);
+      }
+      uint32_t cu = 0;
+      uint64_t a_u = 0, w_u = 0;
+      if (REC) {
+        const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec + kNodeWords)[u];
+        a_u = x.x;
+        w_u = x.y;
+        if (hop) {
+          du = gh.x + gh.y * static_cast<uint32_t>(__popc(word_mask(w_u)));
+          if (MODEL == 1) du += s == 2u ? 0ull : q.k_in * (s == 0u ? word_N(w_u) : word_D(w_u));
+          if (MODEL == 2 && s == 1u)
+            du += q.k_in * (static_cast<uint32_t>(u == centre) - word_R(w_u));
+        }
+      } else {
+        cu = static_cast<uint32_t>(cp[s * ps + u]) + 1u;
+        if (hop) {
+          du = gh.x + gh.y * (lut[u] >> 4);
+          if (MODEL == 1 && s < 2u)
+            du += q.k_in * static_cast<uint32_t>(cp[(1u - s) * ps + u]);
+          if (MODEL == 2 && s == 1u)
+            du += q.k_in * (static_cast<uint32_t>(u == centre) - static_cast<uint32_t>(cp[2u * ps + u]));
+          newmax |= cu;
+        }
+      }
+      if (MODEL != 2 && s == 2u && run) {  // R changes the Hill term, here and where it arrives
+        const uint32_t Ru = hop ? (REC ? word_R(w_u) + 1u : cu) : 1u;
+        if (!slow) {  // every count is inside the table
+          if (MODEL == 0) dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
+          const uint64_t d = __ldg(q.hill + Ru) - __ldg(q.hill + (Ru - 1u));
+          if (hop) du += d;
+        } else {
+          if (MODEL == 0) dv += lane_hill(q.hill, tv, R - 1u) - lane_hill(q.hill, tv, R);
+          if (hop) du += lane_hill(q.hill, tv, Ru) - lane_hill(q.hill, tv, Ru - 1u);
+        }
+      }
+      // the sums along both paths.  One lane: all reads, then all stores.  More:
+      // lane pairs take the levels, the even lane v's entry, the odd lane u's
+      // (v's adds both differences where the paths share the entry).
+      if (ONE) {
+        uint64_t nv[LV], nu[LV];
+#pragma unroll
+        for (uint32_t l = 1; l <= SL; ++l) {
+          const uint32_t sh = NODE8 ? (l == 1 ? 9u : l == 2 ? 7u : 5u) : 2u * (LV - l);
+          const uint32_t o = NODE8 ? (l == 1 ? 0u : l == 2 ? 2u : 10u) : level_off(l);
+          const uint32_t iv = v >> sh, iu = u >> sh;
+          nv[l] = tree[o + iv] + dv + (iv == iu ? du : 0ull);
+          nu[l] = tree[o + iu] + du;
+        }
+        if (NODE8) {
+          const uint32_t iv = v >> 2, iu = u >> 2;
+          nv[0] = rec[iv] + dv + (iv == iu ? du : 0ull);
+          nu[0] = rec[iu] + du;
+        }
+        if (run) {
+#pragma unroll
+          for (uint32_t l = 1; l <= SL; ++l) {
+            const uint32_t sh = NODE8 ? (l == 1 ? 9u : l == 2 ? 7u : 5u) : 2u * (LV - l);
+            const uint32_t o = NODE8 ? (l == 1 ? 0u : l == 2 ? 2u : 10u) : level_off(l);
+            const uint32_t iv = v >> sh, iu = u >> sh;
+            tree[o + iv] = nv[l];
+            if (iv != iu) tree[o + iu] = nu[l];
+          }
+          if (NODE8) {
+            rec[v >> 2] = nv[0];
+            if ((v >> 2) != (u >> 2)) rec[u >> 2] = nu[0];
+          }
+        }
+      } else {
+        const bool odd = sl & 1u;
+        const uint32_t me = odd ? u : v, other = odd ? v : u;
+        const uint64_t dme = odd ? du : dv, dot = odd ? 0ull : du;
+        __syncwarp();
+        // level LV of the tree: the voxel totals themselves (shared leaves)
+        constexpr uint32_t kTasks = 2u * (NODE8 ? SL + 1 : REC ? SL : LV);
+        for (uint32_t t = sl; t < kTasks; t += G) {
+          const uint32_t l = (t >> 1) + 1u;
+          const uint32_t sh = !NODE8   ? 2u * (LV - l)
+                              : l == 4 ? 2u
+                              : l == 1 ? 9u
+                              : l == 2 ? 7u
+                                       : 5u;
+          const uint32_t o = NODE8 ? (l == 1 ? 0u : l == 2 ? 2u : 10u) : level_off(l);
+          const uint32_t i1 = me >> sh, i2 = other >> sh;
+          uint64_t* at = (NODE8 && l == 4) ? rec + i1 : tree + o + i1;
+          const bool same = i1 == i2;
+          if (run && !(odd && same)) *at += dme + (same ? dot : 0ull);
+        }
+      }
+      // the two voxels
+      if (REC) {
+        const uint64_t one = word_unit(s);
+        const uint64_t wv2 = MODEL == 0 ? (gain ? w_v + one : w_v - one)
+                                        : pack_voxel(D + dD, N + dN, R + dR, mask);
+        const uint64_t wu2 = w_u + one;
+        if (run && (ONE || sl == 0u)) {
+          reinterpret_cast<ulonglong2*>(rec + kNodeWords)[v] = make_ulonglong2(a_v + dv, wv2);
+        }
+        if (move && (ONE || sl == 1u)) {
+          reinterpret_cast<ulonglong2*>(rec + kNodeWords)[u] = make_ulonglong2(a_u + du, wu2);
+        }
+        if (run && (((wv2 | (hop ? wu2 : 0ull)) & over_mask) != 0ull)) err |= kErrNarrow;
+      } else {
+        if (run && lead) {
+          if (MODEL == 0) {
+            cp[s * ps + v] = static_cast<int32_t>(nc);
+          } else {
+            if (dD) cp[v] = static_cast<int32_t>(D + dD);
+            if (dN) cp[ps + v] = static_cast<int32_t>(N + dN);
+            if (dR) cp[2u * ps + v] = static_cast<int32_t>(R + dR);
+          }
+          if (hop) cp[s * ps + u] = static_cast<int32_t>(cu);
+        }
+      }
+      if (!ONE) __syncwarp();
+      if (sl == i) {
+        Aj = A;
+        log = v | (u << 10) | (code << 20);
+      }
+      if (run) {
+        A += dv + du;
+        m = i + 1u;
+        if (REC) {
+          run = err == 0;
+        } else if (!big && newmax >= (MODEL == 2 || (MODEL == 0 && s != 2u) ? q.small : lim)) {
+          big = paused = true;  // its limits are checked below, the next batch's in it
+          run = false;
+        }
+      }
+      if (slow) {  // cells past those limits: checked exactly
+        if (run && big && past_limits<MODEL>(tv, cp, ps, lut, v, u, centre)) {
+          err |= kErrOverflow;
+          run = false;
+        }
+        if (!ONE) __syncwarp();
+      }
+    }
+    if (!REC && __any_sync(kFull, paused)) {
+      const uint32_t last = ONE ? log : __shfl_sync(kFull, log, base_lane + static_cast<int>(m ? m - 1u : 0u));
+      if (paused && past_limits<MODEL>(tv, cp, ps, lut, last & 1023u, (last >> 10) & 1023u, centre)) {
+        err |= kErrOverflow;
+        paused = false;
+      }
+      __syncwarp();
+    }
+
+    // ---- the waiting times of the applied events, added in order -----------
+    const double tau = tau_from(F53{Em, Ek}, Ek < 0 || Aj == 0ull, Aj | (Aj == 0ull));
+    uint32_t fired = 0;
+    if (ONE) {
+      const double tn = __dadd_rn(tnow, tau);
+      if (m && before(tn, p.dt)) {
+        tnow = tn;
+        fired = 1;
+      }
+    } else {
+      // lane j keeps the time after event j; times only grow, so the events
+      // that fire are the leading ones
+      double t = tnow, mine = tnow;
+      for (uint32_t j = 0; j < G; ++j) {
+        t = __dadd_rn(t, __shfl_sync(kFull, tau, base_lane + static_cast<int>(j)));
+        if (sl == j) mine = t;
+      }
+      const unsigned late = __ballot_sync(kFull, !(sl < m && before(mine, p.dt))) >> base_lane;
+      fired = min(G, static_cast<uint32_t>(__ffs(static_cast<int>(late))) - 1u);
+      const double tl = __shfl_sync(kFull, mine, base_lane + static_cast<int>(fired ? fired - 1u : 0u));
+      if (fired) tnow = tl;
+    }
+    if (fired < m) err &= ~(kErrOverflow | kErrNarrow);  // the event that met a limit did not fire
+    const uint32_t e = e0 + fired;
+    if (have && fired == G && e >= 0xFFFFFFFFu - 32u) err |= kErrEventIndex;
+    const bool fin = have && (err != 0 || fired < m || (m < G && !paused));
+    e0 = e;
+    unsigned out = __ballot_sync(kFull, fin && lead);
+    if (out) {
+      // undo the events past the end of the step, last first (counts only)
+      for (uint32_t j = G; j-- > 0;) {
+        const uint32_t lg = ONE ? log : __shfl_sync(kFull, log, base_lane + static_cast<int>(j));
+        if (fin && lead && j >= fired && j < m) {
+          const uint32_t v = lg & 1023u, u = (lg >> 10) & 1023u, code = lg >> 20;
+          int d[3] = {0, 0, 0};
+          uint32_t s = 3u;  // species that moves back from u
+          if (code >= kEvHop) {
+            s = code - kEvHop;
+            d[s] = 1;
+          } else if (code == kEvBind || code == kEvRelease) {
+            d[1] = code == kEvBind ? 1 : -1;
+            d[0] = MODEL != 2 ? d[1] : 0;
+            d[2] = -d[1];
+          } else {
+            d[code == 4u ? 2u : (code & 1u)] = code <= 1u ? -1 : 1;
+            if (MODEL == 2 && code == 1u) d[2] = 1;
+          }
+          if (REC) {
+            uint64_t* base = rec + kNodeWords + 1u;
+            uint64_t& wv = base[2u * v];
+            wv = pack_voxel(word_D(wv) + d[0], word_N(wv) + d[1], word_R(wv) + d[2], word_mask(wv));
+            if (s < 3u) base[2u * u] -= word_unit(s);
+          } else {
+            for (uint32_t k = 0; k < 3u; ++k) cp[k * ps + v] += d[k];
+            if (s < 3u) cp[s * ps + u] -= 1;
+          }
+        }
+      }
+      __syncwarp();
+      if (REC && fin && lead && (err & kErrNarrow)) {
+        // left as it was, for the 32-bit pass
+        p.redo[atomicAdd(p.redo_n, 1u)] = make_uint2(vidx, cell);
+      } else if (fin && lead) {
+        tv->ev_last[cell] = e;
+        tv->t_last[cell] = tnow;
+        tv->ev_total[cell] += e;
+        if (err) atomicOr(tv->err, err);
+      }
+      // the counts back to the state array, the whole warp one cell at a time
+      out = __ballot_sync(kFull, fin && lead && !(REC && (err & (kErrNarrow | kErrState))));
+      while (out) {
+        const int src = __ffs(out) - 1;
+        out &= out - 1u;
+        const uint32_t sc = ONE ? static_cast<uint32_t>(src) : static_cast<uint32_t>(src) / G;
+        const uint32_t c = __shfl_sync(kFull, cell, src);
+        const uint32_t vi = __shfl_sync(kFull, vidx, src);
+        int32_t* g = p.views[vi].counts + static_cast<size_t>(c) * 3u * V;
+        if (REC) {
+          const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words + kNodeWords;
+          if (vec) {
+            for (uint32_t i = lane; i < nq; i += 32u) {
+              const U64x4 x = load4(from + 8u * i), y = load4(from + 8u * i + 4u);
+              const U64x4 w{x.b, x.d, y.b, y.d};
+              reinterpret_cast<uint4*>(g)[i] =
+                  make_uint4(word_D(w.a), word_D(w.b), word_D(w.c), word_D(w.d));
+              reinterpret_cast<uint4*>(g + V)[i] =
+                  make_uint4(word_N(w.a), word_N(w.b), word_N(w.c), word_N(w.d));
+              reinterpret_cast<uint4*>(g + 2u * V)[i] =
+                  make_uint4(word_R(w.a), word_R(w.b), word_R(w.c), word_R(w.d));
+            }
+          } else {
+            for (uint32_t i = lane; i < V; i += 32u) {
+              const uint64_t w = from[2u * i + 1u];
+              g[i] = static_cast<int32_t>(word_D(w));
+              g[V + i] = static_cast<int32_t>(word_N(w));
+              g[2u * V + i] = static_cast<int32_t>(word_R(w));
+            }
+          }
+        } else {
+          const int32_t* from = reinterpret_cast<const int32_t*>(
+              reinterpret_cast<const uint64_t*>(warp_cells + sc * p.cell_stride + 48) + kCnt + ps);
+          for (uint32_t sp = 0; sp < 3u; ++sp) {
+            if (vec) {
+              for (uint32_t i = lane; i < nq; i += 32u)
+                reinterpret_cast<int4*>(g + sp * V)[i] =
+                    reinterpret_cast<const int4*>(from + sp * ps)[i];
+            } else {
+              for (uint32_t i = lane; i < V; i += 32u) g[sp * V + i] = from[sp * ps + i];
+            }
+          }
+        }
+      }
+      __syncwarp();
+      if (fin) {
+        have = false;
+        err = 0;
+        A = 0;
+      }
+    }
+  }
+}
+
+}  // namespace
+
+}  // namespace tsg

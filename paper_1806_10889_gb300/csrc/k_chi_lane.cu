@@ -1,0 +1,151 @@
+// K_chi, sum-tree form: the Notch-Delta instantiations, the launch plan and
+// the launcher (the kernel template is in chi_lane.cuh).
+#include "chi_lane.cuh"
+
+namespace tsg {
+
+ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, bool one) {
+  // one lane per cell never takes shared leaves: past 110 cells an SM records
+  // are as fast or faster
+  if (V <= 64) {
+    if (leaf == kLeafRecords) return one ? k_chi_lane<0, 3, kLeafRecords, true> : nullptr;
+    return leaf == kLeafShared && !one ? k_chi_lane<0, 3, kLeafShared, false> : nullptr;
+  }
+  if (V <= 256) {
+    if (leaf == kLeafRecords)
+      return one ? k_chi_lane<0, 4, kLeafRecords, true> : k_chi_lane<0, 4, kLeafRecords, false>;
+    return leaf == kLeafShared && !one ? k_chi_lane<0, 4, kLeafShared, false> : nullptr;
+  }
+  if (leaf == kLeafNodes)
+    return one ? k_chi_lane<0, 5, kLeafNodes, true> : k_chi_lane<0, 5, kLeafNodes, false>;
+  if (one) return nullptr;
+  return leaf == kLeafRecords ? k_chi_lane<0, 5, kLeafRecords, false>
+                              : k_chi_lane<0, 5, kLeafShared, false>;
+}
+
+namespace {
+
+ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, bool one) {
+  return model == 2   ? chi_lane_kernel_pm(V, leaf, one)
+         : model == 1 ? chi_lane_kernel_bind(V, leaf, one)
+                      : chi_lane_kernel_nd(V, leaf, one);
+}
+
+}  // namespace
+
+// The shape follows from the cells an SM holds, per.  Chi ms of one step at
+// dt 0.02 (8x8 and 16x16 voxels) and 0.006 (32x32), 60 D + 30 N + 10 R per
+// voxel, by lanes per cell G and leaf (S shared, R records, N nodes), with the
+// best segmented launch in brackets:
+//   per     8x8                          16x16                        32x32
+//    4  S32 .37 S16 .42 [.70]   S32 1.44 S16 1.58 [2.65]     S32 1.91 S16 2.10 [3.2]
+//    8  S32 .43 S16 .43 [.83]   S16 1.59 S32 1.64 [2.89]     S16 2.09 S32 2.16 [3.5]
+//   13  S16 .46 S8 .48  [.85]   S8 1.74 S16 1.82  [3.18]  15 R16 3.35 R8 3.75  [4.9]
+//   27  S8 .55 S4 .62   [.93]   S8 2.04 S4 2.30 R8 2.80 [4.18]  R8 4.05 R16 4.19 [6.7]
+//   60  R4 .73 S4 .73   [1.2]   R8 3.79 R4 3.90   [6.20]  53 R8 5.14 R4 5.58   [12.0]
+//   80  R4 .84 S4 .85   [2.0]   R4 4.27 R1 4.66   [9.67]  75 R4 6.39 R1 7.9    [16.5]
+//  108  R4 1.01 S2 1.02 [2.2]   R1 4.76 R4 4.80   [11.1]     N4 9.08 N1 10.1   [22.2]
+//  150  R1 1.35 R2 1.35 [2.9]   R1 5.26 R2 5.76   [15.1]     N1 11.3 N2 11.9   [30.1]
+//  431  R1 2.03 R2 2.83 [7.3]   R1 11.4 R2 12.9   [39.4]     N2 25.4 N1 25.9   [82.7]
+// Few cells: one chain of events sets the time, and more lanes per cell take
+// more of the draws off it.  Many: the instructions issued per event do, and
+// one lane per cell issues the fewest.
+LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
+  LanePlan pl;
+  int dev = 0, sms = 0;
+  if (cells == 0 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return pl;
+  const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
+  const uint64_t per = (cells + static_cast<uint64_t>(sms) - 1) / static_cast<uint64_t>(sms);
+  pl.G = per <= 4 ? 32u : per <= (lv == 5 ? 22u : 12u) ? 16u : per <= 56 ? 8u : per <= 110 ? 4u : 1u;
+  // Leaves: in shared memory while one wave of cells fits there; else records,
+  // and past one wave of those (32x32 voxels, 2.7 KB of sums a cell) nodes.
+  constexpr uint64_t kWave = 216 * 1024;  // an SM's shared memory less what blocks reserve
+  const uint32_t nq = (V + 3u) / 4u;
+  const uint32_t sums = 48u + (lv == 3 ? 160u : lv == 4 ? 672u : 2720u);
+  const uint32_t shared = sums + 20u * 4u * nq;
+  pl.leaf = pl.G > 1 && per * shared <= kWave   ? kLeafShared
+            : lv < 5 || per * sums <= kWave     ? kLeafRecords
+                                                : kLeafNodes;
+  const uint32_t raw = pl.leaf == kLeafShared    ? shared
+                       : pl.leaf == kLeafRecords ? sums
+                                                 : 48u + 42u * 8u;
+  // an odd multiple of 16 bytes: lanes reading the same entry of their cells
+  // start on different shared-memory banks
+  pl.cell_stride = ((raw + 15u) & ~15u) | 16u;
+  pl.lut_bytes = 128u + ((4u * nq + 15u) & ~15u);
+  pl.wpb = pl.G == 1 ? 2u : 1u;
+  pl.smem = pl.lut_bytes + static_cast<size_t>(pl.wpb) * (32u / pl.G) * pl.cell_stride;
+  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G == 1);
+  int per_sm = 0;
+  // the limit is the device's, not this plan's: plans of other cell sizes
+  // share the kernel
+  if (!k || pl.smem > kMaxSmem ||
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * static_cast<int>(pl.wpb),
+                                                    pl.smem) != cudaSuccess ||
+      per_sm < 1) {
+    pl.G = 0;
+    return pl;
+  }
+  const uint64_t per_block = static_cast<uint64_t>(pl.wpb) * (32u / pl.G);
+  const uint64_t need = (cells + per_block - 1) / per_block;
+  const uint64_t cap = static_cast<uint64_t>(sms) * static_cast<uint64_t>(per_sm);
+  pl.blocks = static_cast<uint32_t>(need < cap ? need : cap);
+  if (pl.leaf != kLeafShared)
+    pl.scratch_bytes = static_cast<size_t>(pl.blocks) * per_block *
+                       (8u * nq + (pl.leaf == kLeafNodes ? 256u : 0u)) * sizeof(uint64_t);
+  return pl;
+}
+
+cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_views,
+                            const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
+                            uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
+                            uint32_t step_off, double dt, cudaStream_t stream, int priority) {
+  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G == 1);
+  const LaneArgs a{d_views, d_items, d_counter, d_scratch, redo.items, redo.counters + 1, dt,
+                   n_items, step_off, V, n, pl.G, pl.lut_bytes, pl.cell_stride};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pl.blocks);
+  cfg.blockDim = dim3(32u * pl.wpb);
+  cfg.dynamicSmemBytes = pl.smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributePriority;
+  attr[0].val.priority = priority;
+  cfg.attrs = attr;
+  cfg.numAttrs = priority ? 1 : 0;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k, a);
+  if (e != cudaSuccess || pl.leaf == kLeafShared) return e;
+  // the cells that left the packed range, by the segmented kernel from the
+  // state they started the step with (it reads their number from the device)
+  const tissue_launch c = prefix_launch(V, n_items);
+  const int H = static_cast<int>(c.lanes_per_cell);
+  const bool qb = V > static_cast<uint32_t>(H * H);
+  const ChiSegKernel ks =
+      model == 2 ? chi_seg_kernel_pm(H, true, qb) : chi_seg_kernel_nd(H, true, qb);
+  const uint32_t seg_bytes = seg_bytes_for(V, H, true);
+  const size_t smem = static_cast<size_t>(c.warps_per_block) * (32u / c.lanes_per_cell) * seg_bytes;
+  const int threads = 32 * static_cast<int>(c.warps_per_block);
+  int dev = 0, sms = 0, per_sm = 0;
+  if (smem > 48 * 1024 &&
+      (e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(smem))) != cudaSuccess)
+    return e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks, threads, smem)) != cudaSuccess)
+    return e;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  cfg.gridDim = dim3(static_cast<unsigned>(sms * per_sm));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  return cudaLaunchKernelEx(&cfg, ks, d_views, static_cast<const uint2*>(redo.items), n_items,
+                            redo.counters + 2, seg_bytes, step_off, dt,
+                            static_cast<uint2*>(nullptr), static_cast<uint32_t*>(nullptr),
+                            static_cast<const uint32_t*>(redo.counters + 1));
+}
+
+}  // namespace tsg

@@ -17,6 +17,7 @@
 #include <new>
 #include <vector>
 
+#include "chi_lane.h"
 #include "tissue.h"
 #include "tissue_internal.h"
 
@@ -25,11 +26,16 @@ using namespace tsg;
 namespace {
 
 struct ClassPlan {
-  uint32_t V;
+  uint32_t V, n;
   uint32_t lanes, warps_per_block, layout;
   size_t items_off;  // offset (in uint2) into the item buffer
   uint32_t n_items;
   int gen;           // 0: Notch-Delta only; 2: promoter only; 1: both, or a trace is on
+  // the sum-tree launch (lane.G = 0: none), its model code and the offset of
+  // its scratch; it takes the class while the launch shape is a default one
+  LanePlan lane;
+  int lane_model;
+  size_t lane_off;
 };
 
 }  // namespace
@@ -43,6 +49,7 @@ struct tissue_batch {
   uint2* d_items = nullptr;   // chi items of every class, then x-faces, then y-faces
   uint32_t* d_counters = nullptr;  // per class: work counter, redo count, redo-pass work counter
   uint2* d_redo = nullptr;         // cells a class's 16-bit-count pass gives up on
+  uint64_t* d_lane = nullptr;      // the sum-tree launches' scratch, each class its part
   uint32_t* d_io_steps = nullptr;  // checkpoint writes: the members' new step indices
   int* d_io_err = nullptr;         // checkpoint reads: the members' error flags
   int* d_io_bad = nullptr;         // checkpoint writes: a count out of range
@@ -110,6 +117,18 @@ int chi_all(tissue_batch* b, double dt) {
       return TISSUE_E_CUDA;
     // each class has its own part of the redo list (classes may run at once)
     const ChiRedo redo{b->d_redo + p.items_off, counters};
+    const int prio = ov ? (c == 0 ? b->prio_hi : b->prio_lo) : 0;
+    if (p.lane.G && default_shape(p.V, {TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0,
+                                        p.layout})) {
+      if (launch_chi_lane(p.lane, p.lane_model, b->d_views, b->d_items + p.items_off, p.n_items,
+                          counters, b->d_lane + p.lane_off, redo, p.V, p.n, 0u, dt, st, prio) !=
+          cudaSuccess)
+        return TISSUE_E_CUDA;
+      if (mark(b, 4 + c, st) != TISSUE_OK) return TISSUE_E_CUDA;
+      if (ov && c > 0 && cudaEventRecord(b->ev_join[c - 1], st) != cudaSuccess)
+        return TISSUE_E_CUDA;
+      continue;
+    }
     // as for single tissues: a counts-only launch with several voxels per
     // lane takes Notch-Delta classes without a trace; others run the prefix
     // launch of the class (the same trajectories)
@@ -117,7 +136,6 @@ int chi_all(tissue_batch* b, double dt) {
     if (lc.smem_layout == TISSUE_LAYOUT_RECOMPUTE &&
         !recompute_covers(p.V, static_cast<int>(p.lanes), p.gen))
       lc = prefix_launch(p.V, p.n_items);
-    const int prio = ov ? (c == 0 ? b->prio_hi : b->prio_lo) : 0;
     if (launch_chi_seg(b->d_views, b->d_items + p.items_off, p.n_items, counters, p.V,
                        static_cast<int>(lc.lanes_per_cell), static_cast<int>(lc.warps_per_block),
                        0, 0u, dt, lc.smem_layout == TISSUE_LAYOUT_PREFIX, p.gen, &redo, st,
@@ -227,6 +245,7 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
   // chi items by class, largest cells first; faces of both phases
   std::map<uint32_t, std::vector<uint2>, std::greater<uint32_t>> by_v;
   std::map<uint32_t, int> nd_v, pm_v, tr_v;  // per class: members of each model, traced
+  std::map<uint32_t, int> bind_v;            // ... with in-voxel binding
   std::vector<uint2> xf, yf, wm_items;
   for (uint32_t i = 0; i < count; ++i) {
     const tissue_desc& d = info[i].desc;
@@ -234,6 +253,7 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     std::vector<uint2>& list = by_v[V];
     (info[i].view.q.kind == kModelPromoter ? pm_v : nd_v)[V] += 1;
     if (info[i].view.trace != nullptr) tr_v[V] += 1;
+    if (info[i].view.q.k_in || info[i].view.q.k_off) bind_v[V] += 1;
     const uint8_t* wm = info[i].wm_host;
     for (uint32_t c = 0; c < cells; ++c) {
       if (wm && wm[c]) {
@@ -250,6 +270,7 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     }
   }
   std::vector<uint2> items;
+  size_t lane_words = 0;
   for (auto& kv : by_v) {
     if (kv.second.empty()) continue;  // every cell of this size is well-mixed
     ClassPlan p{};
@@ -262,6 +283,11 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     p.n_items = static_cast<uint32_t>(kv.second.size());
     const uint32_t V = kv.first;
     p.gen = (nd_v[V] == 0 && pm_v[V] > 0) ? 2 : (pm_v[V] > 0 || tr_v[V] > 0) ? 1 : 0;
+    while (p.n * p.n < V) ++p.n;
+    p.lane_model = p.gen == 2 ? 2 : bind_v[V] > 0 ? 1 : 0;
+    if (p.gen != 1) p.lane = lane_plan(V, kv.second.size(), p.lane_model);
+    p.lane_off = lane_words;
+    lane_words += ((p.lane.scratch_bytes + 255) & ~static_cast<size_t>(255)) / sizeof(uint64_t);
     items.insert(items.end(), kv.second.begin(), kv.second.end());
     b->classes.push_back(p);
   }
@@ -284,8 +310,17 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
   const size_t counters_bytes =
       (3 * sizeof(uint32_t) * b->classes.size() + 255) & ~static_cast<size_t>(255);
   const size_t total = views_bytes + items_bytes + redo_bytes + counters_bytes + io_bytes + 256;
+  if (lane_words && lib_malloc(reinterpret_cast<void**>(&b->d_lane),
+                               lane_words * sizeof(uint64_t)) != cudaSuccess) {
+    // without scratch those classes keep to the segmented kernel
+    cudaGetLastError();
+    b->d_lane = nullptr;
+    for (ClassPlan& p : b->classes)
+      if (p.lane.scratch_bytes) p.lane.G = 0;
+  }
   if (lib_malloc(reinterpret_cast<void**>(&b->dmem), total) != cudaSuccess) {
     cudaGetLastError();
+    cudaFree(b->d_lane);
     delete b;
     return TISSUE_E_NOMEM;
   }
@@ -303,6 +338,7 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
           cudaSuccess) {
     cudaGetLastError();
     if (b->h_io_steps) cudaFreeHost(b->h_io_steps);
+    cudaFree(b->d_lane);
     cudaFree(b->dmem);
     delete b;
     return TISSUE_E_NOMEM;
@@ -315,6 +351,7 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     drop_side(b);
     cudaFreeHost(b->h_io_steps);
     cudaFreeHost(b->h_io_flags);
+    cudaFree(b->d_lane);
     cudaFree(b->dmem);
     delete b;
     return TISSUE_E_CUDA;
@@ -576,6 +613,7 @@ void tissue_batch_destroy(tissue_batch* b) {
   drop_side(b);
   cudaFreeHost(b->h_io_steps);
   cudaFreeHost(b->h_io_flags);
+  cudaFree(b->d_lane);
   cudaFree(b->dmem);
   delete b;
 }

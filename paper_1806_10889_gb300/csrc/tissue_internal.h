@@ -175,6 +175,11 @@ tissue_launch default_launch(uint32_t V, uint64_t cells);
 // The default among prefix-layout launches (the fallback of a counts-only
 // launch that cannot take a tissue's model).
 tissue_launch prefix_launch(uint32_t V, uint64_t cells);
+// Consumes one armed allocation failure (see lib_malloc), if there is one.
+bool take_alloc_fault();
+// Whether (lanes, warps, layout) is a shape default_launch picks for some
+// number of cells of V voxels: such a launch is left to the library.
+bool default_shape(uint32_t V, const tissue_launch& c);
 void tissue_advance_host_step(tissue* t, uint32_t n);
 void tissue_set_host_step(tissue* t, uint32_t step_index);
 // A latched device error flag as the C ABI's status code.

@@ -11,9 +11,11 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
+#include "chi_lane.h"
 #include "tissue.h"
 #include "tissue_internal.h"
 
@@ -131,16 +133,61 @@ namespace {
 std::atomic<uint32_t> g_fail_allocs{0};
 }  // namespace
 
-cudaError_t tsg::lib_malloc(void** p, size_t bytes) {
+bool tsg::take_alloc_fault() {
   uint32_t n = g_fail_allocs.load();
-  while (n > 0) {
-    if (g_fail_allocs.compare_exchange_weak(n, n - 1)) {
-      *p = nullptr;
-      return cudaErrorMemoryAllocation;
-    }
+  while (n > 0)
+    if (g_fail_allocs.compare_exchange_weak(n, n - 1)) return true;
+  return false;
+}
+
+cudaError_t tsg::lib_malloc(void** p, size_t bytes) {
+  if (take_alloc_fault()) {
+    *p = nullptr;
+    return cudaErrorMemoryAllocation;
   }
   return cudaMalloc(p, bytes);
 }
+
+namespace {
+
+// Scratch of the sum-tree kernel for single tissues: allocated on the
+// tissue's stream for the length of one call, from one pool per device that
+// keeps freed memory (at most what ran at once: about 1.4 GB a stream) until
+// a tissue is destroyed.  Streams never wait for one another's memory.
+constexpr int kMaxDevices = 128;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+bool lane_pool(bool create, cudaMemPool_t* out) {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pool[dev] && create) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = ~0ull;
+    int off = 0;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      cudaMemPoolDestroy(pool);
+      return false;
+    }
+    g_pool[dev] = pool;
+  }
+  *out = g_pool[dev];
+  return *out != nullptr;
+}
+
+}  // namespace
 
 tissue_launch tsg::prefix_launch(uint32_t V, uint64_t cells) {
   // Up to ~1,000 cells the machine is not full and each cell's event chain
@@ -175,10 +222,55 @@ tissue_launch tsg::default_launch(uint32_t V, uint64_t cells) {
   return prefix_launch(V, cells);
 }
 
+bool tsg::default_shape(uint32_t V, const tissue_launch& c) {
+  if (c.kernel != TISSUE_KERNEL_PERSISTENT || c.blocks != 0) return false;
+  for (const uint64_t cells : {uint64_t{1}, kFewCells + 1, uint64_t{1} << 32}) {
+    const tissue_launch d = default_launch(V, cells);
+    if (c.lanes_per_cell == d.lanes_per_cell && c.warps_per_block == d.warps_per_block &&
+        c.smem_layout == d.smem_layout)
+      return true;
+  }
+  return false;
+}
+
 namespace {
 
+// The sum-tree launch of one call's steps: plan.G = 0 when the call keeps to
+// the segmented kernel (another launch shape, a trace, or no scratch to be
+// had: an allocation that fails, a stream being captured).
+struct LaneCall {
+  LanePlan plan;
+  int model = 0;
+  uint64_t* scratch = nullptr;
+  cudaStream_t stream = nullptr;
+
+  LaneCall(tissue* t, uint32_t V) : stream(t->stream) {
+    if (t->d_trace != nullptr || !default_shape(V, t->cfg)) return;
+    model = t->q.kind == kModelPromoter ? 2 : (t->q.k_in || t->q.k_off) ? 1 : 0;
+    plan = lane_plan(V, static_cast<uint64_t>(t->d.width) * t->d.height - t->wm_cells, model);
+    if (plan.G == 0 || plan.scratch_bytes == 0) return;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaMemPool_t pool = nullptr;
+    void* p = nullptr;
+    if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+        take_alloc_fault() || !lane_pool(true, &pool) ||
+        cudaMallocFromPoolAsync(&p, plan.scratch_bytes, pool, stream) != cudaSuccess) {
+      cudaGetLastError();
+      plan.G = 0;
+      return;
+    }
+    scratch = static_cast<uint64_t*>(p);
+  }
+  ~LaneCall() {
+    if (scratch) cudaFreeAsync(scratch, stream);
+  }
+  LaneCall(const LaneCall&) = delete;
+  LaneCall& operator=(const LaneCall&) = delete;
+};
+
 // chi for step offset i, in the tissue's launch configuration.
-cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, uint32_t i, double dt) {
+cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, const LaneCall& lane, uint32_t i,
+                           double dt) {
   tissue_launch c = t->cfg;
   if (c.kernel == TISSUE_KERNEL_PERSISTENT) {
     const uint32_t cells = t->d.width * t->d.height;
@@ -197,6 +289,10 @@ cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, uint32_t i, double dt
     e = cudaMemsetAsync(t->d_work, 0, 3 * sizeof(uint32_t), t->stream);
     if (e != cudaSuccess) return e;
     const ChiRedo redo{t->d_redo, t->d_work};
+    if (lane.plan.G)
+      return launch_chi_lane(lane.plan, lane.model, t->d_view,
+                             t->wm_cells ? t->d_lat_items : nullptr, cells - t->wm_cells, t->d_work,
+                             lane.scratch, redo, v.V, v.n, i, dt, t->stream);
     const bool pre = c.smem_layout == TISSUE_LAYOUT_PREFIX;
     return launch_chi_seg(t->d_view, t->wm_cells ? t->d_lat_items : nullptr, cells - t->wm_cells,
                           t->d_work, v.V, static_cast<int>(c.lanes_per_cell),
@@ -208,11 +304,11 @@ cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, uint32_t i, double dt
 
 // One splitting step at step offset i.  `mark`, if given, is recorded right
 // before and right after the chi launch (for the timed variant).
-int enqueue_split_step(tissue* t, const TissueView& v, uint32_t i, double dt, cudaEvent_t before,
-                       cudaEvent_t after) {
+int enqueue_split_step(tissue* t, const TissueView& v, const LaneCall& lane, uint32_t i, double dt,
+                       cudaEvent_t before, cudaEvent_t after) {
   auto chi = [&]() -> bool {
     if (before && cudaEventRecord(before, t->stream) != cudaSuccess) return false;
-    if (launch_chi_cfg(t, v, i, dt) != cudaSuccess) return false;
+    if (launch_chi_cfg(t, v, lane, i, dt) != cudaSuccess) return false;
     return !after || cudaEventRecord(after, t->stream) == cudaSuccess;
   };
   if (t->scheme == TISSUE_SPLIT_LIE) {
@@ -485,8 +581,9 @@ int tissue_step(tissue* t, double dt, uint32_t n_steps) {
   if (!(dt > 0.0) || !std::isfinite(dt) || !launch_fits_model(t)) return TISSUE_E_ARG;
   if (n_steps == 0) return TISSUE_OK;
   const TissueView v = view_of(t);
+  const LaneCall lane(t, v.V);
   for (uint32_t i = 0; i < n_steps; ++i) {
-    const int rc = enqueue_split_step(t, v, i, dt, nullptr, nullptr);
+    const int rc = enqueue_split_step(t, v, lane, i, dt, nullptr, nullptr);
     if (rc != TISSUE_OK) return rc;
   }
   if (launch_step_advance(t->d_step, n_steps, t->stream) != cudaSuccess) return TISSUE_E_CUDA;
@@ -505,9 +602,10 @@ int tissue_step_timed(tissue* t, double dt, uint32_t n_steps, double* ms_chi, do
   for (auto& e : ev)
     if (cudaEventCreate(&e) != cudaSuccess) rc = TISSUE_E_CUDA;
   const TissueView v = view_of(t);
+  const LaneCall lane(t, v.V);
   for (uint32_t i = 0; i < n_steps && rc == TISSUE_OK; ++i) {
     if (cudaEventRecord(ev[4 * i], t->stream) != cudaSuccess) rc = TISSUE_E_CUDA;
-    if (rc == TISSUE_OK) rc = enqueue_split_step(t, v, i, dt, ev[4 * i + 1], ev[4 * i + 2]);
+    if (rc == TISSUE_OK) rc = enqueue_split_step(t, v, lane, i, dt, ev[4 * i + 1], ev[4 * i + 2]);
     if (rc == TISSUE_OK && cudaEventRecord(ev[4 * i + 3], t->stream) != cudaSuccess)
       rc = TISSUE_E_CUDA;
   }
@@ -676,6 +774,8 @@ void tissue_destroy(tissue* t) {
   cudaStreamSynchronize(t->stream);
   if (t->d_trace_len) cudaFree(t->d_trace_len);
   cudaFree(t->scratch);
+  cudaMemPool_t pool = nullptr;
+  if (lane_pool(false, &pool)) cudaMemPoolTrimTo(pool, 0);
   delete t;
 }
 
