@@ -27,25 +27,30 @@
 // segmented kernel); cells of up to 256 voxels that fill the chip by issue
 // (32 warp instructions per event with G = 1 against 171 and 227, 8x8 and
 // 16x16 voxels); larger ones by random accesses to L2 and DRAM (a dependent
-// 64-byte read and write per lane reaches 25 G/s in DRAM, 42 G/s in L2, and an
-// event makes about three).  Chi ms per step, before -> with this kernel: 2x2
-// cells of 8x8 voxels 2.9 -> 1.53, 64x64 of 16x16 21.1 -> 10.4, 48x48 of 32x32
-// 77.5 -> 52.9, 256x256 of 8x8 33.4 -> 7.9, 256x256 of 32x32 611 -> 187.
+// read and write per lane reaches 25 G/s in DRAM, 42 G/s in L2, and an event
+// makes two).  Chi ms per step, before -> with this kernel: 2x2 cells of 8x8
+// voxels 2.9 -> 1.53, 64x64 of 16x16 21.1 -> 10.4, 48x48 of 32x32 77.5 -> 52.9,
+// 256x256 of 8x8 33.4 -> 7.9, 256x256 of 32x32 611 -> 136.
 //
 // Template parameters: MODEL 0 Notch-Delta without in-voxel binding (k_in =
 // k_off = 0), 1 Notch-Delta, 2 promoter; LV the levels of the tree (V <= 4^LV,
-// LV = 3, 4, 5); LEAF where the voxels live (chi_lane.h): in shared memory
-// (20 bytes a voxel and the sums: the shortest chain), or in a scratch array,
-// total and packed counts side by side so that a quad is one aligned 64-byte
-// block (about a hundred bytes to 2.8 KB of sums a cell stay in shared memory,
-// and hundreds of cells fit on an SM); ONE: G = 1 at compile time.
+// LV = 3, 4, 5); LEAF where the voxels live (chi_lane.h): shared memory (20
+// bytes a voxel and the sums: the shortest chain), or a scratch array with the
+// upper sums in shared memory, so that hundreds of cells fit on an SM --
+// records, total and packed counts of a voxel side by side, a quad one aligned
+// 64-byte block; or sectors, 32 bytes a quad with its sum and 16-bit counts,
+// the four quads under a shared sum one 128-byte line that an event reads
+// whole, the four totals of the chosen quad recomputed, each changed quad one
+// full sector written (256x256 cells of 32x32 voxels: 174 ms with records and a
+// level of quad sums beside them, 490 DRAM bytes an event; 128 ms with sectors);
+// ONE: G = 1 at compile time.
 //
 // Limits.  Counts below the tissue's `small` keep every total below 2^52
 // unchecked, and R below kLaneHill reads the Hill table unchecked.  With
 // shared leaves a cell past either goes on with exact checks; a packed cell
-// (20 bits a count) is left untouched and goes to the redo list, which the
-// launcher runs through the segmented kernel from the same state and random
-// streams.
+// (20 or 16 bits a count) is left untouched and goes to the redo list, which
+// the launcher runs through the segmented kernel from the same state and
+// random streams.
 #pragma once
 #include "chi_lane.h"
 #include "tissue_dev.cuh"
@@ -179,6 +184,26 @@ __device__ __forceinline__ U64x4 load4(const uint64_t* p) {
   return r;
 }
 
+__device__ __forceinline__ void store4(uint64_t* p, const U64x4& x) {
+  asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};"
+               :
+               : "l"(p), "l"(x.a), "l"(x.b), "l"(x.c), "l"(x.d)
+               : "memory");
+}
+
+// Sectors: the counts of a quad's four voxels, 16 bits each.
+__device__ __forceinline__ uint64_t pack4(const uint32_t* c) {
+  return static_cast<uint64_t>((c[0] & 0xFFFFu) | (c[1] << 16)) |
+         (static_cast<uint64_t>((c[2] & 0xFFFFu) | (c[3] << 16)) << 32);
+}
+__device__ __forceinline__ uint32_t field16(uint64_t w, uint32_t k) {
+  const uint32_t h = (k & 2u) ? static_cast<uint32_t>(w >> 32) : static_cast<uint32_t>(w);
+  return (k & 1u) ? h >> 16 : h & 0xFFFFu;
+}
+__device__ __forceinline__ uint4 unpack4(uint64_t w) {
+  return make_uint4(field16(w, 0), field16(w, 1), field16(w, 2), field16(w, 3));
+}
+
 // A voxel of the scratch array in one word: D in bits 0..19, N in 20..39, R
 // in 40..59, the neighbour mask in 60..63.
 __device__ __forceinline__ uint64_t pack_voxel(uint32_t D, uint32_t N, uint32_t R, uint32_t mask) {
@@ -214,13 +239,13 @@ constexpr uint32_t kEvBind = 5u, kEvRelease = 6u, kEvHop = 8u;  // 0..4: channel
 template <int MODEL, int LV, int LEAF, bool ONE>
 __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ? 7 : 14) k_chi_lane(const LaneArgs p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  static_assert(!ONE || LEAF != kLeafShared, "one lane per cell: records or nodes");
+  static_assert(!ONE || LEAF != kLeafShared, "one lane per cell: leaves in the scratch array");
   constexpr bool REC = LEAF != kLeafShared;   // voxels in the scratch array, packed
-  constexpr bool NODE8 = LEAF == kLeafNodes;  // with the quads' sums, eight to a node
+  constexpr bool SEC = LEAF == kLeafSectors;  // ... as counts and quad sums, no voxel totals
   constexpr uint32_t NQ = 1u << (2 * (LV - 1));  // quads of a full tree
-  // levels kept in shared memory above the quads' sums (NODE8: 2, 8, 32
-  // entries), or down to them
-  constexpr int SL = NODE8 ? LV - 2 : LV - 1;
+  // the levels of sums in shared memory: down to the quads' (sectors: down to
+  // those of four quads)
+  constexpr int SL = SEC ? LV - 2 : LV - 1;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const uint32_t G = ONE ? 1u : p.G;
   const uint32_t slot = ONE ? lane : lane / G, sl = ONE ? 0u : lane % G;
@@ -246,7 +271,8 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
                                       : d == 2 ? -static_cast<int>(n)
                                                : static_cast<int>(n));
   }
-  for (uint32_t v = threadIdx.x; v < nq * 4u; v += blockDim.x) {
+  const uint32_t nl = (nq + 3u) >> 2;  // lines of four quads (sectors)
+  for (uint32_t v = threadIdx.x; v < (SEC ? nl * 16u : nq * 4u); v += blockDim.x) {
     const uint32_t vy = v / n, vx = v - vy * n;
     const uint32_t m = static_cast<uint32_t>(vx > 0) | (static_cast<uint32_t>(vx < n - 1) << 1) |
                        (static_cast<uint32_t>(vy > 0) << 2) |
@@ -264,10 +290,9 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
   uint64_t* tree = reinterpret_cast<uint64_t*>(cs + 48);
   constexpr uint32_t kCnt = level_off(LV);  // shared leaves: entry of the voxel totals
   int32_t* cp = reinterpret_cast<int32_t*>(tree + kCnt + ps);
-  // a cell's scratch: NODE8 its quad sums, 256 of them; then 2 words per voxel,
-  // its total and its counts
-  constexpr uint32_t kNodeWords = NODE8 ? 256u : 0u;
-  const uint32_t rec_words = kNodeWords + 8u * nq;
+  // a cell's scratch: 2 words per voxel, its total and its counts (records);
+  // or 4 words per quad, its sum and its counts of D, N and R (sectors)
+  const uint32_t rec_words = SEC ? 16u * nl : 8u * nq;
   uint64_t* warp_rec =
       REC ? p.scratch + (static_cast<size_t>(blockIdx.x) * (blockDim.x >> 5) + wib) * slots * rec_words
           : nullptr;
@@ -279,6 +304,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
   bool have = false, done = false;
   uint32_t cell = 0, vidx = 0, step = 0, word3 = 0, key0 = 0, key1 = 0, e0 = 0;
   uint64_t A = 0, over_mask = 0;
+  uint32_t lim_dn = 0, lim_r = 0;  // sectors: the counts' limits
   double tnow = 0.0;
   int err = 0;
   uint32_t lim = 0;
@@ -353,15 +379,17 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
               }
               if (REC) {
                 // past the packed word's range: to the redo list
-                nbig |= (d[i] | m[i]) >= kWordCount;
+                nbig |= (d[i] | m[i]) >= (SEC ? kSectorCount : kWordCount);
                 wd[i] = pack_voxel(d[i], m[i], r[i] & 0xFFFFFu, mk & 15u);
               }
               a[i] = lane_total<MODEL>(nr, ntv, d[i], m[i], r[i], nn, ctr);
             }
             S += a[i];
           }
-          if (REC) {
-            ulonglong2* o = reinterpret_cast<ulonglong2*>(nrec + kNodeWords) + 4u * qi;
+          if (SEC) {
+            store4(nrec + 4u * qi, U64x4{S, pack4(d), pack4(m), pack4(r)});
+          } else if (REC) {
+            ulonglong2* o = reinterpret_cast<ulonglong2*>(nrec) + 4u * qi;
 #pragma unroll
             for (int i = 0; i < 4; ++i) o[i] = make_ulonglong2(a[i], wd[i]);
           } else {
@@ -372,35 +400,23 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
             reinterpret_cast<uint4*>(ncp + ps)[qi] = make_uint4(m[0], m[1], m[2], m[3]);
             reinterpret_cast<uint4*>(ncp + 2u * ps)[qi] = make_uint4(r[0], r[1], r[2], r[3]);
           }
+        } else if (SEC && qi < 4u * nl) {
+          store4(nrec + 4u * qi, U64x4{0ull, 0ull, 0ull, 0ull});
         }
         // the sums above the quads (entries past the last quad are zero)
-        if (NODE8) {
-          nrec[qi] = S;
-          uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
-          x += __shfl_xor_sync(kFull, x, 2);
-          x += __shfl_xor_sync(kFull, x, 4);
-          if ((lane & 7) == 0) ntree[10u + (qi >> 3)] = x;  // 32 sums of 8 quads
-          x += __shfl_xor_sync(kFull, x, 8);
-          x += __shfl_xor_sync(kFull, x, 16);
-          if (lane == 0) ntree[2u + (qi >> 5)] = x;         // 8 sums of 32
-          total += x;
-          if ((k & 3u) == 3u && lane == 0) ntree[k >> 2] = (k == 3u) ? total : total - pair;
-          if (k == 3u) pair = total;
-        } else {
-          if (qi < NQ) ntree[level_off(LV - 1) + qi] = S;
-          uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
-          x += __shfl_xor_sync(kFull, x, 2);
-          if (qi < NQ && (lane & 3) == 0) ntree[level_off(LV - 2) + (qi >> 2)] = x;
-          x += __shfl_xor_sync(kFull, x, 4);
-          x += __shfl_xor_sync(kFull, x, 8);
-          if (LV >= 4 && (lane & 15) == 0) ntree[level_off(LV >= 4 ? LV - 3 : 1) + (qi >> 4)] = x;
-          x += __shfl_xor_sync(kFull, x, 16);
-          if (LV == 5) {
-            pair = (k & 1u) ? pair + x : x;
-            if ((k & 1u) && lane == 0) ntree[k >> 1] = pair;
-          }
-          total += x;
+        if (!SEC && qi < NQ) ntree[level_off(LV - 1) + qi] = S;
+        uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
+        x += __shfl_xor_sync(kFull, x, 2);
+        if (qi < NQ && (lane & 3) == 0) ntree[level_off(LV - 2) + (qi >> 2)] = x;
+        x += __shfl_xor_sync(kFull, x, 4);
+        x += __shfl_xor_sync(kFull, x, 8);
+        if (LV >= 4 && (lane & 15) == 0) ntree[level_off(LV >= 4 ? LV - 3 : 1) + (qi >> 4)] = x;
+        x += __shfl_xor_sync(kFull, x, 16);
+        if (LV == 5) {
+          pair = (k & 1u) ? pair + x : x;
+          if ((k & 1u) && lane == 0) ntree[k >> 1] = pair;
         }
+        total += x;
       }
       const bool any_ovf = __any_sync(kFull, ovf), any_bad = __any_sync(kFull, bad_state);
       nbig = __any_sync(kFull, nbig);
@@ -422,9 +438,11 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         have = true;
         if (REC) {
           // the bits a count has once it reaches its limit (a power of two)
-          const uint32_t lc = min(q.small, kWordCount), lr = MODEL == 2 ? lc : min(q.small, kLaneHill);
+          const uint32_t lc = min(q.small, SEC ? kSectorCount : kWordCount), lr = MODEL == 2 ? lc : min(q.small, kLaneHill);
           const uint32_t mc = 0xFFFFFu & ~(lc - 1u), mr = 0xFFFFFu & ~(lr - 1u);
           over_mask = pack_voxel(mc, mc, mr, 0u);
+          lim_dn = lc;
+          lim_r = lr;
         }
       }
     }
@@ -448,39 +466,60 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
       uint64_t r = __umul64hi(R64, A);
       // descent to a quad
       uint32_t idx = 0;
-      if (NODE8) {
-        const uint64_t s0 = tree[0];
-        idx = r >= s0 ? 1u : 0u;
-        r -= idx ? s0 : 0ull;
 #pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + (l ? 10u : 2u)) + 2u * idx;
-          const ulonglong2 x = nd[0], y = nd[1];
-          idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
-        }
-        // eight quad sums: the half, then the quad
-        const U64x4 x = load4(rec + 8u * idx), y = load4(rec + 8u * idx + 4u);
-        const uint64_t half = (x.a + x.b) + (x.c + x.d);
-        const bool up = r >= half;
-        r -= up ? half : 0ull;
-        idx = 8u * idx + (up ? 4u : 0u) +
-              pick_child<!ONE>(up ? y.a : x.a, up ? y.b : x.b, up ? y.c : x.c, r);
-      } else {
-#pragma unroll
-        for (uint32_t l = 1; l < LV; ++l) {
-          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) + 2u * idx;
-          const ulonglong2 x = nd[0], y = nd[1];
-          idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
-        }
+      for (uint32_t l = 1; l <= SL; ++l) {
+        const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) + 2u * idx;
+        const ulonglong2 x = nd[0], y = nd[1];
+        idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+      }
+      U64x4 sec{};  // sectors: the quad's sum and its counts of D, N and R
+      if (SEC) {
+        idx = min(idx, nl - 1u);
+        const uint64_t* line = rec + 16u * idx;
+        const U64x4 x0 = load4(line), x1 = load4(line + 4), x2 = load4(line + 8),
+                    x3 = load4(line + 12);
+        const uint32_t k = pick_child<!ONE>(x0.a, x1.a, x2.a, r);
+        idx = 4u * idx + k;
+        sec.a = k == 0u ? x0.a : k == 1u ? x1.a : k == 2u ? x2.a : x3.a;
+        sec.b = k == 0u ? x0.b : k == 1u ? x1.b : k == 2u ? x2.b : x3.b;
+        sec.c = k == 0u ? x0.c : k == 1u ? x1.c : k == 2u ? x2.c : x3.c;
+        sec.d = k == 0u ? x0.d : k == 1u ? x1.d : k == 2u ? x2.d : x3.d;
       }
       if (kChecked && run && idx >= nq) err |= kErrBounds;
       idx = min(idx, nq - 1u);  // never past the cell's quads, whatever the sums hold
       // the voxel, its total, counts and neighbours
       uint64_t a_v, w_v = 0;
       uint32_t v, D, N, R, mask, nn;
-      if (REC) {
-        const U64x4 x = load4(rec + kNodeWords + 8u * idx);
-        const U64x4 y = load4(rec + kNodeWords + 8u * idx + 4u);
+      if (SEC) {
+        const uint32_t mk4 = *reinterpret_cast<const uint32_t*>(lut + 4u * idx);
+        uint64_t a[4];
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j) {
+          const uint32_t Dj = field16(sec.b, j), Nj = field16(sec.c, j), Rj = field16(sec.d, j);
+          const uint32_t nj = (mk4 >> (8u * j + 4u)) & 7u;
+          uint64_t t = (q.gD + q.hD * nj) * Dj + (q.gN + q.hN * nj) * Nj;
+          if (MODEL == 2) {
+            const uint32_t F = static_cast<uint32_t>(4u * idx + j == centre) - Rj;
+            t += q.tD * F + q.kd * Rj + q.k_in * (static_cast<uint64_t>(Nj) * F);
+          } else {
+            // R < kLaneHill in a cell that runs; the mask is for idle lanes
+            t += (q.gR + q.k_off + q.hR * nj) * Rj + __ldg(q.hill + (Rj & (kHillTab - 1u))) + q.kN;
+            if (MODEL == 1) t += q.k_in * (static_cast<uint64_t>(Dj) * Nj);
+          }
+          a[j] = t;
+        }
+        const uint32_t k = pick_child<!ONE>(a[0], a[1], a[2], r);
+        a_v = k == 0u ? a[0] : k == 1u ? a[1] : k == 2u ? a[2] : a[3];
+        v = 4u * idx + k;
+        D = field16(sec.b, k);
+        N = field16(sec.c, k);
+        R = field16(sec.d, k);
+        const uint32_t mk = (mk4 >> (8u * k)) & 0xFFu;
+        mask = mk & 15u;
+        nn = mk >> 4;
+      } else if (REC) {
+        const U64x4 x = load4(rec + 8u * idx);
+        const U64x4 y = load4(rec + 8u * idx + 4u);
         const uint32_t k = pick_child<!ONE>(x.a, x.c, y.a, r);
         a_v = k == 0u ? x.a : k == 1u ? x.c : k == 2u ? y.a : y.c;
         w_v = k == 0u ? x.b : k == 1u ? x.d : k == 2u ? y.b : y.d;
@@ -584,8 +623,20 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
       }
       uint32_t cu = 0;
       uint64_t a_u = 0, w_u = 0;
-      if (REC) {
-        const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec + kNodeWords)[u];
+      U64x4 su{};  // sectors: u's quad
+      if (SEC) {
+        su = load4(rec + 4u * (u >> 2));
+        const uint32_t k = u & 3u;
+        cu = (s == 0u ? field16(su.b, k) : s == 1u ? field16(su.c, k) : field16(su.d, k)) + 1u;
+        if (hop) {
+          du = gh.x + gh.y * (lut[u] >> 4);
+          if (MODEL == 1 && s < 2u)
+            du += q.k_in * (s == 0u ? field16(su.c, k) : field16(su.b, k));
+          if (MODEL == 2 && s == 1u)
+            du += q.k_in * (static_cast<uint32_t>(u == centre) - field16(su.d, k));
+        }
+      } else if (REC) {
+        const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec)[u];
         a_u = x.x;
         w_u = x.y;
         if (hop) {
@@ -606,7 +657,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         }
       }
       if (MODEL != 2 && s == 2u && run) {  // R changes the Hill term, here and where it arrives
-        const uint32_t Ru = hop ? (REC ? word_R(w_u) + 1u : cu) : 1u;
+        const uint32_t Ru = hop ? (REC && !SEC ? word_R(w_u) + 1u : cu) : 1u;
         if (!slow) {  // every count is inside the table
           if (MODEL == 0) dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
           const uint64_t d = __ldg(q.hill + Ru) - __ldg(q.hill + (Ru - 1u));
@@ -623,29 +674,16 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         uint64_t nv[LV], nu[LV];
 #pragma unroll
         for (uint32_t l = 1; l <= SL; ++l) {
-          const uint32_t sh = NODE8 ? (l == 1 ? 9u : l == 2 ? 7u : 5u) : 2u * (LV - l);
-          const uint32_t o = NODE8 ? (l == 1 ? 0u : l == 2 ? 2u : 10u) : level_off(l);
-          const uint32_t iv = v >> sh, iu = u >> sh;
-          nv[l] = tree[o + iv] + dv + (iv == iu ? du : 0ull);
-          nu[l] = tree[o + iu] + du;
-        }
-        if (NODE8) {
-          const uint32_t iv = v >> 2, iu = u >> 2;
-          nv[0] = rec[iv] + dv + (iv == iu ? du : 0ull);
-          nu[0] = rec[iu] + du;
+          const uint32_t iv = v >> (2u * (LV - l)), iu = u >> (2u * (LV - l));
+          nv[l] = tree[level_off(l) + iv] + dv + (iv == iu ? du : 0ull);
+          nu[l] = tree[level_off(l) + iu] + du;
         }
         if (run) {
 #pragma unroll
           for (uint32_t l = 1; l <= SL; ++l) {
-            const uint32_t sh = NODE8 ? (l == 1 ? 9u : l == 2 ? 7u : 5u) : 2u * (LV - l);
-            const uint32_t o = NODE8 ? (l == 1 ? 0u : l == 2 ? 2u : 10u) : level_off(l);
-            const uint32_t iv = v >> sh, iu = u >> sh;
-            tree[o + iv] = nv[l];
-            if (iv != iu) tree[o + iu] = nu[l];
-          }
-          if (NODE8) {
-            rec[v >> 2] = nv[0];
-            if ((v >> 2) != (u >> 2)) rec[u >> 2] = nu[0];
+            const uint32_t iv = v >> (2u * (LV - l)), iu = u >> (2u * (LV - l));
+            tree[level_off(l) + iv] = nv[l];
+            if (iv != iu) tree[level_off(l) + iu] = nu[l];
           }
         }
       } else {
@@ -654,32 +692,53 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         const uint64_t dme = odd ? du : dv, dot = odd ? 0ull : du;
         __syncwarp();
         // level LV of the tree: the voxel totals themselves (shared leaves)
-        constexpr uint32_t kTasks = 2u * (NODE8 ? SL + 1 : REC ? SL : LV);
+        constexpr uint32_t kTasks = 2u * (REC ? SL : LV);
         for (uint32_t t = sl; t < kTasks; t += G) {
           const uint32_t l = (t >> 1) + 1u;
-          const uint32_t sh = !NODE8   ? 2u * (LV - l)
-                              : l == 4 ? 2u
-                              : l == 1 ? 9u
-                              : l == 2 ? 7u
-                                       : 5u;
-          const uint32_t o = NODE8 ? (l == 1 ? 0u : l == 2 ? 2u : 10u) : level_off(l);
-          const uint32_t i1 = me >> sh, i2 = other >> sh;
-          uint64_t* at = (NODE8 && l == 4) ? rec + i1 : tree + o + i1;
+          const uint32_t i1 = me >> (2u * (LV - l)), i2 = other >> (2u * (LV - l));
+          uint64_t* at = tree + level_off(l) + i1;
           const bool same = i1 == i2;
           if (run && !(odd && same)) *at += dme + (same ? dot : 0ull);
         }
       }
       // the two voxels
-      if (REC) {
+      if (SEC) {
+        const uint64_t at = 1ull << (16u * (v & 3u)), to = hop ? 1ull << (16u * (u & 3u)) : 0ull;
+        const uint64_t to0 = s == 0u ? to : 0ull, to1 = s == 1u ? to : 0ull;
+        const uint64_t to2 = s == 2u ? to : 0ull;
+        uint64_t c0, c1, c2;  // the changes at v
+        if (MODEL == 0) {
+          const uint64_t c = gain ? at : 0ull - at;
+          c0 = s == 0u ? c : 0ull;
+          c1 = s == 1u ? c : 0ull;
+          c2 = s == 2u ? c : 0ull;
+        } else {
+          c0 = dD > 0 ? at : dD < 0 ? 0ull - at : 0ull;
+          c1 = dN > 0 ? at : dN < 0 ? 0ull - at : 0ull;
+          c2 = dR > 0 ? at : dR < 0 ? 0ull - at : 0ull;
+        }
+        const bool same = (v >> 2) == (u >> 2);
+        if (run && (ONE || sl == 0u))
+          store4(rec + 4u * (v >> 2),
+                 same ? U64x4{sec.a + dv + du, sec.b + c0 + to0, sec.c + c1 + to1, sec.d + c2 + to2}
+                      : U64x4{sec.a + dv, sec.b + c0, sec.c + c1, sec.d + c2});
+        if (move && !same && (ONE || sl == 1u))
+          store4(rec + 4u * (u >> 2), U64x4{su.a + du, su.b + to0, su.c + to1, su.d + to2});
+        const uint32_t lim_s = s == 2u ? lim_r : lim_dn;
+        bool over = hop && cu >= lim_s;
+        if (MODEL == 0) over = over || nc >= lim_s;
+        else over = over || max(D + dD, N + dN) >= lim_dn || R + dR >= lim_r;
+        if (run && over) err |= kErrNarrow;
+      } else if (REC) {
         const uint64_t one = word_unit(s);
         const uint64_t wv2 = MODEL == 0 ? (gain ? w_v + one : w_v - one)
                                         : pack_voxel(D + dD, N + dN, R + dR, mask);
         const uint64_t wu2 = w_u + one;
         if (run && (ONE || sl == 0u)) {
-          reinterpret_cast<ulonglong2*>(rec + kNodeWords)[v] = make_ulonglong2(a_v + dv, wv2);
+          reinterpret_cast<ulonglong2*>(rec)[v] = make_ulonglong2(a_v + dv, wv2);
         }
         if (move && (ONE || sl == 1u)) {
-          reinterpret_cast<ulonglong2*>(rec + kNodeWords)[u] = make_ulonglong2(a_u + du, wu2);
+          reinterpret_cast<ulonglong2*>(rec)[u] = make_ulonglong2(a_u + du, wu2);
         }
         if (run && (((wv2 | (hop ? wu2 : 0ull)) & over_mask) != 0ull)) err |= kErrNarrow;
       } else {
@@ -773,8 +832,13 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
             d[code == 4u ? 2u : (code & 1u)] = code <= 1u ? -1 : 1;
             if (MODEL == 2 && code == 1u) d[2] = 1;
           }
-          if (REC) {
-            uint64_t* base = rec + kNodeWords + 1u;
+          if (SEC) {
+            uint64_t* qv = rec + 4u * (v >> 2) + 1u;
+            for (uint32_t k = 0; k < 3u; ++k)
+              qv[k] += static_cast<uint64_t>(static_cast<int64_t>(d[k])) << (16u * (v & 3u));
+            if (s < 3u) rec[4u * (u >> 2) + 1u + s] -= 1ull << (16u * (u & 3u));
+          } else if (REC) {
+            uint64_t* base = rec + 1u;
             uint64_t& wv = base[2u * v];
             wv = pack_voxel(word_D(wv) + d[0], word_N(wv) + d[1], word_R(wv) + d[2], word_mask(wv));
             if (s < 3u) base[2u * u] -= word_unit(s);
@@ -803,8 +867,23 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         const uint32_t c = __shfl_sync(kFull, cell, src);
         const uint32_t vi = __shfl_sync(kFull, vidx, src);
         int32_t* g = p.views[vi].counts + static_cast<size_t>(c) * 3u * V;
-        if (REC) {
-          const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words + kNodeWords;
+        if (SEC) {
+          const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words;
+          if (vec) {
+            for (uint32_t i = lane; i < nq; i += 32u) {
+              const U64x4 x = load4(from + 4u * i);
+              reinterpret_cast<uint4*>(g)[i] = unpack4(x.b);
+              reinterpret_cast<uint4*>(g + V)[i] = unpack4(x.c);
+              reinterpret_cast<uint4*>(g + 2u * V)[i] = unpack4(x.d);
+            }
+          } else {
+            for (uint32_t i = lane; i < V; i += 32u)
+              for (uint32_t sp = 0; sp < 3u; ++sp)
+                g[sp * V + i] =
+                    static_cast<int32_t>(field16(from[4u * (i >> 2) + 1u + sp], i & 3u));
+          }
+        } else if (REC) {
+          const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words;
           if (vec) {
             for (uint32_t i = lane; i < nq; i += 32u) {
               const U64x4 x = load4(from + 8u * i), y = load4(from + 8u * i + 4u);

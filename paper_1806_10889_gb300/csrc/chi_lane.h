@@ -7,10 +7,11 @@ namespace tsg {
 constexpr int kMaxSmem = 227 * 1024;  // dynamic shared memory a block may ask for
 // Where a cell's voxels live during the step.
 constexpr int kLeafShared = 0;   // shared memory: totals and 32-bit counts
-constexpr int kLeafRecords = 1;  // the scratch array, packed; every sum in shared memory
-constexpr int kLeafNodes = 2;    // the scratch array, with the lowest level of the sums
+constexpr int kLeafRecords = 1;  // scratch array: 64 bytes a quad, totals and packed counts
+constexpr int kLeafSectors = 2;  // scratch array: 32 bytes a quad, its sum and 16-bit counts
 constexpr uint32_t kLaneHill = 2048;  // R below this reads the Hill table unchecked (R + 1 too)
-constexpr uint32_t kWordCount = 1u << 19;  // counts a packed voxel holds stay below
+constexpr uint32_t kWordCount = 1u << 19;    // counts of a record stay below
+constexpr uint32_t kSectorCount = 1u << 16;  // counts of a sector
 
 struct LaneArgs {
   const TissueView* views;

@@ -5,22 +5,18 @@
 namespace tsg {
 
 ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, bool one) {
-  // one lane per cell never takes shared leaves: past 110 cells an SM records
-  // are as fast or faster
-  if (V <= 64) {
-    if (leaf == kLeafRecords) return one ? k_chi_lane<0, 3, kLeafRecords, true> : nullptr;
-    return leaf == kLeafShared && !one ? k_chi_lane<0, 3, kLeafShared, false> : nullptr;
-  }
-  if (V <= 256) {
-    if (leaf == kLeafRecords)
-      return one ? k_chi_lane<0, 4, kLeafRecords, true> : k_chi_lane<0, 4, kLeafRecords, false>;
-    return leaf == kLeafShared && !one ? k_chi_lane<0, 4, kLeafShared, false> : nullptr;
-  }
-  if (leaf == kLeafNodes)
-    return one ? k_chi_lane<0, 5, kLeafNodes, true> : k_chi_lane<0, 5, kLeafNodes, false>;
-  if (one) return nullptr;
-  return leaf == kLeafRecords ? k_chi_lane<0, 5, kLeafRecords, false>
-                              : k_chi_lane<0, 5, kLeafShared, false>;
+  const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
+  if (leaf == kLeafShared && !one)
+    return lv == 3   ? k_chi_lane<0, 3, kLeafShared, false>
+           : lv == 4 ? k_chi_lane<0, 4, kLeafShared, false>
+                     : k_chi_lane<0, 5, kLeafShared, false>;
+  if (leaf == kLeafRecords && lv == 3 && one) return k_chi_lane<0, 3, kLeafRecords, true>;
+  if (leaf == kLeafRecords && lv == 4 && !one) return k_chi_lane<0, 4, kLeafRecords, false>;
+  if (leaf == kLeafRecords && lv == 5 && !one) return k_chi_lane<0, 5, kLeafRecords, false>;
+  if (leaf == kLeafSectors && lv == 4 && one) return k_chi_lane<0, 4, kLeafSectors, true>;
+  if (leaf == kLeafSectors && lv == 5)
+    return one ? k_chi_lane<0, 5, kLeafSectors, true> : k_chi_lane<0, 5, kLeafSectors, false>;
+  return nullptr;
 }
 
 namespace {
@@ -35,21 +31,22 @@ ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, bool one) {
 
 // The shape follows from the cells an SM holds, per.  Chi ms of one step at
 // dt 0.02 (8x8 and 16x16 voxels) and 0.006 (32x32), 60 D + 30 N + 10 R per
-// voxel, by lanes per cell G and leaf (S shared, R records, N nodes), with the
-// best segmented launch in brackets:
+// voxel, by leaf (S shared, R records, X sectors) and lanes per cell, with the
+// segmented kernel's default launch in brackets:
 //   per     8x8                          16x16                        32x32
 //    4  S32 .37 S16 .42 [.70]   S32 1.44 S16 1.58 [2.65]     S32 1.91 S16 2.10 [3.2]
 //    8  S32 .43 S16 .43 [.83]   S16 1.59 S32 1.64 [2.89]     S16 2.09 S32 2.16 [3.5]
 //   13  S16 .46 S8 .48  [.85]   S8 1.74 S16 1.82  [3.18]  15 R16 3.35 R8 3.75  [4.9]
 //   27  S8 .55 S4 .62   [.93]   S8 2.04 S4 2.30 R8 2.80 [4.18]  R8 4.05 R16 4.19 [6.7]
-//   60  R4 .73 S4 .73   [1.2]   R8 3.79 R4 3.90   [6.20]  53 R8 5.14 R4 5.58   [12.0]
-//   80  R4 .84 S4 .85   [2.0]   R4 4.27 R1 4.66   [9.67]  75 R4 6.39 R1 7.9    [16.5]
-//  108  R4 1.01 S2 1.02 [2.2]   R1 4.76 R4 4.80   [11.1]     N4 9.08 N1 10.1   [22.2]
-//  150  R1 1.35 R2 1.35 [2.9]   R1 5.26 R2 5.76   [15.1]     N1 11.3 N2 11.9   [30.1]
-//  431  R1 2.03 R2 2.83 [7.3]   R1 11.4 R2 12.9   [39.4]     N2 25.4 N1 25.9   [82.7]
+//   60  S4 .73          [1.2]   X4 3.67 R8 3.79 R4 3.90 [6.20] 53 R8 5.1 X4 5.5 [12.0]
+//   80  S4 .85          [2.0]   R4 4.33 X4 4.64   [9.67]  75 X4 6.7 X1 7.6 R8 8.6 [16.5]
+//  108  S4 1.05         [2.2]   X1 4.75 R4 4.84   [11.1]     X4 8.2 X1 8.6     [22.2]
+//  150  R1 1.35 S4 1.50 [2.9]   R1 5.3 X1 5.7     [15.1]     X1 9.6 X2 9.6     [30.1]
+//  431  R1 2.03 X1 2.7  [7.3]   X1 9.7 R1 11.7    [39.4]     X1 19.2 X2 20.6   [82.7]
 // Few cells: one chain of events sets the time, and more lanes per cell take
 // more of the draws off it.  Many: the instructions issued per event do, and
-// one lane per cell issues the fewest.
+// one lane per cell issues the fewest; past L2's size the random accesses to
+// DRAM do, and a sector makes two reads and two writes an event.
 LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   LanePlan pl;
   int dev = 0, sms = 0;
@@ -58,23 +55,29 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
     return pl;
   const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
   const uint64_t per = (cells + static_cast<uint64_t>(sms) - 1) / static_cast<uint64_t>(sms);
-  pl.G = per <= 4 ? 32u : per <= (lv == 5 ? 22u : 12u) ? 16u : per <= 56 ? 8u : per <= 110 ? 4u : 1u;
-  // Leaves: in shared memory while one wave of cells fits there; else records,
-  // and past one wave of those (32x32 voxels, 2.7 KB of sums a cell) nodes.
+  pl.G = per <= 4                      ? 32u
+         : per <= (lv == 5 ? 22u : 12u) ? 16u
+         : per <= 56                    ? 8u
+         : per <= (lv == 3 ? 110u : 100u) ? 4u
+                                          : 1u;
+  // Leaves: in shared memory while one wave of cells fits there (the shortest
+  // chain); else records, whose totals need no recomputing; past L2's size, or
+  // where their sums (2.7 KB a cell of 32x32 voxels) would leave SMs short of
+  // cells, sectors, half the bytes and a quarter of the sums.
   constexpr uint64_t kWave = 216 * 1024;  // an SM's shared memory less what blocks reserve
   const uint32_t nq = (V + 3u) / 4u;
   const uint32_t sums = 48u + (lv == 3 ? 160u : lv == 4 ? 672u : 2720u);
   const uint32_t shared = sums + 20u * 4u * nq;
-  pl.leaf = pl.G > 1 && per * shared <= kWave   ? kLeafShared
-            : lv < 5 || per * sums <= kWave     ? kLeafRecords
-                                                : kLeafNodes;
+  pl.leaf = pl.G > 1 && per * shared <= kWave       ? kLeafShared
+            : lv == 3 || (lv == 4 && pl.G > 1) || (lv == 5 && pl.G > 4) ? kLeafRecords
+                                                                     : kLeafSectors;
   const uint32_t raw = pl.leaf == kLeafShared    ? shared
                        : pl.leaf == kLeafRecords ? sums
-                                                 : 48u + 42u * 8u;
+                                                 : 48u + (lv == 4 ? 160u : 672u);
   // an odd multiple of 16 bytes: lanes reading the same entry of their cells
   // start on different shared-memory banks
   pl.cell_stride = ((raw + 15u) & ~15u) | 16u;
-  pl.lut_bytes = 128u + ((4u * nq + 15u) & ~15u);
+  pl.lut_bytes = 128u + 16u * ((nq + 3u) / 4u);
   pl.wpb = pl.G == 1 ? 2u : 1u;
   pl.smem = pl.lut_bytes + static_cast<size_t>(pl.wpb) * (32u / pl.G) * pl.cell_stride;
   const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G == 1);
@@ -96,7 +99,8 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   pl.blocks = static_cast<uint32_t>(need < cap ? need : cap);
   if (pl.leaf != kLeafShared)
     pl.scratch_bytes = static_cast<size_t>(pl.blocks) * per_block *
-                       (8u * nq + (pl.leaf == kLeafNodes ? 256u : 0u)) * sizeof(uint64_t);
+                       (pl.leaf == kLeafRecords ? 8u * nq : 16u * ((nq + 3u) / 4u)) *
+                       sizeof(uint64_t);
   return pl;
 }
 

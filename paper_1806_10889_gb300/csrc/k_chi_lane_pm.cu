@@ -5,20 +5,18 @@
 namespace tsg {
 
 ChiLaneKernel chi_lane_kernel_pm(uint32_t V, int leaf, bool one) {
-  if (V <= 64) {
-    if (leaf == kLeafRecords) return one ? k_chi_lane<2, 3, kLeafRecords, true> : nullptr;
-    return leaf == kLeafShared && !one ? k_chi_lane<2, 3, kLeafShared, false> : nullptr;
-  }
-  if (V <= 256) {
-    if (leaf == kLeafRecords)
-      return one ? k_chi_lane<2, 4, kLeafRecords, true> : k_chi_lane<2, 4, kLeafRecords, false>;
-    return leaf == kLeafShared && !one ? k_chi_lane<2, 4, kLeafShared, false> : nullptr;
-  }
-  if (leaf == kLeafNodes)
-    return one ? k_chi_lane<2, 5, kLeafNodes, true> : k_chi_lane<2, 5, kLeafNodes, false>;
-  if (one) return nullptr;
-  return leaf == kLeafRecords ? k_chi_lane<2, 5, kLeafRecords, false>
-                              : k_chi_lane<2, 5, kLeafShared, false>;
+  const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
+  if (leaf == kLeafShared && !one)
+    return lv == 3   ? k_chi_lane<2, 3, kLeafShared, false>
+           : lv == 4 ? k_chi_lane<2, 4, kLeafShared, false>
+                     : k_chi_lane<2, 5, kLeafShared, false>;
+  if (leaf == kLeafRecords && lv == 3 && one) return k_chi_lane<2, 3, kLeafRecords, true>;
+  if (leaf == kLeafRecords && lv == 4 && !one) return k_chi_lane<2, 4, kLeafRecords, false>;
+  if (leaf == kLeafRecords && lv == 5 && !one) return k_chi_lane<2, 5, kLeafRecords, false>;
+  if (leaf == kLeafSectors && lv == 4 && one) return k_chi_lane<2, 4, kLeafSectors, true>;
+  if (leaf == kLeafSectors && lv == 5)
+    return one ? k_chi_lane<2, 5, kLeafSectors, true> : k_chi_lane<2, 5, kLeafSectors, false>;
+  return nullptr;
 }
 
 }  // namespace tsg

@@ -1,6 +1,6 @@
 """The sum-tree chi kernel in every form its launch plan picks -- 32 to 1
-lanes per cell, leaves in shared memory, in packed records or in records with
-nodes -- against the oracle, bit for bit: counts, per-cell event counts and
+lanes per cell, leaves in shared memory, in packed records or in sectors --
+against the oracle, bit for bit: counts, per-cell event counts and
 binary64 times.  The plan follows from the cell size and the cells per SM, so
 the tissues here are just wide enough, with cells of ragged sizes.  Some
 cells hold counts past what the packed records and the unchecked Hill lookups
@@ -60,10 +60,10 @@ def _compare(g, spec, ref, ne, tl, ctx):
     assert np.array_equal(gtl.view(np.uint64), tl.view(np.uint64)), f"{ctx}: event times"
 
 
-# (cells per SM, n): shared leaves at 32, 16, 8 and 4 lanes; records at 8, 4
-# and 1; nodes at 4 and 1 (V = 4, 25, 64, 81, 256, 289 and 1,024)
+# (cells per SM, n, dt): shared leaves at 32, 16, 8 and 4 lanes; records at 16,
+# 8, 4 and 1; sectors at 4 and 1 (V = 4, 25, 49, 64, 81, 256, 289, 324 and 1,024)
 FORMS = [(1, 2, 0.3), (8, 5, 0.1), (20, 7, 0.1), (100, 5, 0.02), (8, 16, 0.02), (30, 9, 0.02),
-         (45, 16, 0.01), (105, 9, 0.01), (120, 2, 0.1), (120, 8, 0.01), (120, 9, 0.01),
+         (45, 16, 0.01), (98, 9, 0.01), (120, 2, 0.1), (120, 8, 0.01), (120, 9, 0.01),
          (3, 17, 0.02), (9, 18, 0.02), (30, 17, 0.01), (85, 17, 0.005), (112, 17, 0.005),
          (2, 32, 0.01), (16, 32, 0.005)]
 
