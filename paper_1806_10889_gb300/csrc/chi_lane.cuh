@@ -1,13 +1,17 @@
 // K_chi, sum-tree form: the intracellular module chi (arXiv 1806.10889,
 // Sec. II-A1) over a work list of cells, G = 1..32 lanes of a warp per cell.
 //
-// Every cell keeps a tree of propensity sums, four children per node: the
-// voxel totals are the leaves, S_{LV-1}[q] the total of the four voxels of
-// quad q, S_l[i] that of four entries of S_{l+1}; S_1 has four entries.  An
-// event descends from the root in the direct method's voxel-major order,
+// Every cell keeps a tree of propensity sums.  With up to four lanes per cell
+// a node has four children: the voxel totals are the leaves, S_{LV-1}[q] the
+// total of the four voxels of quad q, S_l[i] that of four entries of S_{l+1};
+// S_1 has four entries.  With eight lanes and more the upper nodes are as wide
+// as the cell's lanes (8 or 16): a lane holds the prefix before its child, one
+// compare, ballot and population count find the child (11 instructions for 3 or
+// 4 bits, 26 for 2 in a four-ary node), the root's prefixes stay in registers,
+// and an update is one predicated addition per lane.  An event descends from the root in the direct method's voxel-major order,
 // finds the channel inside the voxel in closed form, changes one or two
-// voxels and adds the two differences along their paths: 350 to 500
-// instructions of one lane, with nothing in them to share out over lanes.  The
+// voxels and adds the two differences along their paths: 250 to 500
+// instructions, the most of which no lane can take off another.  The
 // segmented kernel (chi_seg.cuh) finds a voxel with ballots and scans over 8
 // to 32 lanes, and its event loop (600 to 900 instructions) serves one to four
 // cells; here an instruction serves up to 32 (G = 1).
@@ -17,19 +21,20 @@
 // next G (about 360 instructions), and computes its waiting time (120).  The
 // waiting time only decides where the cell stops.  So the G events are applied
 // first, the total propensity A before each kept by its lane, then all G
-// waiting times are computed at once and added in order; the events past the
-// end of the step are undone (at most G a cell and step, on the counts only:
-// the sums are not used again).  The updates of the sums are shared out too,
-// an entry to a lane.
+// waiting times are computed at once and added in order (by a scan of integers
+// while the time's exponent stays the same); the events past the end of the
+// step are undone (at most G a cell and step, on the counts only: the sums are
+// not used again).
 //
 // Bound (one GB300, from ncu): few cells by the event chain -- one warp alone
-// issues every 3.6 cycles, 1,320 cycles an event with G = 32 (2,530 in the
-// segmented kernel); cells of up to 256 voxels that fill the chip by issue
+// issues every 3.9 cycles, 260 instructions and 1,010 cycles an event with G =
+// 32 (2,530 cycles in the segmented kernel; 371 and 1,320 with four-ary nodes
+// and the times added one by one); cells of up to 256 voxels that fill the chip by issue
 // (32 warp instructions per event with G = 1 against 171 and 227, 8x8 and
 // 16x16 voxels); larger ones by random accesses to L2 and DRAM (a dependent
 // read and write per lane reaches 25 G/s in DRAM, 42 G/s in L2, and an event
 // makes two).  Chi ms per step, before -> with this kernel: 2x2 cells of 8x8
-// voxels 2.9 -> 1.53, 64x64 of 16x16 21.1 -> 10.4, 48x48 of 32x32 77.5 -> 52.9,
+// voxels 2.9 -> 1.17, 64x64 of 16x16 21.1 -> 9.3, 48x48 of 32x32 77.5 -> 45.0,
 // 256x256 of 8x8 33.4 -> 7.9, 256x256 of 32x32 611 -> 136.
 //
 // Template parameters: MODEL 0 Notch-Delta without in-voxel binding (k_in =
@@ -227,18 +232,54 @@ __device__ __forceinline__ uint64_t word_unit(uint32_t s) {
   return (static_cast<uint64_t>(hi) << 32) | lo;
 }
 
-// First entry of level l of a four-ary tree whose levels follow one another:
-// (4^l - 4) / 3.
-__device__ __forceinline__ constexpr uint32_t level_off(uint32_t l) {
-  return (0x55555555u & ((1u << (2u * l)) - 1u)) - 1u;
+// tau in units of the last place of a binary64 t with exponent field te, rounded
+// to nearest; `tie` when it lies half-way, or when tau is not below 2^53 of
+// them (t and tau both >= 0; sums below 2^63 stay exact).
+__device__ __forceinline__ uint64_t ulps_of(double tau, int te, bool& tie) {
+  const uint64_t b = static_cast<uint64_t>(__double_as_longlong(tau));
+  const int sh = te - static_cast<int>(b >> 52);
+  const uint64_t m = b == 0ull ? 0ull : ((b & ((1ull << 52) - 1ull)) | (1ull << 52));
+  if (sh <= 0) {
+    tie = sh < 0;
+    return m;
+  }
+  if (sh > 54) return 0ull;  // below half a unit
+  const uint64_t half = 1ull << (sh - 1), up = m + half;
+  tie = (up & ((half << 1) - 1ull)) == 0ull && m != 0ull;
+  return up >> sh;
 }
 
 // Event codes of the undo log.
 constexpr uint32_t kEvBind = 5u, kEvRelease = 6u, kEvHop = 8u;  // 0..4: channel; 8 + species: hop
 
-template <int MODEL, int LV, int LEAF, bool ONE>
-__global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ? 7 : 14) k_chi_lane(const LaneArgs p) {
+// The child of a lane-wide node that r falls into: lane l of the cell holds the
+// exclusive prefix x of child l (of R, from lane `base` on), so the child is
+// the last whose prefix is at most r (children of sum 0 share their prefix
+// with the next and are passed over).
+template <int R>
+__device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base) {
+  const unsigned b = __ballot_sync(kFull, r >= x) >> base;
+  const int k = __popc((b | 1u) & ((1u << R) - 1u)) - 1;
+  r -= __shfl_sync(kFull, x, base + k);
+  return static_cast<uint32_t>(k);
+}
+
+template <int MODEL, int LV, int LEAF, int G>
+__global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G == 1 ? 7 : 14)
+    k_chi_lane(const LaneArgs p) {
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool ONE = G == 1;
+  // Lane-wide nodes (8 lanes per cell and more): the root's prefixes, one a
+  // lane, in registers; below it one level of nodes of RAD prefixes in shared
+  // memory, down to voxels (VMID), quads or (FOUR) four quads.
+  constexpr bool WIDE = G >= 8;
+  constexpr uint32_t RAD = G >= 16 ? 16u : 8u;
+  constexpr uint32_t RV = (1u << (2 * LV)) / RAD;  // voxels under a root entry
+  constexpr bool MID = WIDE && RV > 4u;
+  constexpr uint32_t MV = MID ? RV / RAD : 1u;     // ... under an entry of the level below
+  constexpr bool VMID = MID && MV == 1u, FOUR = MID && MV == 16u;
+  constexpr uint32_t kMid = RAD, kFour = RAD + RAD * RAD;
+  static_assert(!VMID || LEAF == kLeafShared, "voxel prefixes: shared leaves");
   static_assert(!ONE || LEAF != kLeafShared, "one lane per cell: leaves in the scratch array");
   constexpr bool REC = LEAF != kLeafShared;   // voxels in the scratch array, packed
   constexpr bool SEC = LEAF == kLeafSectors;  // ... as counts and quad sums, no voxel totals
@@ -247,10 +288,10 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
   // those of four quads)
   constexpr int SL = SEC ? LV - 2 : LV - 1;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const uint32_t G = ONE ? 1u : p.G;
-  const uint32_t slot = ONE ? lane : lane / G, sl = ONE ? 0u : lane % G;
-  const uint32_t slots = ONE ? 32u : 32u / G;
-  const int base_lane = ONE ? lane : lane - static_cast<int>(sl);
+  const uint32_t slot = static_cast<uint32_t>(lane) / G, sl = static_cast<uint32_t>(lane) % G;
+  constexpr uint32_t slots = 32u / G;
+  const int base_lane = lane - static_cast<int>(sl);
+  const uint32_t li = sl % RAD;  // this lane's entry of a lane-wide node
   const bool lead = sl == 0u;
   const uint32_t V = p.V, n = p.n, nq = (V + 3u) >> 2;
   const uint32_t ps = nq * 4u;  // distance between the planes of D, N and R (shared leaves)
@@ -288,7 +329,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
   unsigned char* cs = warp_cells + slot * p.cell_stride;
   const ulonglong2* rates = reinterpret_cast<const ulonglong2*>(cs);
   uint64_t* tree = reinterpret_cast<uint64_t*>(cs + 48);
-  constexpr uint32_t kCnt = level_off(LV);  // shared leaves: entry of the voxel totals
+  constexpr uint32_t kCnt = lane_sum_words(LV, LEAF, G);  // shared leaves: the voxel totals
   int32_t* cp = reinterpret_cast<int32_t*>(tree + kCnt + ps);
   // a cell's scratch: 2 words per voxel, its total and its counts (records);
   // or 4 words per quad, its sum and its counts of D, N and R (sectors)
@@ -304,6 +345,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
   bool have = false, done = false;
   uint32_t cell = 0, vidx = 0, step = 0, word3 = 0, key0 = 0, key1 = 0, e0 = 0;
   uint64_t A = 0, over_mask = 0;
+  uint64_t X1 = 0;  // lane-wide nodes: the root's prefix of entry li
   uint32_t lim_dn = 0, lim_r = 0;  // sectors: the counts' limits
   double tnow = 0.0;
   int err = 0;
@@ -317,7 +359,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
     while (want) {
       const int src = __ffs(want) - 1;
       want &= want - 1u;
-      const uint32_t sc = ONE ? static_cast<uint32_t>(src) : static_cast<uint32_t>(src) / G;
+      const uint32_t sc = static_cast<uint32_t>(src) / G;
       uint32_t it = 0;
       if (lane == src) it = atomicAdd(p.counter, 1u);
       it = __shfl_sync(kFull, it, src);
@@ -343,7 +385,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
       uint64_t total = 0, pair = 0;
       for (uint32_t k = 0; k < (NQ + 31u) / 32u; ++k) {
         const uint32_t qi = static_cast<uint32_t>(lane) + 32u * k;
-        uint64_t S = 0;
+        uint64_t S = 0, a[4] = {0ull, 0ull, 0ull, 0ull};
         if (qi < nq) {
           uint32_t d[4] = {0, 0, 0, 0}, m[4] = {0, 0, 0, 0}, r[4] = {0, 0, 0, 0};
           if (vec) {
@@ -362,11 +404,10 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
                 r[i] = static_cast<uint32_t>(g[2u * V + 4u * qi + i]);
               }
           }
-          uint64_t a[4], wd[4];
+          uint64_t wd[4];
 #pragma unroll
           for (uint32_t i = 0; i < 4u; ++i) {
             const uint32_t v = 4u * qi + i;
-            a[i] = 0ull;
             wd[i] = 0ull;
             if (v < V) {
               const uint32_t mk = lut[v], nn = mk >> 4;
@@ -404,6 +445,35 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
           store4(nrec + 4u * qi, U64x4{0ull, 0ull, 0ull, 0ull});
         }
         // the sums above the quads (entries past the last quad are zero)
+        if (WIDE) {
+          constexpr uint32_t W = RV / 4u;  // quads under a root entry
+          uint64_t I = S;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t x = __shfl_up_sync(kFull, I, o);
+            if (lane >= o) I += x;
+          }
+          const uint64_t E = I - S;
+          const uint64_t first = __shfl_sync(kFull, E, lane & ~static_cast<int>(W - 1u));
+          if (qi < NQ) {
+            if (qi % W == 0u) ntree[qi / W] = total + first;
+            if (VMID) {
+              uint64_t x = E - first;
+#pragma unroll
+              for (uint32_t i = 0; i < 4u; ++i) {
+                ntree[kMid + 4u * qi + i] = x;
+                x += a[i];
+              }
+            } else if (FOUR) {
+              if (qi % 4u == 0u) ntree[kMid + qi / 4u] = E - first;
+              ntree[kFour + qi] = S;
+            } else if (MID) {
+              ntree[kMid + qi] = E - first;
+            }
+          }
+          total += __shfl_sync(kFull, I, 31);
+          continue;
+        }
         if (!SEC && qi < NQ) ntree[level_off(LV - 1) + qi] = S;
         uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
         x += __shfl_xor_sync(kFull, x, 2);
@@ -420,7 +490,9 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
       }
       const bool any_ovf = __any_sync(kFull, ovf), any_bad = __any_sync(kFull, bad_state);
       nbig = __any_sync(kFull, nbig);
+      __syncwarp();
       if (slot == sc) {
+        if (WIDE) X1 = ntree[li];
         q = nr;
         tv = ntv;
         cell = w.y;
@@ -461,16 +533,34 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
     uint32_t m = 0;         // events applied
     uint64_t Aj = 0;        // the total propensity before this lane's event
     uint32_t log = 0;       // this lane's event: v, u, code
-    for (uint32_t i = 0; i < G; ++i) {
-      const uint64_t R64 = ONE ? Rb : __shfl_sync(kFull, Rb, base_lane + static_cast<int>(i));
+    uint64_t Rn = ONE ? Rb : __shfl_sync(kFull, Rb, base_lane);  // the next event's random bits
+    for (uint32_t i = 0; i < static_cast<uint32_t>(G); ++i) {
+      const uint64_t R64 = Rn;
+      if (!ONE) Rn = __shfl_sync(kFull, Rb, base_lane + static_cast<int>((i + 1u) % G));
       uint64_t r = __umul64hi(R64, A);
       // descent to a quad
-      uint32_t idx = 0;
+      uint32_t idx = 0, kv = 0, pv = 0;
+      uint64_t xm = 0;
+      if (WIDE) {
+        kv = pick_lane<RAD>(X1, r, base_lane);
+        idx = kv;
+        if (MID) {
+          xm = tree[kMid + kv * RAD + li];
+          pv = pick_lane<RAD>(xm, r, base_lane);
+          idx = kv * RAD + pv;
+        }
+        if (FOUR) {
+          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + kFour) + 2u * idx;
+          const ulonglong2 x = nd[0], y = nd[1];
+          idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        }
+      } else {
 #pragma unroll
-      for (uint32_t l = 1; l <= SL; ++l) {
-        const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) + 2u * idx;
-        const ulonglong2 x = nd[0], y = nd[1];
-        idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        for (uint32_t l = 1; l <= SL; ++l) {
+          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) + 2u * idx;
+          const ulonglong2 x = nd[0], y = nd[1];
+          idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        }
       }
       U64x4 sec{};  // sectors: the quad's sum and its counts of D, N and R
       if (SEC) {
@@ -485,8 +575,9 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         sec.c = k == 0u ? x0.c : k == 1u ? x1.c : k == 2u ? x2.c : x3.c;
         sec.d = k == 0u ? x0.d : k == 1u ? x1.d : k == 2u ? x2.d : x3.d;
       }
-      if (kChecked && run && idx >= nq) err |= kErrBounds;
-      idx = min(idx, nq - 1u);  // never past the cell's quads, whatever the sums hold
+      // never past the cell's quads (or voxels), whatever the sums hold
+      if (kChecked && run && idx >= (VMID ? 4u * nq : nq)) err |= kErrBounds;
+      idx = min(idx, (VMID ? 4u * nq : nq) - 1u);
       // the voxel, its total, counts and neighbours
       uint64_t a_v, w_v = 0;
       uint32_t v, D, N, R, mask, nn;
@@ -530,9 +621,12 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         mask = word_mask(w_v);
         nn = __popc(mask);
       } else {
-        const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + kCnt) + 2u * idx;
-        const ulonglong2 x = nd[0], y = nd[1];
-        v = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        v = idx;
+        if (!VMID) {
+          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + kCnt) + 2u * idx;
+          const ulonglong2 x = nd[0], y = nd[1];
+          v = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
+        }
         a_v = tree[kCnt + v];
         D = static_cast<uint32_t>(cp[v]);
         N = static_cast<uint32_t>(cp[ps + v]);
@@ -608,6 +702,11 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         }
       }
       const bool move = run && hop;
+      // lane-wide nodes: u's entry in each, and what is there
+      const uint32_t ku = u / RV, pu = u / MV % RAD;
+      uint64_t xu = 0, fq = 0;
+      if (MID) xu = tree[kMid + ku * RAD + li];
+      if (FOUR) fq = tree[kFour + ((sl & 1u) ? u >> 2 : v >> 2)];
       // differences of the totals of v and u
       const ulonglong2 gh = rates[s];
       uint64_t dv, du = 0;
@@ -647,6 +746,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         }
       } else {
         cu = static_cast<uint32_t>(cp[s * ps + u]) + 1u;
+        if (WIDE) a_u = tree[kCnt + u];
         if (hop) {
           du = gh.x + gh.y * (lut[u] >> 4);
           if (MODEL == 1 && s < 2u)
@@ -667,10 +767,33 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
           if (hop) du += lane_hill(q.hill, tv, Ru) - lane_hill(q.hill, tv, Ru - 1u);
         }
       }
-      // the sums along both paths.  One lane: all reads, then all stores.  More:
-      // lane pairs take the levels, the even lane v's entry, the odd lane u's
-      // (v's adds both differences where the paths share the entry).
-      if (ONE) {
+      // the sums along both paths.  Lane-wide nodes: every lane its entry, where
+      // it comes after v's or u's.  Otherwise, one lane: all reads, then all
+      // stores; more: lane pairs take the levels, the even lane v's entry, the
+      // odd lane u's (v's adds both differences where the paths share the entry).
+      if (WIDE) {
+        const bool same = kv == ku;
+        const uint64_t dvm = li > pv ? dv : 0ull, dum = li > pu ? du : 0ull;
+        xm += dvm + (same ? dum : 0ull);
+        xu += dum;
+        if (run) X1 += (li > kv ? dv : 0ull) + (li > ku ? du : 0ull);
+        __syncwarp();
+        if (run) {
+          if (MID && sl < RAD) {
+            tree[kMid + kv * RAD + li] = xm;
+            if (!same) tree[kMid + ku * RAD + li] = xu;
+          }
+          if (FOUR && sl < 2u) {
+            const bool sq = (v >> 2) == (u >> 2);
+            if (sl == 0u) tree[kFour + (v >> 2)] = fq + dv + (sq ? du : 0ull);
+            else if (!sq) tree[kFour + (u >> 2)] = fq + du;
+          }
+          if (!REC) {
+            if (sl == 0u) tree[kCnt + v] = a_v + dv;
+            if (sl == 1u && hop) tree[kCnt + u] = a_u + du;
+          }
+        }
+      } else if (ONE) {
         uint64_t nv[LV], nu[LV];
 #pragma unroll
         for (uint32_t l = 1; l <= SL; ++l) {
@@ -795,15 +918,32 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
         fired = 1;
       }
     } else {
-      // lane j keeps the time after event j; times only grow, so the events
-      // that fire are the leading ones
-      double t = tnow, mine = tnow;
-      for (uint32_t j = 0; j < G; ++j) {
-        t = __dadd_rn(t, __shfl_sync(kFull, tau, base_lane + static_cast<int>(j)));
-        if (sl == j) mine = t;
+      // Lane j's time after event j.  While t stays in one binade a binary64
+      // sum t + tau is t's bits plus tau rounded to t's last place (ties
+      // apart), whatever t is: the rounded taus are integers, and a scan adds
+      // them.  Otherwise one addition after the other.
+      const uint64_t tb = static_cast<uint64_t>(__double_as_longlong(tnow));
+      bool tie = false;
+      const uint64_t ulps = ulps_of(tau, static_cast<int>(tb >> 52), tie);
+      uint64_t sum = ulps;
+#pragma unroll
+      for (int o = 1; o < G; o <<= 1) {
+        const uint64_t x = __shfl_up_sync(kFull, sum, o, G);
+        if (static_cast<int>(sl) >= o) sum += x;
       }
+      double mine = __longlong_as_double(static_cast<long long>(tb + sum));
+      const bool same = ((tb + sum) >> 52) == (tb >> 52) && !tie && tb != 0ull;
+      if (!__all_sync(kFull, same || !have)) {
+        double t = tnow;
+#pragma unroll
+        for (uint32_t j = 0; j < static_cast<uint32_t>(G); ++j) {
+          t = __dadd_rn(t, __shfl_sync(kFull, tau, base_lane + static_cast<int>(j)));
+          if (sl == j) mine = t;
+        }
+      }
+      // times only grow, so the events that fire are the leading ones
       const unsigned late = __ballot_sync(kFull, !(sl < m && before(mine, p.dt))) >> base_lane;
-      fired = min(G, static_cast<uint32_t>(__ffs(static_cast<int>(late))) - 1u);
+      fired = min(static_cast<uint32_t>(G), static_cast<uint32_t>(__ffs(static_cast<int>(late))) - 1u);
       const double tl = __shfl_sync(kFull, mine, base_lane + static_cast<int>(fired ? fired - 1u : 0u));
       if (fired) tnow = tl;
     }
@@ -863,7 +1003,7 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
       while (out) {
         const int src = __ffs(out) - 1;
         out &= out - 1u;
-        const uint32_t sc = ONE ? static_cast<uint32_t>(src) : static_cast<uint32_t>(src) / G;
+        const uint32_t sc = static_cast<uint32_t>(src) / G;
         const uint32_t c = __shfl_sync(kFull, cell, src);
         const uint32_t vi = __shfl_sync(kFull, vidx, src);
         int32_t* g = p.views[vi].counts + static_cast<size_t>(c) * 3u * V;
@@ -925,6 +1065,35 @@ __global__ void __launch_bounds__(ONE ? 64 : 32, LEAF == kLeafShared ? 1 : ONE ?
       }
     }
   }
+}
+
+// The instantiations the launch plan picks from.
+template <int MODEL>
+ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G) {
+  const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
+#define LANE_CASE(L, F, N) \
+  if (lv == L && leaf == F && G == N) return k_chi_lane<MODEL, L, F, N>
+  LANE_CASE(3, kLeafShared, 32);
+  LANE_CASE(3, kLeafShared, 16);
+  LANE_CASE(3, kLeafShared, 8);
+  LANE_CASE(3, kLeafShared, 4);
+  LANE_CASE(3, kLeafRecords, 1);
+  LANE_CASE(4, kLeafShared, 32);
+  LANE_CASE(4, kLeafShared, 16);
+  LANE_CASE(4, kLeafShared, 8);
+  LANE_CASE(4, kLeafShared, 4);
+  LANE_CASE(4, kLeafRecords, 8);
+  LANE_CASE(4, kLeafRecords, 4);
+  LANE_CASE(4, kLeafSectors, 1);
+  LANE_CASE(5, kLeafShared, 32);
+  LANE_CASE(5, kLeafShared, 16);
+  LANE_CASE(5, kLeafShared, 8);
+  LANE_CASE(5, kLeafRecords, 16);
+  LANE_CASE(5, kLeafRecords, 8);
+  LANE_CASE(5, kLeafSectors, 4);
+  LANE_CASE(5, kLeafSectors, 1);
+#undef LANE_CASE
+  return nullptr;
 }
 
 }  // namespace

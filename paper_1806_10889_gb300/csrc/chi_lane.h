@@ -13,6 +13,22 @@ constexpr uint32_t kLaneHill = 2048;  // R below this reads the Hill table unche
 constexpr uint32_t kWordCount = 1u << 19;    // counts of a record stay below
 constexpr uint32_t kSectorCount = 1u << 16;  // counts of a sector
 
+// First entry of level l of a four-ary tree whose levels follow one another:
+// (4^l - 4) / 3.
+__host__ __device__ constexpr uint32_t level_off(uint32_t l) {
+  return (0x55555555u & ((1u << (2u * l)) - 1u)) - 1u;
+}
+// 64-bit words of sums a cell keeps in shared memory: cells of up to 4^lv
+// voxels, G lanes each.  G < 8: a four-ary tree down to the quads (sectors: to
+// four quads).  G >= 8: lane-wide nodes of R = 8 or 16 entries -- a root's copy,
+// R nodes below it unless the root's entries are quads, and the quads' sums
+// where those nodes' entries are four quads.
+__host__ __device__ constexpr uint32_t lane_sum_words(int lv, int leaf, int G) {
+  if (G < 8) return level_off(leaf == kLeafSectors ? lv - 1 : lv);
+  const uint32_t R = G >= 16 ? 16u : 8u, under = (1u << (2 * lv)) / R;
+  return R + (under > 4u ? R * R : 0u) + (under / R == 16u ? 256u : 0u);
+}
+
 struct LaneArgs {
   const TissueView* views;
   const uint2* items;  // (tissue, cell); nullptr: the cells of views[0] in order
@@ -23,7 +39,6 @@ struct LaneArgs {
   double dt;
   uint32_t n_items, step_off;
   uint32_t V, n;       // of every listed cell
-  uint32_t G;          // lanes per cell
   uint32_t lut_bytes, cell_stride;
 };
 
@@ -42,9 +57,9 @@ cudaError_t launch_chi_lane(const LanePlan& plan, int model, const TissueView* d
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
                             uint32_t step_off, double dt, cudaStream_t stream, int priority = 0);
 using ChiLaneKernel = void (*)(const LaneArgs);
-// one: G = 1; nullptr where not built.
-ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, bool one);      // k_chi_lane.cu
-ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, bool one);    // k_chi_lane_bind.cu
-ChiLaneKernel chi_lane_kernel_pm(uint32_t V, int leaf, bool one);      // k_chi_lane_pm.cu
+// nullptr where not built.
+ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G);    // k_chi_lane.cu
+ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G);  // k_chi_lane_bind.cu
+ChiLaneKernel chi_lane_kernel_pm(uint32_t V, int leaf, uint32_t G);    // k_chi_lane_pm.cu
 
 }  // namespace tsg

@@ -4,27 +4,16 @@
 
 namespace tsg {
 
-ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, bool one) {
-  const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
-  if (leaf == kLeafShared && !one)
-    return lv == 3   ? k_chi_lane<0, 3, kLeafShared, false>
-           : lv == 4 ? k_chi_lane<0, 4, kLeafShared, false>
-                     : k_chi_lane<0, 5, kLeafShared, false>;
-  if (leaf == kLeafRecords && lv == 3 && one) return k_chi_lane<0, 3, kLeafRecords, true>;
-  if (leaf == kLeafRecords && lv == 4 && !one) return k_chi_lane<0, 4, kLeafRecords, false>;
-  if (leaf == kLeafRecords && lv == 5 && !one) return k_chi_lane<0, 5, kLeafRecords, false>;
-  if (leaf == kLeafSectors && lv == 4 && one) return k_chi_lane<0, 4, kLeafSectors, true>;
-  if (leaf == kLeafSectors && lv == 5)
-    return one ? k_chi_lane<0, 5, kLeafSectors, true> : k_chi_lane<0, 5, kLeafSectors, false>;
-  return nullptr;
+ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G) {
+  return lane_instance<0>(V, leaf, G);
 }
 
 namespace {
 
-ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, bool one) {
-  return model == 2   ? chi_lane_kernel_pm(V, leaf, one)
-         : model == 1 ? chi_lane_kernel_bind(V, leaf, one)
-                      : chi_lane_kernel_nd(V, leaf, one);
+ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G) {
+  return model == 2   ? chi_lane_kernel_pm(V, leaf, G)
+         : model == 1 ? chi_lane_kernel_bind(V, leaf, G)
+                      : chi_lane_kernel_nd(V, leaf, G);
 }
 
 }  // namespace
@@ -56,7 +45,7 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
   const uint64_t per = (cells + static_cast<uint64_t>(sms) - 1) / static_cast<uint64_t>(sms);
   pl.G = per <= 4                      ? 32u
-         : per <= (lv == 5 ? 22u : 12u) ? 16u
+         : per <= (lv == 5 ? 26u : 17u) ? 16u
          : per <= 56                    ? 8u
          : per <= (lv == 3 ? 110u : 100u) ? 4u
                                           : 1u;
@@ -66,21 +55,21 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   // cells, sectors, half the bytes and a quarter of the sums.
   constexpr uint64_t kWave = 216 * 1024;  // an SM's shared memory less what blocks reserve
   const uint32_t nq = (V + 3u) / 4u;
-  const uint32_t sums = 48u + (lv == 3 ? 160u : lv == 4 ? 672u : 2720u);
-  const uint32_t shared = sums + 20u * 4u * nq;
-  pl.leaf = pl.G > 1 && per * shared <= kWave       ? kLeafShared
+  auto bytes = [&](int leaf) {  // shared memory of a cell
+    return 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(pl.G)) +
+           (leaf == kLeafShared ? 20u * 4u * nq : 0u);
+  };
+  pl.leaf = pl.G > 1 && per * bytes(kLeafShared) <= kWave               ? kLeafShared
             : lv == 3 || (lv == 4 && pl.G > 1) || (lv == 5 && pl.G > 4) ? kLeafRecords
                                                                      : kLeafSectors;
-  const uint32_t raw = pl.leaf == kLeafShared    ? shared
-                       : pl.leaf == kLeafRecords ? sums
-                                                 : 48u + (lv == 4 ? 160u : 672u);
+  const uint32_t raw = bytes(pl.leaf);
   // an odd multiple of 16 bytes: lanes reading the same entry of their cells
   // start on different shared-memory banks
   pl.cell_stride = ((raw + 15u) & ~15u) | 16u;
   pl.lut_bytes = 128u + 16u * ((nq + 3u) / 4u);
   pl.wpb = pl.G == 1 ? 2u : 1u;
   pl.smem = pl.lut_bytes + static_cast<size_t>(pl.wpb) * (32u / pl.G) * pl.cell_stride;
-  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G == 1);
+  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G);
   int per_sm = 0;
   // the limit is the device's, not this plan's: plans of other cell sizes
   // share the kernel
@@ -108,9 +97,9 @@ cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_v
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
                             uint32_t step_off, double dt, cudaStream_t stream, int priority) {
-  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G == 1);
+  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G);
   const LaneArgs a{d_views, d_items, d_counter, d_scratch, redo.items, redo.counters + 1, dt,
-                   n_items, step_off, V, n, pl.G, pl.lut_bytes, pl.cell_stride};
+                   n_items, step_off, V, n, pl.lut_bytes, pl.cell_stride};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.blocks);
   cfg.blockDim = dim3(32u * pl.wpb);

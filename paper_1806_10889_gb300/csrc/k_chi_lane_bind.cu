@@ -4,19 +4,8 @@
 
 namespace tsg {
 
-ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, bool one) {
-  const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
-  if (leaf == kLeafShared && !one)
-    return lv == 3   ? k_chi_lane<1, 3, kLeafShared, false>
-           : lv == 4 ? k_chi_lane<1, 4, kLeafShared, false>
-                     : k_chi_lane<1, 5, kLeafShared, false>;
-  if (leaf == kLeafRecords && lv == 3 && one) return k_chi_lane<1, 3, kLeafRecords, true>;
-  if (leaf == kLeafRecords && lv == 4 && !one) return k_chi_lane<1, 4, kLeafRecords, false>;
-  if (leaf == kLeafRecords && lv == 5 && !one) return k_chi_lane<1, 5, kLeafRecords, false>;
-  if (leaf == kLeafSectors && lv == 4 && one) return k_chi_lane<1, 4, kLeafSectors, true>;
-  if (leaf == kLeafSectors && lv == 5)
-    return one ? k_chi_lane<1, 5, kLeafSectors, true> : k_chi_lane<1, 5, kLeafSectors, false>;
-  return nullptr;
+ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G) {
+  return lane_instance<1>(V, leaf, G);
 }
 
 }  // namespace tsg
