@@ -209,6 +209,10 @@ __device__ __forceinline__ uint4 unpack4(uint64_t w) {
   return make_uint4(field16(w, 0), field16(w, 1), field16(w, 2), field16(w, 3));
 }
 
+__device__ __forceinline__ void add64(uint64_t* p, uint64_t x) {
+  atomicAdd(reinterpret_cast<unsigned long long*>(p), static_cast<unsigned long long>(x));
+}
+
 // A voxel of the scratch array in one word: D in bits 0..19, N in 20..39, R
 // in 40..59, the neighbour mask in 60..63.
 __device__ __forceinline__ uint64_t pack_voxel(uint32_t D, uint32_t N, uint32_t R, uint32_t mask) {
@@ -645,8 +649,10 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
       // channel: hops are the last but the in-voxel bindings in channel order
       const bool ctr = MODEL == 2 && v == centre;
       const uint32_t F = MODEL == 2 ? static_cast<uint32_t>(ctr) - R : 0u;
-      const uint64_t X = MODEL == 2 ? static_cast<uint64_t>(N) * F : static_cast<uint64_t>(D) * N;
-      const uint64_t y17 = MODEL ? q.k_in * X : 0ull;
+      // F is 0 or 1
+      const uint64_t y17 = MODEL == 2 ? (F ? q.k_in * N : 0ull)
+                           : MODEL    ? q.k_in * (static_cast<uint64_t>(D) * N)
+                                      : 0ull;
       const uint64_t y18 = MODEL == 1 ? q.k_off * R : 0ull;
       const uint64_t UD = q.hD * D, UN = q.hN * N, UR = MODEL == 2 ? 0ull : q.hR * R;
       const uint64_t HD = UD * nn, H2 = HD + UN * nn, H3 = MODEL == 2 ? H2 : H2 + UR * nn;
@@ -658,6 +664,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
       bool gain = false;                    // ... and whether by +1 at v
       uint32_t code = kEvHop + s, u = v;
       int dD = 0, dN = 0, dR = 0;           // MODEL 1, 2: the changes at v
+      bool several = false;                 // ... of more than one species
       if (hop) {
         const uint64_t unit = z2 ? UR : z1 ? UN : UD, unit2 = unit + unit;
         const uint64_t z3 = z0 - (z2 ? H2 : z1 ? HD : 0ull);
@@ -676,8 +683,8 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
         const uint64_t gDD = q.gD * D, gNN = q.gN * N;
         uint64_t c0, c1;
         if (MODEL == 2) {
-          c0 = q.tD * F;
-          c1 = c0 + q.kd * R;
+          c0 = F ? q.tD : 0ull;
+          c1 = c0 + (R ? q.kd : 0ull);
         } else {
           c1 = y - q.gR * R - gNN - gDD;
           c0 = c1 - q.kN;
@@ -692,6 +699,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
           dD = ch == 0u ? 1 : ch == 2u ? -1 : 0;
           dN = ch == 1u ? 1 : ch == 3u ? -1 : 0;
           dR = ch == 4u ? -1 : (MODEL == 2 && ch == 1u) ? -1 : 0;
+          several = (MODEL == 2 && ch == 1u) || r >= top;
           if (r >= top) {
             const bool rel = MODEL == 1 && r >= top + y17;  // R -> D + N
             code = rel ? kEvRelease : kEvBind;
@@ -711,14 +719,21 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
       const ulonglong2 gh = rates[s];
       uint64_t dv, du = 0;
       uint32_t nc = 0, newmax = 0;
-      if (MODEL == 0) {
-        const uint64_t c = gh.x + gh.y * nn;
+      {
+        // one molecule of s more or less: a voxel's total is affine in D and in
+        // N (R's Hill term follows below)
+        uint64_t c = gh.x + gh.y * nn;
+        if (MODEL == 1) c += s == 2u ? 0ull : q.k_in * (s == 0u ? N : D);
+        if (MODEL == 2) c += s == 1u && F ? q.k_in : 0ull;
         dv = gain ? c : 0ull - c;
+      }
+      if (MODEL == 0) {
         nc = (s == 0u ? D : s == 1u ? N : R) + (gain ? 1u : 0xFFFFFFFFu);
         newmax = nc;
       } else {
-        dv = lane_total<MODEL>(q, tv, D + dD, N + dN, R + dR, nn, ctr) - a_v;
         newmax = (D + dD) | (N + dN) | (R + dR);
+        // binding, unbinding: two or three species change
+        if (several) dv = lane_total<MODEL>(q, tv, D + dD, N + dN, R + dR, nn, ctr) - a_v;
       }
       uint32_t cu = 0;
       uint64_t a_u = 0, w_u = 0;
@@ -756,14 +771,14 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
           newmax |= cu;
         }
       }
-      if (MODEL != 2 && s == 2u && run) {  // R changes the Hill term, here and where it arrives
+      if (MODEL != 2 && s == 2u && run && !several) {  // R changes the Hill term, here and where it arrives
         const uint32_t Ru = hop ? (REC && !SEC ? word_R(w_u) + 1u : cu) : 1u;
         if (!slow) {  // every count is inside the table
-          if (MODEL == 0) dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
+          dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
           const uint64_t d = __ldg(q.hill + Ru) - __ldg(q.hill + (Ru - 1u));
           if (hop) du += d;
         } else {
-          if (MODEL == 0) dv += lane_hill(q.hill, tv, R - 1u) - lane_hill(q.hill, tv, R);
+          dv += lane_hill(q.hill, tv, R - 1u) - lane_hill(q.hill, tv, R);
           if (hop) du += lane_hill(q.hill, tv, Ru) - lane_hill(q.hill, tv, Ru - 1u);
         }
       }
@@ -954,38 +969,40 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
     e0 = e;
     unsigned out = __ballot_sync(kFull, fin && lead);
     if (out) {
-      // undo the events past the end of the step, last first (counts only)
-      for (uint32_t j = G; j-- > 0;) {
-        const uint32_t lg = ONE ? log : __shfl_sync(kFull, log, base_lane + static_cast<int>(j));
-        if (fin && lead && j >= fired && j < m) {
-          const uint32_t v = lg & 1023u, u = (lg >> 10) & 1023u, code = lg >> 20;
-          int d[3] = {0, 0, 0};
-          uint32_t s = 3u;  // species that moves back from u
-          if (code >= kEvHop) {
-            s = code - kEvHop;
-            d[s] = 1;
-          } else if (code == kEvBind || code == kEvRelease) {
-            d[1] = code == kEvBind ? 1 : -1;
-            d[0] = MODEL != 2 ? d[1] : 0;
-            d[2] = -d[1];
-          } else {
-            d[code == 4u ? 2u : (code & 1u)] = code <= 1u ? -1 : 1;
-            if (MODEL == 2 && code == 1u) d[2] = 1;
-          }
-          if (SEC) {
-            uint64_t* qv = rec + 4u * (v >> 2) + 1u;
-            for (uint32_t k = 0; k < 3u; ++k)
-              qv[k] += static_cast<uint64_t>(static_cast<int64_t>(d[k])) << (16u * (v & 3u));
-            if (s < 3u) rec[4u * (u >> 2) + 1u + s] -= 1ull << (16u * (u & 3u));
-          } else if (REC) {
-            uint64_t* base = rec + 1u;
-            uint64_t& wv = base[2u * v];
-            wv = pack_voxel(word_D(wv) + d[0], word_N(wv) + d[1], word_R(wv) + d[2], word_mask(wv));
-            if (s < 3u) base[2u * u] -= word_unit(s);
-          } else {
-            for (uint32_t k = 0; k < 3u; ++k) cp[k * ps + v] += d[k];
-            if (s < 3u) cp[s * ps + u] -= 1;
-          }
+      // undo the events past the end of the step (counts only), every lane its
+      // own: the changes commute
+      if (fin && sl >= fired && sl < m) {
+        const uint32_t v = log & 1023u, u = (log >> 10) & 1023u, code = log >> 20;
+        int cD = 0, cN = 0, cR = 0;  // back at v
+        if (code == kEvBind || code == kEvRelease) {
+          cN = code == kEvBind ? 1 : -1;
+          cD = MODEL != 2 ? cN : 0;
+          cR = -cN;
+        } else {
+          const uint32_t s = code >= kEvHop ? code - kEvHop : code == 4u ? 2u : (code & 1u);
+          const int c = code <= 1u ? -1 : 1;
+          cD = s == 0u ? c : 0;
+          cN = s == 1u ? c : 0;
+          cR = s == 2u || (MODEL == 2 && code == 1u) ? 1 : 0;
+        }
+        const uint32_t su = code - kEvHop;  // hops: the species taken back from u
+        if (SEC) {
+          uint64_t* w = rec + 4u * (v >> 2) + 1u;
+          const uint32_t sh = 16u * (v & 3u);
+          if (cD) add64(w, static_cast<uint64_t>(static_cast<int64_t>(cD)) << sh);
+          if (cN) add64(w + 1, static_cast<uint64_t>(static_cast<int64_t>(cN)) << sh);
+          if (cR) add64(w + 2, static_cast<uint64_t>(static_cast<int64_t>(cR)) << sh);
+          if (code >= kEvHop) add64(rec + 4u * (u >> 2) + 1u + su, 0ull - (1ull << (16u * (u & 3u))));
+        } else if (REC) {
+          add64(rec + 2u * v + 1u, word_unit(0) * static_cast<uint64_t>(static_cast<int64_t>(cD)) +
+                                       word_unit(1) * static_cast<uint64_t>(static_cast<int64_t>(cN)) +
+                                       word_unit(2) * static_cast<uint64_t>(static_cast<int64_t>(cR)));
+          if (code >= kEvHop) add64(rec + 2u * u + 1u, 0ull - word_unit(su));
+        } else {
+          if (cD) atomicAdd(cp + v, cD);
+          if (cN) atomicAdd(cp + ps + v, cN);
+          if (cR) atomicAdd(cp + 2u * ps + v, cR);
+          if (code >= kEvHop) atomicAdd(cp + su * ps + u, -1);
         }
       }
       __syncwarp();
