@@ -58,6 +58,7 @@
 // random streams.
 #pragma once
 #include "chi_lane.h"
+#include "early_launch.cuh"
 #include "tissue_dev.cuh"
 
 namespace tsg {
@@ -325,6 +326,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
     lut[v] = static_cast<unsigned char>(m | (__popc(m) << 4));
   }
   __syncthreads();
+  early_launch();
 
   // A cell's shared memory: the rates {g, h} of D, N and R, the sums, and with
   // shared leaves the voxel totals (the tree's last level) and the counts.
@@ -347,6 +349,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
   const TissueView* tv = p.views + (p.items ? p.items[0].x : 0u);
   q.hill = tv->q.hill;
   bool have = false, done = false;
+  int started = 0;
   uint32_t cell = 0, vidx = 0, step = 0, word3 = 0, key0 = 0, key1 = 0, e0 = 0;
   uint64_t A = 0, over_mask = 0;
   uint64_t X1 = 0;  // lane-wide nodes: the root's prefix of entry li
@@ -364,9 +367,18 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
       const int src = __ffs(want) - 1;
       want &= want - 1u;
       const uint32_t sc = static_cast<uint32_t>(src) / G;
-      uint32_t it = 0;
-      if (lane == src) it = atomicAdd(p.counter, 1u);
-      it = __shfl_sync(kFull, it, src);
+      // the first item by position, further ones by the counter (never read when
+      // one wave takes all)
+      const uint32_t places = gridDim.x * (blockDim.x >> 5) * slots;
+      uint32_t it = (blockIdx.x * (blockDim.x >> 5) + wib) * slots + sc;
+      if (__shfl_sync(kFull, started, src)) {
+        it = p.n_items;
+        if (places < p.n_items) {
+          if (lane == src) it = places + atomicAdd(p.counter, 1u);
+          it = __shfl_sync(kFull, it, src);
+        }
+      }
+      if (slot == sc) started = 1;
       if (it >= p.n_items) {
         if (slot == sc) done = true;
         continue;

@@ -32,7 +32,7 @@ __host__ __device__ constexpr uint32_t lane_sum_words(int lv, int leaf, int G) {
 struct LaneArgs {
   const TissueView* views;
   const uint2* items;  // (tissue, cell); nullptr: the cells of views[0] in order
-  uint32_t* counter;   // work counter, zero before the launch
+  uint32_t* counter;   // work counter, zero before a launch of more cells than places
   uint64_t* scratch;   // the resident cells' records (plans with scratch_bytes > 0)
   uint2* redo;         // with records: cells whose counts pass the packed range
   uint32_t* redo_n;
@@ -47,6 +47,8 @@ struct LanePlan {
   int leaf = kLeafShared;
   uint32_t lut_bytes = 0, cell_stride = 0;
   size_t smem = 0, scratch_bytes = 0;
+  bool small = false;     // at most one block per SM
+  bool counters = false;  // the launch uses the work and redo counters (cleared before it)
 };
 
 // The plan for `cells` cells of V voxels; model 0: Notch-Delta without
@@ -55,7 +57,8 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model);
 cudaError_t launch_chi_lane(const LanePlan& plan, int model, const TissueView* d_views,
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
-                            uint32_t step_off, double dt, cudaStream_t stream, int priority = 0);
+                            uint32_t step_off, double dt, cudaStream_t stream, int priority = 0,
+                            bool early = false);
 using ChiLaneKernel = void (*)(const LaneArgs);
 // nullptr where not built.
 ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G);    // k_chi_lane.cu

@@ -86,6 +86,8 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   const uint64_t need = (cells + per_block - 1) / per_block;
   const uint64_t cap = static_cast<uint64_t>(sms) * static_cast<uint64_t>(per_sm);
   pl.blocks = static_cast<uint32_t>(need < cap ? need : cap);
+  pl.small = need <= static_cast<uint64_t>(sms);
+  pl.counters = need > cap || pl.leaf != kLeafShared;
   if (pl.leaf != kLeafShared)
     pl.scratch_bytes = static_cast<size_t>(pl.blocks) * per_block *
                        (pl.leaf == kLeafRecords ? 8u * nq : 16u * ((nq + 3u) / 4u)) *
@@ -96,7 +98,7 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
 cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_views,
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
-                            uint32_t step_off, double dt, cudaStream_t stream, int priority) {
+                            uint32_t step_off, double dt, cudaStream_t stream, int priority, bool early) {
   const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G);
   const LaneArgs a{d_views, d_items, d_counter, d_scratch, redo.items, redo.counters + 1, dt,
                    n_items, step_off, V, n, pl.lut_bytes, pl.cell_stride};
@@ -110,6 +112,11 @@ cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_v
   attr[0].val.priority = priority;
   cfg.attrs = attr;
   cfg.numAttrs = priority ? 1 : 0;
+  if (early) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 1;
+  }
   cudaError_t e = cudaLaunchKernelEx(&cfg, k, a);
   if (e != cudaSuccess || pl.leaf == kLeafShared) return e;
   // the cells that left the packed range, by the segmented kernel from the

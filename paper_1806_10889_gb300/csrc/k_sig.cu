@@ -15,6 +15,7 @@
 //
 // This file also holds the initial-state kernel (Poisson counts by CDF
 // inversion), the Hill-production table and the step-counter update.
+#include "early_launch.cuh"
 #include "tissue_dev.cuh"
 
 namespace tsg {
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(256) k_sig(const TissueView t, const int axis,
   const uint32_t W = t.width, H = t.height;
   const uint32_t nfaces = axis == 0 ? (W - 1) * H : W * (H - 1);
   const uint32_t f = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  early_launch();
   if (f >= nfaces) return;  // whole warp
   sig_face(t, axis == 0 ? (f / (W - 1)) * W + f % (W - 1) : f, axis, tag, step_off, dt);
 }
@@ -254,12 +256,20 @@ __global__ void k_step_advance(uint32_t* step, uint32_t n) {
 }  // namespace
 
 cudaError_t launch_sig(const TissueView& t, int axis, uint32_t tag, uint32_t step_off, double dt,
-                       cudaStream_t stream) {
+                       cudaStream_t stream, bool early) {
   const uint32_t nfaces = axis == 0 ? (t.width - 1) * t.height : t.width * (t.height - 1);
   if (nfaces == 0) return cudaSuccess;
   constexpr int kWarps = 8;
-  k_sig<<<(nfaces + kWarps - 1) / kWarps, 32 * kWarps, 0, stream>>>(t, axis, tag, step_off, dt);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((nfaces + kWarps - 1) / kWarps);
+  cfg.blockDim = dim3(32 * kWarps);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_sig, t, axis, tag, step_off, dt);
 }
 
 cudaError_t launch_sig_list(const TissueView* d_views, const uint2* d_items, uint32_t n_items,

@@ -113,13 +113,16 @@ int chi_all(tissue_batch* b, double dt) {
     const cudaStream_t st = (ov && c > 0) ? b->side[c - 1] : b->stream;
     if (ov && c > 0 && cudaStreamWaitEvent(st, b->ev_fork, 0) != cudaSuccess) return TISSUE_E_CUDA;
     uint32_t* counters = b->d_counters + 3 * c;
-    if (cudaMemsetAsync(counters, 0, 3 * sizeof(uint32_t), st) != cudaSuccess)
+    const bool tree =
+        p.lane.G &&
+        default_shape(p.V, {TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0, p.layout});
+    if ((!tree || p.lane.counters) &&
+        cudaMemsetAsync(counters, 0, 3 * sizeof(uint32_t), st) != cudaSuccess)
       return TISSUE_E_CUDA;
     // each class has its own part of the redo list (classes may run at once)
     const ChiRedo redo{b->d_redo + p.items_off, counters};
     const int prio = ov ? (c == 0 ? b->prio_hi : b->prio_lo) : 0;
-    if (p.lane.G && default_shape(p.V, {TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0,
-                                        p.layout})) {
+    if (tree) {
       if (launch_chi_lane(p.lane, p.lane_model, b->d_views, b->d_items + p.items_off, p.n_items,
                           counters, b->d_lane + p.lane_off, redo, p.V, p.n, 0u, dt, st, prio) !=
           cudaSuccess)

@@ -187,8 +187,10 @@ int error_code_of(int flag);
 int seg_lanes_for(uint32_t V, int want);
 
 // tag: the Philox stream tag of this face phase (kTagSx, kTagSy, kTagSx2, kTagSy2).
+// early: the launch may start before the one before it in the stream ends
+// (early_launch.cuh).
 cudaError_t launch_sig(const TissueView& t, int axis, uint32_t tag, uint32_t step_off, double dt,
-                       cudaStream_t stream);
+                       cudaStream_t stream, bool early = false);
 cudaError_t launch_step_advance(uint32_t* step, uint32_t n, cudaStream_t stream);
 cudaError_t launch_selftest_time(uint64_t n, uint64_t seed, unsigned long long* mismatches,
                                  cudaStream_t stream);

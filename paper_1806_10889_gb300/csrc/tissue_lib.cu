@@ -261,6 +261,8 @@ struct LaneCall {
     }
     scratch = static_cast<uint64_t*>(p);
   }
+  // a small tissue's launches may each start before the last has ended
+  bool early() const { return plan.G != 0 && plan.small; }
   ~LaneCall() {
     if (scratch) cudaFreeAsync(scratch, stream);
   }
@@ -286,13 +288,15 @@ cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, const LaneCall& lane,
       e = launch_chi_wm(t->d_view, t->d_wm_items, t->wm_cells, v.V, i, dt, t->stream);
       if (e != cudaSuccess) return e;
     }
-    e = cudaMemsetAsync(t->d_work, 0, 3 * sizeof(uint32_t), t->stream);
-    if (e != cudaSuccess) return e;
+    if (lane.plan.G == 0 || lane.plan.counters) {
+      e = cudaMemsetAsync(t->d_work, 0, 3 * sizeof(uint32_t), t->stream);
+      if (e != cudaSuccess) return e;
+    }
     const ChiRedo redo{t->d_redo, t->d_work};
     if (lane.plan.G)
       return launch_chi_lane(lane.plan, lane.model, t->d_view,
                              t->wm_cells ? t->d_lat_items : nullptr, cells - t->wm_cells, t->d_work,
-                             lane.scratch, redo, v.V, v.n, i, dt, t->stream);
+                             lane.scratch, redo, v.V, v.n, i, dt, t->stream, 0, lane.early());
     const bool pre = c.smem_layout == TISSUE_LAYOUT_PREFIX;
     return launch_chi_seg(t->d_view, t->wm_cells ? t->d_lat_items : nullptr, cells - t->wm_cells,
                           t->d_work, v.V, static_cast<int>(c.lanes_per_cell),
@@ -311,16 +315,15 @@ int enqueue_split_step(tissue* t, const TissueView& v, const LaneCall& lane, uin
     if (launch_chi_cfg(t, v, lane, i, dt) != cudaSuccess) return false;
     return !after || cudaEventRecord(after, t->stream) == cudaSuccess;
   };
+  auto sig = [&](int axis, uint32_t tag, double d) {
+    return launch_sig(v, axis, tag, i, d, t->stream, lane.early()) == cudaSuccess;
+  };
   if (t->scheme == TISSUE_SPLIT_LIE) {
-    if (!chi() || launch_sig(v, 0, kTagSx, i, dt, t->stream) != cudaSuccess ||
-        launch_sig(v, 1, kTagSy, i, dt, t->stream) != cudaSuccess)
-      return TISSUE_E_CUDA;
+    if (!chi() || !sig(0, kTagSx, dt) || !sig(1, kTagSy, dt)) return TISSUE_E_CUDA;
   } else {
     const double h = dt * 0.5;
-    if (launch_sig(v, 0, kTagSx, i, h, t->stream) != cudaSuccess ||
-        launch_sig(v, 1, kTagSy, i, h, t->stream) != cudaSuccess || !chi() ||
-        launch_sig(v, 1, kTagSy2, i, h, t->stream) != cudaSuccess ||
-        launch_sig(v, 0, kTagSx2, i, h, t->stream) != cudaSuccess)
+    if (!sig(0, kTagSx, h) || !sig(1, kTagSy, h) || !chi() || !sig(1, kTagSy2, h) ||
+        !sig(0, kTagSx2, h))
       return TISSUE_E_CUDA;
   }
   return TISSUE_OK;

@@ -119,17 +119,23 @@ def test_no_scratch_or_a_capture_runs_the_segmented_kernel():
     bt.close()
     b.close()
 
-    s = torch.cuda.Stream()
-    c = Tissue(spec, stream=s)
-    c.sync()
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph, stream=s):
-        c.step(dt, 1)
-    graph.replay()
-    graph.replay()
-    torch.cuda.synchronize()
-    _compare(c, spec, want, wne, wtl, "captured")
-    c.close()
+    # captured: the large tissue without scratch, a small one with early launches
+    for sp, steps in ((spec, 1), (TissueSpec(3, 3, 8, seed=93), 3)):
+        ref = Tissue(sp)
+        ref.step(dt, 2 * steps)
+        want, (wne, wtl) = ref.read_counts(), ref.read_stats()
+        ref.close()
+        s = torch.cuda.Stream()
+        c = Tissue(sp, stream=s)
+        c.sync()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            c.step(dt, steps)
+        graph.replay()
+        graph.replay()
+        torch.cuda.synchronize()
+        _compare(c, sp, want, wne, wtl, "captured")
+        c.close()
 
 
 def test_two_streams_step_large_tissues_at_once():
