@@ -45,10 +45,10 @@
 // records, total and packed counts of a voxel side by side, a quad one aligned
 // 64-byte block; or sectors, 32 bytes a quad with its sum and 16-bit counts,
 // the four quads under a shared sum one 128-byte line that an event reads
-// whole, the four totals of the chosen quad recomputed, each changed quad one
-// full sector written (256x256 cells of 32x32 voxels: 174 ms with records and a
-// level of quad sums beside them, 490 DRAM bytes an event; 128 ms with sectors);
-// ONE: G = 1 at compile time.
+// whole, the four totals of the chosen quad recomputed, the sum and the changed
+// count of one or two quads written (256x256 cells of 32x32 voxels: 174 ms with
+// records and a level of quad sums beside them, 490 DRAM bytes an event; 122 ms
+// and 217 bytes with sectors); G.
 //
 // Limits.  Counts below the tissue's `small` keep every total below 2^52
 // unchecked, and R below kLaneHill reads the Hill table unchecked.  With
@@ -269,8 +269,13 @@ __device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base)
   return static_cast<uint32_t>(k);
 }
 
+// Registers: shared leaves as many as they take (150 to 170; shared memory or
+// the number of cells bounds the warps); one lane per cell of more than 256
+// voxels up to 255 (shared memory holds 8 warps an SM anyway); else 128, so that
+// 14 to 16 warps fit an SM.
 template <int MODEL, int LV, int LEAF, int G>
-__global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G == 1 ? 7 : 14)
+__global__ void __launch_bounds__(G == 1 ? 64 : 32,
+                                  LEAF == kLeafShared ? 1 : G > 1 ? 14 : LV == 5 ? 4 : 7)
     k_chi_lane(const LaneArgs p) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr bool ONE = G == 1;
@@ -758,18 +763,17 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
         if (several) dv = lane_total<MODEL>(q, tv, D + dD, N + dN, R + dR, nn, ctr) - a_v;
       }
       uint32_t cu = 0;
-      uint64_t a_u = 0, w_u = 0;
-      U64x4 su{};  // sectors: u's quad
+      uint64_t a_u = 0, w_u = 0;  // records: u's total and word; sectors: its quad's sum and counts
       if (SEC) {
-        su = load4(rec + 4u * (u >> 2));
-        const uint32_t k = u & 3u;
-        cu = (s == 0u ? field16(su.b, k) : s == 1u ? field16(su.c, k) : field16(su.d, k)) + 1u;
+        const uint64_t* uq = rec + 4u * (u >> 2);
+        a_u = uq[0];
+        w_u = uq[1u + s];
+        cu = field16(w_u, u & 3u) + 1u;
         if (hop) {
           du = gh.x + gh.y * (lut[u] >> 4);
-          if (MODEL == 1 && s < 2u)
-            du += q.k_in * (s == 0u ? field16(su.c, k) : field16(su.b, k));
+          if (MODEL == 1 && s < 2u) du += q.k_in * field16(uq[2u - s], u & 3u);
           if (MODEL == 2 && s == 1u)
-            du += q.k_in * (static_cast<uint32_t>(u == centre) - field16(su.d, k));
+            du += q.k_in * (static_cast<uint32_t>(u == centre) - field16(uq[3], u & 3u));
         }
       } else if (REC) {
         const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec)[u];
@@ -831,19 +835,17 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
           }
         }
       } else if (ONE) {
-        uint64_t nv[LV], nu[LV];
-#pragma unroll
-        for (uint32_t l = 1; l <= SL; ++l) {
-          const uint32_t iv = v >> (2u * (LV - l)), iu = u >> (2u * (LV - l));
-          nv[l] = tree[level_off(l) + iv] + dv + (iv == iu ? du : 0ull);
-          nu[l] = tree[level_off(l) + iu] + du;
-        }
         if (run) {
+          // v's entries, then u's: one may be the other
 #pragma unroll
-          for (uint32_t l = 1; l <= SL; ++l) {
-            const uint32_t iv = v >> (2u * (LV - l)), iu = u >> (2u * (LV - l));
-            tree[level_off(l) + iv] = nv[l];
-            if (iv != iu) tree[level_off(l) + iu] = nu[l];
+          for (int side = 0; side < 2; ++side) {
+            uint64_t x[SL];
+#pragma unroll
+            for (uint32_t l = 1; l <= SL; ++l)
+              x[l - 1] = tree[level_off(l) + ((side ? u : v) >> (2u * (LV - l)))];
+#pragma unroll
+            for (uint32_t l = 1; l <= SL; ++l)
+              tree[level_off(l) + ((side ? u : v) >> (2u * (LV - l)))] = x[l - 1] + (side ? du : dv);
           }
         }
       } else {
@@ -863,27 +865,26 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32, LEAF == kLeafShared ? 1 : G 
       }
       // the two voxels
       if (SEC) {
+        // the quad's sum and the changed species' counts, here and at u
         const uint64_t at = 1ull << (16u * (v & 3u)), to = hop ? 1ull << (16u * (u & 3u)) : 0ull;
-        const uint64_t to0 = s == 0u ? to : 0ull, to1 = s == 1u ? to : 0ull;
-        const uint64_t to2 = s == 2u ? to : 0ull;
-        uint64_t c0, c1, c2;  // the changes at v
-        if (MODEL == 0) {
-          const uint64_t c = gain ? at : 0ull - at;
-          c0 = s == 0u ? c : 0ull;
-          c1 = s == 1u ? c : 0ull;
-          c2 = s == 2u ? c : 0ull;
-        } else {
-          c0 = dD > 0 ? at : dD < 0 ? 0ull - at : 0ull;
-          c1 = dN > 0 ? at : dN < 0 ? 0ull - at : 0ull;
-          c2 = dR > 0 ? at : dR < 0 ? 0ull - at : 0ull;
-        }
         const bool same = (v >> 2) == (u >> 2);
-        if (run && (ONE || sl == 0u))
-          store4(rec + 4u * (v >> 2),
-                 same ? U64x4{sec.a + dv + du, sec.b + c0 + to0, sec.c + c1 + to1, sec.d + c2 + to2}
-                      : U64x4{sec.a + dv, sec.b + c0, sec.c + c1, sec.d + c2});
-        if (move && !same && (ONE || sl == 1u))
-          store4(rec + 4u * (u >> 2), U64x4{su.a + du, su.b + to0, su.c + to1, su.d + to2});
+        uint64_t* vq = rec + 4u * (v >> 2);
+        const uint64_t w = (s == 0u ? sec.b : s == 1u ? sec.c : sec.d) + (gain ? at : 0ull - at);
+        if (run && (ONE || sl == 0u)) {
+          vq[0] = sec.a + dv + (same ? du : 0ull);
+          if (MODEL != 0 && several) {
+            vq[1] = sec.b + (dD > 0 ? at : dD < 0 ? 0ull - at : 0ull);
+            vq[2] = sec.c + (dN > 0 ? at : 0ull - at);
+            vq[3] = sec.d + (dR > 0 ? at : 0ull - at);
+          } else {
+            vq[1u + s] = w + (same ? to : 0ull);
+          }
+        }
+        if (move && !same && (ONE || sl == 1u)) {
+          uint64_t* uq = rec + 4u * (u >> 2);
+          uq[0] = a_u + du;
+          uq[1u + s] = w_u + to;
+        }
         const uint32_t lim_s = s == 2u ? lim_r : lim_dn;
         bool over = hop && cu >= lim_s;
         if (MODEL == 0) over = over || nc >= lim_s;
