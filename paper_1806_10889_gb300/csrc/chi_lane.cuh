@@ -22,7 +22,8 @@
 // waiting time only decides where the cell stops.  So the G events are applied
 // first, the total propensity A before each kept by its lane, then all G
 // waiting times are computed at once and added in order (by a scan of integers
-// while the time's exponent stays the same); the events past the end of the
+// while the time's exponent stays the same).  With few warps on an SM a helper
+// warp beside each draws a batch ahead of it; the events past the end of the
 // step are undone (at most G a cell and step, on the counts only: the sums are
 // not used again).
 //
@@ -155,6 +156,18 @@ __device__ __noinline__ bool past_limits(const TissueView* tv, const int32_t* cp
   return o;
 }
 
+// What the two warps of a block with a helper exchange.
+struct LaneExchange {
+  uint64_t Em[2][32], Rb[2][32];
+  int Ek[2][32];
+  uint32_t stream[2][32][7];  // step, cell, word 3, key, next event, whether new
+  int done, swap;
+  int pad[2];
+};
+static_assert(sizeof(LaneExchange) == kExchangeBytes, "chi_lane.h");
+
+__device__ __forceinline__ void pair_barrier() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+
 // The child of a node that r falls into: k = the number of leading children
 // whose running sum is at most r; r becomes the remainder inside it.  WIDE
 // compares with the three running sums at once (the shorter chain, for few
@@ -271,11 +284,14 @@ __device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base)
 
 // Registers: shared leaves as many as they take (150 to 170; shared memory or
 // the number of cells bounds the warps); one lane per cell of more than 256
-// voxels up to 255 (shared memory holds 8 warps an SM anyway); else 128, so that
-// 14 to 16 warps fit an SM.
-template <int MODEL, int LV, int LEAF, int G>
-__global__ void __launch_bounds__(G == 1 ? 64 : 32,
-                                  LEAF == kLeafShared ? 1 : G > 1 ? 14 : LV == 5 ? 4 : 7)
+// voxels up to 255 (shared memory holds 8 warps an SM anyway); with a helper 168
+// (12 warps); else 128, so that 14 to 16 warps fit an SM.
+template <int MODEL, int LV, int LEAF, int G, bool HELP>
+__global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                  ? 6
+                                                            : LEAF == kLeafShared ? 1
+                                                            : G > 1               ? 14
+                                                            : LV == 5             ? 4
+                                                                                  : 7)
     k_chi_lane(const LaneArgs p) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr bool ONE = G == 1;
@@ -297,7 +313,8 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
   // the levels of sums in shared memory: down to the quads' (sectors: down to
   // those of four quads)
   constexpr int SL = SEC ? LV - 2 : LV - 1;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  int wib = threadIdx.x >> 5;
   const uint32_t slot = static_cast<uint32_t>(lane) / G, sl = static_cast<uint32_t>(lane) % G;
   constexpr uint32_t slots = 32u / G;
   const int base_lane = lane - static_cast<int>(sl);
@@ -307,10 +324,21 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
   const uint32_t ps = nq * 4u;  // distance between the planes of D, N and R (shared leaves)
   const uint32_t centre = MODEL == 2 ? (n >> 1) * n + (n >> 1) : 0u;
   const bool vec = (V & 3u) == 0u;
+  const uint32_t warps = HELP ? 1u : blockDim.x >> 5;  // that run cells
 
   // offsets u - v of the m-th existing direction for each neighbour mask, then
   // (shared leaves) the voxels' masks: bits 0..3, and their number: bits 4..6
   int16_t* hop_off = reinterpret_cast<int16_t*>(smem);
+  LaneExchange* ex = reinterpret_cast<LaneExchange*>(smem + p.lut_bytes - sizeof(LaneExchange));
+  if (HELP && threadIdx.x == 0) {
+    unsigned w;
+    asm volatile("mov.u32 %0, %%warpid;" : "=r"(w));
+    // every other pair of blocks the other way round, so that the warps that run
+    // cells spread over the SM's four schedulers (one half of them otherwise:
+    // 64x64 cells 9.3 -> 12.2 ms)
+    ex->swap = static_cast<int>((w >> 2) & 1u);
+    ex->done = 0;
+  }
   unsigned char* lut = smem + 128;
   for (uint32_t i = threadIdx.x; i < 64u; i += blockDim.x) {
     uint32_t b = i >> 2;
@@ -333,6 +361,33 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
   __syncthreads();
   early_launch();
 
+  // The helper warp: draws for the events after those in hand, a batch ahead.
+  // Per phase (one barrier of both warps) it takes the new cells' streams and
+  // leaves the draws for the next phase; buffers and streams alternate.
+  if (HELP) wib ^= ex->swap;
+  if (HELP && wib == 1) {
+    uint32_t hs[5] = {}, he = 0;
+    for (uint32_t ph = 0;; ph ^= 1u) {
+      pair_barrier();
+      if (ex->done) return;
+      const uint32_t* d = ex->stream[ph][slot];
+      if (d[6]) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) hs[k] = d[k];
+        he = d[5];
+      } else {
+        he += G;
+      }
+      uint64_t m_, r_;
+      int k_;
+      draw_event(he + G + sl, hs[0], hs[1], hs[2], hs[3], hs[4], m_, k_, r_);
+      ex->Em[ph ^ 1u][lane] = m_;
+      ex->Rb[ph ^ 1u][lane] = r_;
+      ex->Ek[ph ^ 1u][lane] = k_;
+    }
+  }
+  uint32_t phase = 0;
+
   // A cell's shared memory: the rates {g, h} of D, N and R, the sums, and with
   // shared leaves the voxel totals (the tree's last level) and the counts.
   unsigned char* warp_cells =
@@ -346,7 +401,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
   // or 4 words per quad, its sum and its counts of D, N and R (sectors)
   const uint32_t rec_words = SEC ? 16u * nl : 8u * nq;
   uint64_t* warp_rec =
-      REC ? p.scratch + (static_cast<size_t>(blockIdx.x) * (blockDim.x >> 5) + wib) * slots * rec_words
+      REC ? p.scratch + (static_cast<size_t>(blockIdx.x) * warps + wib) * slots * rec_words
           : nullptr;
   uint64_t* rec = warp_rec + static_cast<size_t>(slot) * rec_words;
 
@@ -355,6 +410,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
   q.hill = tv->q.hill;
   bool have = false, done = false;
   int started = 0;
+  uint32_t e_next = 0xFFFFFFFFu;  // the event the helper's next draws start with
   uint32_t cell = 0, vidx = 0, step = 0, word3 = 0, key0 = 0, key1 = 0, e0 = 0;
   uint64_t A = 0, over_mask = 0;
   uint64_t X1 = 0;  // lane-wide nodes: the root's prefix of entry li
@@ -374,8 +430,8 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
       const uint32_t sc = static_cast<uint32_t>(src) / G;
       // the first item by position, further ones by the counter (never read when
       // one wave takes all)
-      const uint32_t places = gridDim.x * (blockDim.x >> 5) * slots;
-      uint32_t it = (blockIdx.x * (blockDim.x >> 5) + wib) * slots + sc;
+      const uint32_t places = gridDim.x * warps * slots;
+      uint32_t it = (blockIdx.x * warps + wib) * slots + sc;
       if (__shfl_sync(kFull, started, src)) {
         it = p.n_items;
         if (places < p.n_items) {
@@ -525,6 +581,7 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
         A = total;
         tnow = 0.0;
         e0 = 0;
+        e_next = 0xFFFFFFFFu;
         big = nbig;
         lim = min(nr.small, kLaneHill);
         err = any_bad ? kErrState : any_ovf ? kErrOverflow : (REC && nbig) ? kErrNarrow : 0;
@@ -540,12 +597,52 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
       }
     }
     __syncwarp();
-    if (__all_sync(kFull, done)) break;
+    if (__all_sync(kFull, done)) {
+      if (HELP) {
+        if (lane == 0) ex->done = 1;
+        __syncwarp();
+        pair_barrier();
+      }
+      break;
+    }
 
     // ---- draws: lane j of a cell, event e0 + j -----------------------------
     uint64_t Em, Rb;
     int Ek;
-    draw_event(e0 + sl, step, cell, word3, key0, key1, Em, Ek, Rb);
+    if (HELP) {
+      const bool fresh = have && e0 != e_next;  // a new cell, or a batch cut short
+      if (lead) {
+        uint32_t* d = ex->stream[phase][slot];
+        if (fresh) {
+          d[0] = step;
+          d[1] = cell;
+          d[2] = word3;
+          d[3] = key0;
+          d[4] = key1;
+          d[5] = e0;
+        }
+        d[6] = fresh ? 1u : 0u;
+      }
+      __syncwarp();
+      pair_barrier();
+      Em = ex->Em[phase][lane];
+      Rb = ex->Rb[phase][lane];
+      Ek = ex->Ek[phase][lane];
+      phase ^= 1u;
+      if (__any_sync(kFull, fresh)) {
+        uint64_t m_, r_;
+        int k_;
+        draw_event(e0 + sl, step, cell, word3, key0, key1, m_, k_, r_);
+        if (fresh) {
+          Em = m_;
+          Ek = k_;
+          Rb = r_;
+        }
+      }
+      e_next = e0 + G;
+    } else {
+      draw_event(e0 + sl, step, cell, word3, key0, key1, Em, Ek, Rb);
+    }
 
     // ---- G events of every cell, the whole warp in step --------------------
     bool run = have && err == 0;
@@ -1109,29 +1206,35 @@ __global__ void __launch_bounds__(G == 1 ? 64 : 32,
 
 // The instantiations the launch plan picks from.
 template <int MODEL>
-ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G) {
+ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, bool helper) {
   const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
-#define LANE_CASE(L, F, N) \
-  if (lv == L && leaf == F && G == N) return k_chi_lane<MODEL, L, F, N>
-  LANE_CASE(3, kLeafShared, 32);
-  LANE_CASE(3, kLeafShared, 16);
-  LANE_CASE(3, kLeafShared, 8);
-  LANE_CASE(3, kLeafShared, 4);
-  LANE_CASE(3, kLeafRecords, 1);
-  LANE_CASE(4, kLeafShared, 32);
-  LANE_CASE(4, kLeafShared, 16);
-  LANE_CASE(4, kLeafShared, 8);
-  LANE_CASE(4, kLeafShared, 4);
-  LANE_CASE(4, kLeafRecords, 8);
-  LANE_CASE(4, kLeafRecords, 4);
-  LANE_CASE(4, kLeafSectors, 1);
-  LANE_CASE(5, kLeafShared, 32);
-  LANE_CASE(5, kLeafShared, 16);
-  LANE_CASE(5, kLeafShared, 8);
-  LANE_CASE(5, kLeafRecords, 16);
-  LANE_CASE(5, kLeafRecords, 8);
-  LANE_CASE(5, kLeafSectors, 4);
-  LANE_CASE(5, kLeafSectors, 1);
+#define LANE_CASE(L, F, N, H) \
+  if (lv == L && leaf == F && G == N && helper == H) return k_chi_lane<MODEL, L, F, N, H>
+  LANE_CASE(3, kLeafShared, 32, true);
+  LANE_CASE(3, kLeafShared, 16, true);
+  LANE_CASE(3, kLeafShared, 16, false);
+  LANE_CASE(3, kLeafShared, 8, true);
+  LANE_CASE(3, kLeafShared, 8, false);
+  LANE_CASE(3, kLeafShared, 4, false);
+  LANE_CASE(3, kLeafRecords, 1, false);
+  LANE_CASE(4, kLeafShared, 32, true);
+  LANE_CASE(4, kLeafShared, 16, true);
+  LANE_CASE(4, kLeafShared, 16, false);
+  LANE_CASE(4, kLeafShared, 8, true);
+  LANE_CASE(4, kLeafShared, 8, false);
+  LANE_CASE(4, kLeafShared, 4, false);
+  LANE_CASE(4, kLeafRecords, 8, false);
+  LANE_CASE(4, kLeafRecords, 4, false);
+  LANE_CASE(4, kLeafSectors, 1, false);
+  LANE_CASE(5, kLeafShared, 32, true);
+  LANE_CASE(5, kLeafShared, 16, true);
+  LANE_CASE(5, kLeafShared, 8, false);
+  LANE_CASE(5, kLeafRecords, 16, true);
+  LANE_CASE(5, kLeafRecords, 16, false);
+  LANE_CASE(5, kLeafRecords, 8, false);
+  LANE_CASE(5, kLeafSectors, 4, false);
+  LANE_CASE(5, kLeafSectors, 1, true);
+  LANE_CASE(5, kLeafSectors, 1, false);
 #undef LANE_CASE
   return nullptr;
 }

@@ -4,16 +4,16 @@
 
 namespace tsg {
 
-ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G) {
-  return lane_instance<0>(V, leaf, G);
+ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G, bool helper) {
+  return lane_instance<0>(V, leaf, G, helper);
 }
 
 namespace {
 
-ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G) {
-  return model == 2   ? chi_lane_kernel_pm(V, leaf, G)
-         : model == 1 ? chi_lane_kernel_bind(V, leaf, G)
-                      : chi_lane_kernel_nd(V, leaf, G);
+ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G, bool helper) {
+  return model == 2   ? chi_lane_kernel_pm(V, leaf, G, helper)
+         : model == 1 ? chi_lane_kernel_bind(V, leaf, G, helper)
+                      : chi_lane_kernel_nd(V, leaf, G, helper);
 }
 
 }  // namespace
@@ -49,34 +49,48 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
          : per <= 56                    ? 8u
          : per <= (lv == 3 ? 110u : 100u) ? 4u
                                           : 1u;
+  // A helper warp that draws ahead while at most six warps an SM run cells: the
+  // draws leave the chain, and twelve warps still have the registers they take.
+  // Chi ms, without -> with: 2x2 cells of 8x8 voxels 1.19 -> 1.14, 60x50 of 16x16
+  // 8.34 -> 7.70, 60 uneven tissues (26,802 cells of 32x32) 146.7 -> 133.9; at
+  // seven warps (64x64 of 16x16, 128 registers) 9.34 -> 9.40.
+  const uint64_t runs = (cells * pl.G + 31u) / 32u;  // warps that run cells
+  const bool few = runs <= 6u * static_cast<uint64_t>(sms) && (pl.G >= 8 || (pl.G == 1 && lv == 5));
+  const uint32_t nq = (V + 3u) / 4u;
+  const uint64_t places = 32u / pl.G;  // cells a warp runs
   // Leaves: in shared memory while one wave of cells fits there (the shortest
   // chain); else records, whose totals need no recomputing; past L2's size, or
   // where their sums (2.7 KB a cell of 32x32 voxels) would leave SMs short of
   // cells, sectors, half the bytes and a quarter of the sums.
-  constexpr uint64_t kWave = 216 * 1024;  // an SM's shared memory less what blocks reserve
-  const uint32_t nq = (V + 3u) / 4u;
-  auto bytes = [&](int leaf) {  // shared memory of a cell
-    return 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(pl.G)) +
-           (leaf == kLeafShared ? 20u * 4u * nq : 0u);
+  auto shape = [&](int leaf, bool helper) {
+    const uint32_t cell = 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(pl.G)) +
+                          (leaf == kLeafShared ? 20u * 4u * nq : 0u);
+    // an odd multiple of 16 bytes: lanes reading the same entry of their cells
+    // start on different shared-memory banks
+    pl.cell_stride = ((cell + 15u) & ~15u) | 16u;
+    pl.lut_bytes = 128u + 16u * ((nq + 3u) / 4u) + (helper ? kExchangeBytes : 0u);
+    pl.leaf = leaf;
+    pl.helper = helper;
+    pl.wpb = pl.G == 1 && !helper ? 2u : 1u;
+    pl.threads = helper ? 64u : 32u * pl.wpb;
+    pl.smem = pl.lut_bytes + static_cast<size_t>(pl.wpb * places) * pl.cell_stride;
+    // whether one wave holds every cell (a block reserves 1 KB more)
+    return lane_kernel(model, V, leaf, pl.G, helper) != nullptr && pl.smem <= kMaxSmem &&
+           (per + pl.wpb * places - 1) / (pl.wpb * places) * (pl.smem + 1024u) <= 228u * 1024u;
   };
-  pl.leaf = pl.G > 1 && per * bytes(kLeafShared) <= kWave               ? kLeafShared
-            : lv == 3 || (lv == 4 && pl.G > 1) || (lv == 5 && pl.G > 4) ? kLeafRecords
-                                                                     : kLeafSectors;
-  const uint32_t raw = bytes(pl.leaf);
-  // an odd multiple of 16 bytes: lanes reading the same entry of their cells
-  // start on different shared-memory banks
-  pl.cell_stride = ((raw + 15u) & ~15u) | 16u;
-  pl.lut_bytes = 128u + 16u * ((nq + 3u) / 4u);
-  pl.wpb = pl.G == 1 ? 2u : 1u;
-  pl.smem = pl.lut_bytes + static_cast<size_t>(pl.wpb) * (32u / pl.G) * pl.cell_stride;
-  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G);
+  const int spill = lv == 3 || (lv == 4 && pl.G > 1) || (lv == 5 && pl.G > 4) ? kLeafRecords
+                                                                             : kLeafSectors;
+  if (!(few && shape(kLeafShared, true)) && !shape(kLeafShared, false) &&
+      !(few && shape(spill, true)))
+    shape(spill, false);
+  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G, pl.helper);
   int per_sm = 0;
   // the limit is the device's, not this plan's: plans of other cell sizes
   // share the kernel
   if (!k || pl.smem > kMaxSmem ||
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) !=
           cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * static_cast<int>(pl.wpb),
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, static_cast<int>(pl.threads),
                                                     pl.smem) != cudaSuccess ||
       per_sm < 1) {
     pl.G = 0;
@@ -99,12 +113,12 @@ cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_v
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
                             uint32_t step_off, double dt, cudaStream_t stream, int priority, bool early) {
-  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G);
+  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G, pl.helper);
   const LaneArgs a{d_views, d_items, d_counter, d_scratch, redo.items, redo.counters + 1, dt,
                    n_items, step_off, V, n, pl.lut_bytes, pl.cell_stride};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.blocks);
-  cfg.blockDim = dim3(32u * pl.wpb);
+  cfg.blockDim = dim3(pl.threads);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];

@@ -4,8 +4,8 @@
 
 namespace tsg {
 
-ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G) {
-  return lane_instance<1>(V, leaf, G);
+ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G, bool helper) {
+  return lane_instance<1>(V, leaf, G, helper);
 }
 
 }  // namespace tsg
