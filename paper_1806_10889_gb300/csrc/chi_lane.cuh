@@ -161,6 +161,7 @@ struct LaneExchange {
   uint64_t Em[2][32], Rb[2][32];
   int Ek[2][32];
   uint32_t stream[2][32][7];  // step, cell, word 3, key, next event, whether new
+  uint32_t home[32][6];       // the cell's step, number, word 3, key, tissue
   int done, swap;
   int pad[2];
 };
@@ -284,10 +285,11 @@ __device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base)
 
 // Registers: shared leaves as many as they take (150 to 170; shared memory or
 // the number of cells bounds the warps); one lane per cell of more than 256
-// voxels up to 255 (shared memory holds 8 warps an SM anyway); with a helper 168
-// (12 warps); else 128, so that 14 to 16 warps fit an SM.
-template <int MODEL, int LV, int LEAF, int G, bool HELP>
-__global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                  ? 6
+// voxels up to 255 (shared memory holds 8 warps an SM anyway); with a helper of
+// HELP blocks an SM 168 (six, 12 warps) or 128 (eight); else 128, so that 14 to
+// 16 warps fit an SM.
+template <int MODEL, int LV, int LEAF, int G, int HELP>
+__global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                  ? HELP
                                                             : LEAF == kLeafShared ? 1
                                                             : G > 1               ? 14
                                                             : LV == 5             ? 4
@@ -295,6 +297,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     k_chi_lane(const LaneArgs p) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr bool ONE = G == 1;
+  // rates read from shared memory by every event rather than held in registers:
+  // MODEL 0 then fits 128 of them but for four words (the others gain nothing)
+  constexpr bool kLean = MODEL == 0 && LEAF == kLeafShared && HELP == 8;
   // Lane-wide nodes (8 lanes per cell and more): the root's prefixes, one a
   // lane, in registers; below it one level of nodes of RAD prefixes in shared
   // memory, down to voxels (VMID), quads or (FOUR) four quads.
@@ -387,6 +392,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     }
   }
   uint32_t phase = 0;
+  uint32_t* home = HELP ? ex->home[slot] : nullptr;
 
   // A cell's shared memory: the rates {g, h} of D, N and R, the sums, and with
   // shared leaves the voxel totals (the tree's last level) and the counts.
@@ -572,12 +578,20 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         if (WIDE) X1 = ntree[li];
         q = nr;
         tv = ntv;
-        cell = w.y;
-        vidx = w.x;
         step = *ntv->step + p.step_off;
+        cell = w.y;
+        word3 = ntv->tissue_id | (kTagChi << 24);
         key0 = static_cast<uint32_t>(ntv->seed);
         key1 = static_cast<uint32_t>(ntv->seed >> 32);
-        word3 = ntv->tissue_id | (kTagChi << 24);
+        vidx = w.x;
+        if (HELP && lead) {
+          home[0] = step;
+          home[1] = cell;
+          home[2] = word3;
+          home[3] = key0;
+          home[4] = key1;
+          home[5] = vidx;
+        }
         A = total;
         tnow = 0.0;
         e0 = 0;
@@ -607,38 +621,34 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     }
 
     // ---- draws: lane j of a cell, event e0 + j -----------------------------
-    uint64_t Em, Rb;
-    int Ek;
+    uint64_t Em = 0, Rb = 0;
+    int Ek = 0;
+    const uint64_t* bits = nullptr;  // helper: the batch's random bits
     if (HELP) {
       const bool fresh = have && e0 != e_next;  // a new cell, or a batch cut short
       if (lead) {
         uint32_t* d = ex->stream[phase][slot];
         if (fresh) {
-          d[0] = step;
-          d[1] = cell;
-          d[2] = word3;
-          d[3] = key0;
-          d[4] = key1;
+#pragma unroll
+          for (int k = 0; k < 5; ++k) d[k] = home[k];
           d[5] = e0;
         }
         d[6] = fresh ? 1u : 0u;
       }
       __syncwarp();
       pair_barrier();
-      Em = ex->Em[phase][lane];
-      Rb = ex->Rb[phase][lane];
-      Ek = ex->Ek[phase][lane];
-      phase ^= 1u;
       if (__any_sync(kFull, fresh)) {
         uint64_t m_, r_;
         int k_;
-        draw_event(e0 + sl, step, cell, word3, key0, key1, m_, k_, r_);
+        draw_event(e0 + sl, home[0], home[1], home[2], home[3], home[4], m_, k_, r_);
         if (fresh) {
-          Em = m_;
-          Ek = k_;
-          Rb = r_;
+          ex->Em[phase][lane] = m_;
+          ex->Ek[phase][lane] = k_;
+          ex->Rb[phase][lane] = r_;
         }
+        __syncwarp();
       }
+      bits = ex->Rb[phase] + base_lane;
       e_next = e0 + G;
     } else {
       draw_event(e0 + sl, step, cell, word3, key0, key1, Em, Ek, Rb);
@@ -651,7 +661,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     uint32_t m = 0;         // events applied
     uint64_t Aj = 0;        // the total propensity before this lane's event
     uint32_t log = 0;       // this lane's event: v, u, code
-    uint64_t Rn = ONE ? Rb : __shfl_sync(kFull, Rb, base_lane);  // the next event's random bits
+    uint64_t Rn = HELP ? bits[0] : ONE ? Rb : __shfl_sync(kFull, Rb, base_lane);  // the next event's random bits
     // A whole warp on a cell: near the end of the step no more events than are
     // likely left (A (dt - t) are expected), so that a short step does not undo
     // most of 32 (2x2 cells, dt 1e-9: 34 us -> 22 us a step).
@@ -664,7 +674,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     }
     for (uint32_t i = 0; i < batch; ++i) {
       const uint64_t R64 = Rn;
-      if (!ONE) Rn = __shfl_sync(kFull, Rb, base_lane + static_cast<int>((i + 1u) % G));
+      if (!ONE)
+        Rn = HELP ? bits[(i + 1u) % G]
+                  : __shfl_sync(kFull, Rb, base_lane + static_cast<int>((i + 1u) % G));
       uint64_t r = __umul64hi(R64, A);
       // descent to a quad
       uint32_t idx = 0, kv = 0, pv = 0;
@@ -778,7 +790,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
                            : MODEL    ? q.k_in * (static_cast<uint64_t>(D) * N)
                                       : 0ull;
       const uint64_t y18 = MODEL == 1 ? q.k_off * R : 0ull;
-      const uint64_t UD = q.hD * D, UN = q.hN * N, UR = MODEL == 2 ? 0ull : q.hR * R;
+      const uint64_t UD = (kLean ? rates[0].y : q.hD) * D, UN = (kLean ? rates[1].y : q.hN) * N;
+      const uint64_t UR = MODEL == 2 ? 0ull : (kLean ? rates[2].y : q.hR) * R;
       const uint64_t HD = UD * nn, H2 = HD + UN * nn, H3 = MODEL == 2 ? H2 : H2 + UR * nn;
       const uint64_t top = a_v - y17 - y18, y = top - H3;
       const bool hop = r >= y && (MODEL == 0 || r < top);
@@ -804,14 +817,14 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           dR = s == 2u ? -1 : 0;
         }
       } else {
-        const uint64_t gDD = q.gD * D, gNN = q.gN * N;
+        const uint64_t gDD = (kLean ? rates[0].x : q.gD) * D, gNN = (kLean ? rates[1].x : q.gN) * N;
         uint64_t c0, c1;
         if (MODEL == 2) {
           c0 = F ? q.tD : 0ull;
           c1 = c0 + (R ? q.kd : 0ull);
         } else {
-          c1 = y - q.gR * R - gNN - gDD;
-          c0 = c1 - q.kN;
+          c1 = y - (kLean ? rates[2].x * R - y18 : q.gR * R) - gNN - gDD;
+          c0 = c1 - (kLean ? tv->q.kN : q.kN);
         }
         const uint64_t c2 = c1 + gDD, c3 = c2 + gNN;
         const uint32_t ch = static_cast<uint32_t>(r >= c0) + static_cast<uint32_t>(r >= c1) +
@@ -1044,6 +1057,11 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     }
 
     // ---- the waiting times of the applied events, added in order -----------
+    if (HELP) {
+      Em = ex->Em[phase][lane];
+      Ek = ex->Ek[phase][lane];
+      phase ^= 1u;
+    }
     const double tau = tau_from(F53{Em, Ek}, Ek < 0 || Aj == 0ull, Aj | (Aj == 0ull));
     uint32_t fired = 0;
     if (ONE) {
@@ -1128,11 +1146,12 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       __syncwarp();
       if (REC && fin && lead && (err & kErrNarrow)) {
         // left as it was, for the 32-bit pass
-        p.redo[atomicAdd(p.redo_n, 1u)] = make_uint2(vidx, cell);
+        p.redo[atomicAdd(p.redo_n, 1u)] = make_uint2(HELP ? home[5] : vidx, HELP ? home[1] : cell);
       } else if (fin && lead) {
-        tv->ev_last[cell] = e;
-        tv->t_last[cell] = tnow;
-        tv->ev_total[cell] += e;
+        const uint32_t c = HELP ? home[1] : cell;
+        tv->ev_last[c] = e;
+        tv->t_last[c] = tnow;
+        tv->ev_total[c] += e;
         if (err) atomicOr(tv->err, err);
       }
       // the counts back to the state array, the whole warp one cell at a time
@@ -1141,8 +1160,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         const int src = __ffs(out) - 1;
         out &= out - 1u;
         const uint32_t sc = static_cast<uint32_t>(src) / G;
-        const uint32_t c = __shfl_sync(kFull, cell, src);
-        const uint32_t vi = __shfl_sync(kFull, vidx, src);
+        const uint32_t c = HELP ? ex->home[sc][1] : __shfl_sync(kFull, cell, src);
+        const uint32_t vi = HELP ? ex->home[sc][5] : __shfl_sync(kFull, vidx, src);
         int32_t* g = p.views[vi].counts + static_cast<size_t>(c) * 3u * V;
         if (SEC) {
           const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words;
@@ -1206,35 +1225,38 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
 
 // The instantiations the launch plan picks from.
 template <int MODEL>
-ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, bool helper) {
+ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
 #define LANE_CASE(L, F, N, H) \
   if (lv == L && leaf == F && G == N && helper == H) return k_chi_lane<MODEL, L, F, N, H>
-  LANE_CASE(3, kLeafShared, 32, true);
-  LANE_CASE(3, kLeafShared, 16, true);
-  LANE_CASE(3, kLeafShared, 16, false);
-  LANE_CASE(3, kLeafShared, 8, true);
-  LANE_CASE(3, kLeafShared, 8, false);
-  LANE_CASE(3, kLeafShared, 4, false);
-  LANE_CASE(3, kLeafRecords, 1, false);
-  LANE_CASE(4, kLeafShared, 32, true);
-  LANE_CASE(4, kLeafShared, 16, true);
-  LANE_CASE(4, kLeafShared, 16, false);
-  LANE_CASE(4, kLeafShared, 8, true);
-  LANE_CASE(4, kLeafShared, 8, false);
-  LANE_CASE(4, kLeafShared, 4, false);
-  LANE_CASE(4, kLeafRecords, 8, false);
-  LANE_CASE(4, kLeafRecords, 4, false);
-  LANE_CASE(4, kLeafSectors, 1, false);
-  LANE_CASE(5, kLeafShared, 32, true);
-  LANE_CASE(5, kLeafShared, 16, true);
-  LANE_CASE(5, kLeafShared, 8, false);
-  LANE_CASE(5, kLeafRecords, 16, true);
-  LANE_CASE(5, kLeafRecords, 16, false);
-  LANE_CASE(5, kLeafRecords, 8, false);
-  LANE_CASE(5, kLeafSectors, 4, false);
-  LANE_CASE(5, kLeafSectors, 1, true);
-  LANE_CASE(5, kLeafSectors, 1, false);
+  LANE_CASE(3, kLeafShared, 32, 6);
+  LANE_CASE(3, kLeafShared, 16, 6);
+  LANE_CASE(3, kLeafShared, 16, 0);
+  LANE_CASE(3, kLeafShared, 8, 6);
+  if (MODEL != 1) LANE_CASE(3, kLeafShared, 8, 8);
+  LANE_CASE(3, kLeafShared, 8, 0);
+  LANE_CASE(3, kLeafShared, 4, 0);
+  LANE_CASE(3, kLeafRecords, 1, 0);
+  LANE_CASE(4, kLeafShared, 32, 6);
+  LANE_CASE(4, kLeafShared, 16, 6);
+  LANE_CASE(4, kLeafShared, 16, 0);
+  LANE_CASE(4, kLeafShared, 8, 6);
+  if (MODEL != 1) LANE_CASE(4, kLeafShared, 8, 8);
+  LANE_CASE(4, kLeafShared, 8, 0);
+  LANE_CASE(4, kLeafShared, 4, 0);
+  LANE_CASE(4, kLeafRecords, 8, 0);
+  LANE_CASE(4, kLeafRecords, 4, 0);
+  LANE_CASE(4, kLeafSectors, 1, 0);
+  LANE_CASE(5, kLeafShared, 32, 6);
+  LANE_CASE(5, kLeafShared, 16, 6);
+  LANE_CASE(5, kLeafShared, 8, 0);
+  LANE_CASE(5, kLeafRecords, 16, 6);
+  LANE_CASE(5, kLeafRecords, 16, 8);
+  LANE_CASE(5, kLeafRecords, 16, 0);
+  LANE_CASE(5, kLeafRecords, 8, 0);
+  LANE_CASE(5, kLeafSectors, 4, 0);
+  LANE_CASE(5, kLeafSectors, 1, 6);
+  LANE_CASE(5, kLeafSectors, 1, 0);
 #undef LANE_CASE
   return nullptr;
 }

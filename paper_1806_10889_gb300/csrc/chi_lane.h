@@ -30,7 +30,7 @@ __host__ __device__ constexpr uint32_t lane_sum_words(int lv, int leaf, int G) {
 }
 
 // Shared memory that the two warps of a block with a helper exchange through.
-constexpr uint32_t kExchangeBytes = 2 * 32 * (8 + 8 + 4 + 28) + 16;
+constexpr uint32_t kExchangeBytes = 2 * 32 * (8 + 8 + 4 + 28) + 32 * 24 + 16;
 
 struct LaneArgs {
   const TissueView* views;
@@ -48,7 +48,7 @@ struct LaneArgs {
 struct LanePlan {
   uint32_t G = 0, wpb = 0, threads = 0, blocks = 0;  // G = 0: this launch stays with the segmented kernel
   int leaf = kLeafShared;
-  bool helper = false;    // two warps a block: one runs cells, one draws ahead
+  uint32_t helper = 0;    // two warps a block: one runs cells, one draws ahead; blocks an SM
   uint32_t lut_bytes = 0, cell_stride = 0;
   size_t smem = 0, scratch_bytes = 0;
   bool small = false;     // at most one block per SM
@@ -66,8 +66,8 @@ cudaError_t launch_chi_lane(const LanePlan& plan, int model, const TissueView* d
 using ChiLaneKernel = void (*)(const LaneArgs);
 // nullptr where not built.
 // k_chi_lane.cu, k_chi_lane_bind.cu, k_chi_lane_pm.cu
-ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G, bool helper);
-ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G, bool helper);
-ChiLaneKernel chi_lane_kernel_pm(uint32_t V, int leaf, uint32_t G, bool helper);
+ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G, uint32_t helper);
+ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G, uint32_t helper);
+ChiLaneKernel chi_lane_kernel_pm(uint32_t V, int leaf, uint32_t G, uint32_t helper);
 
 }  // namespace tsg

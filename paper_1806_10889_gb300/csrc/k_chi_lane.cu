@@ -4,13 +4,13 @@
 
 namespace tsg {
 
-ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G, bool helper) {
+ChiLaneKernel chi_lane_kernel_nd(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   return lane_instance<0>(V, leaf, G, helper);
 }
 
 namespace {
 
-ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G, bool helper) {
+ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   return model == 2   ? chi_lane_kernel_pm(V, leaf, G, helper)
          : model == 1 ? chi_lane_kernel_bind(V, leaf, G, helper)
                       : chi_lane_kernel_nd(V, leaf, G, helper);
@@ -49,20 +49,25 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
          : per <= 56                    ? 8u
          : per <= (lv == 3 ? 110u : 100u) ? 4u
                                           : 1u;
-  // A helper warp that draws ahead while at most six warps an SM run cells: the
-  // draws leave the chain, and twelve warps still have the registers they take.
-  // Chi ms, without -> with: 2x2 cells of 8x8 voxels 1.19 -> 1.14, 60x50 of 16x16
-  // 8.34 -> 7.70, 60 uneven tissues (26,802 cells of 32x32) 146.7 -> 133.9; at
-  // seven warps (64x64 of 16x16, 128 registers) 9.34 -> 9.40.
+  // A helper warp that draws ahead while at most eight warps an SM run cells: the
+  // draws leave the chain.  Up to six, twelve warps have the registers they want
+  // (168).  Chi ms, without -> with: 2x2 cells of 8x8 voxels 1.19 -> 1.14, 60x50 of
+  // 16x16 8.34 -> 7.70, 60 uneven tissues (26,802 cells of 32x32) 146.7 -> 133.9.
+  // Seven and eight leave 128: 64x64 of 16x16 9.35 -> 9.12, promoter 7.41 -> 6.95,
+  // 64x64 of 8x8 3.83 -> 3.69, 48x48 of 32x32 (records) 45.05 -> 44.36; with
+  // in-voxel binding the spills cost more (16x16 9.74 -> 10.01) and it is not
+  // built for 8 lanes; below six warps 128 registers cost 2% (7.68 -> 7.81).
   const uint64_t runs = (cells * pl.G + 31u) / 32u;  // warps that run cells
-  const bool few = runs <= 6u * static_cast<uint64_t>(sms) && (pl.G >= 8 || (pl.G == 1 && lv == 5));
+  const uint32_t few = runs <= 6u * static_cast<uint64_t>(sms)   ? 6u
+                       : runs <= 8u * static_cast<uint64_t>(sms) ? 8u
+                                                                 : 0u;
   const uint32_t nq = (V + 3u) / 4u;
   const uint64_t places = 32u / pl.G;  // cells a warp runs
   // Leaves: in shared memory while one wave of cells fits there (the shortest
   // chain); else records, whose totals need no recomputing; past L2's size, or
   // where their sums (2.7 KB a cell of 32x32 voxels) would leave SMs short of
   // cells, sectors, half the bytes and a quarter of the sums.
-  auto shape = [&](int leaf, bool helper) {
+  auto shape = [&](int leaf, uint32_t helper) {
     const uint32_t cell = 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(pl.G)) +
                           (leaf == kLeafShared ? 20u * 4u * nq : 0u);
     // an odd multiple of 16 bytes: lanes reading the same entry of their cells
@@ -80,9 +85,9 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   };
   const int spill = lv == 3 || (lv == 4 && pl.G > 1) || (lv == 5 && pl.G > 4) ? kLeafRecords
                                                                              : kLeafSectors;
-  if (!(few && shape(kLeafShared, true)) && !shape(kLeafShared, false) &&
-      !(few && shape(spill, true)))
-    shape(spill, false);
+  if (!(few && shape(kLeafShared, few)) && !shape(kLeafShared, 0) &&
+      !(few && shape(spill, few)))
+    shape(spill, 0);
   const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G, pl.helper);
   int per_sm = 0;
   // the limit is the device's, not this plan's: plans of other cell sizes

@@ -4,7 +4,7 @@
 
 namespace tsg {
 
-ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G, bool helper) {
+ChiLaneKernel chi_lane_kernel_bind(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   return lane_instance<1>(V, leaf, G, helper);
 }
 
