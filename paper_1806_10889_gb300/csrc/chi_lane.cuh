@@ -290,7 +290,7 @@ __device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base)
 // 16 warps fit an SM.
 template <int MODEL, int LV, int LEAF, int G, int HELP>
 __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                  ? HELP
-                                                            : LEAF == kLeafShared ? 1
+                                                            : LEAF == kLeafShared ? 12
                                                             : G > 1               ? 14
                                                             : LV == 5             ? 4
                                                                                   : 7)
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   constexpr bool VMID = MID && MV == 1u, FOUR = MID && MV == 16u;
   constexpr uint32_t kMid = RAD, kFour = RAD + RAD * RAD;
   static_assert(!VMID || LEAF == kLeafShared, "voxel prefixes: shared leaves");
-  static_assert(!ONE || LEAF != kLeafShared, "one lane per cell: leaves in the scratch array");
+  static_assert(ONE ? LEAF != kLeafShared : LEAF != kLeafSectors, "one lane per cell: leaves in the scratch array; sectors: one lane per cell");
   constexpr bool REC = LEAF != kLeafShared;   // voxels in the scratch array, packed
   constexpr bool SEC = LEAF == kLeafSectors;  // ... as counts and quad sums, no voxel totals
   constexpr uint32_t NQ = 1u << (2 * (LV - 1));  // quads of a full tree
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         const uint64_t* line = rec + 16u * idx;
         const U64x4 x0 = load4(line), x1 = load4(line + 4), x2 = load4(line + 8),
                     x3 = load4(line + 12);
-        const uint32_t k = pick_child<!ONE>(x0.a, x1.a, x2.a, r);
+        const uint32_t k = pick_child<false>(x0.a, x1.a, x2.a, r);
         idx = 4u * idx + k;
         sec.a = k == 0u ? x0.a : k == 1u ? x1.a : k == 2u ? x2.a : x3.a;
         sec.b = k == 0u ? x0.b : k == 1u ? x1.b : k == 2u ? x2.b : x3.b;
@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           }
           a[j] = t;
         }
-        const uint32_t k = pick_child<!ONE>(a[0], a[1], a[2], r);
+        const uint32_t k = pick_child<false>(a[0], a[1], a[2], r);
         a_v = k == 0u ? a[0] : k == 1u ? a[1] : k == 2u ? a[2] : a[3];
         v = 4u * idx + k;
         D = field16(sec.b, k);
@@ -869,8 +869,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         newmax = nc;
       } else {
         newmax = (D + dD) | (N + dN) | (R + dR);
-        // binding, unbinding: two or three species change
-        if (several) dv = lane_total<MODEL>(q, tv, D + dD, N + dN, R + dR, nn, ctr) - a_v;
+        // binding, unbinding: two or three species change (not for lanes without a
+        // cell: what they read can send the Hill term to its slow path)
+        if (several && run) dv = lane_total<MODEL>(q, tv, D + dD, N + dN, R + dR, nn, ctr) - a_v;
       }
       uint32_t cu = 0;
       uint64_t a_u = 0, w_u = 0;  // records: u's total and word; sectors: its quad's sum and counts
@@ -1231,30 +1232,30 @@ ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   if (lv == L && leaf == F && G == N && helper == H) return k_chi_lane<MODEL, L, F, N, H>
   LANE_CASE(3, kLeafShared, 32, 6);
   LANE_CASE(3, kLeafShared, 16, 6);
-  LANE_CASE(3, kLeafShared, 16, 0);
   LANE_CASE(3, kLeafShared, 8, 6);
   if (MODEL != 1) LANE_CASE(3, kLeafShared, 8, 8);
   LANE_CASE(3, kLeafShared, 8, 0);
   LANE_CASE(3, kLeafShared, 4, 0);
+  LANE_CASE(3, kLeafRecords, 1, 8);
+  LANE_CASE(3, kLeafRecords, 1, 6);
   LANE_CASE(3, kLeafRecords, 1, 0);
   LANE_CASE(4, kLeafShared, 32, 6);
   LANE_CASE(4, kLeafShared, 16, 6);
-  LANE_CASE(4, kLeafShared, 16, 0);
   LANE_CASE(4, kLeafShared, 8, 6);
   if (MODEL != 1) LANE_CASE(4, kLeafShared, 8, 8);
   LANE_CASE(4, kLeafShared, 8, 0);
   LANE_CASE(4, kLeafShared, 4, 0);
   LANE_CASE(4, kLeafRecords, 8, 0);
   LANE_CASE(4, kLeafRecords, 4, 0);
+  LANE_CASE(4, kLeafSectors, 1, 8);
+  LANE_CASE(4, kLeafSectors, 1, 6);
   LANE_CASE(4, kLeafSectors, 1, 0);
   LANE_CASE(5, kLeafShared, 32, 6);
   LANE_CASE(5, kLeafShared, 16, 6);
-  LANE_CASE(5, kLeafShared, 8, 0);
   LANE_CASE(5, kLeafRecords, 16, 6);
   LANE_CASE(5, kLeafRecords, 16, 8);
   LANE_CASE(5, kLeafRecords, 16, 0);
   LANE_CASE(5, kLeafRecords, 8, 0);
-  LANE_CASE(5, kLeafSectors, 4, 0);
   LANE_CASE(5, kLeafSectors, 1, 6);
   LANE_CASE(5, kLeafSectors, 1, 0);
 #undef LANE_CASE

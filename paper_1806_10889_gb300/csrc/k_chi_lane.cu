@@ -18,24 +18,28 @@ ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G, uint32_t 
 
 }  // namespace
 
-// The shape follows from the cells an SM holds, per.  Chi ms of one step at
-// dt 0.02 (8x8 and 16x16 voxels) and 0.006 (32x32), 60 D + 30 N + 10 R per
-// voxel, by leaf (S shared, R records, X sectors) and lanes per cell, with the
-// segmented kernel's default launch in brackets:
-//   per     8x8                          16x16                        32x32
-//    4  S32 .37 S16 .42 [.70]   S32 1.44 S16 1.58 [2.65]     S32 1.91 S16 2.10 [3.2]
-//    8  S32 .43 S16 .43 [.83]   S16 1.59 S32 1.64 [2.89]     S16 2.09 S32 2.16 [3.5]
-//   13  S16 .46 S8 .48  [.85]   S8 1.74 S16 1.82  [3.18]  15 R16 3.35 R8 3.75  [4.9]
-//   27  S8 .55 S4 .62   [.93]   S8 2.04 S4 2.30 R8 2.80 [4.18]  R8 4.05 R16 4.19 [6.7]
-//   60  S4 .73          [1.2]   X4 3.67 R8 3.79 R4 3.90 [6.20] 53 R8 5.1 X4 5.5 [12.0]
-//   80  S4 .85          [2.0]   R4 4.33 X4 4.64   [9.67]  75 X4 6.7 X1 7.6 R8 8.6 [16.5]
-//  108  S4 1.05         [2.2]   X1 4.75 R4 4.84   [11.1]     X4 8.2 X1 8.6     [22.2]
-//  150  R1 1.35 S4 1.50 [2.9]   R1 5.3 X1 5.7     [15.1]     X1 9.6 X2 9.6     [30.1]
-//  431  R1 2.03 X1 2.7  [7.3]   X1 9.7 R1 11.7    [39.4]     X1 19.2 X2 20.6   [82.7]
-// Few cells: one chain of events sets the time, and more lanes per cell take
-// more of the draws off it.  Many: the instructions issued per event do, and
-// one lane per cell issues the fewest; past L2's size the random accesses to
-// DRAM do, and a sector makes two reads and two writes an event.
+// The shape follows from the cells an SM holds: the most lanes per cell with
+// which one wave runs them all (12 or 16 warps an SM).  Few cells: one chain of
+// events sets the time, and more lanes per cell take more of the draws off it.
+// Many: the instructions issued per event do, and one lane per cell issues the
+// fewest; past L2's size the random accesses to DRAM do, and a sector makes two
+// reads and two writes an event.  Chi ms of one step at dt 0.02 (8x8 and 16x16
+// voxels) and 0.006 (32x32), 60 D + 30 N + 10 R per voxel, by cells per SM; leaf
+// (S shared, R records, X sectors) and lanes per cell; in parentheses the next
+// shape, in brackets the segmented kernel's default launch:
+//         8x8                          16x16                        32x32
+//    4  S32 .26 (S16 .28) [.65]    S32 1.05 (S16 1.12) [2.6]    S32 1.39 (S16 1.43) [3.1]
+//    6  S16 .29 (S32 .29) [.71]    S16 1.15 (S32 1.22) [2.8]    S16 1.48 (S32 1.60) [3.5]
+//   12  S16 .34 (S8 .35)  [.79]    S16 1.34 (S8 1.36)  [3.1]    R16 2.68 (R8 3.68)  [4.0]
+//   32  S8 .42  (S4 .54)  [.87]    S8 1.68  (S4 2.09)  [4.1]    R16 3.55 (R8 4.03)  [6.7]
+//   48  S8 .52  (S4 .63)  [.98]  44 R8 2.93 (R4 3.60)  [5.2]  33 R8 4.26 (R16 5.5)  [9.8]
+//   64  S4 .64  (S8 .91)  [1.2]    R8 3.36  (R4 3.69)  [6.1]    R8 5.13  (X1 6.4)  [13.3]
+//   96  S4 .76  (R1 1.15) [2.0]  65 R4 3.93 (R8 5.0)   [8.7]  65 X1 6.45 (R8 7.7)  [15.2]
+//  128  R1 1.06           [2.2]    R4 4.58  (X1 5.24) [12.1]
+//  150  R1 1.12 (R4 1.36) [2.8]    X1 5.17  (R4 7.2)  [15.0]    X1 8.2             [30.1]
+//  431  R1 1.79           [7.0]    X1 9.0             [39.1]    X1 18.1            [84.0]
+// Cells of 10x10 voxels fit shared memory longer: 50 to 64 an SM take S4 (.98,
+// R8 1.13 to 1.20).
 LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   LanePlan pl;
   int dev = 0, sms = 0;
@@ -44,31 +48,36 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
     return pl;
   const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
   const uint64_t per = (cells + static_cast<uint64_t>(sms) - 1) / static_cast<uint64_t>(sms);
-  pl.G = per <= 4                      ? 32u
-         : per <= (lv == 5 ? 26u : 17u) ? 16u
-         : per <= 56                    ? 8u
-         : per <= (lv == 3 ? 110u : 100u) ? 4u
-                                          : 1u;
+  const uint32_t G = per <= 4                                        ? 32u
+                     : per <= (lv == 5 ? 32u : 12u)                  ? 16u
+                     : per <= (lv == 3 ? 48u : 64u)                  ? 8u
+                     : per <= (lv == 3 ? 96u : lv == 4 ? 128u : 64u) ? 4u
+                                                                     : 1u;
   // A helper warp that draws ahead while at most eight warps an SM run cells: the
   // draws leave the chain.  Up to six, twelve warps have the registers they want
   // (168).  Chi ms, without -> with: 2x2 cells of 8x8 voxels 1.19 -> 1.14, 60x50 of
   // 16x16 8.34 -> 7.70, 60 uneven tissues (26,802 cells of 32x32) 146.7 -> 133.9.
+  // One lane per cell, 190 cells of 16x16 an SM: 5.81 -> 5.24.
   // Seven and eight leave 128: 64x64 of 16x16 9.35 -> 9.12, promoter 7.41 -> 6.95,
   // 64x64 of 8x8 3.83 -> 3.69, 48x48 of 32x32 (records) 45.05 -> 44.36; with
   // in-voxel binding the spills cost more (16x16 9.74 -> 10.01) and it is not
   // built for 8 lanes; below six warps 128 registers cost 2% (7.68 -> 7.81).
-  const uint64_t runs = (cells * pl.G + 31u) / 32u;  // warps that run cells
+  const uint64_t runs = (cells * G + 31u) / 32u;  // warps that run cells
   const uint32_t few = runs <= 6u * static_cast<uint64_t>(sms)   ? 6u
                        : runs <= 8u * static_cast<uint64_t>(sms) ? 8u
                                                                  : 0u;
   const uint32_t nq = (V + 3u) / 4u;
-  const uint64_t places = 32u / pl.G;  // cells a warp runs
+  int per_sm = 0;  // blocks an SM holds
   // Leaves: in shared memory while one wave of cells fits there (the shortest
-  // chain); else records, whose totals need no recomputing; past L2's size, or
-  // where their sums (2.7 KB a cell of 32x32 voxels) would leave SMs short of
-  // cells, sectors, half the bytes and a quarter of the sums.
-  auto shape = [&](int leaf, uint32_t helper) {
-    const uint32_t cell = 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(pl.G)) +
+  // chain, also with four lanes per cell instead of eight); else records, whose
+  // totals need no recomputing; for one lane per cell, where L2's size and the
+  // sums in shared memory (2.7 KB a cell of 32x32 voxels) bound the cells in
+  // flight, sectors: half the bytes and a quarter of the sums (8x8 keeps records,
+  // 9.0 against 10.7 ms for 256x256 cells).
+  auto shape = [&](uint32_t G, int leaf, uint32_t helper) {
+    const uint64_t places = 32u / G;  // cells a warp runs
+    pl.G = G;
+    const uint32_t cell = 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(G)) +
                           (leaf == kLeafShared ? 20u * 4u * nq : 0u);
     // an odd multiple of 16 bytes: lanes reading the same entry of their cells
     // start on different shared-memory banks
@@ -76,28 +85,27 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
     pl.lut_bytes = 128u + 16u * ((nq + 3u) / 4u) + (helper ? kExchangeBytes : 0u);
     pl.leaf = leaf;
     pl.helper = helper;
-    pl.wpb = pl.G == 1 && !helper ? 2u : 1u;
+    pl.wpb = G == 1 && !helper ? 2u : 1u;
     pl.threads = helper ? 64u : 32u * pl.wpb;
     pl.smem = pl.lut_bytes + static_cast<size_t>(pl.wpb * places) * pl.cell_stride;
-    // whether one wave holds every cell (a block reserves 1 KB more)
-    return lane_kernel(model, V, leaf, pl.G, helper) != nullptr && pl.smem <= kMaxSmem &&
-           (per + pl.wpb * places - 1) / (pl.wpb * places) * (pl.smem + 1024u) <= 228u * 1024u;
+    // The answer: whether one wave holds every cell.  The shared-memory limit is
+    // the device's, not this plan's: plans of other cell sizes share the kernel.
+    const ChiLaneKernel k = lane_kernel(model, V, leaf, G, helper);
+    per_sm = 0;
+    if (!k || pl.smem > kMaxSmem ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, static_cast<int>(pl.threads),
+                                                      pl.smem) != cudaSuccess)
+      per_sm = 0;
+    return per <= static_cast<uint64_t>(per_sm) * pl.wpb * places;
   };
-  const int spill = lv == 3 || (lv == 4 && pl.G > 1) || (lv == 5 && pl.G > 4) ? kLeafRecords
-                                                                             : kLeafSectors;
-  if (!(few && shape(kLeafShared, few)) && !shape(kLeafShared, 0) &&
-      !(few && shape(spill, few)))
-    shape(spill, 0);
-  const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G, pl.helper);
-  int per_sm = 0;
-  // the limit is the device's, not this plan's: plans of other cell sizes
-  // share the kernel
-  if (!k || pl.smem > kMaxSmem ||
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, static_cast<int>(pl.threads),
-                                                    pl.smem) != cudaSuccess ||
-      per_sm < 1) {
+  const int spill = G == 1 && lv > 3 ? kLeafSectors : kLeafRecords;
+  if (!(few && shape(G, kLeafShared, few)) && !shape(G, kLeafShared, 0) &&
+      !(G == 8 && shape(4, kLeafShared, 0)) && !(few && shape(G, spill, few)) &&
+      !shape(G, spill, 0) && per_sm < 1)
+    shape(G, kLeafShared, 0);
+  if (per_sm < 1) {
     pl.G = 0;
     return pl;
   }

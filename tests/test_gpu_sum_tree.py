@@ -63,7 +63,7 @@ def _compare(g, spec, ref, ne, tl, ctx):
 # (cells per SM, n, dt): shared leaves at 32, 16, 8 and 4 lanes; records at 16,
 # 8, 4 and 1; sectors at 4 and 1 (V = 4, 25, 49, 64, 81, 256, 289, 324 and 1,024)
 FORMS = [(1, 2, 0.3), (8, 5, 0.1), (20, 7, 0.1), (100, 5, 0.02), (8, 16, 0.02), (30, 9, 0.02),
-         (28, 8, 0.02), (28, 16, 0.01),
+         (28, 8, 0.02), (28, 16, 0.01), (40, 9, 0.02), (90, 8, 0.01), (140, 9, 0.01), (50, 17, 0.01),
          (45, 16, 0.01), (98, 9, 0.01), (120, 2, 0.1), (120, 8, 0.01), (120, 9, 0.01),
          (3, 17, 0.02), (9, 18, 0.02), (30, 17, 0.01), (85, 17, 0.005), (112, 17, 0.005),
          (2, 32, 0.01), (16, 32, 0.005)]
