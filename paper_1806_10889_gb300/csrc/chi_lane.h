@@ -46,9 +46,9 @@ struct LaneArgs {
 };
 
 struct LanePlan {
-  uint32_t G = 0, wpb = 0, threads = 0, blocks = 0;  // G = 0: this launch stays with the segmented kernel
+  uint32_t G = 0, wpb = 0, threads = 0, blocks = 0;  // G = 0: stays with the segmented kernel
   int leaf = kLeafShared;
-  uint32_t helper = 0;    // two warps a block: one runs cells, one draws ahead; blocks an SM
+  uint32_t helper = 0;    // blocks an SM of two warps, one of which draws ahead; 0: none
   uint32_t lut_bytes = 0, cell_stride = 0;
   size_t smem = 0, scratch_bytes = 0;
   bool small = false;     // at most one block per SM
@@ -56,8 +56,9 @@ struct LanePlan {
 };
 
 // The plan for `cells` cells of V voxels; model 0: Notch-Delta without
-// in-voxel binding, 1: Notch-Delta, 2: promoter.
-LanePlan lane_plan(uint32_t V, uint64_t cells, int model);
+// in-voxel binding, 1: Notch-Delta, 2: promoter.  `beside`: warps of launches
+// that run at the same time and come first.
+LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside = 0);
 cudaError_t launch_chi_lane(const LanePlan& plan, int model, const TissueView* d_views,
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,

@@ -40,7 +40,7 @@ ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G, uint32_t 
 //  431  R1 1.79           [7.0]    X1 9.0             [39.1]    X1 18.1            [84.0]
 // Cells of 10x10 voxels fit shared memory longer: 50 to 64 an SM take S4 (.98,
 // R8 1.13 to 1.20).
-LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
+LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
   LanePlan pl;
   int dev = 0, sms = 0;
   if (cells == 0 || cudaGetDevice(&dev) != cudaSuccess ||
@@ -62,7 +62,10 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
   // 64x64 of 8x8 3.83 -> 3.69, 48x48 of 32x32 (records) 45.05 -> 44.36; with
   // in-voxel binding the spills cost more (16x16 9.74 -> 10.01) and it is not
   // built for 8 lanes; below six warps 128 registers cost 2% (7.68 -> 7.81).
-  const uint64_t runs = (cells * G + 31u) / 32u;  // warps that run cells
+  // Classes of a batch share the SMs, the first ahead of the others, which run
+  // in what it leaves: a helper there takes warps and issue slots from it (60
+  // uneven tissues, helpers in all three classes 138.8, with this count 132.9).
+  const uint64_t runs = beside + (cells * G + 31u) / 32u;
   const uint32_t few = runs <= 6u * static_cast<uint64_t>(sms)   ? 6u
                        : runs <= 8u * static_cast<uint64_t>(sms) ? 8u
                                                                  : 0u;
@@ -125,7 +128,8 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model) {
 cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_views,
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
-                            uint32_t step_off, double dt, cudaStream_t stream, int priority, bool early) {
+                            uint32_t step_off, double dt, cudaStream_t stream, int priority,
+                            bool early) {
   const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G, pl.helper);
   const LaneArgs a{d_views, d_items, d_counter, d_scratch, redo.items, redo.counters + 1, dt,
                    n_items, step_off, V, n, pl.lut_bytes, pl.cell_stride};

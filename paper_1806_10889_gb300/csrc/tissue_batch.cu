@@ -274,6 +274,7 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
   }
   std::vector<uint2> items;
   size_t lane_words = 0;
+  uint64_t lane_warps = 0;  // of the classes before: all run at the same time
   for (auto& kv : by_v) {
     if (kv.second.empty()) continue;  // every cell of this size is well-mixed
     ClassPlan p{};
@@ -288,7 +289,8 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     p.gen = (nd_v[V] == 0 && pm_v[V] > 0) ? 2 : (pm_v[V] > 0 || tr_v[V] > 0) ? 1 : 0;
     while (p.n * p.n < V) ++p.n;
     p.lane_model = p.gen == 2 ? 2 : bind_v[V] > 0 ? 1 : 0;
-    if (p.gen != 1) p.lane = lane_plan(V, kv.second.size(), p.lane_model);
+    if (p.gen != 1) p.lane = lane_plan(V, kv.second.size(), p.lane_model, lane_warps);
+    if (p.lane.G) lane_warps += static_cast<uint64_t>(p.lane.blocks) * (p.lane.threads / 32u);
     p.lane_off = lane_words;
     lane_words += ((p.lane.scratch_bytes + 255) & ~static_cast<size_t>(255)) / sizeof(uint64_t);
     items.insert(items.end(), kv.second.begin(), kv.second.end());
