@@ -95,6 +95,21 @@ CHI_IPE = {
         "batch:V64/H8/rec/qb0/nd/u32": (239.3, 0.5607),
     },
 }
+# The same of the sum-tree chi kernel, which runs default launch shapes in a form
+# that follows from the cell size and the number of cells (its warps serve up to
+# 32 cells): per workload and cell size, with its own sources.
+TREE_SOURCES = ["chi_lane.cuh", "chi_lane.h", "tissue_dev.cuh", "k_chi_lane.cu",
+                "k_chi_lane_bind.cu", "k_chi_lane_pm.cu"]
+TREE_IPE = {
+    "sources": "2b3a23066718a2fc",
+    "kernels": {
+        "batch:V1024": (42.4, 146.6),
+        "batch:V256": (40.1, 78.7),
+        "batch:V64": (34.0, 23.0),
+        "medium:V256": (98.3, 0.314),
+        "large:V1024": (42.6, 147.4),
+    },
+}
 
 
 def _code_of(name: str, text: str) -> str:
@@ -108,17 +123,17 @@ def _code_of(name: str, text: str) -> str:
     return "\n".join(ln for ln in lines if ln.strip())
 
 
-def chi_sources_sha(read=None) -> str:
-    """SHA-256 over the persistent chi kernel's code (comments stripped) and
-    the nvcc flags.  read(name) returns a source's text (default: the files
-    in csrc/)."""
+def chi_sources_sha(read=None, files=None) -> str:
+    """SHA-256 over a chi kernel's code (default: the persistent one's;
+    comments stripped) and the nvcc flags.  read(name) returns a source's text
+    (default: the files in csrc/)."""
     from paper_1806_10889_gb300.build import NVCC_FLAGS
     if read is None:
         def read(name):
             with open(os.path.join(CSRC, name)) as fh:
                 return fh.read()
     h = hashlib.sha256()
-    for f in CHI_SOURCES:
+    for f in files or CHI_SOURCES:
         h.update(f.encode() + b"\0" + _code_of(f, read(f)).encode())
     h.update(" ".join(x for x in NVCC_FLAGS if not x.startswith("-I")).encode())
     return h.hexdigest()[:16]
@@ -133,10 +148,38 @@ def chi_kernel_key(V: int, lanes: int, layout: int, model: str = "nd") -> str:
             f"{'u16' if narrow else 'u32'}")
 
 
+def chi_launch_key(V: int, lanes: int, warps_per_block: int, layout: int) -> str:
+    """What a Notch-Delta launch of this shape runs: the sum-tree kernel for the
+    default shapes of the cell size, else the persistent kernel's
+    instantiation."""
+    few = (32, 2, 0)
+    default = {few, (8, 4, 0)} if V <= 64 else {few, (16, 4, 0), (8, 2, 1)} if V <= 256 else \
+        {few, (16, 2, 1)}
+    if (lanes, warps_per_block, layout) in default:
+        return f"V{V}/tree"
+    return chi_kernel_key(V, lanes, layout)
+
+
+def chi_kernel_name(key: str) -> str:
+    return f"{'k_chi_lane' if key.endswith('/tree') else 'k_chi_seg'} {key}"
+
+
+def chi_launches(key: str, cells: int) -> int:
+    """Kernels of one chi phase: the launch, and a second one for cells past
+    the range of packed counts, where there are any (the persistent kernel's
+    16-bit counts; the sum-tree kernel from 128 cells an SM up, which it keeps
+    packed at every cell size)."""
+    return 1 + int(cells > 128 * 152 if key.endswith("/tree") else key.endswith("u16"))
+
+
 def chi_ipe(workload: str, key: str):
     """(warp instructions per chi event, DRAM bytes per chi event) of a kernel
     instantiation on a workload, or None when unmeasured or measured on other
     kernel sources."""
+    if key.endswith("/tree"):
+        if TREE_IPE["sources"] != chi_sources_sha(files=TREE_SOURCES):
+            return None
+        return TREE_IPE["kernels"].get(f"{workload}:{key[:-5]}")
     if CHI_IPE["sources"] != chi_sources_sha():
         return None
     return CHI_IPE["kernels"].get(f"{workload}:{key}")
@@ -254,7 +297,7 @@ def issue_roofline(workload: str, chi_events: float, chi_ms: float, key: str, V:
     hbm = 24 * V * cells * steps / chi_s / 1e9 if chi_s > 0 else 0.0
     m = chi_ipe(workload, key)
     out = {"bound": "alu", "unit": "Gwarp-inst/s", "peak": ISSUE_PEAK_GINST,
-           "peak_source": "152 SMs x 4 issue/clk x 2.070 GHz", "kernel": f"k_chi_seg {key}",
+           "peak_source": "152 SMs x 4 issue/clk x 2.070 GHz", "kernel": chi_kernel_name(key),
            "chi_events_per_s": rate, "launch_ms": chi_ms / max(launches, 1),
            "hbm_gbs": hbm, "hbm_frac": hbm / peaks["hbm_gbs"], "hbm_peak_source": peak_kind}
     if m is None:
@@ -263,6 +306,9 @@ def issue_roofline(workload: str, chi_events: float, chi_ms: float, key: str, V:
         return out
     ipe, traffic_per_event = m
     ach = rate * ipe / 1e9
+    if traffic_per_event is not None:
+        dram = rate * traffic_per_event / 1e9
+        out.update({"dram_gbs": dram, "dram_frac": dram / peaks["hbm_gbs"]})
     out.update({"achieved": ach, "frac": ach / ISSUE_PEAK_GINST, "inst_per_event": ipe,
                 "traffic": (traffic_per_event * chi_events / max(launches, 1)
                             if traffic_per_event is not None else None)})
@@ -420,7 +466,7 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
     per_class, inst, traffic, stale = [], 0.0, 0.0, False
     for ci, c in enumerate(classes):
         idx = [i for i, r in enumerate(runs) if r.tissue.V == c["V"]]
-        key = chi_kernel_key(c["V"], c["lanes_per_cell"], c["smem_layout"])
+        key = chi_launch_key(c["V"], c["lanes_per_cell"], c["warps_per_block"], c["smem_layout"])
         ev_c = float(d_ev[idx, 0].sum())
         m = chi_ipe("batch", key)
         if m is None:
@@ -430,7 +476,7 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
             traffic = None if traffic is None or m[1] is None else traffic + ev_c * m[1]
         per_class.append({"V": c["V"], "cells": c["cells"], "tissues": len(idx),
                           "launch": [c["lanes_per_cell"], c["warps_per_block"], c["smem_layout"]],
-                          "kernel": f"k_chi_seg {key}",
+                          "kernel": chi_kernel_name(key),
                           "span_ms_per_step": class_ms[ci] / args.steps,
                           "chi_events_per_step": ev_c / args.steps,
                           "inst_per_event": None if m is None else m[0]})
@@ -440,7 +486,8 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
     hbm = sum(24 * c["V"] * c["cells"] for c in classes) * args.steps / chi_s / 1e9
     roofline = {"bound": "alu", "unit": "Gwarp-inst/s", "peak": ISSUE_PEAK_GINST,
                 "peak_source": "152 SMs x 4 issue/clk x 2.070 GHz",
-                "kernel": "k_chi_seg, one launch per cell-size class, " +
+                "kernel": " + ".join(sorted({c["kernel"].split()[0] for c in per_class})) +
+                          ", one launch per cell-size class, " +
                           ("overlapped" if bt.overlap else "one after another"),
                 "chi_events_per_s": chi_events / chi_s, "launch_ms": chi_ms / args.steps,
                 "hbm_gbs": hbm, "hbm_frac": hbm / peaks["hbm_gbs"], "hbm_peak_source": peak_kind}
@@ -452,6 +499,9 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
         roofline.update({"achieved": ach, "frac": ach / ISSUE_PEAK_GINST,
                          "inst_per_event": inst / chi_events,
                          "traffic": None if traffic is None else traffic / args.steps})
+        if traffic is not None:
+            roofline.update({"dram_gbs": traffic / chi_s / 1e9,
+                             "dram_frac": traffic / chi_s / 1e9 / peaks["hbm_gbs"]})
 
     # end to end through the C ABI: every tissue's state from pinned host
     # memory before each step, back to pinned host memory after it (the
@@ -576,11 +626,12 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
         "cpu_baseline": cpu,
         "parity_checked": None if cpu is None else cpu["parity_checked"],
     }
-    # our kernels per step: per class the chi launch (and, for cells of more
-    # than 256 voxels with 16-bit counts, its 32-bit redo pass), both face
-    # phases and the step-counter update
-    per_step = sum(1 + int(chi_kernel_key(c["V"], c["lanes_per_cell"], c["smem_layout"])
-                           .endswith("u16")) for c in classes) + 3
+    # our kernels per step: per class the chi launch (and the pass over cells
+    # past the range of packed counts), both face phases and the step-counter
+    # update
+    per_step = sum(chi_launches(chi_launch_key(c["V"], c["lanes_per_cell"], c["warps_per_block"],
+                                               c["smem_layout"]), c["cells"])
+                   for c in classes) + 3
     out["gpu_launches"] = per_step * args.steps
     return out
 
@@ -653,7 +704,7 @@ def medium_leg(args) -> dict:
     nbytes = spec.state_ints * 4
     g.close()
 
-    key = chi_kernel_key(spec.V, launch[1], launch[4]) if launch[0] == 1 else "warp"
+    key = chi_launch_key(spec.V, launch[1], launch[2], launch[4]) if launch[0] == 1 else "warp"
     out = {"metric": MEDIUM_METRIC, "value": events / (total_ms / 1e3), "unit": UNIT,
            "workload": f"tissue {spec.width}x{spec.height} cells of {spec.n}x{spec.n} voxels, "
                        f"Notch-Delta model, dt {args.dt}, burn-in {args.burn_in} time units, "
@@ -754,7 +805,8 @@ def large_leg(args) -> dict:
     burn = int(round(args.large_burn_in / lg.dt))
     r = _timed_tissue(lg.tissue, lg.dt, burn, args.large_steps, flush=False)
     cl = r["chi_launch"]
-    key = chi_kernel_key(lg.tissue.V, cl["lanes_per_cell"], cl["smem_layout"])
+    key = chi_launch_key(lg.tissue.V, cl["lanes_per_cell"], cl["warps_per_block"],
+                         cl["smem_layout"])
     r["roofline"] = issue_roofline("large", r.pop("chi_ev"), r.pop("chi_ms"), key, lg.tissue.V,
                                    lg.tissue.cells, args.large_steps, args.large_steps)
     r["workload"] = (f"tissue 256x256 cells of 32x32 voxels, Notch-Delta model, dt 0.1, "
@@ -949,7 +1001,10 @@ def run_profile(args) -> dict:
     instructions and DRAM bytes per event.  Workloads: "batch" (a subset of
     the batch with every cell-size class), "medium" and "large".  Under ncu,
     skip the chi launches of the burn-in and warm-up (launches_before in the
-    output) and capture launches_per_step x steps of them."""
+    output) and capture launches_per_step x steps of them.  The batch runs a
+    subset of its tissues for --profile-class shapes (instructions per event do
+    not depend on the number of cells there), else all of them (the sum-tree
+    kernel's form does)."""
     import torch
 
     from paper_1806_10889_gb300.batching import Batch
@@ -957,7 +1012,7 @@ def run_profile(args) -> dict:
 
     if args.profile_chi == "batch":
         runs = batch_runs()
-        idx = profile_subset(runs)
+        idx = profile_subset(runs) if args.profile_class else list(range(len(runs)))
         sub = [runs[i] for i in idx]
         burn_time = args.batch_burn_in
     else:
@@ -986,8 +1041,9 @@ def run_profile(args) -> dict:
         classes = [{"V": g.spec.V, "lanes_per_cell": la[1], "warps_per_block": la[2],
                     "smem_layout": la[4], "cells": g.spec.cells}]
         step, sync = g.step, g.sync
-    keys = [chi_kernel_key(c["V"], c["lanes_per_cell"], c["smem_layout"]) for c in classes]
-    per_step = sum(1 + int(k.endswith("u16")) for k in keys)
+    keys = [chi_launch_key(c["V"], c["lanes_per_cell"], c["warps_per_block"], c["smem_layout"])
+            for c in classes]
+    per_step = sum(chi_launches(k, c["cells"]) for k, c in zip(keys, classes))
     burn = int(round(burn_time / dt))
     step(dt, burn + args.warmup)
     sync()
@@ -1009,7 +1065,8 @@ def run_profile(args) -> dict:
             "classes": [dict(c, key=k) for c, k in zip(classes, keys)],
             "chi_launches_per_step": per_step,
             "launches_before": per_step * (burn + args.warmup),
-            "chi_events_per_step_by_class": steps, "sources": chi_sources_sha()}
+            "chi_events_per_step_by_class": steps, "sources": chi_sources_sha(),
+            "tree_sources": chi_sources_sha(files=TREE_SOURCES)}
 
 
 # ---------------------------------------------------------------------------

@@ -232,7 +232,7 @@ typedef struct {
  * launch on a 152-SM GB300).  While the shape is one of these defaults, for
  * whatever number of cells, the library may run the step with its sum-tree
  * kernel instead, in a form that fits the number of cells; it uses up to
- * 1.4 GB of device memory for the length of a call, and keeps to the shape
+ * 0.35 GB of device memory for the length of a call, and keeps to the shape
  * when that cannot be had, while a trace is on, and in a stream capture that
  * would need it.  Another shape is run as it is.  A recompute launch with
  * more voxels per block than lanes that the tissue's model cannot take (the
@@ -410,7 +410,9 @@ int tissue_trace_end(tissue* t);
 /* Host-side fault injection for tests: the next n device allocations the
  * library makes (tissue_create, tissue_batch_create, tissue_trace_begin)
  * fail as an out-of-memory cudaMalloc would (TISSUE_E_NOMEM), without
- * touching the GPU.  n = 0 disarms it. */
+ * touching the GPU.  n = 0 disarms it.  The scratch of a tissue's step
+ * (tissue_step, tissue_step_timed) and of a batch's classes count too; without
+ * it the step runs the same on the segmented kernel and nothing fails. */
 int tissue_debug_fail_allocs(uint32_t n);
 
 /* Release library scratch (not the caller's buffer or stream). */

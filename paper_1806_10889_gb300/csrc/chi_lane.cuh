@@ -8,13 +8,13 @@
 // as the cell's lanes (8 or 16): a lane holds the prefix before its child, one
 // compare, ballot and population count find the child (11 instructions for 3 or
 // 4 bits, 26 for 2 in a four-ary node), the root's prefixes stay in registers,
-// and an update is one predicated addition per lane.  An event descends from the root in the direct method's voxel-major order,
-// finds the channel inside the voxel in closed form, changes one or two
-// voxels and adds the two differences along their paths: 250 to 500
-// instructions, the most of which no lane can take off another.  The
-// segmented kernel (chi_seg.cuh) finds a voxel with ballots and scans over 8
-// to 32 lanes, and its event loop (600 to 900 instructions) serves one to four
-// cells; here an instruction serves up to 32 (G = 1).
+// and an update is one predicated addition per lane.  An event descends from the
+// root in the direct method's voxel-major order, finds the channel inside the
+// voxel in closed form, changes one or two voxels and adds the two differences
+// along their paths: 250 to 500 instructions, the most of which no lane can take
+// off another.  The segmented kernel (chi_seg.cuh) finds a voxel with ballots and
+// scans over 8 to 32 lanes, and its event loop (600 to 900 instructions) serves
+// one to four cells; here an instruction serves up to 32 (G = 1).
 //
 // What the G lanes of a cell share out is the work that does not depend on
 // the state: lane j of the cell draws the random numbers of event j of the
@@ -22,21 +22,24 @@
 // waiting time only decides where the cell stops.  So the G events are applied
 // first, the total propensity A before each kept by its lane, then all G
 // waiting times are computed at once and added in order (by a scan of integers
-// while the time's exponent stays the same).  With few warps on an SM a helper
-// warp beside each draws a batch ahead of it; the events past the end of the
+// while the time's exponent stays the same); the events past the end of the
 // step are undone (at most G a cell and step, on the counts only: the sums are
-// not used again).
+// not used again).  With few warps on an SM a helper warp beside each draws a
+// batch ahead of it.
 //
-// Bound (one GB300, from ncu): few cells by the event chain -- one warp alone
+// Bound (one GB300, from ncu).  Few cells: the event chain -- one warp alone
 // issues every 3.9 cycles, 260 instructions and 1,010 cycles an event with G =
 // 32 (2,530 cycles in the segmented kernel; 371 and 1,320 with four-ary nodes
-// and the times added one by one); cells of up to 256 voxels that fill the chip by issue
-// (32 warp instructions per event with G = 1 against 171 and 227, 8x8 and
-// 16x16 voxels); larger ones by random accesses to L2 and DRAM (a dependent
-// read and write per lane reaches 25 G/s in DRAM, 42 G/s in L2, and an event
-// makes two).  Chi ms per step, before -> with this kernel: 2x2 cells of 8x8
-// voxels 2.9 -> 1.17, 64x64 of 16x16 21.1 -> 9.3, 48x48 of 32x32 77.5 -> 45.0,
-// 256x256 of 8x8 33.4 -> 7.9, 256x256 of 32x32 611 -> 136.
+// and the times added one by one).  Cells of up to 256 voxels that fill the
+// chip: issue (34 and 40 warp instructions an event with G = 1, 8x8 and 16x16
+// voxels, 44 to 48% of the peak; 171 and 227 segmented) beside their scattered
+// accesses (57% of the L1 wavefronts).  Larger ones that do: shared memory
+// holds 8 warps an SM, 6 cycles an instruction of which 2.3 wait for the
+// scattered leaves (43 instructions and 147 DRAM bytes an event, 1.4 TB/s; a
+// dependent read and write a lane reaches 25 G/s in DRAM, an event makes two).
+// Chi ms per step, segmented -> this kernel: 2x2 cells of 8x8 voxels 2.9 ->
+// 1.10, 64x64 of 16x16 21.1 -> 9.1, 48x48 of 32x32 77.5 -> 44.4, 256x256 of 8x8
+// 33.4 -> 7.9, 256x256 of 32x32 611 -> 122.
 //
 // Template parameters: MODEL 0 Notch-Delta without in-voxel binding (k_in =
 // k_off = 0), 1 Notch-Delta, 2 promoter; LV the levels of the tree (V <= 4^LV,
@@ -49,7 +52,9 @@
 // whole, the four totals of the chosen quad recomputed, the sum and the changed
 // count of one or two quads written (256x256 cells of 32x32 voxels: 174 ms with
 // records and a level of quad sums beside them, 490 DRAM bytes an event; 122 ms
-// and 217 bytes with sectors); G.
+// and 147 bytes with sectors; 132 ms with 32 bits a voxel and the sums of all
+// four quads recomputed, 260 instructions more); G lanes per cell; HELP blocks
+// an SM with a helper warp, 0: none.
 //
 // Limits.  Counts below the tissue's `small` keep every total below 2^52
 // unchecked, and R below kLaneHill reads the Hill table unchecked.  With
@@ -283,11 +288,10 @@ __device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base)
   return static_cast<uint32_t>(k);
 }
 
-// Registers: shared leaves as many as they take (150 to 170; shared memory or
-// the number of cells bounds the warps); one lane per cell of more than 256
-// voxels up to 255 (shared memory holds 8 warps an SM anyway); with a helper of
-// HELP blocks an SM 168 (six, 12 warps) or 128 (eight); else 128, so that 14 to
-// 16 warps fit an SM.
+// Registers: shared leaves 168 (12 warps an SM; beyond, more lanes' worth of cells
+// take records); one lane per cell of more than 256 voxels up to 255 (shared
+// memory holds 8 warps an SM anyway); with a helper of HELP blocks an SM 168 (six,
+// 12 warps) or 128 (eight); else 128, so that 14 to 16 warps fit an SM.
 template <int MODEL, int LV, int LEAF, int G, int HELP>
 __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                  ? HELP
                                                             : LEAF == kLeafShared ? 12
@@ -311,7 +315,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   constexpr bool VMID = MID && MV == 1u, FOUR = MID && MV == 16u;
   constexpr uint32_t kMid = RAD, kFour = RAD + RAD * RAD;
   static_assert(!VMID || LEAF == kLeafShared, "voxel prefixes: shared leaves");
-  static_assert(ONE ? LEAF != kLeafShared : LEAF != kLeafSectors, "one lane per cell: leaves in the scratch array; sectors: one lane per cell");
+  static_assert(ONE ? LEAF != kLeafShared : LEAF != kLeafSectors,
+                "one lane per cell: leaves in the scratch array; sectors: one lane per cell");
   constexpr bool REC = LEAF != kLeafShared;   // voxels in the scratch array, packed
   constexpr bool SEC = LEAF == kLeafSectors;  // ... as counts and quad sums, no voxel totals
   constexpr uint32_t NQ = 1u << (2 * (LV - 1));  // quads of a full tree

@@ -152,7 +152,7 @@ namespace {
 
 // Scratch of the sum-tree kernel for single tissues: allocated on the
 // tissue's stream for the length of one call, from one pool per device that
-// keeps freed memory (at most what ran at once: about 1.4 GB a stream) until
+// keeps freed memory (at most what ran at once: 0.35 GB a stream) until
 // a tissue is destroyed.  Streams never wait for one another's memory.
 constexpr int kMaxDevices = 128;
 std::mutex g_pool_mu;
