@@ -38,14 +38,16 @@
 // scattered leaves (43 instructions and 147 DRAM bytes an event, 1.4 TB/s; a
 // dependent read and write a lane reaches 25 G/s in DRAM, an event makes two).
 // Chi ms per step, segmented -> this kernel: 2x2 cells of 8x8 voxels 2.9 ->
-// 1.10, 64x64 of 16x16 21.1 -> 9.1, 48x48 of 32x32 77.5 -> 44.4, 256x256 of 8x8
+// 1.10, 64x64 of 16x16 21.1 -> 9.1, 48x48 of 32x32 77.5 -> 31.0, 256x256 of 8x8
 // 33.4 -> 7.9, 256x256 of 32x32 611 -> 122.
 //
 // Template parameters: MODEL 0 Notch-Delta without in-voxel binding (k_in =
 // k_off = 0), 1 Notch-Delta, 2 promoter; LV the levels of the tree (V <= 4^LV,
 // LV = 3, 4, 5); LEAF where the voxels live (chi_lane.h): shared memory (20
-// bytes a voxel and the sums: the shortest chain), or a scratch array with the
-// upper sums in shared memory, so that hundreds of cells fit on an SM --
+// bytes a voxel and the sums: the shortest chain); planes there, 16-bit counts
+// and no totals (6 bytes a voxel: two to four times the cells; four lanes
+// recompute the totals of the chosen quad, one each); or a scratch array with
+// the upper sums in shared memory, so that hundreds of cells fit on an SM --
 // records, total and packed counts of a voxel side by side, a quad one aligned
 // 64-byte block; or sectors, 32 bytes a quad with its sum and 16-bit counts,
 // the four quads under a shared sum one 128-byte line that an event reads
@@ -55,6 +57,10 @@
 // and 147 bytes with sectors; 132 ms with 32 bits a voxel and the sums of all
 // four quads recomputed, 260 instructions more); G lanes per cell; HELP blocks
 // an SM with a helper warp, 0: none.
+//
+// Planes against records: 48x48 cells of 32x32 voxels 44.2 -> 31.0 ms, 76x76 of
+// 16x16 13.8 -> 11.1, 113x113 of them 19.8 -> 15.9 (an event's two dependent
+// accesses to L2, 400 cycles each and more under load, become shared memory's 30).
 //
 // Limits.  Counts below the tissue's `small` keep every total below 2^52
 // unchecked, and R below kLaneHill reads the Hill table unchecked.  With
@@ -317,7 +323,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   static_assert(!VMID || LEAF == kLeafShared, "voxel prefixes: shared leaves");
   static_assert(ONE ? LEAF != kLeafShared : LEAF != kLeafSectors,
                 "one lane per cell: leaves in the scratch array; sectors: one lane per cell");
-  constexpr bool REC = LEAF != kLeafShared;   // voxels in the scratch array, packed
+  constexpr bool PLN = LEAF == kLeafPlanes;   // 16-bit counts in shared memory, no voxel totals
+  static_assert(!PLN || G == 4 || (MID && MV == 4u), "planes: sums down to quads");
+  constexpr bool REC = LEAF != kLeafShared;   // counts in a packed range (else: scratch array)
   constexpr bool SEC = LEAF == kLeafSectors;  // ... as counts and quad sums, no voxel totals
   constexpr uint32_t NQ = 1u << (2 * (LV - 1));  // quads of a full tree
   // the levels of sums in shared memory: down to the quads' (sectors: down to
@@ -410,9 +418,10 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   int32_t* cp = reinterpret_cast<int32_t*>(tree + kCnt + ps);
   // a cell's scratch: 2 words per voxel, its total and its counts (records);
   // or 4 words per quad, its sum and its counts of D, N and R (sectors)
+  uint16_t* hp = reinterpret_cast<uint16_t*>(tree + kCnt);  // planes: the counts
   const uint32_t rec_words = SEC ? 16u * nl : 8u * nq;
   uint64_t* warp_rec =
-      REC ? p.scratch + (static_cast<size_t>(blockIdx.x) * warps + wib) * slots * rec_words
+      REC && !PLN ? p.scratch + (static_cast<size_t>(blockIdx.x) * warps + wib) * slots * rec_words
           : nullptr;
   uint64_t* rec = warp_rec + static_cast<size_t>(slot) * rec_words;
 
@@ -508,7 +517,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
               }
               if (REC) {
                 // past the packed word's range: to the redo list
-                nbig |= (d[i] | m[i]) >= (SEC ? kSectorCount : kWordCount);
+                nbig |= PLN ? max(d[i], m[i]) >= kPlaneCount
+                            : (d[i] | m[i]) >= (SEC ? kSectorCount : kWordCount);
                 wd[i] = pack_voxel(d[i], m[i], r[i] & 0xFFFFFu, mk & 15u);
               }
               a[i] = lane_total<MODEL>(nr, ntv, d[i], m[i], r[i], nn, ctr);
@@ -517,6 +527,11 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           }
           if (SEC) {
             store4(nrec + 4u * qi, U64x4{S, pack4(d), pack4(m), pack4(r)});
+          } else if (PLN) {
+            uint64_t* o = ntree + kCnt;
+            o[qi] = pack4(d);
+            o[nq + qi] = pack4(m);
+            o[2u * nq + qi] = pack4(r);
           } else if (REC) {
             ulonglong2* o = reinterpret_cast<ulonglong2*>(nrec) + 4u * qi;
 #pragma unroll
@@ -607,7 +622,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         have = true;
         if (REC) {
           // the bits a count has once it reaches its limit (a power of two)
-          const uint32_t lc = min(q.small, SEC ? kSectorCount : kWordCount), lr = MODEL == 2 ? lc : min(q.small, kLaneHill);
+          const uint32_t lc = min(q.small, PLN ? kPlaneCount : SEC ? kSectorCount : kWordCount), lr = MODEL == 2 ? lc : min(q.small, kLaneHill);
           const uint32_t mc = 0xFFFFFu & ~(lc - 1u), mr = 0xFFFFFu & ~(lr - 1u);
           over_mask = pack_voxel(mc, mc, mr, 0u);
           lim_dn = lc;
@@ -753,6 +768,38 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         const uint32_t mk = (mk4 >> (8u * k)) & 0xFFu;
         mask = mk & 15u;
         nn = mk >> 4;
+      } else if (PLN) {
+        // lane j of every four computes the quad's voxel j; the prefixes find v
+        const uint32_t vj = 4u * idx + (sl & 3u);
+        const uint32_t Dj = hp[vj], Nj = hp[ps + vj], Rj = hp[2u * ps + vj];
+        const uint32_t mk = lut[vj], nj = mk >> 4;
+        uint64_t t = (q.gD + q.hD * nj) * Dj + (q.gN + q.hN * nj) * Nj;
+        if (MODEL == 2) {
+          const uint32_t Fj = static_cast<uint32_t>(vj == centre) - Rj;
+          t += q.tD * Fj + q.kd * Rj + q.k_in * (static_cast<uint64_t>(Nj) * Fj);
+        } else {
+          // R < kLaneHill in a cell that runs; the mask is for idle lanes
+          t += (q.gR + q.k_off + q.hR * nj) * Rj + __ldg(q.hill + (Rj & (kHillTab - 1u))) + q.kN;
+          if (MODEL == 1) t += q.k_in * (static_cast<uint64_t>(Dj) * Nj);
+        }
+        uint64_t in = t;
+        uint64_t z = __shfl_up_sync(kFull, in, 1, 4);
+        if (sl & 3u) in += z;
+        z = __shfl_up_sync(kFull, in, 2, 4);
+        if (sl & 2u) in += z;
+        const uint64_t ex4 = in - t;
+        const unsigned b4 = __ballot_sync(kFull, r >= ex4) >> base_lane;
+        const int k = __popc((b4 | 1u) & 15u) - 1;
+        r -= __shfl_sync(kFull, ex4, base_lane + k);
+        a_v = __shfl_sync(kFull, t, base_lane + k);
+        const uint32_t dn = __shfl_sync(kFull, Dj | (Nj << 16), base_lane + k);
+        const uint32_t rm = __shfl_sync(kFull, Rj | (mk << 16), base_lane + k);
+        v = 4u * idx + static_cast<uint32_t>(k);
+        D = dn & 0xFFFFu;
+        N = dn >> 16;
+        R = rm & 0xFFFFu;
+        mask = (rm >> 16) & 15u;
+        nn = rm >> 20;
       } else if (REC) {
         const U64x4 x = load4(rec + 8u * idx);
         const U64x4 y = load4(rec + 8u * idx + 4u);
@@ -891,6 +938,14 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           if (MODEL == 2 && s == 1u)
             du += q.k_in * (static_cast<uint32_t>(u == centre) - field16(uq[3], u & 3u));
         }
+      } else if (PLN) {
+        cu = hp[s * ps + u] + 1u;
+        if (hop) {
+          du = gh.x + gh.y * (lut[u] >> 4);
+          if (MODEL == 1 && s < 2u) du += q.k_in * hp[(1u - s) * ps + u];
+          if (MODEL == 2 && s == 1u)
+            du += q.k_in * (static_cast<uint32_t>(u == centre) - hp[2u * ps + u]);
+        }
       } else if (REC) {
         const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec)[u];
         a_u = x.x;
@@ -914,7 +969,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         }
       }
       if (MODEL != 2 && s == 2u && run && !several) {  // R changes the Hill term, here and where it arrives
-        const uint32_t Ru = hop ? (REC && !SEC ? word_R(w_u) + 1u : cu) : 1u;
+        const uint32_t Ru = hop ? (REC && !SEC && !PLN ? word_R(w_u) + 1u : cu) : 1u;
         if (!slow) {  // every count is inside the table
           dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
           const uint64_t d = __ldg(q.hill + Ru) - __ldg(q.hill + (Ru - 1u));
@@ -1000,6 +1055,22 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           uint64_t* uq = rec + 4u * (u >> 2);
           uq[0] = a_u + du;
           uq[1u + s] = w_u + to;
+        }
+        const uint32_t lim_s = s == 2u ? lim_r : lim_dn;
+        bool over = hop && cu >= lim_s;
+        if (MODEL == 0) over = over || nc >= lim_s;
+        else over = over || max(D + dD, N + dN) >= lim_dn || R + dR >= lim_r;
+        if (run && over) err |= kErrNarrow;
+      } else if (PLN) {
+        if (run && lead) {
+          if (MODEL == 0) {
+            hp[s * ps + v] = static_cast<uint16_t>(nc);
+          } else {
+            if (dD) hp[v] = static_cast<uint16_t>(D + dD);
+            if (dN) hp[ps + v] = static_cast<uint16_t>(N + dN);
+            if (dR) hp[2u * ps + v] = static_cast<uint16_t>(R + dR);
+          }
+          if (hop) hp[s * ps + u] = static_cast<uint16_t>(cu);
         }
         const uint32_t lim_s = s == 2u ? lim_r : lim_dn;
         bool over = hop && cu >= lim_s;
@@ -1137,6 +1208,17 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           if (cN) add64(w + 1, static_cast<uint64_t>(static_cast<int64_t>(cN)) << sh);
           if (cR) add64(w + 2, static_cast<uint64_t>(static_cast<int64_t>(cR)) << sh);
           if (code >= kEvHop) add64(rec + 4u * (u >> 2) + 1u + su, 0ull - (1ull << (16u * (u & 3u))));
+        } else if (PLN) {
+          // whole 32-bit words: the sum of all changes is in range, so carries
+          // between the halves cancel
+          auto add16 = [&](uint32_t at, int c) {
+            atomicAdd(reinterpret_cast<uint32_t*>(hp) + (at >> 1),
+                      static_cast<uint32_t>(c) << (16u * (at & 1u)));
+          };
+          if (cD) add16(v, cD);
+          if (cN) add16(ps + v, cN);
+          if (cR) add16(2u * ps + v, cR);
+          if (code >= kEvHop) add16(su * ps + u, -1);
         } else if (REC) {
           add64(rec + 2u * v + 1u, word_unit(0) * static_cast<uint64_t>(static_cast<int64_t>(cD)) +
                                        word_unit(1) * static_cast<uint64_t>(static_cast<int64_t>(cN)) +
@@ -1183,6 +1265,18 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
               for (uint32_t sp = 0; sp < 3u; ++sp)
                 g[sp * V + i] =
                     static_cast<int32_t>(field16(from[4u * (i >> 2) + 1u + sp], i & 3u));
+          }
+        } else if (PLN) {
+          const uint64_t* from =
+              reinterpret_cast<const uint64_t*>(warp_cells + sc * p.cell_stride + 48) + kCnt;
+          for (uint32_t sp = 0; sp < 3u; ++sp) {
+            if (vec) {
+              for (uint32_t i = lane; i < nq; i += 32u)
+                reinterpret_cast<uint4*>(g + sp * V)[i] = unpack4(from[sp * nq + i]);
+            } else {
+              for (uint32_t i = lane; i < V; i += 32u)
+                g[sp * V + i] = static_cast<int32_t>(field16(from[sp * nq + (i >> 2)], i & 3u));
+            }
           }
         } else if (REC) {
           const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words;
@@ -1238,7 +1332,7 @@ ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   LANE_CASE(3, kLeafShared, 32, 6);
   LANE_CASE(3, kLeafShared, 16, 6);
   LANE_CASE(3, kLeafShared, 8, 6);
-  if (MODEL != 1) LANE_CASE(3, kLeafShared, 8, 8);
+  if constexpr (MODEL != 1) LANE_CASE(3, kLeafShared, 8, 8);
   LANE_CASE(3, kLeafShared, 8, 0);
   LANE_CASE(3, kLeafShared, 4, 0);
   LANE_CASE(3, kLeafRecords, 1, 8);
@@ -1247,18 +1341,21 @@ ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   LANE_CASE(4, kLeafShared, 32, 6);
   LANE_CASE(4, kLeafShared, 16, 6);
   LANE_CASE(4, kLeafShared, 8, 6);
-  if (MODEL != 1) LANE_CASE(4, kLeafShared, 8, 8);
+  if constexpr (MODEL != 1) LANE_CASE(4, kLeafShared, 8, 8);
   LANE_CASE(4, kLeafShared, 8, 0);
   LANE_CASE(4, kLeafShared, 4, 0);
-  LANE_CASE(4, kLeafRecords, 8, 0);
   LANE_CASE(4, kLeafRecords, 4, 0);
   LANE_CASE(4, kLeafSectors, 1, 8);
   LANE_CASE(4, kLeafSectors, 1, 6);
   LANE_CASE(4, kLeafSectors, 1, 0);
   LANE_CASE(5, kLeafShared, 32, 6);
   LANE_CASE(5, kLeafShared, 16, 6);
-  LANE_CASE(5, kLeafRecords, 16, 6);
-  LANE_CASE(5, kLeafRecords, 16, 8);
+  LANE_CASE(5, kLeafPlanes, 16, 6);
+  LANE_CASE(5, kLeafPlanes, 16, 8);
+  LANE_CASE(5, kLeafPlanes, 16, 0);
+  LANE_CASE(4, kLeafPlanes, 8, 0);
+  LANE_CASE(4, kLeafPlanes, 4, 0);
+  LANE_CASE(3, kLeafPlanes, 4, 0);
   LANE_CASE(5, kLeafRecords, 16, 0);
   LANE_CASE(5, kLeafRecords, 8, 0);
   LANE_CASE(5, kLeafSectors, 1, 6);

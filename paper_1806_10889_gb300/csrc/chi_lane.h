@@ -9,9 +9,11 @@ constexpr int kMaxSmem = 227 * 1024;  // dynamic shared memory a block may ask f
 constexpr int kLeafShared = 0;   // shared memory: totals and 32-bit counts
 constexpr int kLeafRecords = 1;  // scratch array: 64 bytes a quad, totals and packed counts
 constexpr int kLeafSectors = 2;  // scratch array: 32 bytes a quad, its sum and 16-bit counts
+constexpr int kLeafPlanes = 3;   // shared memory: three planes of 16-bit counts
 constexpr uint32_t kLaneHill = 2048;  // R below this reads the Hill table unchecked (R + 1 too)
 constexpr uint32_t kWordCount = 1u << 19;    // counts of a record stay below
 constexpr uint32_t kSectorCount = 1u << 16;  // counts of a sector
+constexpr uint32_t kPlaneCount = 0xFFFFu;    // ... and of a plane, below what 16 bits hold
 
 // First entry of level l of a four-ary tree whose levels follow one another:
 // (4^l - 4) / 3.
@@ -37,7 +39,7 @@ struct LaneArgs {
   const uint2* items;  // (tissue, cell); nullptr: the cells of views[0] in order
   uint32_t* counter;   // work counter, zero before a launch of more cells than places
   uint64_t* scratch;   // the resident cells' records (plans with scratch_bytes > 0)
-  uint2* redo;         // with records: cells whose counts pass the packed range
+  uint2* redo;         // unless shared leaves: cells whose counts pass the packed range
   uint32_t* redo_n;
   double dt;
   uint32_t n_items, step_off;

@@ -25,21 +25,22 @@ ChiLaneKernel lane_kernel(int model, uint32_t V, int leaf, uint32_t G, uint32_t 
 // fewest; past L2's size the random accesses to DRAM do, and a sector makes two
 // reads and two writes an event.  Chi ms of one step at dt 0.02 (8x8 and 16x16
 // voxels) and 0.006 (32x32), 60 D + 30 N + 10 R per voxel, by cells per SM; leaf
-// (S shared, R records, X sectors) and lanes per cell; in parentheses the next
-// shape, in brackets the segmented kernel's default launch:
+// (S shared, P planes, R records, X sectors) and lanes per cell; in parentheses
+// the next shape, in brackets the segmented kernel's default launch:
 //         8x8                          16x16                        32x32
 //    4  S32 .26 (S16 .28) [.65]    S32 1.05 (S16 1.12) [2.6]    S32 1.39 (S16 1.43) [3.1]
 //    6  S16 .29 (S32 .29) [.71]    S16 1.15 (S32 1.22) [2.8]    S16 1.48 (S32 1.60) [3.5]
-//   12  S16 .34 (S8 .35)  [.79]    S16 1.34 (S8 1.36)  [3.1]    R16 2.68 (R8 3.68)  [4.0]
+//   12  S16 .34 (S8 .35)  [.79]    S16 1.34 (S8 1.36)  [3.1]    P16 1.92 (R16 2.68) [4.0]
+//   24                           27 S8 1.68 (S4 2.10)  [4.1]    P16 2.47 (R16 3.3)  [6.1]
 //   32  S8 .42  (S4 .54)  [.87]    S8 1.68  (S4 2.09)  [4.1]    R16 3.55 (R8 4.03)  [6.7]
-//   48  S8 .52  (S4 .63)  [.98]  44 R8 2.93 (R4 3.60)  [5.2]  33 R8 4.26 (R16 5.5)  [9.8]
-//   64  S4 .64  (S8 .91)  [1.2]    R8 3.36  (R4 3.69)  [6.1]    R8 5.13  (X1 6.4)  [13.3]
-//   96  S4 .76  (R1 1.15) [2.0]  65 R4 3.93 (R8 5.0)   [8.7]  65 X1 6.45 (R8 7.7)  [15.2]
-//  128  R1 1.06           [2.2]    R4 4.58  (X1 5.24) [12.1]
+//   48  S8 .52  (S4 .63)  [.98]  44 P8 2.28 (R8 2.93)  [5.2]  33 R8 4.26 (R16 5.5)  [9.8]
+//   64  S4 .63  (S8 .91)  [1.2]    P8 2.82  (R8 3.36)  [6.1]    R8 5.13  (X1 6.4)  [13.3]
+//   88  S4 .76  (R1 1.15) [2.0]    P4 3.25  (R4 4.1)   [9.7]  65 X1 6.45 (R8 7.7)  [15.2]
+//  128  P4 .92  (R1 1.06) [2.2]    R4 4.58  (X1 5.24) [12.1]
 //  150  R1 1.12 (R4 1.36) [2.8]    X1 5.17  (R4 7.2)  [15.0]    X1 8.2             [30.1]
 //  431  R1 1.79           [7.0]    X1 9.0             [39.1]    X1 18.1            [84.0]
 // Cells of 10x10 voxels fit shared memory longer: 50 to 64 an SM take S4 (.98,
-// R8 1.13 to 1.20).
+// R8 1.13 to 1.20), 81 to 128 P4.
 LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
   LanePlan pl;
   int dev = 0, sms = 0;
@@ -48,18 +49,18 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
     return pl;
   const int lv = V <= 64 ? 3 : V <= 256 ? 4 : 5;
   const uint64_t per = (cells + static_cast<uint64_t>(sms) - 1) / static_cast<uint64_t>(sms);
-  const uint32_t G = per <= 4                                        ? 32u
-                     : per <= (lv == 5 ? 32u : 12u)                  ? 16u
-                     : per <= (lv == 3 ? 48u : 64u)                  ? 8u
-                     : per <= (lv == 3 ? 96u : lv == 4 ? 128u : 64u) ? 4u
-                                                                     : 1u;
+  const uint32_t G = per <= 4                       ? 32u
+                     : per <= (lv == 5 ? 32u : 12u) ? 16u
+                     : per <= (lv == 3 ? 48u : 64u) ? 8u
+                     : per <= 128 && lv < 5         ? 4u
+                                                    : 1u;
   // A helper warp that draws ahead while at most eight warps an SM run cells: the
   // draws leave the chain.  Up to six, twelve warps have the registers they want
   // (168).  Chi ms, without -> with: 2x2 cells of 8x8 voxels 1.19 -> 1.14, 60x50 of
   // 16x16 8.34 -> 7.70, 60 uneven tissues (26,802 cells of 32x32) 146.7 -> 133.9.
   // One lane per cell, 190 cells of 16x16 an SM: 5.81 -> 5.24.
   // Seven and eight leave 128: 64x64 of 16x16 9.35 -> 9.12, promoter 7.41 -> 6.95,
-  // 64x64 of 8x8 3.83 -> 3.69, 48x48 of 32x32 (records) 45.05 -> 44.36; with
+  // 64x64 of 8x8 3.83 -> 3.69, 48x48 of 32x32 (records, then) 45.05 -> 44.36; with
   // in-voxel binding the spills cost more (16x16 9.74 -> 10.01) and it is not
   // built for 8 lanes; below six warps 128 registers cost 2% (7.68 -> 7.81).
   // Classes of a batch share the SMs, the first ahead of the others, which run
@@ -72,8 +73,10 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
   const uint32_t nq = (V + 3u) / 4u;
   int per_sm = 0;  // blocks an SM holds
   // Leaves: in shared memory while one wave of cells fits there (the shortest
-  // chain, also with four lanes per cell instead of eight); else records, whose
-  // totals need no recomputing; for one lane per cell, where L2's size and the
+  // chain, also with four lanes per cell instead of eight); else as planes there
+  // (cells of 16x16, 37 to 64 an SM: planes 2.28 to 2.82 ms, records 2.9 to 3.4;
+  // where S8 fits, 2.09); else records, whose totals need no recomputing, in the scratch
+  // array; for one lane per cell, where L2's size and the
   // sums in shared memory (2.7 KB a cell of 32x32 voxels) bound the cells in
   // flight, sectors: half the bytes and a quarter of the sums (8x8 keeps records,
   // 9.0 against 10.7 ms for 256x256 cells).
@@ -81,7 +84,7 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
     const uint64_t places = 32u / G;  // cells a warp runs
     pl.G = G;
     const uint32_t cell = 48u + 8u * lane_sum_words(lv, leaf, static_cast<int>(G)) +
-                          (leaf == kLeafShared ? 20u * 4u * nq : 0u);
+                          (leaf == kLeafShared ? 80u : leaf == kLeafPlanes ? 24u : 0u) * nq;
     // an odd multiple of 16 bytes: lanes reading the same entry of their cells
     // start on different shared-memory banks
     pl.cell_stride = ((cell + 15u) & ~15u) | 16u;
@@ -105,7 +108,8 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
   };
   const int spill = G == 1 && lv > 3 ? kLeafSectors : kLeafRecords;
   if (!(few && shape(G, kLeafShared, few)) && !shape(G, kLeafShared, 0) &&
-      !(G == 8 && shape(4, kLeafShared, 0)) && !(few && shape(G, spill, few)) &&
+      !(G == 8 && shape(4, kLeafShared, 0)) &&
+      !(few && shape(G, kLeafPlanes, few)) && !shape(G, kLeafPlanes, 0) && !(few && shape(G, spill, few)) &&
       !shape(G, spill, 0) && per_sm < 1)
     shape(G, kLeafShared, 0);
   if (per_sm < 1) {
@@ -118,7 +122,7 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
   pl.blocks = static_cast<uint32_t>(need < cap ? need : cap);
   pl.small = need <= static_cast<uint64_t>(sms);
   pl.counters = need > cap || pl.leaf != kLeafShared;
-  if (pl.leaf != kLeafShared)
+  if (pl.leaf == kLeafRecords || pl.leaf == kLeafSectors)
     pl.scratch_bytes = static_cast<size_t>(pl.blocks) * per_block *
                        (pl.leaf == kLeafRecords ? 8u * nq : 16u * ((nq + 3u) / 4u)) *
                        sizeof(uint64_t);

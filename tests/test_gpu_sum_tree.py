@@ -66,7 +66,7 @@ FORMS = [(1, 2, 0.3), (8, 5, 0.1), (20, 7, 0.1), (100, 5, 0.02), (8, 16, 0.02), 
          (28, 8, 0.02), (28, 16, 0.01), (40, 9, 0.02), (90, 8, 0.01), (140, 9, 0.01), (50, 17, 0.01),
          (45, 16, 0.01), (98, 9, 0.01), (120, 2, 0.1), (120, 8, 0.01), (120, 9, 0.01),
          (3, 17, 0.02), (9, 18, 0.02), (30, 17, 0.01), (85, 17, 0.005), (112, 17, 0.005),
-         (2, 32, 0.01), (16, 32, 0.005)]
+         (2, 32, 0.01), (16, 32, 0.005), (11, 32, 0.005), (24, 31, 0.005), (60, 15, 0.01)]
 
 
 @pytest.mark.parametrize("model", ["plain", "binding", "promoter"])
@@ -89,7 +89,7 @@ def test_every_form_matches_oracle(per_sm, n, dt, model):
 def test_no_scratch_or_a_capture_runs_the_segmented_kernel():
     """A tissue or batch that cannot have the records' scratch gives the same
     results by the other kernel; so does a step captured into a graph."""
-    spec = _spec(112, 9, "plain")
+    spec = _spec(140, 9, "plain")
     dt = 0.01
     ref = Tissue(spec)
     ref.step(dt, 2)
