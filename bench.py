@@ -95,7 +95,8 @@ CHI_IPE = {
         "batch:V64/H8/rec/qb0/nd/u32": (239.3, 0.5607),
     },
 }
-# The same of the sum-tree chi kernel, which runs default launch shapes in a form
+# The same of the sum-tree chi kernel (profiles/k_chi_lane_inst_per_event.md),
+# which runs default launch shapes in a form
 # that follows from the cell size and the number of cells (its warps serve up to
 # 32 cells): per workload and cell size, with its own sources.
 TREE_SOURCES = ["chi_lane.cuh", "chi_lane.h", "tissue_dev.cuh", "k_chi_lane.cu",

@@ -66,7 +66,8 @@ FORMS = [(1, 2, 0.3), (8, 5, 0.1), (20, 7, 0.1), (100, 5, 0.02), (8, 16, 0.02), 
          (28, 8, 0.02), (28, 16, 0.01), (40, 9, 0.02), (90, 8, 0.01), (140, 9, 0.01), (50, 17, 0.01),
          (45, 16, 0.01), (98, 9, 0.01), (120, 2, 0.1), (120, 8, 0.01), (120, 9, 0.01),
          (3, 17, 0.02), (9, 18, 0.02), (30, 17, 0.01), (85, 17, 0.005), (112, 17, 0.005),
-         (2, 32, 0.01), (16, 32, 0.005), (11, 32, 0.005), (24, 31, 0.005), (60, 15, 0.01)]
+         (2, 32, 0.01), (16, 32, 0.005), (11, 32, 0.005), (24, 31, 0.005), (60, 15, 0.01),
+         (120, 16, 0.004), (30, 32, 0.002)]
 
 
 @pytest.mark.parametrize("model", ["plain", "binding", "promoter"])
