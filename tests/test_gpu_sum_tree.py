@@ -1,5 +1,5 @@
 """The sum-tree chi kernel in every form its launch plan picks -- 32 to 1
-lanes per cell, leaves in shared memory, in packed records or in sectors --
+lanes per cell, leaves in shared memory, in planes, records or sectors --
 against the oracle, bit for bit: counts, per-cell event counts and
 binary64 times.  The plan follows from the cell size and the cells per SM, so
 the tissues here are just wide enough, with cells of ragged sizes.  Some
@@ -60,8 +60,8 @@ def _compare(g, spec, ref, ne, tl, ctx):
     assert np.array_equal(gtl.view(np.uint64), tl.view(np.uint64)), f"{ctx}: event times"
 
 
-# (cells per SM, n, dt): shared leaves at 32, 16, 8 and 4 lanes; records at 16,
-# 8, 4 and 1; sectors at 4 and 1 (V = 4, 25, 49, 64, 81, 256, 289, 324 and 1,024)
+# (cells per SM, n, dt): shared leaves at 32, 16, 8 and 4 lanes; planes at 16, 8
+# and 4; records at 16, 8, 4 and 1; sectors at 1 (V = 4 to 1,024)
 FORMS = [(1, 2, 0.3), (8, 5, 0.1), (20, 7, 0.1), (100, 5, 0.02), (8, 16, 0.02), (30, 9, 0.02),
          (28, 8, 0.02), (28, 16, 0.01), (40, 9, 0.02), (90, 8, 0.01), (140, 9, 0.01), (50, 17, 0.01),
          (45, 16, 0.01), (98, 9, 0.01), (120, 2, 0.1), (120, 8, 0.01), (120, 9, 0.01),
@@ -122,7 +122,8 @@ def test_no_scratch_or_a_capture_runs_the_segmented_kernel():
     b.close()
 
     # captured: the large tissue without scratch, a small one with early launches
-    for sp, steps in ((spec, 1), (TissueSpec(3, 3, 8, seed=93), 3)):
+    # and one whose planes need none
+    for sp, steps in ((spec, 1), (_spec(60, 15, "plain"), 1), (TissueSpec(3, 3, 8, seed=93), 3)):
         ref = Tissue(sp)
         ref.step(dt, 2 * steps)
         want, (wne, wtl) = ref.read_counts(), ref.read_stats()
@@ -142,7 +143,7 @@ def test_no_scratch_or_a_capture_runs_the_segmented_kernel():
 
 def test_two_streams_step_large_tissues_at_once():
     """Two tissues on two streams, each with its own scratch in flight."""
-    specs = [_spec(112, 9, "plain"), _spec(120, 8, "binding")]
+    specs = [_spec(140, 9, "plain"), _spec(140, 8, "binding")]
     dt = 0.01
     want = []
     for s in specs:
@@ -157,3 +158,23 @@ def test_two_streams_step_large_tissues_at_once():
     for t, x in zip(ts, want):
         assert np.array_equal(t.read_counts(), x)
         t.close()
+
+
+@pytest.mark.parametrize("per_sm,n,dt", [(60, 15, 0.002), (70, 16, 0.002), (11, 32, 0.001)])
+def test_planes_meet_their_range_within_a_step(per_sm, n, dt):
+    """Counts just below what 16 bits hold, whose neighbours' molecules hop in:
+    some cells pass the range within the step (and are run again by the 32-bit
+    pass), others only in the events that the end of the step undoes."""
+    spec = _spec(per_sm, n, "plain")
+    d, m = orc_desc(spec), orc_model(spec)
+    ref = O.init_counts(d)
+    x = ref.reshape(spec.cells, 3, spec.V)
+    for c in range(8):
+        x[c, c % 2, 2 * c:2 * c + 2] = 65534 - c
+    g = Tissue(spec)
+    g.write_counts(ref, 0)
+    for k in range(2):
+        ne, tl = O.step(d, m, ref, k, 1, dt)
+        g.step(dt, 1)
+        _compare(g, spec, ref, ne, tl, f"{spec.width}x{spec.height}x{n} step {k}")
+    g.close()
