@@ -71,6 +71,7 @@
 #pragma once
 #include "chi_lane.h"
 #include "early_launch.cuh"
+#include "pair_end.h"
 #include "tissue_dev.cuh"
 
 namespace tsg {
@@ -173,8 +174,8 @@ struct LaneExchange {
   int Ek[2][32];
   uint32_t stream[2][32][7];  // step, cell, word 3, key, next event, whether new
   uint32_t home[32][6];       // the cell's step, number, word 3, key, tissue
-  int done, swap;
-  int pad[2];
+  PairEnd end;
+  int swap, pad;
 };
 static_assert(sizeof(LaneExchange) == kExchangeBytes, "chi_lane.h");
 
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     // cells spread over the SM's four schedulers (one half of them otherwise:
     // 64x64 cells 9.3 -> 12.2 ms)
     ex->swap = static_cast<int>((w >> 2) & 1u);
-    ex->done = 0;
+    ex->end.clear();
   }
   unsigned char* lut = smem + 128;
   for (uint32_t i = threadIdx.x; i < 64u; i += blockDim.x) {
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     uint32_t hs[5] = {}, he = 0;
     for (uint32_t ph = 0;; ph ^= 1u) {
       pair_barrier();
-      if (ex->done) return;
+      if (ex->end.reached(ph)) return;
       const uint32_t* d = ex->stream[ph][slot];
       if (d[6]) {
 #pragma unroll
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     __syncwarp();
     if (__all_sync(kFull, done)) {
       if (HELP) {
-        if (lane == 0) ex->done = 1;
+        if (lane == 0) ex->end.announce(phase);
         __syncwarp();
         pair_barrier();
       }
