@@ -30,7 +30,8 @@ struct ClassPlan {
   uint32_t lanes, warps_per_block, layout;
   size_t items_off;  // offset (in uint2) into the item buffer
   uint32_t n_items;
-  int gen;           // 0: Notch-Delta only; 2: promoter only; 1: both, or a trace is on
+  // 0: Notch-Delta only; 2: promoter only, traced or not; 1: both, or Notch-Delta traced
+  int gen;
   // the sum-tree launch (lane.G = 0: none), its model code and the offset of
   // its scratch; it takes the class while the launch shape is a default one
   LanePlan lane;
@@ -289,7 +290,9 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     p.gen = (nd_v[V] == 0 && pm_v[V] > 0) ? 2 : (pm_v[V] > 0 || tr_v[V] > 0) ? 1 : 0;
     while (p.n * p.n < V) ++p.n;
     p.lane_model = p.gen == 2 ? 2 : bind_v[V] > 0 ? 1 : 0;
-    if (p.gen != 1) p.lane = lane_plan(V, kv.second.size(), p.lane_model, lane_warps);
+    // the sum-tree kernel writes no trace (a traced class of promoter members
+    // has gen 2 like an untraced one)
+    if (p.gen != 1 && tr_v[V] == 0) p.lane = lane_plan(V, kv.second.size(), p.lane_model, lane_warps);
     if (p.lane.G) lane_warps += static_cast<uint64_t>(p.lane.blocks) * (p.lane.threads / 32u);
     p.lane_off = lane_words;
     lane_words += ((p.lane.scratch_bytes + 255) & ~static_cast<size_t>(255)) / sizeof(uint64_t);
