@@ -142,20 +142,21 @@ cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_v
   cfg.blockDim = dim3(pl.threads);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributePriority;
   attr[0].val.priority = priority;
-  cfg.attrs = attr;
-  cfg.numAttrs = priority ? 1 : 0;
-  if (early) {
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 1;
-  }
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  // the priority, if there is one, and the early start
+  cfg.attrs = priority ? attr : attr + 1;
+  cfg.numAttrs = (priority ? 1u : 0u) + (early ? 1u : 0u);
   cudaError_t e = cudaLaunchKernelEx(&cfg, k, a);
   if (e != cudaSuccess || pl.leaf == kLeafShared) return e;
   // the cells that left the packed range, by the segmented kernel from the
-  // state they started the step with (it reads their number from the device)
+  // state they started the step with (it reads their number from the device, and
+  // does not wait for the launch before: never early)
+  cfg.attrs = attr;
+  cfg.numAttrs = priority ? 1 : 0;
   const tissue_launch c = prefix_launch(V, n_items);
   const int H = static_cast<int>(c.lanes_per_cell);
   const bool qb = V > static_cast<uint32_t>(H * H);

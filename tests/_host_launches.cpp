@@ -1,0 +1,96 @@
+// The host side of the chi launches on a machine without a GPU: the launch code
+// linked against a CUDA runtime that only records.  Devices have 152 SMs; a
+// kernel's occupancy is what its shared memory and its launch bounds allow.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+
+#include <cuda_runtime.h>
+template <class T>
+T atomicAdd(T* p, T x);  // named by an inline device function
+#include "chi_lane.h"
+
+namespace {
+
+std::map<const void*, std::string>& names() {
+  static std::map<const void*, std::string> m;
+  return m;
+}
+bool record = false;  // print launches
+
+// The template arguments of a sum-tree kernel.
+bool lane_args(const std::string& n, int a[5]) {
+  const size_t at = n.find("k_chi_laneI");
+  return at != std::string::npos &&
+         std::sscanf(n.c_str() + at, "k_chi_laneILi%dELi%dELi%dELi%dELi%dE", a, a + 1, a + 2, a + 3,
+                     a + 4) == 5;
+}
+
+}  // namespace
+
+extern "C" {
+void** __cudaRegisterFatBinary(void*) {
+  static void* handle;
+  return &handle;
+}
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, uint3*, uint3*,
+                            dim3*, dim3*, int*) {
+  names()[host] = name;
+}
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+cudaError_t cudaGetDevice(int* d) {
+  *d = 0;
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) {
+  *v = 152;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* k,
+                                                                   int threads, size_t smem,
+                                                                   unsigned) {
+  int a[5];
+  int by_regs = 2048 / threads / 4;
+  if (lane_args(names()[k], a))
+    by_regs = a[4] ? a[4] : a[2] == tsg::kLeafShared ? 12 : a[3] > 1 ? 14 : a[1] == 5 ? 4 : 7;
+  const int by_smem = static_cast<int>(228 * 1024 / (smem + 1024));
+  *n = by_regs < by_smem ? by_regs : by_smem;
+  return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* k, void**) {
+  if (!record) return cudaSuccess;
+  int early = 0, priority = 0;
+  for (unsigned i = 0; i < c->numAttrs; ++i) {
+    if (c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization)
+      early = c->attrs[i].val.programmaticStreamSerializationAllowed;
+    if (c->attrs[i].id == cudaLaunchAttributePriority) priority = c->attrs[i].val.priority;
+  }
+  const std::string& n = names()[k];
+  std::printf("%s early %d priority %d\n",
+              n.find("k_chi_lane") != std::string::npos ? "tree" : "segmented", early, priority);
+  return cudaSuccess;
+}
+}
+
+// The launches of one chi phase whose cells are packed, so that there is a pass
+// over those past the packed range.
+static int launches(int priority, bool early) {
+  tsg::LanePlan pl = tsg::lane_plan(1024, 30 * 152, 0);
+  if (pl.G == 0 || pl.leaf == tsg::kLeafShared) return 1;
+  record = true;
+  return tsg::launch_chi_lane(pl, 0, nullptr, nullptr, 30 * 152, nullptr, nullptr,
+                              tsg::ChiRedo{nullptr, nullptr}, 1024, 32, 0, 0.1, nullptr, priority,
+                              early) != cudaSuccess;
+}
+
+int main(int argc, char** argv) {
+  if (argc == 4 && !std::strcmp(argv[1], "launches"))
+    return launches(std::atoi(argv[2]), std::atoi(argv[3]) != 0);
+  return 2;
+}
