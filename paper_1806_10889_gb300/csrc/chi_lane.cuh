@@ -1331,7 +1331,9 @@ ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
 #define LANE_CASE(L, F, N, H) \
   if (lv == L && leaf == F && G == N && helper == H) return k_chi_lane<MODEL, L, F, N, H>
   LANE_CASE(3, kLeafShared, 32, 6);
+  LANE_CASE(3, kLeafShared, 32, 0);
   LANE_CASE(3, kLeafShared, 16, 6);
+  LANE_CASE(3, kLeafShared, 16, 0);
   LANE_CASE(3, kLeafShared, 8, 6);
   if constexpr (MODEL != 1) LANE_CASE(3, kLeafShared, 8, 8);
   LANE_CASE(3, kLeafShared, 8, 0);
@@ -1340,7 +1342,9 @@ ChiLaneKernel lane_instance(uint32_t V, int leaf, uint32_t G, uint32_t helper) {
   LANE_CASE(3, kLeafRecords, 1, 6);
   LANE_CASE(3, kLeafRecords, 1, 0);
   LANE_CASE(4, kLeafShared, 32, 6);
+  LANE_CASE(4, kLeafShared, 32, 0);
   LANE_CASE(4, kLeafShared, 16, 6);
+  LANE_CASE(4, kLeafShared, 16, 0);
   LANE_CASE(4, kLeafShared, 8, 6);
   if constexpr (MODEL != 1) LANE_CASE(4, kLeafShared, 8, 8);
   LANE_CASE(4, kLeafShared, 8, 0);

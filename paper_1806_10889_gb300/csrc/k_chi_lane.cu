@@ -106,12 +106,26 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
       per_sm = 0;
     return per <= static_cast<uint64_t>(per_sm) * pl.wpb * places;
   };
-  const int spill = G == 1 && lv > 3 ? kLeafSectors : kLeafRecords;
-  if (!(few && shape(G, kLeafShared, few)) && !shape(G, kLeafShared, 0) &&
-      !(G == 8 && shape(4, kLeafShared, 0)) &&
-      !(few && shape(G, kLeafPlanes, few)) && !shape(G, kLeafPlanes, 0) && !(few && shape(G, spill, few)) &&
-      !shape(G, spill, 0) && per_sm < 1)
-    shape(G, kLeafShared, 0);
+  // A helper is asked for first.
+  auto fits = [&](uint32_t G, int leaf) {
+    return (few && shape(G, leaf, few)) || shape(G, leaf, 0);
+  };
+  // The first form, in the order above, that holds all cells; one that holds some
+  // of them if none does.
+  auto any_form = [&](uint32_t G) {
+    return fits(G, kLeafShared) || (G == 8 && shape(4, kLeafShared, 0)) || fits(G, kLeafPlanes) ||
+           fits(G, G == 1 && lv > 3 ? kLeafSectors : kLeafRecords) || per_sm >= 1 ||
+           (shape(G, kLeafShared, 0), per_sm >= 1);
+  };
+  // A small class beside others that leave no helper: up to 256 voxels 32 and 16
+  // lanes without one, whose blocks are the smallest and find room beside the
+  // first class's (1,500 cells of 32x32 with 500 of 16x16 and 500 of 8x8: the chi
+  // phase 11.1 ms, with 8 lanes 13.8, with the segmented kernel 10.8; 3,500 of
+  // 16x16 with 500 of 15x15: 4.1, 5.8, 6.4).  Above, 32 lanes take 25 KB a cell and
+  // wait for the first class to end (6,400 of 32x32 with 400 of 31x31: 30.0 ms):
+  // not built, the next narrower form, planes, takes them (25.0; segmented 25.8; beside
+  // 1,600 of 32x32 20.9, 23.2 and 34.9).
+  for (uint32_t g = G; g >= 1u && !any_form(g);) g /= 2u;
   if (per_sm < 1) {
     pl.G = 0;
     return pl;

@@ -89,7 +89,23 @@ static int launches(int priority, bool early) {
                               early) != cudaSuccess;
 }
 
+// Every class a batch may hold, behind up to a chip full of other warps: the
+// plans that have no kernel, and those whose blocks do not hold all cells.
+static int plans() {
+  for (uint32_t n = 2; n <= 32; ++n)
+    for (int model = 0; model < 3; ++model)
+      for (uint64_t cells = 1; cells < 200000; cells += 1 + cells / 4)
+        for (uint64_t beside : {0, 100, 152 * 5, 152 * 6, 152 * 7, 152 * 8 - 1, 152 * 8, 152 * 16, 40000}) {
+          const tsg::LanePlan pl = tsg::lane_plan(n * n, cells, model, beside);
+          if (pl.G == 0 || pl.blocks == 0 || pl.smem > tsg::kMaxSmem)
+            std::printf("V %u model %d cells %llu beside %llu: G %u\n", n * n, model,
+                        (unsigned long long)cells, (unsigned long long)beside, pl.G);
+        }
+  return 0;
+}
+
 int main(int argc, char** argv) {
+  if (argc == 2 && !std::strcmp(argv[1], "plans")) return plans();
   if (argc == 4 && !std::strcmp(argv[1], "launches"))
     return launches(std::atoi(argv[2]), std::atoi(argv[3]) != 0);
   return 2;

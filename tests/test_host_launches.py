@@ -39,3 +39,9 @@ def test_the_pass_over_the_packed_ranges_rest_never_starts_early(probe, priority
     first, *rest = probe("launches", priority, 0)
     assert first == f"tree early 0 priority {priority}"
     assert all(x == f"segmented early 0 priority {priority}" for x in rest)
+
+
+def test_every_class_has_a_sum_tree_plan(probe):
+    """Every cell size, model and number of cells, alone and behind the launches of
+    other classes that fill the chip."""
+    assert probe("plans") == []
