@@ -171,12 +171,19 @@ cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_v
   // does not wait for the launch before: never early)
   cfg.attrs = attr;
   cfg.numAttrs = priority ? 1 : 0;
-  const tissue_launch c = prefix_launch(V, n_items);
+  // in the shape that kernel has by default for as many cells: where every cell is
+  // past the packed range, the time it takes alone (N at 70,000 a voxel, 256x180
+  // cells of 16x16 voxels 59.9 -> 50.0 ms against the prefix layout, 128x160 of
+  // 32x32 88.5 -> 70.8)
+  tissue_launch c = default_launch(V, n_items);
+  if (c.smem_layout == TISSUE_LAYOUT_RECOMPUTE &&
+      !recompute_covers(V, static_cast<int>(c.lanes_per_cell), model == 2 ? 2 : 0))
+    c = prefix_launch(V, n_items);
   const int H = static_cast<int>(c.lanes_per_cell);
-  const bool qb = V > static_cast<uint32_t>(H * H);
+  const bool qb = V > static_cast<uint32_t>(H * H), pre = c.smem_layout == TISSUE_LAYOUT_PREFIX;
   const ChiSegKernel ks =
-      model == 2 ? chi_seg_kernel_pm(H, true, qb) : chi_seg_kernel_nd(H, true, qb);
-  const uint32_t seg_bytes = seg_bytes_for(V, H, true);
+      model == 2 ? chi_seg_kernel_pm(H, pre, qb) : chi_seg_kernel_nd(H, pre, qb);
+  const uint32_t seg_bytes = seg_bytes_for(V, H, pre);
   const size_t smem = static_cast<size_t>(c.warps_per_block) * (32u / c.lanes_per_cell) * seg_bytes;
   const int threads = 32 * static_cast<int>(c.warps_per_block);
   int dev = 0, sms = 0, per_sm = 0;
