@@ -64,10 +64,17 @@
 //
 // Limits.  Counts below the tissue's `small` keep every total below 2^52
 // unchecked, and R below kLaneHill reads the Hill table unchecked.  With
-// shared leaves a cell past either goes on with exact checks; a packed cell
-// (20 or 16 bits a count) is left untouched and goes to the redo list, which
-// the launcher runs through the segmented kernel from the same state and
-// random streams.
+// shared leaves a cell past either goes on with exact checks.  A packed cell
+// (20 or 16 bits a count) goes on with limits of its own, taken from its largest
+// counts when it is loaded and again when one is met (pick_limits; the event
+// loop compares with them all the same, so that this costs a running tissue
+// nothing).  Only where there are none -- counts past their field, R past the
+// Hill table, totals near 2^52 -- it is left untouched and goes to the redo list,
+// which the launcher runs through the segmented kernel from the same state and
+// random streams.  Cells past `small` (hops at 100 and 600 D a voxel), redone and
+// with their own limits: 256x180 of 16x16 voxels 55.5 -> 9.5 ms, 48x48 of 32x32
+// 28.2 -> 6.9, 256x256 of 8x8 40.8 -> 8.6; with 2,500 R a voxel 54.1 -> 10.5 and,
+// 128x160 of 32x32, 63.0 -> 10.0.
 #pragma once
 #include "chi_lane.h"
 #include "early_launch.cuh"
@@ -149,6 +156,52 @@ __device__ __noinline__ bool exact_ovf(const TissueView* tv, uint32_t D, uint32_
   a += mul_lim(q.k_in, X, ovf);
   a += mul_lim(q.k_off, R, ovf);
   return ovf || (a >> 52) != 0ull;
+}
+
+// Limits of a cell's counts of D, N and R.
+struct Limits {
+  uint32_t D, N, R;
+};
+
+// The limits of a cell with packed counts, from the largest it holds: while every
+// count stays below them, no total reaches 2^52, no count leaves its field
+// (`most`) and no R the Hill table (most_r).  As a rule that is the tissue's
+// `small`.  A cell past it gets limits of its own: records, compared by their
+// bits, the next power of two each; else one for D and N and one for R, the
+// largest counts times what 2^52 leaves room for (a total grows at most with
+// the square of that; in single precision, 3% below).  False where there are
+// none: the cell goes to the redo list.
+template <int MODEL, int LEAF>
+__device__ __forceinline__ bool pick_limits(const TissueView* tv, Limits m, Limits& l) {
+  constexpr uint32_t most = LEAF == kLeafRecords ? kWordCount : kHalfCount;
+  constexpr uint32_t most_r = MODEL == 2               ? most
+                              : LEAF == kLeafRecords ? kHillTab
+                                                     : kHillTab - 1u;
+  const QRates& q = tv->q;
+  if (LEAF != kLeafRecords) m.D = m.N = max(m.D, m.N);
+  l.D = l.N = min(q.small, most);
+  l.R = min(q.small, most_r);
+  if (max(m.D, m.N) < l.D && m.R < l.R) return true;
+  if (max(m.D, m.N) >= most || m.R >= most_r) return false;
+  auto up = [](uint32_t x) { return LEAF == kLeafRecords ? 2u << (31 - __clz(x | 1)) : x + 1u; };
+  l = Limits{up(m.D), up(m.N), up(m.R)};
+  const float fD = static_cast<float>(l.D), fN = static_cast<float>(l.N);
+  float a = __ull2float_rn(q.gD + 4u * q.hopD) * fD + __ull2float_rn(q.gN + 4u * q.hopN) * fN;
+  if (MODEL == 2) {
+    a += __ull2float_rn(q.tD + q.kd) + __ull2float_rn(q.k_in) * fN;
+  } else {
+    a += __ull2float_rn(q.gR + q.k_off + 4u * q.hopR) * static_cast<float>(l.R) +
+         __ull2float_rn(__ldg(q.hill) + q.kN);  // the table falls with R
+    if (MODEL == 1) a += __ull2float_rn(q.k_in) * (fD * fN);
+  }
+  float f = 0x1.fp51f / a;
+  if (!(f >= 1.0f)) return false;
+  if (LEAF != kLeafRecords) {
+    f = fminf(MODEL == 1 ? sqrtf(f) : f, 64.0f) * 0.99f;
+    l.D = l.N = min(most, max(l.D, static_cast<uint32_t>(fD * f)));
+    l.R = min(most_r, max(l.R, static_cast<uint32_t>(static_cast<float>(l.R) * f)));
+  }
+  return true;
 }
 
 // Whether the event that changed v (and u) took a count past its maximum or
@@ -438,6 +491,16 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   uint32_t lim_dn = 0, lim_r = 0;  // sectors: the counts' limits
   double tnow = 0.0;
   int err = 0;
+  // records: the bits a count has once it reaches its limit (a power of two)
+  auto set_limits = [&](const Limits& l) {
+    over_mask = pack_voxel(0xFFFFFu & ~(l.D - 1u), 0xFFFFFu & ~(l.N - 1u), 0xFFFFFu & ~(l.R - 1u), 0u);
+    lim_dn = l.D;
+    lim_r = l.R;
+  };
+  auto warp_max = [](const Limits& m) {
+    return Limits{__reduce_max_sync(kFull, m.D), __reduce_max_sync(kFull, m.N),
+                  __reduce_max_sync(kFull, m.R)};
+  };
   uint32_t lim = 0;
   bool big = false;  // shared leaves: the cell holds, or held, a D or N of `small` or an R of
                      // `lim` or more
@@ -480,6 +543,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             : lane == 1 ? make_ulonglong2(nr.gN, nr.hN)
                         : make_ulonglong2(nr.gR + (MODEL == 1 ? nr.k_off : 0ull), nr.hR);
       bool ovf = false, bad_state = false, nbig = false;
+      Limits top{0, 0, 0};  // packed counts: the largest
       uint64_t total = 0, pair = 0;
       for (uint32_t k = 0; k < (NQ + 31u) / 32u; ++k) {
         const uint32_t qi = static_cast<uint32_t>(lane) + 32u * k;
@@ -511,15 +575,16 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
               const uint32_t mk = lut[v], nn = mk >> 4;
               const bool ctr = MODEL == 2 && v == centre;
               if (MODEL == 2 && r[i] > static_cast<uint32_t>(ctr)) bad_state = true;
-              if (MODEL != 2 && r[i] >= kLaneHill) nbig = true;
-              if ((d[i] | m[i] | r[i]) >= nr.small) {
-                nbig = true;
-                if (!REC) ovf |= exact_ovf<MODEL>(ntv, d[i], m[i], r[i], nn, ctr);
+              if (REC) {
+                top = Limits{max(top.D, d[i]), max(top.N, m[i]), max(top.R, r[i])};
+              } else {
+                if (MODEL != 2 && r[i] >= kLaneHill) nbig = true;
+                if ((d[i] | m[i] | r[i]) >= nr.small) {
+                  nbig = true;
+                  ovf |= exact_ovf<MODEL>(ntv, d[i], m[i], r[i], nn, ctr);
+                }
               }
               if (REC) {
-                // past the packed word's range: to the redo list
-                nbig |= PLN ? max(d[i], m[i]) >= kPlaneCount
-                            : (d[i] | m[i]) >= (SEC ? kSectorCount : kWordCount);
                 wd[i] = pack_voxel(d[i], m[i], r[i] & 0xFFFFFu, mk & 15u);
               }
               a[i] = lane_total<MODEL>(nr, ntv, d[i], m[i], r[i], nn, ctr);
@@ -594,6 +659,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       }
       const bool any_ovf = __any_sync(kFull, ovf), any_bad = __any_sync(kFull, bad_state);
       nbig = __any_sync(kFull, nbig);
+      Limits nlim{1, 1, 1};
+      if (REC) nbig = !pick_limits<MODEL, LEAF>(ntv, warp_max(top), nlim);
       __syncwarp();
       if (slot == sc) {
         if (WIDE) X1 = ntree[li];
@@ -621,14 +688,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         lim = min(nr.small, kLaneHill);
         err = any_bad ? kErrState : any_ovf ? kErrOverflow : (REC && nbig) ? kErrNarrow : 0;
         have = true;
-        if (REC) {
-          // the bits a count has once it reaches its limit (a power of two)
-          const uint32_t lc = min(q.small, PLN ? kPlaneCount : SEC ? kSectorCount : kWordCount), lr = MODEL == 2 ? lc : min(q.small, kLaneHill);
-          const uint32_t mc = 0xFFFFFu & ~(lc - 1u), mr = 0xFFFFFu & ~(lr - 1u);
-          over_mask = pack_voxel(mc, mc, mr, 0u);
-          lim_dn = lc;
-          lim_r = lr;
-        }
+        if (REC) set_limits(nlim);
       }
     }
     __syncwarp();
@@ -754,7 +814,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             const uint32_t F = static_cast<uint32_t>(4u * idx + j == centre) - Rj;
             t += q.tD * F + q.kd * Rj + q.k_in * (static_cast<uint64_t>(Nj) * F);
           } else {
-            // R < kLaneHill in a cell that runs; the mask is for idle lanes
+            // R < kHillTab in a cell that runs; the mask is for idle lanes
             t += (q.gR + q.k_off + q.hR * nj) * Rj + __ldg(q.hill + (Rj & (kHillTab - 1u))) + q.kN;
             if (MODEL == 1) t += q.k_in * (static_cast<uint64_t>(Dj) * Nj);
           }
@@ -779,7 +839,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           const uint32_t Fj = static_cast<uint32_t>(vj == centre) - Rj;
           t += q.tD * Fj + q.kd * Rj + q.k_in * (static_cast<uint64_t>(Nj) * Fj);
         } else {
-          // R < kLaneHill in a cell that runs; the mask is for idle lanes
+          // R < kHillTab in a cell that runs; the mask is for idle lanes
           t += (q.gR + q.k_off + q.hR * nj) * Rj + __ldg(q.hill + (Rj & (kHillTab - 1u))) + q.kN;
           if (MODEL == 1) t += q.k_in * (static_cast<uint64_t>(Dj) * Nj);
         }
@@ -970,7 +1030,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         }
       }
       if (MODEL != 2 && s == 2u && run && !several) {  // R changes the Hill term, here and where it arrives
-        const uint32_t Ru = hop ? (REC && !SEC && !PLN ? word_R(w_u) + 1u : cu) : 1u;
+        // (records: the event that leaves the table reads its end; its cell is redone)
+        const uint32_t Ru = hop ? (REC && !SEC && !PLN ? min(word_R(w_u) + 1u, kHillTab - 1u) : cu) : 1u;
         if (!slow) {  // every count is inside the table
           dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
           const uint64_t d = __ldg(q.hill + Ru) - __ldg(q.hill + (Ru - 1u));
@@ -1181,10 +1242,41 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     if (fired < m) err &= ~(kErrOverflow | kErrNarrow);  // the event that met a limit did not fire
     const uint32_t e = e0 + fired;
     if (have && fired == batch && e >= 0xFFFFFFFFu - 32u) err |= kErrEventIndex;
-    const bool fin = have && (err != 0 || fired < m || (m < batch && !paused));
+    bool fin = have && (err != 0 || fired < m || (m < batch && !paused));
     e0 = e;
     unsigned out = __ballot_sync(kFull, fin && lead);
     if (out) {
+      if (REC) {
+        // cells that met a limit: other limits, from what they hold now, the whole
+        // warp one cell at a time
+        for (unsigned met = __ballot_sync(kFull, fin && lead && (err & kErrNarrow) && m); met;
+             met &= met - 1u) {
+          const uint32_t sc = static_cast<uint32_t>(__ffs(met) - 1) / G;
+          const uint64_t* words =
+              PLN ? reinterpret_cast<const uint64_t*>(warp_cells + sc * p.cell_stride + 48) + kCnt
+                  : warp_rec + static_cast<size_t>(sc) * rec_words;
+          Limits now{0, 0, 0}, next{1, 1, 1};
+#pragma unroll 1
+          for (uint32_t i = lane; i < V; i += 32u) {
+            uint32_t D, N, R;
+            if (LEAF == kLeafRecords) {
+              const uint64_t w = words[2u * i + 1u];
+              D = word_D(w), N = word_N(w), R = word_R(w);
+            } else {
+              const uint64_t* x = SEC ? words + 4u * (i >> 2) + 1u : words + (i >> 2);
+              const uint32_t dist = SEC ? 1u : nq, k = i & 3u;
+              D = field16(x[0], k), N = field16(x[dist], k), R = field16(x[2u * dist], k);
+            }
+            now = Limits{max(now.D, D), max(now.N, N), max(now.R, R)};
+          }
+          now = warp_max(now);
+          if (slot == sc && pick_limits<MODEL, LEAF>(tv, now, next)) {
+            set_limits(next);
+            err &= ~kErrNarrow;
+            fin = err != 0;
+          }
+        }
+      }
       // undo the events past the end of the step (counts only), every lane its
       // own: the changes commute
       if (fin && sl >= fired && sl < m) {

@@ -10,10 +10,10 @@ constexpr int kLeafShared = 0;   // shared memory: totals and 32-bit counts
 constexpr int kLeafRecords = 1;  // scratch array: 64 bytes a quad, totals and packed counts
 constexpr int kLeafSectors = 2;  // scratch array: 32 bytes a quad, its sum and 16-bit counts
 constexpr int kLeafPlanes = 3;   // shared memory: three planes of 16-bit counts
-constexpr uint32_t kLaneHill = 2048;  // R below this reads the Hill table unchecked (R + 1 too)
+// Shared leaves: R below this reads the Hill table unchecked (R + 1 too).
+constexpr uint32_t kLaneHill = 2048;
 constexpr uint32_t kWordCount = 1u << 19;    // counts of a record stay below
-constexpr uint32_t kSectorCount = 1u << 16;  // counts of a sector
-constexpr uint32_t kPlaneCount = 0xFFFFu;    // ... and of a plane, below what 16 bits hold
+constexpr uint32_t kHalfCount = 0xFFFFu;     // ... of a sector or a plane, below what 16 bits hold
 
 // First entry of level l of a four-ary tree whose levels follow one another:
 // (4^l - 4) / 3.
