@@ -111,7 +111,10 @@ typedef struct {
 size_t tissue_state_bytes(const tissue_desc* desc);
 
 /* Bytes the library itself allocates for one tissue (statistics, flags,
- * tables), for memory-budget admission.  0 for an invalid descriptor. */
+ * tables) as long as it exists, for memory-budget admission.  0 for an invalid
+ * descriptor.  What a step takes beside them, where it is to be had, is in
+ * tissue_get_chi_info and tissue_batch_get_chi_info; a batch keeps to a limit
+ * (tissue_batch_create_within). */
 size_t tissue_scratch_bytes(const tissue_desc* desc);
 
 /* Bind a tissue to a caller-owned device buffer (>= tissue_state_bytes,
@@ -241,6 +244,19 @@ typedef struct {
 int tissue_set_launch_config(tissue* t, const tissue_launch* config);
 int tissue_get_launch_config(const tissue* t, tissue_launch* config);
 
+/* What the lattice chi of a step runs (with the launch shape, model and trace
+ * that are set now, outside a stream capture). */
+typedef struct {
+  uint32_t sum_tree;       /* 1: the sum-tree kernel; 0: the launch shape's own */
+  uint32_t lanes_per_cell; /* lanes it runs a cell on */
+  uint32_t launches;       /* kernels it launches a step */
+  uint32_t reserved;
+  uint64_t scratch_bytes;  /* device memory it takes beside tissue_scratch_bytes: a tissue
+                            * for the length of a call (the step runs the shape's own
+                            * kernel when there is none), a batch while it exists */
+} tissue_chi_info;
+int tissue_get_chi_info(const tissue* t, tissue_chi_info* info);
+
 /* ---- Batching: many tissues in one persistent launch per step ----------
  * The members keep their own buffers, models, statistics and step indices;
  * one batch step runs chi for the cells of every member with the persistent
@@ -258,6 +274,12 @@ typedef struct tissue_batch tissue_batch;
  * which is not graph-captured).  Waits for the members' pending work. */
 int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_stream,
                         tissue_batch** out);
+
+/* The same with at most scratch_limit bytes for its sum-tree launches: classes,
+ * largest cells first, whose launch needs more than is left run their launch
+ * shape's own kernel.  tissue_batch_create sets no limit. */
+int tissue_batch_create_within(tissue* const* members, uint32_t count, void* cuda_stream,
+                               size_t scratch_limit, tissue_batch** out);
 
 /* Launch shape of the chi launch of the class of cells with V voxels:
  * 8, 16 or 32 lanes per cell, 1..8 warps per block (1..4 with the recompute
@@ -314,6 +336,10 @@ int tissue_batch_read_counts(tissue_batch* b, int32_t* const* host);
 int tissue_batch_class_info(const tissue_batch* b, uint32_t i, uint32_t* V,
                             uint32_t* lanes_per_cell, uint32_t* warps_per_block,
                             uint32_t* smem_layout, uint32_t* cells);
+
+/* What class i's chi runs; its scratch_bytes are held while the batch exists,
+ * also while the class has a launch shape that does not use them. */
+int tissue_batch_get_chi_info(const tissue_batch* b, uint32_t i, tissue_chi_info* info);
 
 /* Diagnostic timing of batch steps (a measurement aid; the paper has no
  * counterpart).  With on = 1 every following step records CUDA events on the

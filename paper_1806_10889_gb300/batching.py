@@ -9,11 +9,13 @@ from __future__ import annotations
 
 import ctypes as C
 
-from .tissue import Tissue, TissueError, _check, lib
+from .tissue import ChiInfo, Tissue, TissueError, _check, lib
 
 
 class Batch:
-    def __init__(self, members: list[Tissue], stream=None):
+    def __init__(self, members: list[Tissue], stream=None, scratch_limit: int | None = None):
+        """scratch_limit: most bytes its sum-tree launches may hold (None: no
+        limit); classes past it run their launch shape's own kernel."""
         import torch
         if not members:
             raise ValueError("a batch needs at least one tissue")
@@ -24,8 +26,10 @@ class Batch:
         self._h = C.c_void_p()
         self.timing = False  # tissue_batch_set_timing's state
         self.overlap = True  # tissue_batch_set_overlap's state
-        _check(lib().tissue_batch_create(arr, len(members), C.c_void_p(self.stream.cuda_stream),
-                                         C.byref(self._h)), "tissue_batch_create")
+        limit = C.c_size_t(-1).value if scratch_limit is None else max(0, int(scratch_limit))
+        _check(lib().tissue_batch_create_within(arr, len(members),
+                                                C.c_void_p(self.stream.cuda_stream), limit,
+                                                C.byref(self._h)), "tissue_batch_create_within")
 
     def set_class_launch(self, V: int, lanes_per_cell: int, warps_per_block: int,
                          smem_layout: int = 0):
@@ -94,6 +98,18 @@ class Batch:
             out.append({"V": V, "lanes_per_cell": lanes, "warps_per_block": wpb,
                         "smem_layout": layout, "cells": cells})
         return out
+
+    def chi_info(self, i: int) -> dict:
+        """What class i's chi runs (as Tissue.chi_info); its scratch_bytes are
+        held while the batch exists."""
+        c = ChiInfo()
+        _check(lib().tissue_batch_get_chi_info(self._h, i, C.byref(c)),
+               "tissue_batch_get_chi_info")
+        return c.as_dict()
+
+    def scratch_bytes(self) -> int:
+        """Device memory the batch's sum-tree launches hold."""
+        return sum(self.chi_info(i)["scratch_bytes"] for i in range(self.info()[1]))
 
     def set_timing(self, on: bool) -> None:
         """Record device times of each following step (a measurement aid)."""

@@ -66,6 +66,9 @@ cudaError_t launch_chi_lane(const LanePlan& plan, int model, const TissueView* d
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,
                             uint32_t step_off, double dt, cudaStream_t stream, int priority = 0,
                             bool early = false);
+// What a launch of the plan, or of a shape of the segmented kernel, runs.
+tissue_chi_info lane_info(const LanePlan& plan);
+tissue_chi_info seg_info(const tissue_launch& shape, uint32_t V, int gen);
 using ChiLaneKernel = void (*)(const LaneArgs);
 // nullptr where not built.
 // k_chi_lane.cu, k_chi_lane_bind.cu, k_chi_lane_pm.cu

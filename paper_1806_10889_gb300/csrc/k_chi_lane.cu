@@ -143,6 +143,18 @@ LanePlan lane_plan(uint32_t V, uint64_t cells, int model, uint64_t beside) {
   return pl;
 }
 
+tissue_chi_info lane_info(const LanePlan& pl) {
+  return tissue_chi_info{1, pl.G, pl.leaf == kLeafShared ? 1u : 2u, 0, pl.scratch_bytes};
+}
+
+tissue_chi_info seg_info(const tissue_launch& c, uint32_t V, int gen) {
+  const int H = static_cast<int>(c.lanes_per_cell);
+  const bool narrow = c.kernel == TISSUE_KERNEL_PERSISTENT && gen == 0 && V > 256 &&
+                      chi_seg_kernel_narrow(H, c.smem_layout == TISSUE_LAYOUT_PREFIX,
+                                            V > static_cast<uint32_t>(H * H));
+  return tissue_chi_info{0, c.lanes_per_cell, narrow ? 2u : 1u, 0, 0};
+}
+
 cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_views,
                             const uint2* d_items, uint32_t n_items, uint32_t* d_counter,
                             uint64_t* d_scratch, const ChiRedo& redo, uint32_t V, uint32_t n,

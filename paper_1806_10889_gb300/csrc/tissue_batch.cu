@@ -13,6 +13,7 @@
 // alone and in any batch.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <map>
 #include <new>
 #include <vector>
@@ -100,6 +101,23 @@ bool overlapped(const tissue_batch* b) {
          b->side.size() + 1 == b->classes.size();
 }
 
+// Whether class p's chi is its sum-tree launch.
+bool runs_tree(const ClassPlan& p) {
+  return p.lane.G &&
+         default_shape(p.V, {TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0, p.layout});
+}
+
+// The segmented launch of class p.  As for single tissues: a counts-only launch
+// with several voxels per lane takes Notch-Delta classes without a trace; others
+// run the prefix launch of the class (the same trajectories).
+tissue_launch seg_launch(const ClassPlan& p) {
+  const tissue_launch lc{TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0, p.layout};
+  return lc.smem_layout == TISSUE_LAYOUT_RECOMPUTE &&
+                 !recompute_covers(p.V, static_cast<int>(p.lanes), p.gen)
+             ? prefix_launch(p.V, p.n_items)
+             : lc;
+}
+
 int chi_all(tissue_batch* b, double dt) {
   if (mark(b, 2) != TISSUE_OK) return TISSUE_E_CUDA;
   if (b->n_wm && launch_chi_wm(b->d_views, b->d_items + b->wm_off, b->n_wm, b->wm_vmax, 0u, dt,
@@ -114,9 +132,7 @@ int chi_all(tissue_batch* b, double dt) {
     const cudaStream_t st = (ov && c > 0) ? b->side[c - 1] : b->stream;
     if (ov && c > 0 && cudaStreamWaitEvent(st, b->ev_fork, 0) != cudaSuccess) return TISSUE_E_CUDA;
     uint32_t* counters = b->d_counters + 3 * c;
-    const bool tree =
-        p.lane.G &&
-        default_shape(p.V, {TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0, p.layout});
+    const bool tree = runs_tree(p);
     if ((!tree || p.lane.counters) &&
         cudaMemsetAsync(counters, 0, 3 * sizeof(uint32_t), st) != cudaSuccess)
       return TISSUE_E_CUDA;
@@ -133,13 +149,7 @@ int chi_all(tissue_batch* b, double dt) {
         return TISSUE_E_CUDA;
       continue;
     }
-    // as for single tissues: a counts-only launch with several voxels per
-    // lane takes Notch-Delta classes without a trace; others run the prefix
-    // launch of the class (the same trajectories)
-    tissue_launch lc{TISSUE_KERNEL_PERSISTENT, p.lanes, p.warps_per_block, 0, p.layout};
-    if (lc.smem_layout == TISSUE_LAYOUT_RECOMPUTE &&
-        !recompute_covers(p.V, static_cast<int>(p.lanes), p.gen))
-      lc = prefix_launch(p.V, p.n_items);
+    const tissue_launch lc = seg_launch(p);
     if (launch_chi_seg(b->d_views, b->d_items + p.items_off, p.n_items, counters, p.V,
                        static_cast<int>(lc.lanes_per_cell), static_cast<int>(lc.warps_per_block),
                        0, 0u, dt, lc.smem_layout == TISSUE_LAYOUT_PREFIX, p.gen, &redo, st,
@@ -231,6 +241,11 @@ extern "C" {
 
 int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_stream,
                         tissue_batch** out) {
+  return tissue_batch_create_within(members, count, cuda_stream, SIZE_MAX, out);
+}
+
+int tissue_batch_create_within(tissue* const* members, uint32_t count, void* cuda_stream,
+                               size_t scratch_limit, tissue_batch** out) {
   if (!out) return TISSUE_E_ARG;
   *out = nullptr;
   if (!members || count == 0) return TISSUE_E_ARG;
@@ -293,9 +308,12 @@ int tissue_batch_create(tissue* const* members, uint32_t count, void* cuda_strea
     // the sum-tree kernel writes no trace (a traced class of promoter members
     // has gen 2 like an untraced one)
     if (p.gen != 1 && tr_v[V] == 0) p.lane = lane_plan(V, kv.second.size(), p.lane_model, lane_warps);
+    // whole blocks of 256 bytes
+    const size_t need = (p.lane.scratch_bytes + 255) & ~static_cast<size_t>(255);
+    if (need > scratch_limit - lane_words * sizeof(uint64_t)) p.lane = LanePlan{};
     if (p.lane.G) lane_warps += static_cast<uint64_t>(p.lane.blocks) * (p.lane.threads / 32u);
     p.lane_off = lane_words;
-    lane_words += ((p.lane.scratch_bytes + 255) & ~static_cast<size_t>(255)) / sizeof(uint64_t);
+    if (p.lane.G) lane_words += need / sizeof(uint64_t);
     items.insert(items.end(), kv.second.begin(), kv.second.end());
     b->classes.push_back(p);
   }
@@ -545,6 +563,14 @@ int tissue_batch_class_info(const tissue_batch* b, uint32_t i, uint32_t* V,
   if (warps_per_block) *warps_per_block = p.warps_per_block;
   if (smem_layout) *smem_layout = p.layout;
   if (cells) *cells = p.n_items;
+  return TISSUE_OK;
+}
+
+int tissue_batch_get_chi_info(const tissue_batch* b, uint32_t i, tissue_chi_info* info) {
+  if (!b || i >= b->classes.size() || !info) return TISSUE_E_ARG;
+  const ClassPlan& p = b->classes[i];
+  *info = runs_tree(p) ? lane_info(p.lane) : seg_info(seg_launch(p), p.V, p.gen);
+  info->scratch_bytes = p.lane.G ? (p.lane.scratch_bytes + 255) & ~static_cast<size_t>(255) : 0;
   return TISSUE_OK;
 }
 

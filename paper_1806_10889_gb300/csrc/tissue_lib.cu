@@ -244,10 +244,14 @@ struct LaneCall {
   uint64_t* scratch = nullptr;
   cudaStream_t stream = nullptr;
 
-  LaneCall(tissue* t, uint32_t V) : stream(t->stream) {
+  explicit LaneCall(const tissue* t) : stream(t->stream) {
+    const uint32_t V = t->d.n * t->d.n;
     if (t->d_trace != nullptr || !default_shape(V, t->cfg)) return;
     model = t->q.kind == kModelPromoter ? 2 : (t->q.k_in || t->q.k_off) ? 1 : 0;
     plan = lane_plan(V, static_cast<uint64_t>(t->d.width) * t->d.height - t->wm_cells, model);
+  }
+  // Its scratch, on the tissue's stream.
+  void take_scratch() {
     if (plan.G == 0 || plan.scratch_bytes == 0) return;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaMemPool_t pool = nullptr;
@@ -270,19 +274,26 @@ struct LaneCall {
   LaneCall& operator=(const LaneCall&) = delete;
 };
 
+// The segmented launch of tissue t.  A counts-only launch with several voxels per
+// lane runs Notch-Delta launches without a trace only; others take the prefix
+// launch of the cell size (the same trajectory, bit for bit).
+int seg_gen(const tissue* t) {
+  return t->q.kind == kModelPromoter ? 2 : t->d_trace != nullptr ? 1 : 0;
+}
+tissue_launch seg_launch(const tissue* t) {
+  const uint32_t V = t->d.n * t->d.n, cells = t->d.width * t->d.height;
+  return t->cfg.kernel == TISSUE_KERNEL_PERSISTENT &&
+                 t->cfg.smem_layout == TISSUE_LAYOUT_RECOMPUTE &&
+                 !recompute_covers(V, static_cast<int>(t->cfg.lanes_per_cell), seg_gen(t))
+             ? prefix_launch(V, cells - t->wm_cells)
+             : t->cfg;
+}
+
 // chi for step offset i, in the tissue's launch configuration.
 cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, const LaneCall& lane, uint32_t i,
                            double dt) {
-  tissue_launch c = t->cfg;
-  if (c.kernel == TISSUE_KERNEL_PERSISTENT) {
+  if (t->cfg.kernel == TISSUE_KERNEL_PERSISTENT) {
     const uint32_t cells = t->d.width * t->d.height;
-    const int gen = t->q.kind == kModelPromoter ? 2 : t->d_trace != nullptr ? 1 : 0;
-    // A counts-only launch with several voxels per lane runs Notch-Delta
-    // launches without a trace only; others take the prefix launch of the
-    // cell size (the same trajectory, bit for bit).
-    if (c.smem_layout == TISSUE_LAYOUT_RECOMPUTE &&
-        !recompute_covers(v.V, static_cast<int>(c.lanes_per_cell), gen))
-      c = prefix_launch(v.V, cells - t->wm_cells);
     cudaError_t e = cudaSuccess;
     if (t->wm_cells) {  // well-mixed cells first, then the lattice cells by list
       e = launch_chi_wm(t->d_view, t->d_wm_items, t->wm_cells, v.V, i, dt, t->stream);
@@ -297,13 +308,14 @@ cudaError_t launch_chi_cfg(tissue* t, const TissueView& v, const LaneCall& lane,
       return launch_chi_lane(lane.plan, lane.model, t->d_view,
                              t->wm_cells ? t->d_lat_items : nullptr, cells - t->wm_cells, t->d_work,
                              lane.scratch, redo, v.V, v.n, i, dt, t->stream, 0, lane.early());
+    const tissue_launch c = seg_launch(t);
     const bool pre = c.smem_layout == TISSUE_LAYOUT_PREFIX;
     return launch_chi_seg(t->d_view, t->wm_cells ? t->d_lat_items : nullptr, cells - t->wm_cells,
                           t->d_work, v.V, static_cast<int>(c.lanes_per_cell),
                           static_cast<int>(c.warps_per_block), static_cast<int>(c.blocks), i, dt,
-                          pre, gen, &redo, t->stream);
+                          pre, seg_gen(t), &redo, t->stream);
   }
-  return launch_chi(v, i, dt, static_cast<int>(c.warps_per_block), t->stream);
+  return launch_chi(v, i, dt, static_cast<int>(t->cfg.warps_per_block), t->stream);
 }
 
 // One splitting step at step offset i.  `mark`, if given, is recorded right
@@ -584,7 +596,8 @@ int tissue_step(tissue* t, double dt, uint32_t n_steps) {
   if (!(dt > 0.0) || !std::isfinite(dt) || !launch_fits_model(t)) return TISSUE_E_ARG;
   if (n_steps == 0) return TISSUE_OK;
   const TissueView v = view_of(t);
-  const LaneCall lane(t, v.V);
+  LaneCall lane(t);
+  lane.take_scratch();
   for (uint32_t i = 0; i < n_steps; ++i) {
     const int rc = enqueue_split_step(t, v, lane, i, dt, nullptr, nullptr);
     if (rc != TISSUE_OK) return rc;
@@ -605,7 +618,8 @@ int tissue_step_timed(tissue* t, double dt, uint32_t n_steps, double* ms_chi, do
   for (auto& e : ev)
     if (cudaEventCreate(&e) != cudaSuccess) rc = TISSUE_E_CUDA;
   const TissueView v = view_of(t);
-  const LaneCall lane(t, v.V);
+  LaneCall lane(t);
+  lane.take_scratch();
   for (uint32_t i = 0; i < n_steps && rc == TISSUE_OK; ++i) {
     if (cudaEventRecord(ev[4 * i], t->stream) != cudaSuccess) rc = TISSUE_E_CUDA;
     if (rc == TISSUE_OK) rc = enqueue_split_step(t, v, lane, i, dt, ev[4 * i + 1], ev[4 * i + 2]);
@@ -725,6 +739,14 @@ int tissue_set_launch_config(tissue* t, const tissue_launch* c) {
 int tissue_get_launch_config(const tissue* t, tissue_launch* c) {
   if (!t || !c) return TISSUE_E_ARG;
   *c = t->cfg;
+  return TISSUE_OK;
+}
+
+int tissue_get_chi_info(const tissue* t, tissue_chi_info* info) {
+  if (!t || !info) return TISSUE_E_ARG;
+  const LaneCall lane(t);
+  *info = lane.plan.G ? lane_info(lane.plan)
+                      : seg_info(seg_launch(t), t->d.n * t->d.n, seg_gen(t));
   return TISSUE_OK;
 }
 

@@ -85,9 +85,11 @@ class Server:
     """Continuous-batching server over one device.
 
     budget_bytes: device memory the server may hold for tissue state and
-    scratch; chunk_steps: steps per batch call between admission points;
-    tuned: optional autotuner result (``autotune.tune_batch``) applied to
-    every batch; keep_counts: return each replica's final counts.
+    scratch (what the active requests leave of it bounds the scratch of the
+    batch's launches, which run another kernel without it); chunk_steps: steps
+    per batch call between admission points; tuned: optional autotuner result
+    (``autotune.tune_batch``) applied to every batch; keep_counts: return each
+    replica's final counts.
     """
 
     def __init__(self, budget_bytes: int, chunk_steps: int = 10, tuned: dict | None = None,
@@ -143,6 +145,7 @@ class Server:
         active: list[_Active] = []
         hashed = []
         batch = None
+        held = 0  # bytes of the batch's scratch
         members_key = None
         t0 = self.clock()
         while pending or active:
@@ -177,6 +180,9 @@ class Server:
                     continue
                 if self.used + need > self.budget:
                     break
+                if batch is not None and self.used + held + need > self.budget:
+                    batch.close()  # the next one holds less
+                    batch, members_key = None, None
                 pending.pop(0)
                 tissues = [Tissue(s) for s in req.replica_specs()]
                 res = results[req.index]
@@ -198,7 +204,9 @@ class Server:
                 tb = self.clock()
                 if batch is not None:
                     batch.close()
-                batch = Batch([t for a in chosen for t in a.tissues])
+                batch = Batch([t for a in chosen for t in a.tissues],
+                              scratch_limit=self.budget - self.used)
+                held = batch.scratch_bytes()
                 if self.tuned:
                     from .autotune import apply_batch
                     apply_batch(batch, self.tuned)
@@ -221,7 +229,7 @@ class Server:
             batch.sync()
             for a in chosen:
                 a.steps_done += k
-            self.peak_used = max(self.peak_used, self.used)
+            self.peak_used = max(self.peak_used, self.used + held)
             if on_round is not None:
                 on_round(self, [a.req.index for a in chosen])
             # 4. retire finished requests

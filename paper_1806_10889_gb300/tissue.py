@@ -70,6 +70,16 @@ class Launch(C.Structure):
                 ("smem_layout", C.c_uint32)]
 
 
+class ChiInfo(C.Structure):
+    _fields_ = [("sum_tree", C.c_uint32), ("lanes_per_cell", C.c_uint32),
+                ("launches", C.c_uint32), ("reserved", C.c_uint32),
+                ("scratch_bytes", C.c_uint64)]
+
+    def as_dict(self) -> dict:
+        return {"sum_tree": bool(self.sum_tree), "lanes_per_cell": int(self.lanes_per_cell),
+                "launches": int(self.launches), "scratch_bytes": int(self.scratch_bytes)}
+
+
 # Every exported symbol of include/tissue.h with (restype, argtypes).
 _P = C.POINTER
 SIGNATURES = {
@@ -97,10 +107,14 @@ SIGNATURES = {
     "tissue_batch_set_splitting": (C.c_int, [C.c_void_p, C.c_uint32]),
     "tissue_set_launch_config": (C.c_int, [C.c_void_p, _P(Launch)]),
     "tissue_get_launch_config": (C.c_int, [C.c_void_p, _P(Launch)]),
+    "tissue_get_chi_info": (C.c_int, [C.c_void_p, _P(ChiInfo)]),
     "tissue_step_noalloc": (C.c_int, [_P(Desc), _P(Model), C.c_void_p, C.c_uint32, C.c_double,
                                       C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p]),
     "tissue_selftest_time": (C.c_int, [C.c_uint64, C.c_uint64, _P(C.c_uint64)]),
     "tissue_batch_create": (C.c_int, [C.c_void_p, C.c_uint32, C.c_void_p, _P(C.c_void_p)]),
+    "tissue_batch_create_within": (C.c_int, [C.c_void_p, C.c_uint32, C.c_void_p, C.c_size_t,
+                                              _P(C.c_void_p)]),
+    "tissue_batch_get_chi_info": (C.c_int, [C.c_void_p, C.c_uint32, _P(ChiInfo)]),
     "tissue_batch_set_class_launch": (C.c_int, [C.c_void_p, C.c_uint32, C.c_uint32, C.c_uint32,
                                                  C.c_uint32]),
     "tissue_batch_step": (C.c_int, [C.c_void_p, C.c_double, C.c_uint32]),
@@ -293,6 +307,14 @@ class Tissue:
         c = Launch()
         _check(lib().tissue_get_launch_config(self._h, C.byref(c)), "tissue_get_launch_config")
         return (c.kernel, c.lanes_per_cell, c.warps_per_block, c.blocks, c.smem_layout)
+
+    def chi_info(self) -> dict:
+        """What the lattice chi of a step runs now: sum_tree (or the launch
+        shape's own kernel), lanes_per_cell, launches a step, and the device
+        memory it takes beside scratch_bytes for the length of a call."""
+        c = ChiInfo()
+        _check(lib().tissue_get_chi_info(self._h, C.byref(c)), "tissue_get_chi_info")
+        return c.as_dict()
 
     def set_splitting(self, scheme: int):
         _check(lib().tissue_set_splitting(self._h, int(scheme)), "tissue_set_splitting")
