@@ -4,11 +4,13 @@ split-step schedule.
 Every candidate runs the same steps from the same state on a clone of the
 work and must end with the same counts and statistics bit for bit (the
 arithmetic is exact, so a variant that differs is a bug, not noise); the
-fastest is kept.  Results are cached per GPU, cell size, tissue size class
-and dt in ``_build/autotune.json`` beside the compiled library.
+fastest is kept.  Results are cached per GPU, library build, cell size, tissue
+size class and dt in ``_build/autotune.json`` beside the compiled library: a
+pick made with other kernels is not taken over.
 """
 from __future__ import annotations
 
+import hashlib
 import json
 import math
 import os
@@ -17,7 +19,7 @@ import threading
 import numpy as np
 
 from .tissue import (KERNEL_PERSISTENT, KERNEL_WARP, LAYOUT_PREFIX, LAYOUT_RECOMPUTE, Tissue,
-                     TissueError)
+                     TissueError, lib, library_path)
 from .workloads import TissueSpec
 
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json")
@@ -60,6 +62,13 @@ def batch_class_candidates(V: int) -> list[tuple]:
 def _gpu_name() -> str:
     import torch
     return torch.cuda.get_device_name()
+
+
+def _build() -> str:
+    """What the compiled kernels are told apart by."""
+    lib()  # builds it where it is missing or stale
+    with open(library_path(), "rb") as f:
+        return hashlib.file_digest(f, "blake2b").hexdigest()[:16]
 
 
 def _load() -> dict:
@@ -106,7 +115,7 @@ def tune_tissue(spec: TissueSpec, dt: float, state: np.ndarray | None = None,
     on_candidate(config, tissue), if given, runs after each candidate's clone
     is set up and before it steps (a hook for tests of the bit-identity
     check)."""
-    key = f"tissue|{_gpu_name()}|V={spec.V}|cells~{_size_class(spec.cells)}|dt={dt}"
+    key = f"tissue|{_gpu_name()}|{_build()}|V={spec.V}|cells~{_size_class(spec.cells)}|dt={dt}"
     if use_cache and candidates is None:
         hit = _load().get(key)
         if hit:
@@ -159,7 +168,7 @@ def tune_batch(members: list[Tissue], dt: float, steps: int = 1, max_clones: int
     by_v: dict[int, list[Tissue]] = {}
     for m in members:
         by_v.setdefault(m.spec.V, []).append(m)
-    key = (f"batch|{_gpu_name()}|dt={dt}|" +
+    key = (f"batch|{_gpu_name()}|{_build()}|dt={dt}|" +
            ",".join(f"{V}:{_size_class(sum(m.spec.cells for m in ms))}"
                     for V, ms in sorted(by_v.items())))
     if use_cache:
