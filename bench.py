@@ -99,7 +99,7 @@ CHI_IPE = {
 # which runs default launch shapes in a form
 # that follows from the cell size and the number of cells (its warps serve up to
 # 32 cells): per workload and cell size, with its own sources.
-TREE_SOURCES = ["chi_lane.cuh", "chi_lane.h", "tissue_dev.cuh", "k_chi_lane.cu",
+TREE_SOURCES = ["chi_lane.cuh", "chi_lane.h", "pair_end.h", "tissue_dev.cuh", "k_chi_lane.cu",
                 "k_chi_lane_bind.cu", "k_chi_lane_pm.cu"]
 TREE_IPE = {
     "sources": "b5e78d1614589eb1",
@@ -149,28 +149,20 @@ def chi_kernel_key(V: int, lanes: int, layout: int, model: str = "nd") -> str:
             f"{'u16' if narrow else 'u32'}")
 
 
-def chi_launch_key(V: int, lanes: int, warps_per_block: int, layout: int) -> str:
-    """What a Notch-Delta launch of this shape runs: the sum-tree kernel for the
-    default shapes of the cell size, else the persistent kernel's
-    instantiation."""
-    few = (32, 2, 0)
-    default = {few, (8, 4, 0)} if V <= 64 else {few, (16, 4, 0), (8, 2, 1)} if V <= 256 else \
-        {few, (16, 2, 1)}
-    if (lanes, warps_per_block, layout) in default:
-        return f"V{V}/tree"
-    return chi_kernel_key(V, lanes, layout)
+def chi_launch_key(V: int, lanes: int, layout: int, sum_tree: bool) -> str:
+    """What a Notch-Delta launch of this shape runs: the sum-tree kernel where the
+    library says so (Tissue.chi_info, Batch.chi_info), else the persistent
+    kernel's instantiation."""
+    return f"V{V}/tree" if sum_tree else chi_kernel_key(V, lanes, layout)
+
+
+def class_key(c: dict, info: dict) -> str:
+    """chi_launch_key of a batch class (Batch.classes(), Batch.chi_info())."""
+    return chi_launch_key(c["V"], c["lanes_per_cell"], c["smem_layout"], info["sum_tree"])
 
 
 def chi_kernel_name(key: str) -> str:
     return f"{'k_chi_lane' if key.endswith('/tree') else 'k_chi_seg'} {key}"
-
-
-def chi_launches(key: str, cells: int) -> int:
-    """Kernels of one chi phase: the launch, and a second one for cells past
-    the range of packed counts, where there are any (the persistent kernel's
-    16-bit counts; the sum-tree kernel from 128 cells an SM up, which it keeps
-    packed at every cell size)."""
-    return 1 + int(cells > 128 * 152 if key.endswith("/tree") else key.endswith("u16"))
 
 
 def chi_ipe(workload: str, key: str):
@@ -423,6 +415,7 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
         bt.step(dt, 1)
     bt.sync()
     classes = bt.classes()
+    chi_info = [bt.chi_info(i) for i in range(len(classes))]
     step0 = members[0].get_step()
     sample = oracle_sample(runs, per_class=args.oracle_per_class) if (
         rank == 0 and world == 1 and not args.no_cpu_baseline) else []
@@ -467,7 +460,7 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
     per_class, inst, traffic, stale = [], 0.0, 0.0, False
     for ci, c in enumerate(classes):
         idx = [i for i, r in enumerate(runs) if r.tissue.V == c["V"]]
-        key = chi_launch_key(c["V"], c["lanes_per_cell"], c["warps_per_block"], c["smem_layout"])
+        key = class_key(c, chi_info[ci])
         ev_c = float(d_ev[idx, 0].sum())
         m = chi_ipe("batch", key)
         if m is None:
@@ -628,11 +621,9 @@ def batch_headline(args, rank: int, world: int, dist) -> dict:
         "parity_checked": None if cpu is None else cpu["parity_checked"],
     }
     # our kernels per step: per class the chi launch (and the pass over cells
-    # past the range of packed counts), both face phases and the step-counter
-    # update
-    per_step = sum(chi_launches(chi_launch_key(c["V"], c["lanes_per_cell"], c["warps_per_block"],
-                                               c["smem_layout"]), c["cells"])
-                   for c in classes) + 3
+    # past the range of packed counts, where its plan has one), both face phases
+    # and the step-counter update
+    per_step = sum(i["launches"] for i in chi_info) + 3
     out["gpu_launches"] = per_step * args.steps
     return out
 
@@ -658,6 +649,7 @@ def medium_leg(args) -> dict:
     if args.kernel == "persistent":
         g.set_launch_config(1, args.lanes, args.chi_wpb or 4, 0, args.layout)
     launch = g.launch_config()
+    sum_tree = g.chi_info()["sum_tree"]
     burn = int(round(args.burn_in / args.dt))
     if burn:
         g.step(args.dt, burn)
@@ -705,7 +697,7 @@ def medium_leg(args) -> dict:
     nbytes = spec.state_ints * 4
     g.close()
 
-    key = chi_launch_key(spec.V, launch[1], launch[2], launch[4]) if launch[0] == 1 else "warp"
+    key = chi_launch_key(spec.V, launch[1], launch[4], sum_tree) if launch[0] == 1 else "warp"
     out = {"metric": MEDIUM_METRIC, "value": events / (total_ms / 1e3), "unit": UNIT,
            "workload": f"tissue {spec.width}x{spec.height} cells of {spec.n}x{spec.n} voxels, "
                        f"Notch-Delta model, dt {args.dt}, burn-in {args.burn_in} time units, "
@@ -766,6 +758,7 @@ def _timed_tissue(spec, dt: float, burn: int, steps: int, flush: bool = True) ->
         chi_ms += c_ms
     ev = g.total_events() - ev0
     launch = g.launch_config()
+    chi_info = g.chi_info()
     g.close()
     return {"events_per_s": float(ev.sum()) / (total_ms / 1e3),
             "chi_events_per_s": float(ev[0]) / (chi_ms / 1e3),
@@ -776,7 +769,7 @@ def _timed_tissue(spec, dt: float, burn: int, steps: int, flush: bool = True) ->
             "steps": steps, "timed_steps_from": k0, "chi_ev": float(ev[0]), "chi_ms": chi_ms,
             "chi_launch": {"kernel": ["warp", "persistent"][launch[0]],
                            "lanes_per_cell": launch[1], "warps_per_block": launch[2],
-                           "smem_layout": launch[4]}}
+                           "smem_layout": launch[4], "sum_tree": chi_info["sum_tree"]}}
 
 
 def promoter_leg(args, run=None) -> dict:
@@ -806,8 +799,7 @@ def large_leg(args) -> dict:
     burn = int(round(args.large_burn_in / lg.dt))
     r = _timed_tissue(lg.tissue, lg.dt, burn, args.large_steps, flush=False)
     cl = r["chi_launch"]
-    key = chi_launch_key(lg.tissue.V, cl["lanes_per_cell"], cl["warps_per_block"],
-                         cl["smem_layout"])
+    key = chi_launch_key(lg.tissue.V, cl["lanes_per_cell"], cl["smem_layout"], cl["sum_tree"])
     r["roofline"] = issue_roofline("large", r.pop("chi_ev"), r.pop("chi_ms"), key, lg.tissue.V,
                                    lg.tissue.cells, args.large_steps, args.large_steps)
     r["workload"] = (f"tissue 256x256 cells of 32x32 voxels, Notch-Delta model, dt 0.1, "
@@ -1032,6 +1024,7 @@ def run_profile(args) -> dict:
             V, lanes, wpb, layout = (int(x) for x in part.split(":"))
             bt.set_class_launch(V, lanes, wpb, layout)
         classes = bt.classes()
+        chi_info = [bt.chi_info(i) for i in range(len(classes))]
         step = bt.step
 
         def sync():
@@ -1041,10 +1034,10 @@ def run_profile(args) -> dict:
         la = g.launch_config()
         classes = [{"V": g.spec.V, "lanes_per_cell": la[1], "warps_per_block": la[2],
                     "smem_layout": la[4], "cells": g.spec.cells}]
+        chi_info = [g.chi_info()]
         step, sync = g.step, g.sync
-    keys = [chi_launch_key(c["V"], c["lanes_per_cell"], c["warps_per_block"], c["smem_layout"])
-            for c in classes]
-    per_step = sum(chi_launches(k, c["cells"]) for k, c in zip(keys, classes))
+    keys = [class_key(c, i) for c, i in zip(classes, chi_info)]
+    per_step = sum(i["launches"] for i in chi_info)
     burn = int(round(burn_time / dt))
     step(dt, burn + args.warmup)
     sync()

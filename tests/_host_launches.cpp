@@ -18,7 +18,8 @@ std::map<const void*, std::string>& names() {
   static std::map<const void*, std::string> m;
   return m;
 }
-bool record = false;  // print launches
+bool record = false;  // print and count launches
+uint32_t launched = 0;
 
 // The template arguments of a sum-tree kernel.
 bool lane_args(const std::string& n, int a[5]) {
@@ -65,6 +66,7 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* k, void**) {
   if (!record) return cudaSuccess;
+  ++launched;
   int early = 0, priority = 0;
   for (unsigned i = 0; i < c->numAttrs; ++i) {
     if (c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization)
@@ -79,14 +81,20 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* k, void
 }
 
 // The launches of one chi phase whose cells are packed, so that there is a pass
-// over those past the packed range.
+// over those past the packed range; then one without.
 static int launches(int priority, bool early) {
-  tsg::LanePlan pl = tsg::lane_plan(1024, 30 * 152, 0);
-  if (pl.G == 0 || pl.leaf == tsg::kLeafShared) return 1;
   record = true;
-  return tsg::launch_chi_lane(pl, 0, nullptr, nullptr, 30 * 152, nullptr, nullptr,
-                              tsg::ChiRedo{nullptr, nullptr}, 1024, 32, 0, 0.1, nullptr, priority,
-                              early) != cudaSuccess;
+  for (const uint32_t cells : {30u * 152u, 152u}) {
+    const tsg::LanePlan pl = tsg::lane_plan(1024, cells, 0);
+    if (pl.G == 0 || (pl.leaf == tsg::kLeafShared) != (cells == 152u)) return 1;
+    launched = 0;
+    if (tsg::launch_chi_lane(pl, 0, nullptr, nullptr, cells, nullptr, nullptr,
+                             tsg::ChiRedo{nullptr, nullptr}, 1024, 32, 0, 0.1, nullptr, priority,
+                             early) != cudaSuccess ||
+        launched != tsg::lane_info(pl).launches)
+      return 1;
+  }
+  return 0;
 }
 
 // Every class a batch may hold, behind up to a chip full of other warps: the
