@@ -398,6 +398,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   const bool vec = (V & 3u) == 0u;
   const uint32_t warps = HELP ? 1u : blockDim.x >> 5;  // that run cells
 
+  // The index i of an array of n (checked build: `oob` when it is out of range).
+  [[maybe_unused]] bool oob = false;
+#define IX(i, n) TSG_IDX(i, n, oob)
   // offsets u - v of the m-th existing direction for each neighbour mask, then
   // (shared leaves) the voxels' masks: bits 0..3, and their number: bits 4..6
   int16_t* hop_off = reinterpret_cast<int16_t*>(smem);
@@ -416,22 +419,35 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     uint32_t b = i >> 2;
     for (uint32_t k = i & 3u; k > 0u; --k) b &= b - 1u;
     const int d = __ffs(static_cast<int>(b)) - 1;
-    hop_off[i] = static_cast<int16_t>(d < 0    ? 0
+    hop_off[IX(i, 64)] = static_cast<int16_t>(d < 0    ? 0
                                       : d == 0 ? -1
                                       : d == 1 ? 1
                                       : d == 2 ? -static_cast<int>(n)
                                                : static_cast<int>(n));
   }
   const uint32_t nl = (nq + 3u) >> 2;  // lines of four quads (sectors)
+  [[maybe_unused]] const uint32_t lut_n = SEC ? nl * 16u : nq * 4u;
   for (uint32_t v = threadIdx.x; v < (SEC ? nl * 16u : nq * 4u); v += blockDim.x) {
     const uint32_t vy = v / n, vx = v - vy * n;
     const uint32_t m = static_cast<uint32_t>(vx > 0) | (static_cast<uint32_t>(vx < n - 1) << 1) |
                        (static_cast<uint32_t>(vy > 0) << 2) |
                        (static_cast<uint32_t>(vy < n - 1) << 3);
-    lut[v] = static_cast<unsigned char>(m | (__popc(m) << 4));
+    lut[IX(v, lut_n)] = static_cast<unsigned char>(m | (__popc(m) << 4));
   }
   __syncthreads();
   early_launch();
+  if (kChecked) {  // the parts of shared memory and of the scratch array
+    uint32_t bytes;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+    const uint32_t cell = 48u + 8u * lane_sum_words(LV, LEAF, G) + (PLN ? 6u : REC ? 0u : 20u) * ps;
+    const uint64_t words = SEC ? 16u * nl : 8u * nq;
+    if (128u + lut_n + (HELP ? kExchangeBytes : 0u) > p.lut_bytes || cell > p.cell_stride ||
+        p.lut_bytes + warps * slots * p.cell_stride > bytes ||
+        (REC && !PLN && gridDim.x * warps * slots * words > p.scratch_words)) {
+      if (threadIdx.x == 0) atomicOr(p.views[0].err, kErrBounds);
+      return;  // the whole block
+    }
+  }
 
   // The helper warp: draws for the events after those in hand, a batch ahead.
   // Per phase (one barrier of both warps) it takes the new cells' streams and
@@ -478,6 +494,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       REC && !PLN ? p.scratch + (static_cast<size_t>(blockIdx.x) * warps + wib) * slots * rec_words
           : nullptr;
   uint64_t* rec = warp_rec + static_cast<size_t>(slot) * rec_words;
+  [[maybe_unused]] const uint32_t tree_n = kCnt + (REC ? 0u : ps);  // words of `tree`
 
   LaneRates<MODEL> q{};
   const TissueView* tv = p.views + (p.items ? p.items[0].x : 0u);
@@ -493,7 +510,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   int err = 0;
   // records: the bits a count has once it reaches its limit (a power of two)
   auto set_limits = [&](const Limits& l) {
-    over_mask = pack_voxel(0xFFFFFu & ~(l.D - 1u), 0xFFFFFu & ~(l.N - 1u), 0xFFFFFu & ~(l.R - 1u), 0u);
+    auto bits = [](uint32_t x) { return 0xFFFFFu & ~(x - 1u); };
+    over_mask = pack_voxel(bits(l.D), bits(l.N), bits(l.R), 0u);
     lim_dn = l.D;
     lim_r = l.R;
   };
@@ -530,6 +548,10 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       }
       const uint2 w = p.items ? p.items[it] : make_uint2(0u, it);
       const TissueView* ntv = p.views + w.x;
+      if (kChecked && (ntv->V != V || w.y >= ntv->width * ntv->height)) {
+        if (lane == 0) atomicOr(ntv->err, kErrBounds);
+        continue;
+      }
       LaneRates<MODEL> nr;
       nr.load(ntv->q);
       const int32_t* g = ntv->counts + static_cast<size_t>(w.y) * 3u * V;
@@ -551,9 +573,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         if (qi < nq) {
           uint32_t d[4] = {0, 0, 0, 0}, m[4] = {0, 0, 0, 0}, r[4] = {0, 0, 0, 0};
           if (vec) {
-            const uint4 x = reinterpret_cast<const uint4*>(g)[qi];
-            const uint4 y = reinterpret_cast<const uint4*>(g + V)[qi];
-            const uint4 z = reinterpret_cast<const uint4*>(g + 2u * V)[qi];
+            const uint4 x = reinterpret_cast<const uint4*>(g)[IX(qi, V / 4u)];
+            const uint4 y = reinterpret_cast<const uint4*>(g + V)[IX(qi, V / 4u)];
+            const uint4 z = reinterpret_cast<const uint4*>(g + 2u * V)[IX(qi, V / 4u)];
             d[0] = x.x, d[1] = x.y, d[2] = x.z, d[3] = x.w;
             m[0] = y.x, m[1] = y.y, m[2] = y.z, m[3] = y.w;
             r[0] = z.x, r[1] = z.y, r[2] = z.z, r[3] = z.w;
@@ -561,9 +583,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
 #pragma unroll
             for (uint32_t i = 0; i < 4u; ++i)
               if (4u * qi + i < V) {
-                d[i] = static_cast<uint32_t>(g[4u * qi + i]);
-                m[i] = static_cast<uint32_t>(g[V + 4u * qi + i]);
-                r[i] = static_cast<uint32_t>(g[2u * V + 4u * qi + i]);
+                d[i] = static_cast<uint32_t>(g[IX(4u * qi + i, 3u * V)]);
+                m[i] = static_cast<uint32_t>(g[IX(V + 4u * qi + i, 3u * V)]);
+                r[i] = static_cast<uint32_t>(g[IX(2u * V + 4u * qi + i, 3u * V)]);
               }
           }
           uint64_t wd[4];
@@ -572,7 +594,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             const uint32_t v = 4u * qi + i;
             wd[i] = 0ull;
             if (v < V) {
-              const uint32_t mk = lut[v], nn = mk >> 4;
+              const uint32_t mk = lut[IX(v, lut_n)], nn = mk >> 4;
               const bool ctr = MODEL == 2 && v == centre;
               if (MODEL == 2 && r[i] > static_cast<uint32_t>(ctr)) bad_state = true;
               if (REC) {
@@ -592,26 +614,27 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             S += a[i];
           }
           if (SEC) {
-            store4(nrec + 4u * qi, U64x4{S, pack4(d), pack4(m), pack4(r)});
+            store4(nrec + 4u * IX(qi, rec_words / 4u), U64x4{S, pack4(d), pack4(m), pack4(r)});
           } else if (PLN) {
             uint64_t* o = ntree + kCnt;
-            o[qi] = pack4(d);
-            o[nq + qi] = pack4(m);
-            o[2u * nq + qi] = pack4(r);
+            o[IX(qi, 3u * nq)] = pack4(d);
+            o[IX(nq + qi, 3u * nq)] = pack4(m);
+            o[IX(2u * nq + qi, 3u * nq)] = pack4(r);
           } else if (REC) {
-            ulonglong2* o = reinterpret_cast<ulonglong2*>(nrec) + 4u * qi;
+            ulonglong2* o = reinterpret_cast<ulonglong2*>(nrec) + 4u * IX(qi, rec_words / 8u);
 #pragma unroll
             for (int i = 0; i < 4; ++i) o[i] = make_ulonglong2(a[i], wd[i]);
           } else {
-            ulonglong2* o = reinterpret_cast<ulonglong2*>(ntree + kCnt) + 2u * qi;
+            ulonglong2* o = reinterpret_cast<ulonglong2*>(ntree + kCnt) + 2u * IX(qi, nq);
             o[0] = make_ulonglong2(a[0], a[1]);
             o[1] = make_ulonglong2(a[2], a[3]);
-            reinterpret_cast<uint4*>(ncp)[qi] = make_uint4(d[0], d[1], d[2], d[3]);
-            reinterpret_cast<uint4*>(ncp + ps)[qi] = make_uint4(m[0], m[1], m[2], m[3]);
-            reinterpret_cast<uint4*>(ncp + 2u * ps)[qi] = make_uint4(r[0], r[1], r[2], r[3]);
+            reinterpret_cast<uint4*>(ncp)[IX(qi, nq)] = make_uint4(d[0], d[1], d[2], d[3]);
+            reinterpret_cast<uint4*>(ncp + ps)[IX(qi, nq)] = make_uint4(m[0], m[1], m[2], m[3]);
+            reinterpret_cast<uint4*>(ncp + 2u * ps)[IX(qi, nq)] =
+                make_uint4(r[0], r[1], r[2], r[3]);
           }
         } else if (SEC && qi < 4u * nl) {
-          store4(nrec + 4u * qi, U64x4{0ull, 0ull, 0ull, 0ull});
+          store4(nrec + 4u * IX(qi, rec_words / 4u), U64x4{0ull, 0ull, 0ull, 0ull});
         }
         // the sums above the quads (entries past the last quad are zero)
         if (WIDE) {
@@ -625,35 +648,36 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           const uint64_t E = I - S;
           const uint64_t first = __shfl_sync(kFull, E, lane & ~static_cast<int>(W - 1u));
           if (qi < NQ) {
-            if (qi % W == 0u) ntree[qi / W] = total + first;
+            if (qi % W == 0u) ntree[IX(qi / W, tree_n)] = total + first;
             if (VMID) {
               uint64_t x = E - first;
 #pragma unroll
               for (uint32_t i = 0; i < 4u; ++i) {
-                ntree[kMid + 4u * qi + i] = x;
+                ntree[IX(kMid + 4u * qi + i, tree_n)] = x;
                 x += a[i];
               }
             } else if (FOUR) {
-              if (qi % 4u == 0u) ntree[kMid + qi / 4u] = E - first;
-              ntree[kFour + qi] = S;
+              if (qi % 4u == 0u) ntree[IX(kMid + qi / 4u, tree_n)] = E - first;
+              ntree[IX(kFour + qi, tree_n)] = S;
             } else if (MID) {
-              ntree[kMid + qi] = E - first;
+              ntree[IX(kMid + qi, tree_n)] = E - first;
             }
           }
           total += __shfl_sync(kFull, I, 31);
           continue;
         }
-        if (!SEC && qi < NQ) ntree[level_off(LV - 1) + qi] = S;
+        if (!SEC && qi < NQ) ntree[IX(level_off(LV - 1) + qi, tree_n)] = S;
         uint64_t x = S + __shfl_xor_sync(kFull, S, 1);
         x += __shfl_xor_sync(kFull, x, 2);
-        if (qi < NQ && (lane & 3) == 0) ntree[level_off(LV - 2) + (qi >> 2)] = x;
+        if (qi < NQ && (lane & 3) == 0) ntree[IX(level_off(LV - 2) + (qi >> 2), tree_n)] = x;
         x += __shfl_xor_sync(kFull, x, 4);
         x += __shfl_xor_sync(kFull, x, 8);
-        if (LV >= 4 && (lane & 15) == 0) ntree[level_off(LV >= 4 ? LV - 3 : 1) + (qi >> 4)] = x;
+        if (LV >= 4 && (lane & 15) == 0)
+          ntree[IX(level_off(LV >= 4 ? LV - 3 : 1) + (qi >> 4), tree_n)] = x;
         x += __shfl_xor_sync(kFull, x, 16);
         if (LV == 5) {
           pair = (k & 1u) ? pair + x : x;
-          if ((k & 1u) && lane == 0) ntree[k >> 1] = pair;
+          if ((k & 1u) && lane == 0) ntree[IX(k >> 1, tree_n)] = pair;
         }
         total += x;
       }
@@ -661,9 +685,11 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       nbig = __any_sync(kFull, nbig);
       Limits nlim{1, 1, 1};
       if (REC) nbig = !pick_limits<MODEL, LEAF>(ntv, warp_max(top), nlim);
+      const bool out_of_range = kChecked && __any_sync(kFull, oob);
+      oob = false;
       __syncwarp();
       if (slot == sc) {
-        if (WIDE) X1 = ntree[li];
+        if (WIDE) X1 = ntree[IX(li, tree_n)];
         q = nr;
         tv = ntv;
         step = *ntv->step + p.step_off;
@@ -687,6 +713,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         big = nbig;
         lim = min(nr.small, kLaneHill);
         err = any_bad ? kErrState : any_ovf ? kErrOverflow : (REC && nbig) ? kErrNarrow : 0;
+        if (out_of_range) err = kErrBounds;
         have = true;
         if (REC) set_limits(nlim);
       }
@@ -754,6 +781,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       batch = min(32u, __reduce_max_sync(kFull, few));  // uniform, for the compiler too
     }
     for (uint32_t i = 0; i < batch; ++i) {
+      [[maybe_unused]] const bool ran = run;
       const uint64_t R64 = Rn;
       if (!ONE)
         Rn = HELP ? bits[(i + 1u) % G]
@@ -766,19 +794,21 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         kv = pick_lane<RAD>(X1, r, base_lane);
         idx = kv;
         if (MID) {
-          xm = tree[kMid + kv * RAD + li];
+          xm = tree[IX(kMid + kv * RAD + li, tree_n)];
           pv = pick_lane<RAD>(xm, r, base_lane);
           idx = kv * RAD + pv;
         }
         if (FOUR) {
-          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + kFour) + 2u * idx;
+          const ulonglong2* nd =
+              reinterpret_cast<const ulonglong2*>(tree + kFour) + 2u * IX(idx, 64);
           const ulonglong2 x = nd[0], y = nd[1];
           idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
         }
       } else {
 #pragma unroll
         for (uint32_t l = 1; l <= SL; ++l) {
-          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) + 2u * idx;
+          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + level_off(l)) +
+                                 2u * IX(idx, 1 << (2u * (l - 1u)));
           const ulonglong2 x = nd[0], y = nd[1];
           idx = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
         }
@@ -786,7 +816,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       U64x4 sec{};  // sectors: the quad's sum and its counts of D, N and R
       if (SEC) {
         idx = min(idx, nl - 1u);
-        const uint64_t* line = rec + 16u * idx;
+        const uint64_t* line = rec + 16u * IX(idx, nl);
         const U64x4 x0 = load4(line), x1 = load4(line + 4), x2 = load4(line + 8),
                     x3 = load4(line + 12);
         const uint32_t k = pick_child<false>(x0.a, x1.a, x2.a, r);
@@ -803,7 +833,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       uint64_t a_v, w_v = 0;
       uint32_t v, D, N, R, mask, nn;
       if (SEC) {
-        const uint32_t mk4 = *reinterpret_cast<const uint32_t*>(lut + 4u * idx);
+        const uint32_t mk4 = *reinterpret_cast<const uint32_t*>(lut + 4u * IX(idx, lut_n / 4u));
         uint64_t a[4];
 #pragma unroll
         for (uint32_t j = 0; j < 4u; ++j) {
@@ -815,7 +845,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             t += q.tD * F + q.kd * Rj + q.k_in * (static_cast<uint64_t>(Nj) * F);
           } else {
             // R < kHillTab in a cell that runs; the mask is for idle lanes
-            t += (q.gR + q.k_off + q.hR * nj) * Rj + __ldg(q.hill + (Rj & (kHillTab - 1u))) + q.kN;
+            t += (q.gR + q.k_off + q.hR * nj) * Rj +
+                 __ldg(q.hill + IX(Rj & (kHillTab - 1u), kHillTab)) + q.kN;
             if (MODEL == 1) t += q.k_in * (static_cast<uint64_t>(Dj) * Nj);
           }
           a[j] = t;
@@ -832,15 +863,17 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       } else if (PLN) {
         // lane j of every four computes the quad's voxel j; the prefixes find v
         const uint32_t vj = 4u * idx + (sl & 3u);
-        const uint32_t Dj = hp[vj], Nj = hp[ps + vj], Rj = hp[2u * ps + vj];
-        const uint32_t mk = lut[vj], nj = mk >> 4;
+        const uint32_t Dj = hp[IX(vj, 3u * ps)], Nj = hp[IX(ps + vj, 3u * ps)],
+                       Rj = hp[IX(2u * ps + vj, 3u * ps)];
+        const uint32_t mk = lut[IX(vj, lut_n)], nj = mk >> 4;
         uint64_t t = (q.gD + q.hD * nj) * Dj + (q.gN + q.hN * nj) * Nj;
         if (MODEL == 2) {
           const uint32_t Fj = static_cast<uint32_t>(vj == centre) - Rj;
           t += q.tD * Fj + q.kd * Rj + q.k_in * (static_cast<uint64_t>(Nj) * Fj);
         } else {
           // R < kHillTab in a cell that runs; the mask is for idle lanes
-          t += (q.gR + q.k_off + q.hR * nj) * Rj + __ldg(q.hill + (Rj & (kHillTab - 1u))) + q.kN;
+          t += (q.gR + q.k_off + q.hR * nj) * Rj +
+               __ldg(q.hill + IX(Rj & (kHillTab - 1u), kHillTab)) + q.kN;
           if (MODEL == 1) t += q.k_in * (static_cast<uint64_t>(Dj) * Nj);
         }
         uint64_t in = t;
@@ -862,8 +895,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         mask = (rm >> 16) & 15u;
         nn = rm >> 20;
       } else if (REC) {
-        const U64x4 x = load4(rec + 8u * idx);
-        const U64x4 y = load4(rec + 8u * idx + 4u);
+        const U64x4 x = load4(rec + 8u * IX(idx, nq));
+        const U64x4 y = load4(rec + 8u * IX(idx, nq) + 4u);
         const uint32_t k = pick_child<!ONE>(x.a, x.c, y.a, r);
         a_v = k == 0u ? x.a : k == 1u ? x.c : k == 2u ? y.a : y.c;
         w_v = k == 0u ? x.b : k == 1u ? x.d : k == 2u ? y.b : y.d;
@@ -876,15 +909,16 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       } else {
         v = idx;
         if (!VMID) {
-          const ulonglong2* nd = reinterpret_cast<const ulonglong2*>(tree + kCnt) + 2u * idx;
+          const ulonglong2* nd =
+              reinterpret_cast<const ulonglong2*>(tree + kCnt) + 2u * IX(idx, nq);
           const ulonglong2 x = nd[0], y = nd[1];
           v = 4u * idx + pick_child<!ONE>(x.x, x.y, y.x, r);
         }
-        a_v = tree[kCnt + v];
-        D = static_cast<uint32_t>(cp[v]);
-        N = static_cast<uint32_t>(cp[ps + v]);
-        R = static_cast<uint32_t>(cp[2u * ps + v]);
-        const uint32_t mk = lut[v];
+        a_v = tree[IX(kCnt + v, tree_n)];
+        D = static_cast<uint32_t>(cp[IX(v, 3u * ps)]);
+        N = static_cast<uint32_t>(cp[IX(ps + v, 3u * ps)]);
+        R = static_cast<uint32_t>(cp[IX(2u * ps + v, 3u * ps)]);
+        const uint32_t mk = lut[IX(v, lut_n)];
         mask = mk & 15u;
         nn = mk >> 4;
       }
@@ -920,7 +954,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         const uint64_t z3 = z0 - (z2 ? H2 : z1 ? HD : 0ull);
         const bool b2 = z3 >= unit2;
         const uint64_t z4 = z3 - (b2 ? unit2 : 0ull);
-        const int off = hop_off[(mask << 2) + (b2 ? 2u : 0u) + (z4 >= unit ? 1u : 0u)];
+        const int off = hop_off[IX((mask << 2) + (b2 ? 2u : 0u) + (z4 >= unit ? 1u : 0u), 64)];
         u = v + static_cast<uint32_t>(off);
         if (kChecked && run && u >= V) err |= kErrBounds;
         u = min(u, V - 1u);
@@ -963,10 +997,10 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       // lane-wide nodes: u's entry in each, and what is there
       const uint32_t ku = u / RV, pu = u / MV % RAD;
       uint64_t xu = 0, fq = 0;
-      if (MID) xu = tree[kMid + ku * RAD + li];
-      if (FOUR) fq = tree[kFour + ((sl & 1u) ? u >> 2 : v >> 2)];
+      if (MID) xu = tree[IX(kMid + ku * RAD + li, tree_n)];
+      if (FOUR) fq = tree[IX(kFour + ((sl & 1u) ? u >> 2 : v >> 2), tree_n)];
       // differences of the totals of v and u
-      const ulonglong2 gh = rates[s];
+      const ulonglong2 gh = rates[IX(s, 3)];
       uint64_t dv, du = 0;
       uint32_t nc = 0, newmax = 0;
       {
@@ -989,26 +1023,26 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       uint32_t cu = 0;
       uint64_t a_u = 0, w_u = 0;  // records: u's total and word; sectors: its quad's sum and counts
       if (SEC) {
-        const uint64_t* uq = rec + 4u * (u >> 2);
+        const uint64_t* uq = rec + 4u * IX(u >> 2, rec_words / 4u);
         a_u = uq[0];
         w_u = uq[1u + s];
         cu = field16(w_u, u & 3u) + 1u;
         if (hop) {
-          du = gh.x + gh.y * (lut[u] >> 4);
+          du = gh.x + gh.y * (lut[IX(u, lut_n)] >> 4);
           if (MODEL == 1 && s < 2u) du += q.k_in * field16(uq[2u - s], u & 3u);
           if (MODEL == 2 && s == 1u)
             du += q.k_in * (static_cast<uint32_t>(u == centre) - field16(uq[3], u & 3u));
         }
       } else if (PLN) {
-        cu = hp[s * ps + u] + 1u;
+        cu = hp[IX(s * ps + u, 3u * ps)] + 1u;
         if (hop) {
-          du = gh.x + gh.y * (lut[u] >> 4);
-          if (MODEL == 1 && s < 2u) du += q.k_in * hp[(1u - s) * ps + u];
+          du = gh.x + gh.y * (lut[IX(u, lut_n)] >> 4);
+          if (MODEL == 1 && s < 2u) du += q.k_in * hp[IX((1u - s) * ps + u, 3u * ps)];
           if (MODEL == 2 && s == 1u)
-            du += q.k_in * (static_cast<uint32_t>(u == centre) - hp[2u * ps + u]);
+            du += q.k_in * (static_cast<uint32_t>(u == centre) - hp[IX(2u * ps + u, 3u * ps)]);
         }
       } else if (REC) {
-        const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec)[u];
+        const ulonglong2 x = reinterpret_cast<const ulonglong2*>(rec)[IX(u, rec_words / 2u)];
         a_u = x.x;
         w_u = x.y;
         if (hop) {
@@ -1018,23 +1052,29 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             du += q.k_in * (static_cast<uint32_t>(u == centre) - word_R(w_u));
         }
       } else {
-        cu = static_cast<uint32_t>(cp[s * ps + u]) + 1u;
-        if (WIDE) a_u = tree[kCnt + u];
+        cu = static_cast<uint32_t>(cp[IX(s * ps + u, 3u * ps)]) + 1u;
+        if (WIDE) a_u = tree[IX(kCnt + u, tree_n)];
         if (hop) {
-          du = gh.x + gh.y * (lut[u] >> 4);
+          du = gh.x + gh.y * (lut[IX(u, lut_n)] >> 4);
           if (MODEL == 1 && s < 2u)
-            du += q.k_in * static_cast<uint32_t>(cp[(1u - s) * ps + u]);
+            du += q.k_in * static_cast<uint32_t>(cp[IX((1u - s) * ps + u, 3u * ps)]);
           if (MODEL == 2 && s == 1u)
-            du += q.k_in * (static_cast<uint32_t>(u == centre) - static_cast<uint32_t>(cp[2u * ps + u]));
+            du += q.k_in * (static_cast<uint32_t>(u == centre) -
+                            static_cast<uint32_t>(cp[IX(2u * ps + u, 3u * ps)]));
           newmax |= cu;
         }
       }
-      if (MODEL != 2 && s == 2u && run && !several) {  // R changes the Hill term, here and where it arrives
+      // R changes the Hill term, here and where it arrives
+      if (MODEL != 2 && s == 2u && run && !several) {
         // (records: the event that leaves the table reads its end; its cell is redone)
-        const uint32_t Ru = hop ? (REC && !SEC && !PLN ? min(word_R(w_u) + 1u, kHillTab - 1u) : cu) : 1u;
+        const uint32_t Ru = !hop                       ? 1u
+                            : LEAF == kLeafRecords ? min(word_R(w_u) + 1u, kHillTab - 1u)
+                                                   : cu;
         if (!slow) {  // every count is inside the table
-          dv += __ldg(q.hill + (R - 1u)) - __ldg(q.hill + R);
-          const uint64_t d = __ldg(q.hill + Ru) - __ldg(q.hill + (Ru - 1u));
+          dv += __ldg(q.hill + IX(R - 1u, kHillTab)) -
+                __ldg(q.hill + IX(R, kHillTab));
+          const uint64_t d = __ldg(q.hill + IX(Ru, kHillTab)) -
+                             __ldg(q.hill + IX(Ru - 1u, kHillTab));
           if (hop) du += d;
         } else {
           dv += lane_hill(q.hill, tv, R - 1u) - lane_hill(q.hill, tv, R);
@@ -1054,17 +1094,17 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         __syncwarp();
         if (run) {
           if (MID && sl < RAD) {
-            tree[kMid + kv * RAD + li] = xm;
-            if (!same) tree[kMid + ku * RAD + li] = xu;
+            tree[IX(kMid + kv * RAD + li, tree_n)] = xm;
+            if (!same) tree[IX(kMid + ku * RAD + li, tree_n)] = xu;
           }
           if (FOUR && sl < 2u) {
             const bool sq = (v >> 2) == (u >> 2);
-            if (sl == 0u) tree[kFour + (v >> 2)] = fq + dv + (sq ? du : 0ull);
-            else if (!sq) tree[kFour + (u >> 2)] = fq + du;
+            if (sl == 0u) tree[IX(kFour + (v >> 2), tree_n)] = fq + dv + (sq ? du : 0ull);
+            else if (!sq) tree[IX(kFour + (u >> 2), tree_n)] = fq + du;
           }
           if (!REC) {
-            if (sl == 0u) tree[kCnt + v] = a_v + dv;
-            if (sl == 1u && hop) tree[kCnt + u] = a_u + du;
+            if (sl == 0u) tree[IX(kCnt + v, tree_n)] = a_v + dv;
+            if (sl == 1u && hop) tree[IX(kCnt + u, tree_n)] = a_u + du;
           }
         }
       } else if (ONE) {
@@ -1075,10 +1115,11 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
             uint64_t x[SL];
 #pragma unroll
             for (uint32_t l = 1; l <= SL; ++l)
-              x[l - 1] = tree[level_off(l) + ((side ? u : v) >> (2u * (LV - l)))];
+              x[l - 1] = tree[IX(level_off(l) + ((side ? u : v) >> (2u * (LV - l))), tree_n)];
 #pragma unroll
             for (uint32_t l = 1; l <= SL; ++l)
-              tree[level_off(l) + ((side ? u : v) >> (2u * (LV - l)))] = x[l - 1] + (side ? du : dv);
+              tree[IX(level_off(l) + ((side ? u : v) >> (2u * (LV - l))), tree_n)] =
+                  x[l - 1] + (side ? du : dv);
           }
         }
       } else {
@@ -1091,7 +1132,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         for (uint32_t t = sl; t < kTasks; t += G) {
           const uint32_t l = (t >> 1) + 1u;
           const uint32_t i1 = me >> (2u * (LV - l)), i2 = other >> (2u * (LV - l));
-          uint64_t* at = tree + level_off(l) + i1;
+          uint64_t* at = tree + IX(level_off(l) + i1, tree_n);
           const bool same = i1 == i2;
           if (run && !(odd && same)) *at += dme + (same ? dot : 0ull);
         }
@@ -1101,7 +1142,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         // the quad's sum and the changed species' counts, here and at u
         const uint64_t at = 1ull << (16u * (v & 3u)), to = hop ? 1ull << (16u * (u & 3u)) : 0ull;
         const bool same = (v >> 2) == (u >> 2);
-        uint64_t* vq = rec + 4u * (v >> 2);
+        uint64_t* vq = rec + 4u * IX(v >> 2, rec_words / 4u);
         const uint64_t w = (s == 0u ? sec.b : s == 1u ? sec.c : sec.d) + (gain ? at : 0ull - at);
         if (run && (ONE || sl == 0u)) {
           vq[0] = sec.a + dv + (same ? du : 0ull);
@@ -1114,7 +1155,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           }
         }
         if (move && !same && (ONE || sl == 1u)) {
-          uint64_t* uq = rec + 4u * (u >> 2);
+          uint64_t* uq = rec + 4u * IX(u >> 2, rec_words / 4u);
           uq[0] = a_u + du;
           uq[1u + s] = w_u + to;
         }
@@ -1126,13 +1167,13 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       } else if (PLN) {
         if (run && lead) {
           if (MODEL == 0) {
-            hp[s * ps + v] = static_cast<uint16_t>(nc);
+            hp[IX(s * ps + v, 3u * ps)] = static_cast<uint16_t>(nc);
           } else {
-            if (dD) hp[v] = static_cast<uint16_t>(D + dD);
-            if (dN) hp[ps + v] = static_cast<uint16_t>(N + dN);
-            if (dR) hp[2u * ps + v] = static_cast<uint16_t>(R + dR);
+            if (dD) hp[IX(v, 3u * ps)] = static_cast<uint16_t>(D + dD);
+            if (dN) hp[IX(ps + v, 3u * ps)] = static_cast<uint16_t>(N + dN);
+            if (dR) hp[IX(2u * ps + v, 3u * ps)] = static_cast<uint16_t>(R + dR);
           }
-          if (hop) hp[s * ps + u] = static_cast<uint16_t>(cu);
+          if (hop) hp[IX(s * ps + u, 3u * ps)] = static_cast<uint16_t>(cu);
         }
         const uint32_t lim_s = s == 2u ? lim_r : lim_dn;
         bool over = hop && cu >= lim_s;
@@ -1145,22 +1186,24 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
                                         : pack_voxel(D + dD, N + dN, R + dR, mask);
         const uint64_t wu2 = w_u + one;
         if (run && (ONE || sl == 0u)) {
-          reinterpret_cast<ulonglong2*>(rec)[v] = make_ulonglong2(a_v + dv, wv2);
+          reinterpret_cast<ulonglong2*>(rec)[IX(v, rec_words / 2u)] =
+              make_ulonglong2(a_v + dv, wv2);
         }
         if (move && (ONE || sl == 1u)) {
-          reinterpret_cast<ulonglong2*>(rec)[u] = make_ulonglong2(a_u + du, wu2);
+          reinterpret_cast<ulonglong2*>(rec)[IX(u, rec_words / 2u)] =
+              make_ulonglong2(a_u + du, wu2);
         }
         if (run && (((wv2 | (hop ? wu2 : 0ull)) & over_mask) != 0ull)) err |= kErrNarrow;
       } else {
         if (run && lead) {
           if (MODEL == 0) {
-            cp[s * ps + v] = static_cast<int32_t>(nc);
+            cp[IX(s * ps + v, 3u * ps)] = static_cast<int32_t>(nc);
           } else {
-            if (dD) cp[v] = static_cast<int32_t>(D + dD);
-            if (dN) cp[ps + v] = static_cast<int32_t>(N + dN);
-            if (dR) cp[2u * ps + v] = static_cast<int32_t>(R + dR);
+            if (dD) cp[IX(v, 3u * ps)] = static_cast<int32_t>(D + dD);
+            if (dN) cp[IX(ps + v, 3u * ps)] = static_cast<int32_t>(N + dN);
+            if (dR) cp[IX(2u * ps + v, 3u * ps)] = static_cast<int32_t>(R + dR);
           }
-          if (hop) cp[s * ps + u] = static_cast<int32_t>(cu);
+          if (hop) cp[IX(s * ps + u, 3u * ps)] = static_cast<int32_t>(cu);
         }
       }
       if (!ONE) __syncwarp();
@@ -1179,16 +1222,26 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         }
       }
       if (slow) {  // cells past those limits: checked exactly
-        if (run && big && past_limits<MODEL>(tv, cp, ps, lut, v, u, centre)) {
+        if (run && big &&
+            past_limits<MODEL>(tv, cp, ps, lut, IX(v, lut_n), IX(u, lut_n), centre)) {
           err |= kErrOverflow;
           run = false;
         }
         if (!ONE) __syncwarp();
       }
+      if (kChecked) {  // an index of the event out of range, on any of the cell's lanes
+        const unsigned bad = __ballot_sync(kFull, oob && ran) >> base_lane;
+        if (bad & (G == 32 ? kFull : (1u << (G & 31)) - 1u)) {
+          err |= kErrBounds;
+          run = false;
+        }
+        oob = false;
+      }
     }
     if (!REC && __any_sync(kFull, paused)) {
       const uint32_t last = ONE ? log : __shfl_sync(kFull, log, base_lane + static_cast<int>(m ? m - 1u : 0u));
-      if (paused && past_limits<MODEL>(tv, cp, ps, lut, last & 1023u, (last >> 10) & 1023u, centre)) {
+      if (paused && past_limits<MODEL>(tv, cp, ps, lut, IX(last & 1023u, lut_n),
+                                       IX((last >> 10) & 1023u, lut_n), centre)) {
         err |= kErrOverflow;
         paused = false;
       }
@@ -1260,10 +1313,11 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           for (uint32_t i = lane; i < V; i += 32u) {
             uint32_t D, N, R;
             if (LEAF == kLeafRecords) {
-              const uint64_t w = words[2u * i + 1u];
+              const uint64_t w = words[IX(2u * i + 1u, rec_words)];
               D = word_D(w), N = word_N(w), R = word_R(w);
             } else {
-              const uint64_t* x = SEC ? words + 4u * (i >> 2) + 1u : words + (i >> 2);
+              const uint64_t* x = SEC ? words + 4u * IX(i >> 2, rec_words / 4u) + 1u
+                                      : words + IX(i >> 2, nq);
               const uint32_t dist = SEC ? 1u : nq, k = i & 3u;
               D = field16(x[0], k), N = field16(x[dist], k), R = field16(x[2u * dist], k);
             }
@@ -1295,17 +1349,18 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
         }
         const uint32_t su = code - kEvHop;  // hops: the species taken back from u
         if (SEC) {
-          uint64_t* w = rec + 4u * (v >> 2) + 1u;
+          uint64_t* w = rec + 4u * IX(v >> 2, rec_words / 4u) + 1u;
           const uint32_t sh = 16u * (v & 3u);
           if (cD) add64(w, static_cast<uint64_t>(static_cast<int64_t>(cD)) << sh);
           if (cN) add64(w + 1, static_cast<uint64_t>(static_cast<int64_t>(cN)) << sh);
           if (cR) add64(w + 2, static_cast<uint64_t>(static_cast<int64_t>(cR)) << sh);
-          if (code >= kEvHop) add64(rec + 4u * (u >> 2) + 1u + su, 0ull - (1ull << (16u * (u & 3u))));
+          if (code >= kEvHop)
+            add64(rec + IX(4u * (u >> 2) + 1u + su, rec_words), 0ull - (1ull << (16u * (u & 3u))));
         } else if (PLN) {
           // whole 32-bit words: the sum of all changes is in range, so carries
           // between the halves cancel
           auto add16 = [&](uint32_t at, int c) {
-            atomicAdd(reinterpret_cast<uint32_t*>(hp) + (at >> 1),
+            atomicAdd(reinterpret_cast<uint32_t*>(hp) + IX(at >> 1, 3u * ps / 2u),
                       static_cast<uint32_t>(c) << (16u * (at & 1u)));
           };
           if (cD) add16(v, cD);
@@ -1313,23 +1368,26 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           if (cR) add16(2u * ps + v, cR);
           if (code >= kEvHop) add16(su * ps + u, -1);
         } else if (REC) {
-          add64(rec + 2u * v + 1u, word_unit(0) * static_cast<uint64_t>(static_cast<int64_t>(cD)) +
-                                       word_unit(1) * static_cast<uint64_t>(static_cast<int64_t>(cN)) +
-                                       word_unit(2) * static_cast<uint64_t>(static_cast<int64_t>(cR)));
-          if (code >= kEvHop) add64(rec + 2u * u + 1u, 0ull - word_unit(su));
+          add64(rec + IX(2u * v + 1u, rec_words),
+                word_unit(0) * static_cast<uint64_t>(static_cast<int64_t>(cD)) +
+                    word_unit(1) * static_cast<uint64_t>(static_cast<int64_t>(cN)) +
+                    word_unit(2) * static_cast<uint64_t>(static_cast<int64_t>(cR)));
+          if (code >= kEvHop) add64(rec + IX(2u * u + 1u, rec_words), 0ull - word_unit(su));
         } else {
-          if (cD) atomicAdd(cp + v, cD);
-          if (cN) atomicAdd(cp + ps + v, cN);
-          if (cR) atomicAdd(cp + 2u * ps + v, cR);
-          if (code >= kEvHop) atomicAdd(cp + su * ps + u, -1);
+          if (cD) atomicAdd(cp + IX(v, 3u * ps), cD);
+          if (cN) atomicAdd(cp + IX(ps + v, 3u * ps), cN);
+          if (cR) atomicAdd(cp + IX(2u * ps + v, 3u * ps), cR);
+          if (code >= kEvHop) atomicAdd(cp + IX(su * ps + u, 3u * ps), -1);
         }
       }
       __syncwarp();
       if (REC && fin && lead && (err & kErrNarrow)) {
         // left as it was, for the 32-bit pass
-        p.redo[atomicAdd(p.redo_n, 1u)] = make_uint2(HELP ? home[5] : vidx, HELP ? home[1] : cell);
+        p.redo[IX(atomicAdd(p.redo_n, 1u), p.n_items)] =
+            make_uint2(HELP ? home[5] : vidx, HELP ? home[1] : cell);
       } else if (fin && lead) {
-        const uint32_t c = HELP ? home[1] : cell;
+        const uint32_t cells = kChecked ? tv->width * tv->height : 0u;
+        const uint32_t c = IX(HELP ? home[1] : cell, cells);
         tv->ev_last[c] = e;
         tv->t_last[c] = tnow;
         tv->ev_total[c] += e;
@@ -1348,16 +1406,17 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words;
           if (vec) {
             for (uint32_t i = lane; i < nq; i += 32u) {
-              const U64x4 x = load4(from + 4u * i);
-              reinterpret_cast<uint4*>(g)[i] = unpack4(x.b);
-              reinterpret_cast<uint4*>(g + V)[i] = unpack4(x.c);
-              reinterpret_cast<uint4*>(g + 2u * V)[i] = unpack4(x.d);
+              const U64x4 x = load4(from + 4u * IX(i, rec_words / 4u));
+              reinterpret_cast<uint4*>(g)[IX(i, V / 4u)] = unpack4(x.b);
+              reinterpret_cast<uint4*>(g + V)[IX(i, V / 4u)] = unpack4(x.c);
+              reinterpret_cast<uint4*>(g + 2u * V)[IX(i, V / 4u)] = unpack4(x.d);
             }
           } else {
             for (uint32_t i = lane; i < V; i += 32u)
               for (uint32_t sp = 0; sp < 3u; ++sp)
-                g[sp * V + i] =
-                    static_cast<int32_t>(field16(from[4u * (i >> 2) + 1u + sp], i & 3u));
+                g[IX(sp * V + i, 3u * V)] =
+                    static_cast<int32_t>(field16(from[IX(4u * (i >> 2) + 1u + sp, rec_words)],
+                                                 i & 3u));
           }
         } else if (PLN) {
           const uint64_t* from =
@@ -1365,31 +1424,34 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           for (uint32_t sp = 0; sp < 3u; ++sp) {
             if (vec) {
               for (uint32_t i = lane; i < nq; i += 32u)
-                reinterpret_cast<uint4*>(g + sp * V)[i] = unpack4(from[sp * nq + i]);
+                reinterpret_cast<uint4*>(g + sp * V)[IX(i, V / 4u)] =
+                    unpack4(from[IX(sp * nq + i, 3u * nq)]);
             } else {
               for (uint32_t i = lane; i < V; i += 32u)
-                g[sp * V + i] = static_cast<int32_t>(field16(from[sp * nq + (i >> 2)], i & 3u));
+                g[IX(sp * V + i, 3u * V)] =
+                    static_cast<int32_t>(field16(from[IX(sp * nq + (i >> 2), 3u * nq)], i & 3u));
             }
           }
         } else if (REC) {
           const uint64_t* from = warp_rec + static_cast<size_t>(sc) * rec_words;
           if (vec) {
             for (uint32_t i = lane; i < nq; i += 32u) {
-              const U64x4 x = load4(from + 8u * i), y = load4(from + 8u * i + 4u);
+              const uint64_t* at = from + 8u * IX(i, rec_words / 8u);
+              const U64x4 x = load4(at), y = load4(at + 4u);
               const U64x4 w{x.b, x.d, y.b, y.d};
-              reinterpret_cast<uint4*>(g)[i] =
+              reinterpret_cast<uint4*>(g)[IX(i, V / 4u)] =
                   make_uint4(word_D(w.a), word_D(w.b), word_D(w.c), word_D(w.d));
-              reinterpret_cast<uint4*>(g + V)[i] =
+              reinterpret_cast<uint4*>(g + V)[IX(i, V / 4u)] =
                   make_uint4(word_N(w.a), word_N(w.b), word_N(w.c), word_N(w.d));
-              reinterpret_cast<uint4*>(g + 2u * V)[i] =
+              reinterpret_cast<uint4*>(g + 2u * V)[IX(i, V / 4u)] =
                   make_uint4(word_R(w.a), word_R(w.b), word_R(w.c), word_R(w.d));
             }
           } else {
             for (uint32_t i = lane; i < V; i += 32u) {
-              const uint64_t w = from[2u * i + 1u];
-              g[i] = static_cast<int32_t>(word_D(w));
-              g[V + i] = static_cast<int32_t>(word_N(w));
-              g[2u * V + i] = static_cast<int32_t>(word_R(w));
+              const uint64_t w = from[IX(2u * i + 1u, rec_words)];
+              g[IX(i, 3u * V)] = static_cast<int32_t>(word_D(w));
+              g[IX(V + i, 3u * V)] = static_cast<int32_t>(word_N(w));
+              g[IX(2u * V + i, 3u * V)] = static_cast<int32_t>(word_R(w));
             }
           }
         } else {
@@ -1398,13 +1460,18 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
           for (uint32_t sp = 0; sp < 3u; ++sp) {
             if (vec) {
               for (uint32_t i = lane; i < nq; i += 32u)
-                reinterpret_cast<int4*>(g + sp * V)[i] =
-                    reinterpret_cast<const int4*>(from + sp * ps)[i];
+                reinterpret_cast<int4*>(g + sp * V)[IX(i, V / 4u)] =
+                    reinterpret_cast<const int4*>(from + sp * ps)[IX(i, nq)];
             } else {
-              for (uint32_t i = lane; i < V; i += 32u) g[sp * V + i] = from[sp * ps + i];
+              for (uint32_t i = lane; i < V; i += 32u)
+                g[IX(sp * V + i, 3u * V)] = from[IX(sp * ps + i, 3u * ps)];
             }
           }
         }
+      }
+      if (kChecked && oob) {
+        atomicOr(tv->err, kErrBounds);
+        oob = false;
       }
       __syncwarp();
       if (fin) {
@@ -1415,6 +1482,8 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     }
   }
 }
+
+#undef IX
 
 // The instantiations the launch plan picks from.
 template <int MODEL>

@@ -45,6 +45,7 @@ struct LaneArgs {
   uint32_t n_items, step_off;
   uint32_t V, n;       // of every listed cell
   uint32_t lut_bytes, cell_stride;
+  uint64_t scratch_words;  // of `scratch` (read by the checked build)
 };
 
 struct LanePlan {

@@ -162,7 +162,8 @@ cudaError_t launch_chi_lane(const LanePlan& pl, int model, const TissueView* d_v
                             bool early) {
   const ChiLaneKernel k = lane_kernel(model, V, pl.leaf, pl.G, pl.helper);
   const LaneArgs a{d_views, d_items, d_counter, d_scratch, redo.items, redo.counters + 1, dt,
-                   n_items, step_off, V, n, pl.lut_bytes, pl.cell_stride};
+                   n_items, step_off, V, n, pl.lut_bytes, pl.cell_stride,
+                   pl.scratch_bytes / sizeof(uint64_t)};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(pl.blocks);
   cfg.blockDim = dim3(pl.threads);

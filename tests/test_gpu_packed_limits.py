@@ -8,6 +8,7 @@ import pytest
 
 import oracle as O
 from paper_1806_10889_gb300 import workloads as W
+from paper_1806_10889_gb300.batching import Batch
 from paper_1806_10889_gb300.workloads import TissueSpec
 from tests._util import orc_desc, orc_model
 
@@ -102,3 +103,36 @@ def test_a_total_past_its_limit_is_reported(per_sm, n):
         g.read_counts()
     assert e.value.code == T.E_OVERFLOW
     g.close()
+
+
+def test_packed_classes_of_a_batch_share_the_redo_list():
+    """Three classes with packed counts (sectors, planes, records) in one batch, some
+    cells of each past their range from the start and within the step."""
+    specs = [_tissue(112, 17), _tissue(45, 16), TissueSpec(140, SMS, 8, seed=97, tissue_id=1),
+             TissueSpec(3, 2, 16, seed=97, tissue_id=2)]
+    dt = 0.004
+    states = []
+    for s in specs:
+        x = O.init_counts(orc_desc(s)).reshape(s.cells, 3, s.V)
+        x[0, 0, 0] = 70000
+        x[1, 2, 1] = 5000
+        x[2, 1, :2] = 65533
+        x[3, 2, :3] = 4094
+        x[4, 0, 0] = 200000
+        states.append(np.ascontiguousarray(x.ravel()))
+    members = [Tissue(s) for s in specs]
+    for g, x in zip(members, states):
+        g.write_counts(x, 0)
+    b = Batch(members)
+    assert [b.chi_info(i)["launches"] for i in range(3)] == [2, 2, 2]
+    for k in range(2):
+        b.step(dt, 1)
+        b.sync()
+        for g, s, x in zip(members, specs, states):
+            ne, tl = O.step(orc_desc(s), orc_model(s), x, k, 1, dt)
+            assert np.array_equal(g.read_counts(), x), (s, k)
+            gne, gtl = g.read_stats()
+            assert np.array_equal(gne, ne) and np.array_equal(gtl.view(np.uint64), tl.view(np.uint64))
+    b.close()
+    for g in members:
+        g.close()
