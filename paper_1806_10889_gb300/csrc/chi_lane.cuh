@@ -526,6 +526,7 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
   for (;;) {
     // ---- slots without a cell take the next work items, one after another --
     unsigned want = __ballot_sync(kFull, !have && !done && lead);
+    const bool loads = want != 0u;  // uniform
     while (want) {
       const int src = __ffs(want) - 1;
       want &= want - 1u;
@@ -770,15 +771,18 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
     uint64_t Aj = 0;        // the total propensity before this lane's event
     uint32_t log = 0;       // this lane's event: v, u, code
     uint64_t Rn = HELP ? bits[0] : ONE ? Rb : __shfl_sync(kFull, Rb, base_lane);  // the next event's random bits
-    // A whole warp on a cell: near the end of the step no more events than are
-    // likely left (A (dt - t) are expected), so that a short step does not undo
-    // most of 32 (2x2 cells, dt 1e-9: 34 us -> 22 us a step).
+    // No more events than are likely left in the step (A (dt - t) are expected), so
+    // that a short one does not undo most of its batch.  A whole warp on a cell asks
+    // before every batch (2x2 cells of 8x8 voxels, dt 1e-9: 34 -> 22 us a step), 8 and
+    // 16 lanes on small cells, which have the fewest events, after a load (40x40 of
+    // 4x4, dt 1e-5: 34 -> 27 us; larger cells: 2% slower with the promoter model).
     uint32_t batch = G;
-    if (G == 32) {
+    if (G == 32 || (LV == 3 && WIDE && loads)) {
       const float left = __double2float_rn(p.dt - tnow) * (__ull2float_rn(A) * 0x1p-32f);
       const uint32_t few =
           left < 32.0f ? static_cast<uint32_t>(left + 3.0f * sqrtf(left)) + 3u : 32u;
-      batch = min(32u, __reduce_max_sync(kFull, few));  // uniform, for the compiler too
+      // uniform, for the compiler too
+      batch = min(static_cast<uint32_t>(G), __reduce_max_sync(kFull, have || G == 32 ? few : 0u));
     }
     for (uint32_t i = 0; i < batch; ++i) {
       [[maybe_unused]] const bool ran = run;
