@@ -158,6 +158,18 @@ constexpr int kMaxDevices = 128;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
 
+// While one lives, this thread's pool calls are allowed beside a stream capture of
+// the program's: a capture in the global mode forbids them on every stream and
+// in every thread, and one that is made all the same invalidates it.  The calls
+// are on a stream that is not being captured, and wait for none that is.
+struct BesideCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  BesideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~BesideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  BesideCapture(const BesideCapture&) = delete;
+  BesideCapture& operator=(const BesideCapture&) = delete;
+};
+
 bool lane_pool(bool create, cudaMemPool_t* out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
@@ -253,6 +265,7 @@ struct LaneCall {
   // Its scratch, on the tissue's stream.
   void take_scratch() {
     if (plan.G == 0 || plan.scratch_bytes == 0) return;
+    const BesideCapture beside;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaMemPool_t pool = nullptr;
     void* p = nullptr;
@@ -268,7 +281,9 @@ struct LaneCall {
   // a small tissue's launches may each start before the last has ended
   bool early() const { return plan.G != 0 && plan.small; }
   ~LaneCall() {
-    if (scratch) cudaFreeAsync(scratch, stream);
+    if (!scratch) return;
+    const BesideCapture beside;
+    cudaFreeAsync(scratch, stream);
   }
   LaneCall(const LaneCall&) = delete;
   LaneCall& operator=(const LaneCall&) = delete;
