@@ -39,7 +39,7 @@
 // dependent read and write a lane reaches 25 G/s in DRAM, an event makes two).
 // Chi ms per step, segmented -> this kernel: 2x2 cells of 8x8 voxels 2.9 ->
 // 1.10, 64x64 of 16x16 21.1 -> 9.1, 48x48 of 32x32 77.5 -> 31.0, 256x256 of 8x8
-// 33.4 -> 7.9, 256x256 of 32x32 611 -> 122.
+// 33.4 -> 7.9, 256x256 of 32x32 611 -> 130.
 //
 // Template parameters: MODEL 0 Notch-Delta without in-voxel binding (k_in =
 // k_off = 0), 1 Notch-Delta, 2 promoter; LV the levels of the tree (V <= 4^LV,
@@ -52,10 +52,10 @@
 // 64-byte block; or sectors, 32 bytes a quad with its sum and 16-bit counts,
 // the four quads under a shared sum one 128-byte line that an event reads
 // whole, the four totals of the chosen quad recomputed, the sum and the changed
-// count of one or two quads written (256x256 cells of 32x32 voxels: 174 ms with
-// records and a level of quad sums beside them, 490 DRAM bytes an event; 122 ms
-// and 147 bytes with sectors; 132 ms with 32 bits a voxel and the sums of all
-// four quads recomputed, 260 instructions more); G lanes per cell; HELP blocks
+// count of one or two quads written (256x256 cells of 32x32 voxels, one state:
+// 186 ms with records and 490 DRAM bytes an event, 136 when sectors took their
+// place; later 122 and 147 bytes, against 132 with 32 bits a voxel and the sums of
+// all four quads recomputed, 260 instructions more); G lanes per cell; HELP blocks
 // an SM with a helper warp, 0: none.
 //
 // Planes against records: 48x48 cells of 32x32 voxels 44.2 -> 31.0 ms, 76x76 of
@@ -349,8 +349,8 @@ __device__ __forceinline__ uint32_t pick_lane(uint64_t x, uint64_t& r, int base)
 }
 
 // Registers: shared leaves 168 (12 warps an SM; beyond, more lanes' worth of cells
-// take records); one lane per cell of more than 256 voxels up to 255 (shared
-// memory holds 8 warps an SM anyway); with a helper of HELP blocks an SM 168 (six,
+// take records); one lane per cell of more than 256 voxels as many as it wants, 130
+// to 151 (shared memory holds 8 warps an SM anyway); with a helper of HELP blocks an SM 168 (six,
 // 12 warps) or 128 (eight); else 128, so that 14 to 16 warps fit an SM.
 template <int MODEL, int LV, int LEAF, int G, int HELP>
 __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                  ? HELP
