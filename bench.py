@@ -102,11 +102,11 @@ CHI_IPE = {
 TREE_SOURCES = ["chi_lane.cuh", "chi_lane.h", "pair_end.h", "tissue_dev.cuh", "k_chi_lane.cu",
                 "k_chi_lane_bind.cu", "k_chi_lane_pm.cu"]
 TREE_IPE = {
-    "sources": "4663ee504c114490",
+    "sources": "574fa24508b224a7",
     "kernels": {
-        "batch:V1024": (42.3, 146.7),
-        "batch:V256": (40.0, 78.6),
-        "batch:V64": (34.0, 23.0),
+        "batch:V1024": (42.5, 146.6),
+        "batch:V256": (40.1, 78.7),
+        "batch:V64": (34.1, 23.0),
         "medium:V256": (98.9, 0.306),
         "large:V1024": (42.6, 147.4),
     },

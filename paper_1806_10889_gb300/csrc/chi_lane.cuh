@@ -535,66 +535,65 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       if (kChecked && (ntv->V != V || w.y >= ntv->width * ntv->height)) {
         atomicOr(ntv->err, kErrBounds);
       } else {
-      q.load(ntv->q);
-      const int32_t* g = ntv->counts + static_cast<size_t>(w.y) * 3u * V;
-      ulonglong2* rt = reinterpret_cast<ulonglong2*>(cs);
-      rt[0] = make_ulonglong2(q.gD, q.hD);
-      rt[1] = make_ulonglong2(q.gN, q.hN);
-      rt[2] = make_ulonglong2(q.gR + (MODEL == 1 ? q.k_off : 0ull), q.hR);
-      bool bad_state = false;
-      Limits top{0, 0, 0};
-      uint64_t four = 0;
-      A = 0;
+        q.load(ntv->q);
+        const int32_t* g = ntv->counts + static_cast<size_t>(w.y) * 3u * V;
+        ulonglong2* rt = reinterpret_cast<ulonglong2*>(cs);
+        rt[0] = make_ulonglong2(q.gD, q.hD);
+        rt[1] = make_ulonglong2(q.gN, q.hN);
+        rt[2] = make_ulonglong2(q.gR + (MODEL == 1 ? q.k_off : 0ull), q.hR);
+        bool bad_state = false;
+        Limits top{0, 0, 0};
+        uint64_t four = 0;
+        A = 0;
 #pragma unroll 1
-      for (uint32_t qi = 0; qi < NQ; ++qi) {
-        uint64_t S = 0;
-        if (qi < nq) {
-          uint32_t d[4] = {0, 0, 0, 0}, m[4] = {0, 0, 0, 0}, r[4] = {0, 0, 0, 0};
-          if (vec) {
-            const uint4 x = reinterpret_cast<const uint4*>(g)[IX(qi, V / 4u)];
-            const uint4 y = reinterpret_cast<const uint4*>(g + V)[IX(qi, V / 4u)];
-            const uint4 z = reinterpret_cast<const uint4*>(g + 2u * V)[IX(qi, V / 4u)];
-            d[0] = x.x, d[1] = x.y, d[2] = x.z, d[3] = x.w;
-            m[0] = y.x, m[1] = y.y, m[2] = y.z, m[3] = y.w;
-            r[0] = z.x, r[1] = z.y, r[2] = z.z, r[3] = z.w;
-          } else {
+        for (uint32_t qi = 0; qi < NQ; ++qi) {
+          uint64_t S = 0;
+          if (qi < nq) {
+            uint32_t d[4] = {0, 0, 0, 0}, m[4] = {0, 0, 0, 0}, r[4] = {0, 0, 0, 0};
+            if (vec) {
+              const uint4 x = reinterpret_cast<const uint4*>(g)[IX(qi, V / 4u)];
+              const uint4 y = reinterpret_cast<const uint4*>(g + V)[IX(qi, V / 4u)];
+              const uint4 z = reinterpret_cast<const uint4*>(g + 2u * V)[IX(qi, V / 4u)];
+              d[0] = x.x, d[1] = x.y, d[2] = x.z, d[3] = x.w;
+              m[0] = y.x, m[1] = y.y, m[2] = y.z, m[3] = y.w;
+              r[0] = z.x, r[1] = z.y, r[2] = z.z, r[3] = z.w;
+            } else {
 #pragma unroll
-            for (uint32_t i = 0; i < 4u; ++i)
-              if (4u * qi + i < V) {
-                d[i] = static_cast<uint32_t>(g[IX(4u * qi + i, 3u * V)]);
-                m[i] = static_cast<uint32_t>(g[IX(V + 4u * qi + i, 3u * V)]);
-                r[i] = static_cast<uint32_t>(g[IX(2u * V + 4u * qi + i, 3u * V)]);
-              }
-          }
-          ulonglong2* o = reinterpret_cast<ulonglong2*>(rec) + 4u * IX(qi, rec_words / 8u);
-#pragma unroll
-          for (uint32_t i = 0; i < 4u; ++i) {
-            const uint32_t v = 4u * qi + i;
-            uint64_t a = 0, wd = 0;
-            if (v < V) {
-              const uint32_t mk = lut[IX(v, lut_n)];
-              const bool ctr = MODEL == 2 && v == centre;
-              bad_state = bad_state || (MODEL == 2 && r[i] > static_cast<uint32_t>(ctr));
-              top = Limits{max(top.D, d[i]), max(top.N, m[i]), max(top.R, r[i])};
-              wd = pack_voxel(d[i], m[i], r[i] & 0xFFFFFu, mk & 15u);
-              a = lane_total<MODEL>(q, ntv, d[i], m[i], r[i], mk >> 4, ctr);
+              for (uint32_t i = 0; i < 4u; ++i)
+                if (4u * qi + i < V) {
+                  d[i] = static_cast<uint32_t>(g[IX(4u * qi + i, 3u * V)]);
+                  m[i] = static_cast<uint32_t>(g[IX(V + 4u * qi + i, 3u * V)]);
+                  r[i] = static_cast<uint32_t>(g[IX(2u * V + 4u * qi + i, 3u * V)]);
+                }
             }
-            o[i] = make_ulonglong2(a, wd);
-            S += a;
+            ulonglong2* o = reinterpret_cast<ulonglong2*>(rec) + 4u * IX(qi, rec_words / 8u);
+#pragma unroll
+            for (uint32_t i = 0; i < 4u; ++i) {
+              const uint32_t v = 4u * qi + i;
+              uint64_t a = 0, wd = 0;
+              if (v < V) {
+                const uint32_t mk = lut[IX(v, lut_n)];
+                const bool ctr = MODEL == 2 && v == centre;
+                bad_state = bad_state || (MODEL == 2 && r[i] > static_cast<uint32_t>(ctr));
+                top = Limits{max(top.D, d[i]), max(top.N, m[i]), max(top.R, r[i])};
+                wd = pack_voxel(d[i], m[i], r[i] & 0xFFFFFu, mk & 15u);
+                a = lane_total<MODEL>(q, ntv, d[i], m[i], r[i], mk >> 4, ctr);
+              }
+              o[i] = make_ulonglong2(a, wd);
+              S += a;
+            }
+          }
+          tree[IX(level_off(2) + qi, tree_n)] = S;
+          four += S;
+          if ((qi & 3u) == 3u) {
+            tree[IX(qi >> 2, tree_n)] = four;
+            A += four;
+            four = 0;
           }
         }
-        tree[IX(level_off(2) + qi, tree_n)] = S;
-        four += S;
-        if ((qi & 3u) == 3u) {
-          tree[IX(qi >> 2, tree_n)] = four;
-          A += four;
-          four = 0;
-        }
-      }
         Limits nlim{1, 1, 1};
-        err = bad_state                                      ? kErrState
-              : !pick_limits<MODEL, LEAF>(ntv, top, nlim) ? kErrNarrow
-                                                             : 0;
+        const bool past = !pick_limits<MODEL, LEAF>(ntv, top, nlim);
+        err = bad_state ? kErrState : past ? kErrNarrow : 0;
         set_limits(nlim);
         if (kChecked && oob) err = kErrBounds;
         oob = false;
@@ -1402,8 +1401,9 @@ __global__ void __launch_bounds__(HELP || G == 1 ? 64 : 32, HELP                
       if (REC) {
         // cells that met a limit: other limits, from what they hold now, the whole
         // warp one cell at a time
-        for (unsigned met = __ballot_sync(kFull, fin && lead && (err & kErrNarrow) && m); met;
-             met &= met - 1u) {
+        unsigned met = __ballot_sync(kFull, fin && lead && (err & kErrNarrow) && m);
+        if (met) __syncwarp();  // the counts that other lanes wrote
+        for (; met; met &= met - 1u) {
           const uint32_t sc = static_cast<uint32_t>(__ffs(met) - 1) / G;
           const uint64_t* words =
               PLN ? reinterpret_cast<const uint64_t*>(warp_cells + sc * p.cell_stride + 48) + kCnt
